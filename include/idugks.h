@@ -52,8 +52,8 @@ typedef enum {
     IDG_ERR_OOM = 4,           /* workspace smaller than idg_workspace_size            */
     IDG_ERR_NONFINITE = 5,     /* the residual became NaN or Inf (sticky until the     */
                                /* next idg_init_uniform or idg_set_state)              */
-    IDG_ERR_TIMEOUT = 6,       /* reserved: no kernel of this library waits on another */
-                               /* thread block, so none is returned                    */
+    IDG_ERR_TIMEOUT = 6,       /* a bounded wait between the warps of one thread block */
+                               /* ran out (no kernel waits on another block)           */
     IDG_ERR_NOT_CONVERGED = 7  /* idg_iterate reached max_iter above tol               */
 } idg_status;
 
@@ -313,19 +313,19 @@ idg_status idg_get_wall(idg_ctx *ctx, int side, double *out5, int cap, int *nfac
 idg_status idg_iterate_profiled(idg_ctx *ctx, void *stream, double *kernel_ms);
 
 /* Launch-shape tuning of the wavefront kernels (after idg_bind_workspace;
- * no effect on results).  IDG_TUNE_SWEEP_TV: discrete velocities per thread
- * block of the micro LU-SGS sweeps (power of two, 1..32, times min(ni, nj)
- * at most 512).  IDG_TUNE_SWEEP_STAGES / IDG_TUNE_MACRO_STAGES: hyperplanes
- * prefetched ahead by the micro / macroscopic sweeps (2, 4 or 8; 2 halves the
- * micro sweeps' shared memory, so more velocity tiles are resident at once
- * on a large velocity grid; the macroscopic sweep takes 2 by default for a
- * float64 block with min(ni, nj) above 213, its records filling shared
- * memory).  Returns
- * IDG_ERR_ARG for a value that is invalid or does not fit in shared memory.
- * IDG_TUNE_SWEEP_VPT: consecutive velocities per thread of the micro sweeps
- * (1, 2 or 4; all instances of a batch must agree).  Any velocity count takes
- * all three: the library stores each cell's velocities rounded up to a
- * multiple of 4, the extra ones being ghost velocities of zero weight at
+ * no effect on results).  IDG_TUNE_SWEEP_TV: threads per cell and block of the
+ * micro LU-SGS sweeps (power of two, 1..32, times min(ni, nj) at most 512);
+ * IDG_TUNE_SWEEP_VPT: consecutive velocities per thread (1, 2 or 4; all
+ * instances of a batch must agree).  On a structured block the sweeps take a
+ * shape by size until one of the two is set (the values read back before are
+ * those of a first setting).  IDG_TUNE_SWEEP_STAGES / IDG_TUNE_MACRO_STAGES:
+ * steps prefetched ahead by the micro / macroscopic sweeps (2, 4 or 8, the
+ * micro sweeps at most what shared memory holds; the macroscopic sweep takes
+ * 2 by default for a float64 block with min(ni, nj) above 213, its records
+ * filling shared memory).  Returns IDG_ERR_ARG for a value that is invalid or
+ * whose macroscopic records do not fit in shared memory.  Any velocity count
+ * takes all of these: the library stores each cell's velocities rounded up to
+ * a multiple of 4, the extra ones being ghost velocities of zero weight at
  * xi = 0 that enter no moment and no flux and never reach the caller.
  * IDG_TUNE_GRAPH (1 default, 0 off): idg_iterate replays chunks of 16
  * iterations (and single iterations) as captured CUDA graphs on a

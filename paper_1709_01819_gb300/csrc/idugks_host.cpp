@@ -604,7 +604,8 @@ size_t layout(idg_ctx *c, char *base, KParams *kp)
     k.crT = L.take<char>(8 * ts * N);
     k.clsgT = L.take<char>(8 * ts * N);
     k.cslotT = L.take<char>(8 * ts * N);
-    k.scode = L.take<int>(32 * N);
+    k.scode = c->unstr ? L.take<int>(32 * N) : nullptr;
+    k.sgeo = c->unstr ? nullptr : L.take<char>(16 * ts * N);
     k.sched = c->unstr ? L.take<int>(4 * c->sched.size()) : nullptr;
     k.sptr = c->unstr ? L.take<int>(4 * c->sptr.size()) : nullptr;
     k.fL = L.take<int>(4 * nf);
@@ -838,11 +839,12 @@ idg_status refresh_plan(idg_ctx *c)
     pl.doff = nullptr;
     pl.dactive = nullptr;
     pl.ninst = 1;
+    idg::sweep_shape(c->kp, c->precision == IDG_FP64);
     idg::blocks_per_instance(c->kp, pl.nblocks);
     if (idg::plan_shapes(&c->kp, 1, c->precision == IDG_FP64, pl))
         return fail(c, IDG_ERR_ARG, "launch shape does not fit in shared memory");
+    if (int rc = idg::configure_sweeps(pl, c->precision == IDG_FP64)) return cuda_fail(c, (cudaError_t)rc, "configure sweeps");
     c->kp.macro_stages = pl.macro_stages;
-    c->kp.sweep_stages = pl.sweep_stages;
     pl.explicit_dugks = (c->flags & IDG_NUM_EXPLICIT) ? 1 : 0;
     cudaError_t e;
     if (c->gstream && (e = cudaStreamSynchronize(c->gstream)) != cudaSuccess) return cuda_fail(c, e, "sync");
@@ -1134,29 +1136,17 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
     std::vector<float> uxf(c->ux.begin(), c->ux.end()), uyf(c->uy.begin(), c->uy.end()),
         wf(c->w.begin(), c->w.end());
     std::vector<double> fgeo8((size_t)8 * c->nf, 0.0), cslot((size_t)8 * c->N, 0.0);
-    // micro sweeps: the role of each slot's neighbour in the forward (dir +1)
-    // and backward (dir -1) sweep: its slot in the previous hyperplane (>= 0),
-    // -2 a ghost or not yet swept, -3 the cell itself, -4 - nb the neighbour
-    // nb across a periodic seam
-    std::vector<int> scode((size_t)8 * c->N, -2);
-    for (int dir = 1, o = 0; dir >= -1; dir -= 2, o += 4 * c->N)
-        for (int q = 0; q < c->N; ++q) {
-            const int d = q % c->ni + q / c->ni;
-            for (int m = 0; m < 4; ++m) {
-                const int nb = c->cnb[4 * q + m];
-                int code = -2;
-                if (nb == q) code = -3;
-                else if (nb >= 0 && (dir > 0 ? nb < q : nb > q)) {
-                    if (c->unstr) {
-                        code = -4 - nb;  // scheduled sweeps read every neighbour from global memory
-                    } else {
-                        const int nbi = nb % c->ni, dp = d - dir;
-                        code = nbi + nb / c->ni == dp ? nbi - std::max(0, dp - (c->nj - 1)) : -4 - nb;
-                    }
+    // scheduled micro sweeps: the role of each slot's neighbour in the forward
+    // (dir +1) and backward (dir -1) sweep: -2 a ghost or not yet swept,
+    // -4 - nb the neighbour nb, already swept
+    std::vector<int> scode(c->unstr ? (size_t)8 * c->N : 0, -2);
+    if (c->unstr)
+        for (int dir = 1, o = 0; dir >= -1; dir -= 2, o += 4 * c->N)
+            for (int q = 0; q < c->N; ++q)
+                for (int m = 0; m < 4; ++m) {
+                    const int nb = c->cnb[4 * q + m];
+                    if (nb >= 0 && (dir > 0 ? nb < q : nb > q)) scode[o + 4 * q + m] = -4 - nb;
                 }
-                scode[o + 4 * q + m] = code;
-            }
-        }
     for (int q = 0; q < c->nf; ++q)
         for (int m = 0; m < 7; ++m) fgeo8[(size_t)8 * q + m] = c->fgeo[(size_t)7 * q + m];
     // micro sweeps: per slot the outward normal scaled by the face length
@@ -1167,10 +1157,29 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
             cslot[8 * q + 2 * m] = s * c->fgeo[(size_t)7 * fi] * S;
             cslot[8 * q + 2 * m + 1] = s * c->fgeo[(size_t)7 * fi + 1] * S;
         }
+    // line micro sweeps: per direction and cell the scaled outward normals of
+    // the slots that the marching thread has not met yet (its own line's next
+    // face; the adjacent lines' faces, the already swept side first); a slot
+    // whose neighbour is the cell itself (a periodic direction one cell wide)
+    // contributes nothing
+    std::vector<double> sgeo(c->unstr ? 0 : (size_t)16 * c->N, 0.0);
+    if (!c->unstr) {
+        const bool cols = c->ni <= c->nj;
+        const int tm = cols ? 0 : 2, wm = cols ? 2 : 0;  // slots towards the previous line / along the line
+        for (int q = 0; q < c->N; ++q)
+            for (int dir = 0; dir < 2; ++dir) {
+                const int slot[3] = {dir ? wm : wm + 1, dir ? tm + 1 : tm, dir ? tm : tm + 1};
+                for (int m = 0; m < 3; ++m)
+                    if (c->cnb[4 * q + slot[m]] != q)
+                        for (int x = 0; x < 2; ++x)
+                            sgeo[8 * ((size_t)dir * c->N + q) + 2 * m + x] = cslot[8 * q + 2 * slot[m] + x];
+            }
+    }
     cudaError_t errs[] = {
         up((double *)k.area, c->area), up((double *)k.dtimp, c->dtimp), up((int *)k.cface, c->cface),
         up((int *)k.cnb, c->cnb), up((int *)k.csign, c->csign), up_storage(c, k.crT, c->cr),
-        up_storage(c, k.clsgT, c->clsg), up_storage(c, k.cslotT, cslot), up((int *)k.scode, scode), up((int *)k.fL, c->fL),
+        up_storage(c, k.clsgT, c->clsg), up_storage(c, k.cslotT, cslot),
+        c->unstr ? up((int *)k.scode, scode) : up_storage(c, k.sgeo, sgeo), up((int *)k.fL, c->fL),
         up((int *)k.fR, c->fR), up((double *)k.fgeo, c->fgeo), up_storage(c, k.fgeoT, fgeo8),
         up((int *)k.fbc, c->fbc), up((int *)k.fside, c->fside),
         up((double *)k.ux, c->ux), up((double *)k.uy, c->uy), up((double *)k.w, c->w),
@@ -1479,6 +1488,7 @@ idg_status idg_iterate(idg_ctx *c, int max_iter, double tol, void *stream, int *
         for (int q = 0; q < n; ++q) c->hist.push_back(buf[q]);
         if (status) {
             if (iters_done) *iters_done = done;
+            if (status == IDG_ERR_TIMEOUT) return fail(c, IDG_ERR_TIMEOUT, "a wait inside a sweep kernel ran out");
             return fail(c, IDG_ERR_NONFINITE, "residual became non-finite");
         }
         double r1 = c->hist.front();
@@ -1539,10 +1549,12 @@ idg_status idg_set_tuning(idg_ctx *c, int key, int value)
         if (value < 1 || value > 32 || (value & (value - 1)) || value * k.sweep_pc > 512)
             return fail(c, IDG_ERR_ARG, "sweep velocities per block %d invalid for %d cell slots", value, k.sweep_pc);
         k.sweep_tv = value;
+        k.sweep_tuned = 1;
     } else if (key == IDG_TUNE_SWEEP_VPT) {
         if ((value != 1 && value != 2 && value != 4) || k.Nv % value)
             return fail(c, IDG_ERR_ARG, "velocities per thread %d must be 1, 2 or 4 and divide %d", value, k.Nv);
         k.sweep_vpt = value;
+        k.sweep_tuned = 1;
     } else if (key == IDG_TUNE_SWEEP_STAGES) {
         if (value != 2 && value != 4 && value != 8) return fail(c, IDG_ERR_ARG, "sweep stages must be 2, 4 or 8");
         k.sweep_stages = value;
@@ -1557,12 +1569,12 @@ idg_status idg_set_tuning(idg_ctx *c, int key, int value)
     } else {
         return fail(c, IDG_ERR_ARG, "unknown tuning key %d", key);
     }
+    idg::sweep_shape(k, c->precision == IDG_FP64);
     idg::Plan trial{};
     idg::blocks_per_instance(k, trial.nblocks);
     if (key == IDG_TUNE_MACRO_KIND && !idg::plan_shapes(&k, 1, c->precision == IDG_FP64, trial))
         k.macro_stages = trial.macro_stages;
-    if (idg::plan_shapes(&k, 1, c->precision == IDG_FP64, trial) ||
-        trial.sweep_stages != k.sweep_stages || trial.macro_stages != k.macro_stages)
+    if (idg::plan_shapes(&k, 1, c->precision == IDG_FP64, trial) || trial.macro_stages != k.macro_stages)
         return fail(c, IDG_ERR_ARG, "launch shape does not fit in shared memory");
     KParams old = c->kp;
     c->kp = k;
@@ -1580,7 +1592,7 @@ idg_status idg_get_tuning(const idg_ctx *c, int key, int *value)
     if (key == IDG_TUNE_GRAPH) *value = c->use_graph;
     else if (key == IDG_TUNE_SWEEP_TV) *value = c->kp.sweep_tv;
     else if (key == IDG_TUNE_SWEEP_VPT) *value = c->kp.sweep_vpt;
-    else if (key == IDG_TUNE_SWEEP_STAGES) *value = c->plan.sweep_stages;
+    else if (key == IDG_TUNE_SWEEP_STAGES) *value = c->kp.sweep_stages;
     else if (key == IDG_TUNE_MACRO_STAGES) *value = c->plan.macro_stages;
     else if (key == IDG_TUNE_MACRO_KIND) *value = c->kp.macro_kind;
     else return IDG_ERR_ARG;
@@ -1771,17 +1783,26 @@ idg_status batch_refresh(idg_batch *b)
 {
     const int n = (int)b->ctx.size();
     b->hparams.resize(n);
+    for (int i = 0; i < n; ++i) b->hparams[i] = b->ctx[i]->kp;
+    // one number of velocities per thread for the whole batch: the tuned one,
+    // or, untuned, the one of an instance with many waves of warps
+    std::vector<KParams> hp = b->hparams;
+    int vpt = b->precision == IDG_FP64 ? 1 : 2;
+    for (int i = 0; i < n; ++i)
+        if (hp[i].sweep_tuned) vpt = hp[i].sweep_vpt;
+    for (int i = 0; i < n; ++i) idg::sweep_shape(hp[i], b->precision == IDG_FP64, vpt);
     std::vector<int> off((size_t)idg::KT_COUNT * (n + 1), 0);
     idg::Plan pl{};
     for (int i = 0; i < n; ++i) {
-        b->hparams[i] = b->ctx[i]->kp;
         int nbk[idg::KT_COUNT];
-        idg::blocks_per_instance(b->hparams[i], nbk);
+        idg::blocks_per_instance(hp[i], nbk);
         for (int t = 0; t < idg::KT_COUNT; ++t) off[(size_t)t * (n + 1) + i + 1] = off[(size_t)t * (n + 1) + i] + nbk[t];
     }
     for (int t = 0; t < idg::KT_COUNT; ++t) pl.nblocks[t] = off[(size_t)t * (n + 1) + n];
-    if (idg::plan_shapes(b->hparams.data(), n, b->precision == IDG_FP64, pl))
+    if (idg::plan_shapes(hp.data(), n, b->precision == IDG_FP64, pl))
         return bfail(b, IDG_ERR_ARG, "batch launch shape does not fit in shared memory");
+    if (int rc = idg::configure_sweeps(pl, b->precision == IDG_FP64))
+        return bfail(b, IDG_ERR_CUDA, "configure sweeps: %s", cudaGetErrorString((cudaError_t)rc));
     pl.dparams = b->dparams;
     pl.doff = b->doff;
     pl.dactive = b->dactive;
@@ -1789,7 +1810,7 @@ idg_status batch_refresh(idg_batch *b)
     cudaError_t e;
     if (b->gstream && (e = cudaStreamSynchronize(b->gstream)) != cudaSuccess)
         return bfail(b, IDG_ERR_CUDA, "sync: %s", cudaGetErrorString(e));
-    if ((e = cudaMemcpy(b->dparams, b->hparams.data(), n * sizeof(KParams), cudaMemcpyHostToDevice)) != cudaSuccess ||
+    if ((e = cudaMemcpy(b->dparams, hp.data(), n * sizeof(KParams), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->doff, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(b->dactive, b->active.data(), n * sizeof(int), cudaMemcpyHostToDevice)) != cudaSuccess)
         return bfail(b, IDG_ERR_CUDA, "batch upload: %s", cudaGetErrorString(e));

@@ -33,6 +33,9 @@ struct KParams {
     const void *clsgT;     // [N][8] T: least-squares weight vector per slot
     const void *cslotT;    // [N][4][2] T: sign*nx*S, sign*ny*S per slot (micro sweeps)
     const int *scode;      // [2][N][4] forward, backward: role of each slot's neighbour in that micro sweep
+                           // (scheduled sweeps of an unstructured mesh; null on a structured block)
+    void *sgeo;            // [2][N][8] T forward, backward: what the line sweeps read of a cell (k_sweep_lines);
+                           // entry 6, the cell's diagonal base, is written every iteration (null if unstructured)
     // faces
     const int *fL, *fR;    // [nf]
     const double *fgeo;    // [nf][7] nx, ny, S, rLx, rLy, rRx, rRy
@@ -81,6 +84,11 @@ struct KParams {
     // launch shape of the wavefront kernels: velocities per CTA and cell
     // slots of the micro sweeps, prefetch depths (hyperplanes; 4 or 8)
     int sweep_tv, sweep_pc, sweep_stages, macro_stages;
+    int sweep_tuned; // 1: sweep_tv or sweep_vpt was set by the caller
+    // line micro sweeps (sweep_shape()): threads per cell of a block and
+    // velocities per thread, sweep_g of those threads neighbours in one warp,
+    // entries of a border ring
+    int sweep_ktv, sweep_kvpt, sweep_g, sweep_ring;
     int sweep_vpt;  // consecutive velocities per thread in the micro sweeps (1, 2, 4)
     int macro_kind; // macroscopic LU-SGS on a structured block: 0 hyperplane slots (k_macro_sweep),
                     // 1 one thread per line of cells (k_macro_lines)
@@ -129,8 +137,14 @@ struct Plan {
     size_t sched_smem;   // shared memory of the scheduled macroscopic sweep (0: increments in global memory)
 };
 
+// launch shape of the micro sweeps: KParams::sweep_ktv, sweep_kvpt, sweep_g,
+// sweep_ring, from the tuned tile or, untuned, by size; vpt > 0 fixes the
+// velocities per thread (one value for all instances of a batch)
+void sweep_shape(KParams &p, bool fp64, int vpt = 0);
+
 // kernel launchers (idugks_kernels.cu)
 int configure_kernels(bool fp64);
+int configure_sweeps(const Plan &plan, bool fp64);  // before a plan's first launch
 void blocks_per_instance(const KParams &p, int out[KT_COUNT]);
 int plan_shapes(const KParams *hp, int n, bool fp64, Plan &plan);
 constexpr int kProfiled = 6;  // timed groups in launch_iteration(events)

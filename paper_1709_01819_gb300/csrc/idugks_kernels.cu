@@ -42,9 +42,9 @@
 //                    (k_macro_sweep_sched on an unstructured mesh; with the
 //                    point-relaxation predictor k_record_residual and n
 //                    launches of k_macro_relax in place of the sweep)
-//   k_micro_residual, k_sweep_fwd, k_sweep_bwd: micro LU-SGS sweeps and
-//                    update (hyperplanes on a structured block, level
-//                    schedules on an unstructured mesh)              [a6-a7]
+//   k_micro_residual, then the micro LU-SGS sweeps and update: k_sweep_lines
+//                    (lines of cells of a structured block) or k_sweep (level
+//                    schedules of an unstructured mesh)              [a6-a7]
 // Explicit DUGKS (Eq. 21) runs the cell and face kernels, then
 // k_explicit_update, k_cell_moments, k_explicit_w and k_record_residual.
 // Data are laid out per cell in four face slots (a triangle's fourth slot is
@@ -1881,6 +1881,12 @@ __global__ void __launch_bounds__(32) k_macro_post(Launch L)
     cp[15] = p.area[c] / p.dtimp[c] + cq;
     T *ct = (T *)p.cellpT + kCellP * c;
     for (int q = 0; q < kCellP; ++q) ct[q] = (T)cp[q];
+    if (p.sgeo) {
+        // the diagonal base where both line sweeps read it
+        T *sg = (T *)p.sgeo + 8 * (size_t)c + 6;
+        sg[0] = (T)cp[15];
+        sg[8 * (size_t)p.N] = (T)cp[15];
+    }
 }
 
 // Point relaxation of the predictor equations (the alternative to LU-SGS the
@@ -2025,12 +2031,10 @@ __global__ void __launch_bounds__(32) k_explicit_w(Launch L)
 //   k_sweep_bwd       Delta_c = Delta*_c + sum_{upper inflow nb} |xi.n| S Delta_nb / D_c,
 //                     f~ += Delta (Eq. 32)
 // with D = Omega/dt_imp + sum_{outflow} xi.n S + 2 Omega/(2 tau' + dt).
-// The sweeps run one CTA per tile of sweep_tv velocities over the i+j
-// hyperplanes; thread (slot, t) owns cell (ilo + slot) of each hyperplane at
-// velocity t.  Everything a step reads except the neighbours' increments is
-// prefetched kStages-1 hyperplanes ahead with cp.async; the previous
-// hyperplane's increments sit in a shared-memory ring, and neighbours across
-// a periodic seam (earlier hyperplanes) are read back from global memory.
+// A structured block's sweeps run lines of cells (k_sweep_lines), an
+// unstructured mesh's the steps of its level schedule (k_sweep: one block per
+// tile of sweep_tv velocities, a thread per (cell of the step, velocity),
+// everything but the neighbours' increments copied kStages-1 steps ahead).
 // ---------------------------------------------------------------------------
 template <class T>
 __global__ void __launch_bounds__(128) k_micro_residual(Launch L)
@@ -2092,13 +2096,11 @@ template <> __device__ __forceinline__ void load16<double>(double (&r)[16], cons
     }
 }
 
-// Role of the neighbour across each slot of a cell in one micro sweep
-// (computed on the host): >= 0 its slot in the previous hyperplane's ring;
-// kOther a ghost or a neighbour not yet swept (outflow only adds to D); kSelf
-// the cell itself across a periodic direction one cell wide (no term at all);
-// <= kSeam the neighbour kSeam - code across a periodic seam (already swept,
-// read from global memory).
-constexpr int kOther = -2, kSelf = -3, kSeam = -4;
+// Role of the neighbour across each slot of a cell in one scheduled micro sweep
+// (computed on the host): <= kSeam the neighbour kSeam - code, already swept and
+// read from global memory; otherwise a ghost or a neighbour not yet swept
+// (outflow only adds to D).
+constexpr int kSeam = -4;
 
 // 8 storage scalars from 16-byte-aligned shared memory
 template <class T> __device__ __forceinline__ void load8(T (&r)[8], const T *s);
@@ -2116,14 +2118,13 @@ template <> __device__ __forceinline__ void load8<double>(double (&r)[8], const 
     }
 }
 
-// shared-memory layout of the micro sweeps (VPT consecutive velocities per thread)
+// shared-memory layout of the scheduled micro sweeps (VPT consecutive velocities per thread)
 template <class T, int kStages, int VPT> struct SweepSmem {
     using T2 = typename V2<T>::t;
     T2 *R;      // [kStages][pc][tv*VPT]  R (forward) / Delta* (backward)
     T2 *F;      // [kStages][pc][tv*VPT]  f~ (backward only)
     T *geo;     // [kStages][pc][8]  per slot: sign*nx*S, sign*ny*S
-    int *code;  // [kStages][pc][4]  per slot: the neighbour's role in this sweep (sweep_codes)
-    T2 *ring;   // [2][pc][tv*VPT]  increments of the previous hyperplane, by slot
+    int *code;  // [kStages][pc][4]  per slot: the neighbour's role in this sweep
     T *D0;      // [kStages][pc]
     __device__ SweepSmem(unsigned char *base, int pc, int tv, bool withF)
     {
@@ -2133,7 +2134,6 @@ template <class T, int kStages, int VPT> struct SweepSmem {
         F = (T2 *)(base + o); if (withF) o += (size_t)kStages * pc * w * sizeof(T2);
         geo = (T *)(base + o); o += (size_t)kStages * pc * 8 * sizeof(T);
         code = (int *)(base + o); o += (size_t)kStages * pc * 4 * sizeof(int);
-        ring = (T2 *)(base + o); o += (size_t)2 * pc * w * sizeof(T2);
         D0 = (T *)(base + o);
     }
 };
@@ -2143,49 +2143,38 @@ template <class T, int kStages, int VPT> static size_t sweep_smem_bytes(int pc, 
     using T2 = typename V2<T>::t;
     const size_t w = (size_t)tv * VPT;
     size_t o = (size_t)kStages * pc * w * sizeof(T2) * (withF ? 2 : 1);
-    o += (size_t)kStages * pc * (8 * sizeof(T) + 4 * sizeof(int));
-    o += (size_t)2 * pc * w * sizeof(T2) + (size_t)kStages * pc * sizeof(T);
+    o += (size_t)kStages * pc * (9 * sizeof(T) + 4 * sizeof(int));
     return o;
 }
 
-// the parameters a sweep touches every step, held in registers
+// the parameters a scheduled sweep touches every step, held in registers
 struct SweepArgs {
-    int Nv, ni, nj, tv, pc;
+    int Nv, tv, pc;
     void *dst, *f;
     const void *cslotT, *cellpT;
-    const int *codes;  // this sweep's [N][4] slot codes
-    const int *sched, *sptr;  // this sweep's schedule (unstructured) or null
+    const int *codes;         // this sweep's [N][4] slot codes
+    const int *sched, *sptr;  // this sweep's schedule
     int nsteps;               // steps of the sweep
 };
 
-// the cell of slot `slot` at step d (a hyperplane i + j = d on a structured
-// block, with its (i, j); the d-th step of the schedule otherwise), -1 past
-// the step's end
-template <bool SCHED> __device__ __forceinline__ int sweep_cell(const SweepArgs &p, int d, int slot, int &i, int &j)
+// the cell of slot `slot` at the d-th step of the schedule, -1 past the step's end
+__device__ __forceinline__ int sweep_cell(const SweepArgs &p, int d, int slot)
 {
-    if (SCHED) {
-        const int b = p.sptr[d];
-        i = j = 0;
-        return slot < p.sptr[d + 1] - b ? p.sched[b + slot] : -1;
-    }
-    const int ilo = max(0, d - (p.nj - 1)), ihi = min(p.ni - 1, d);
-    i = ilo + slot;
-    j = d - i;
-    return i <= ihi ? j * p.ni + i : -1;
+    const int b = p.sptr[d];
+    return slot < p.sptr[d + 1] - b ? p.sched[b + slot] : -1;
 }
 
 // asynchronous copy of one step's data for the thread's cell: its VPT
 // consecutive velocities of R (or Delta*, f~), and the cell's slot geometry
 // and diagonal base spread over the cell's tv threads
-template <class T, int kStages, int VPT, bool SCHED>
-__device__ __forceinline__ void sweep_issue(const SweepArgs &p, const SweepSmem<T, kStages, VPT> &sm, int s, int d,
+template <class T, int kStages, int VPT>
+__device__ __forceinline__ void sweep_issue(const SweepArgs &p, const SweepSmem<T, kStages, VPT> &sm, int s,
                                             int slot, int t, int k0, bool act, bool withF)
 {
     using T2 = typename V2<T>::t;
     const int tv = p.tv, pc = p.pc;
     if (s < p.nsteps) {
-        int ci, cj;
-        const int c = sweep_cell<SCHED>(p, d, slot, ci, cj);
+        const int c = sweep_cell(p, s, slot);
         if (c >= 0) {
             int st = s & (kStages - 1);
             size_t e = ((size_t)st * pc + slot);
@@ -2215,21 +2204,17 @@ __device__ __forceinline__ void sweep_issue(const SweepArgs &p, const SweepSmem<
     cp_commit();
 }
 
-template <class T, bool FWD, int kStages, int VPT, bool SCHED = false>
+// unstructured meshes: the sweeps walk the steps of the level schedule
+template <class T, bool FWD, int kStages, int VPT>
 __global__ void __launch_bounds__(512) k_sweep(Launch L)
 {
     IDG_LOCATE();
     using T2 = typename V2<T>::t;
     extern __shared__ __align__(16) unsigned char smraw[];
-    // SCHED (unstructured mesh): the steps of the schedule; otherwise the i+j
-    // hyperplanes, compiled without any schedule state
-    const SweepArgs a{p.Nv, p.ni, p.nj, p.sweep_tv, p.sweep_pc, p.dst, p.f, p.cslotT, p.cellpT,
-                      p.scode + (FWD ? 0 : 4 * (size_t)p.N),
-                      SCHED ? p.sched + (FWD ? 0 : (size_t)p.N) : nullptr,
-                      SCHED ? p.sptr + (FWD ? 0 : p.nsteps_f + 1) : nullptr,
-                      SCHED ? (FWD ? p.nsteps_f : p.nsteps_b) : p.ni + p.nj - 1};
-    const int tv = a.tv, pc = a.pc, ni = a.ni, nj = a.nj, Nv = a.Nv;
-    const bool per_i = p.per_i, per_j = p.per_j;
+    const SweepArgs a{p.Nv, p.sweep_tv, p.sweep_pc, p.dst, p.f, p.cslotT, p.cellpT,
+                      p.scode + (FWD ? 0 : 4 * (size_t)p.N), p.sched + (FWD ? 0 : (size_t)p.N),
+                      p.sptr + (FWD ? 0 : p.nsteps_f + 1), FWD ? p.nsteps_f : p.nsteps_b};
+    const int tv = a.tv, pc = a.pc, Nv = a.Nv;
     const SweepSmem<T, kStages, VPT> sm(smraw, pc, tv, !FWD);
     const int t = threadIdx.x % tv, slot = threadIdx.x / tv;
     const int k0 = (blk * tv + t) * VPT;  // Nv is a multiple of VPT
@@ -2245,15 +2230,12 @@ __global__ void __launch_bounds__(512) k_sweep(Launch L)
     T2 *f = (T2 *)a.f;
     const int nh = a.nsteps;
     const size_t w = (size_t)tv * VPT;
-    // a schedule lists the backward sweep's steps in processing order
-    auto step_d = [&](int s) { return (FWD || SCHED) ? s : nh - 1 - s; };
-    for (int s = 0; s < kStages - 1; ++s) sweep_issue<T, kStages, VPT, SCHED>(a, sm, s, step_d(s), slot, t, k0, act, !FWD);
+    for (int s = 0; s < kStages - 1; ++s) sweep_issue<T, kStages, VPT>(a, sm, s, slot, t, k0, act, !FWD);
     for (int s = 0; s < nh; ++s) {
         cp_wait<kStages - 2>();
         __syncthreads();
-        sweep_issue<T, kStages, VPT, SCHED>(a, sm, s + kStages - 1, step_d(s + kStages - 1), slot, t, k0, act, !FWD);
-        int i, j;
-        const int c = sweep_cell<SCHED>(a, step_d(s), slot, i, j);
+        sweep_issue<T, kStages, VPT>(a, sm, s + kStages - 1, slot, t, k0, act, !FWD);
+        const int c = sweep_cell(a, s, slot);
         if (c < 0 || !act) continue;
         const size_t e = (size_t)(s & (kStages - 1)) * pc + slot;
         T g[8];
@@ -2263,69 +2245,375 @@ __global__ void __launch_bounds__(512) k_sweep(Launch L)
         const T D0 = sm.D0[e];
         const size_t ck = (size_t)c * Nv + k0;
         const size_t rbase = e * w + (size_t)t * VPT;
-        const size_t rprev = (size_t)((s + 1) & 1) * pc * w + (size_t)t * VPT;
-        // the backward sweep's increments are read back from global memory
-        // only across a periodic seam (the first and last cells of a periodic
-        // direction); elsewhere only f and the ring take them
-        const bool keep = FWD || SCHED || (per_i && (i == 0 || i == ni - 1)) || (per_j && (j == 0 || j == nj - 1));
-        // the step of one cell; SEAM: some neighbour lies across a periodic
-        // seam (read from global memory), otherwise every inflow comes from
-        // the ring
-        auto cell_step = [&](auto seam_tag) {
-            constexpr bool SEAM = decltype(seam_tag)::value;
 #pragma unroll
-            for (int v = 0; v < VPT; ++v) {
-                // slot terms, branch-free: outflow adds (xi.n) S to D, inflow
-                // from the already-swept side adds |xi.n| S Delta_nb
-                T D = D0;
-                T aS[4];
-                bool in[4];
+        for (int v = 0; v < VPT; ++v) {
+            // slot terms, branch-free: outflow adds (xi.n) S to D, inflow
+            // from the already-swept side adds |xi.n| S Delta_nb
+            T D = D0;
+            T aS[4];
+            bool in[4];
 #pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    aS[m] = add_rn(mul_rn(ux[v], g[2 * m]), mul_rn(uy[v], g[2 * m + 1]));
-                    D += (aS[m] > (T)0 && code[m] != kSelf) ? aS[m] : (T)0;
-                    in[m] = aS[m] < (T)0 && (code[m] >= 0 || (SEAM && code[m] <= kSeam));
-                }
-                T2 dn[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    dn[m].x = (T)0;
-                    dn[m].y = (T)0;
-                    if (in[m]) {
-                        if (!SEAM || code[m] >= 0) dn[m] = sm.ring[rprev + (size_t)code[m] * w + v];
-                        else dn[m] = ds[(size_t)(kSeam - code[m]) * Nv + k0 + v];
-                    }
-                }
-                T ag = 0, ah = 0;
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    ag -= aS[m] * dn[m].x;
-                    ah -= aS[m] * dn[m].y;
-                }
-                const T2 r = sm.R[rbase + v];
-                const T iD = rcp_rn(D);
-                T2 o;
-                if (FWD) {
-                    o.x = (r.x + ag) * iD;
-                    o.y = (r.y + ah) * iD;
-                } else {
-                    o.x = r.x + ag * iD;
-                    o.y = r.y + ah * iD;
-                    T2 fv = sm.F[rbase + v];
-                    fv.x += o.x;
-                    fv.y += o.y;
-                    f[ck + v] = fv;
-                }
-                if (keep) ds[ck + v] = o;
-                sm.ring[((size_t)(s & 1) * pc + slot) * w + (size_t)t * VPT + v] = o;
+            for (int m = 0; m < 4; ++m) {
+                aS[m] = add_rn(mul_rn(ux[v], g[2 * m]), mul_rn(uy[v], g[2 * m + 1]));
+                D += aS[m] > (T)0 ? aS[m] : (T)0;
+                in[m] = aS[m] < (T)0 && code[m] <= kSeam;
             }
-        };
-        if (code[0] <= kSeam || code[1] <= kSeam || code[2] <= kSeam || code[3] <= kSeam)
-            cell_step(std::true_type{});
-        else
-            cell_step(std::false_type{});
+            T2 dn[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                dn[m].x = (T)0;
+                dn[m].y = (T)0;
+                if (in[m]) dn[m] = ds[(size_t)(kSeam - code[m]) * Nv + k0 + v];
+            }
+            T ag = 0, ah = 0;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                ag -= aS[m] * dn[m].x;
+                ah -= aS[m] * dn[m].y;
+            }
+            const T2 r = sm.R[rbase + v];
+            const T iD = rcp_rn(D);
+            T2 o;
+            if (FWD) {
+                o.x = (r.x + ag) * iD;
+                o.y = (r.y + ah) * iD;
+            } else {
+                o.x = r.x + ag * iD;
+                o.y = r.y + ah * iD;
+                T2 fv = sm.F[rbase + v];
+                fv.x += o.x;
+                fv.y += o.y;
+                f[ck + v] = fv;
+            }
+            ds[ck + v] = o;
+        }
     }
     cp_wait<0>();
+}
+
+// The micro sweeps of a structured block, a warp per bundle of lines: lines run
+// along the longer axis (w), 32 / G neighbouring lines of the shorter axis (t)
+// by G neighbouring groups of VPT velocities make up a warp, and lane (l, g)
+// marches along line l one cell per step, one step behind line l - 1.  The two
+// swept neighbours of a cell are then the thread's own result of the previous
+// step (registers) and lane l - 1's (a shuffle): no barrier and no shared
+// memory inside a bundle.  The bundles (strips) of a block pass their border
+// line on through a shared-memory ring: every kSweepBlock steps a warp
+// publishes how far it is and waits, if need be, for the strip before it (whose
+// border it reads) and for the strip after it (whose unread entries it must not
+// overwrite).  A strip runs kSweepBlock steps behind the one before on top of
+// their distance in lines, so that a block of steps needs only finished blocks.
+// Everything a step reads is copied PF steps ahead into shared memory
+// (cp.async: the copies of a step are awaited by their group, while loads into
+// registers share the warp's few scoreboards and would wait for one another).
+// A cell's record holds only the normals that the march has not met yet: its next own
+// face and the two faces towards the adjacent lines; the own face behind is the
+// previous cell's, with the opposite sign.
+// Seams: a line's first cell stays in registers for its last one; across a seam
+// between the first and the last line the first line's increments are read from
+// global memory, ordered by the same flags (in one warp by a __syncwarp).
+// Bound by the latency of a step (issue a third of the cycles on 64 lines), on
+// large states by the copies.  Measured against one barrier per hyperplane with
+// all neighbours in shared memory, forward + backward, float32: 64 x 64 cells
+// with 1024 velocities 79 + 84 -> 40 + 39 us, 128 x 128 with 784 234 + 326 ->
+// 89 + 94 us, 121 x 81 with 7921 950 + 1436 -> 495 + 682 us; float64 64 x 64
+// 462 + 467 -> 355 + 355 us.  Loads into registers instead of cp.async took
+// 53 + 51 us on 64 x 64, a warp running through the steps before its first and
+// after its last cell 57 + 61 us.
+constexpr int kSweepBlock = 4;
+
+// progress flags between the warps of one block
+__device__ __forceinline__ void flag_store(int *f, int v)
+{
+    asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(smem_addr(f)), "r"(v) : "memory");
+}
+__device__ __forceinline__ int flag_load(const int *f)
+{
+    int v;
+    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_addr(f)) : "memory");
+    return v;
+}
+// waits until *f >= need (seen: what the last poll found).  The warps of a block
+// run at the same time, so the wait ends; should it not (2^22 polls), the status
+// word is raised and the sweep goes on.
+__device__ __forceinline__ void flag_wait(const int *f, int need, int &seen, int *status)
+{
+    for (int n = 0; seen < need; ++n) {
+        seen = flag_load(f);
+        if (n > (1 << 22)) {
+            *status = 6;
+            seen = 0x7fffffff;
+        }
+    }
+}
+
+// 1 / x to within an ulp in float32 (one Newton step on the approximation; x is
+// a positive sum of areas and rates, far from the ends of the range), correctly
+// rounded in float64
+__device__ __forceinline__ float rcp_nr(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+__device__ __forceinline__ double rcp_nr(double x) { return __drcp_rn(x); }
+
+// VPT consecutive T2 / the 8-entry record, by the widest loads
+template <int VPT> __device__ __forceinline__ void ld_vec(float2 (&o)[VPT], const float2 *s)
+{
+    if constexpr (VPT == 1) {
+        o[0] = *s;
+    } else {
+#pragma unroll
+        for (int v = 0; v < VPT; v += 2) {
+            const float4 a = *reinterpret_cast<const float4 *>(s + v);
+            o[v] = make_float2(a.x, a.y);
+            o[v + 1] = make_float2(a.z, a.w);
+        }
+    }
+}
+template <int VPT> __device__ __forceinline__ void ld_vec(double2 (&o)[VPT], const double2 *s)
+{
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) o[v] = s[v];
+}
+// predicated stores to global (GLOBAL) or shared memory, without a branch
+template <bool GLOBAL, int VPT> __device__ __forceinline__ void st_vec(float2 *d, const float2 (&x)[VPT], bool on)
+{
+    if constexpr (VPT == 1) {
+        if constexpr (GLOBAL)
+            asm volatile("{.reg .pred p; setp.ne.s32 p, %3, 0; @p st.global.v2.f32 [%0], {%1, %2};}" ::"l"(d), "f"(x[0].x), "f"(x[0].y), "r"((int)on) : "memory");
+        else
+            asm volatile("{.reg .pred p; setp.ne.s32 p, %3, 0; @p st.shared.v2.f32 [%0], {%1, %2};}" ::"r"(smem_addr(d)), "f"(x[0].x), "f"(x[0].y), "r"((int)on) : "memory");
+    } else {
+#pragma unroll
+        for (int v = 0; v < VPT; v += 2) {
+            if constexpr (GLOBAL)
+                asm volatile("{.reg .pred p; setp.ne.s32 p, %5, 0; @p st.global.v4.f32 [%0], {%1, %2, %3, %4};}" ::"l"(d + v), "f"(x[v].x), "f"(x[v].y), "f"(x[v + 1].x), "f"(x[v + 1].y), "r"((int)on) : "memory");
+            else
+                asm volatile("{.reg .pred p; setp.ne.s32 p, %5, 0; @p st.shared.v4.f32 [%0], {%1, %2, %3, %4};}" ::"r"(smem_addr(d + v)), "f"(x[v].x), "f"(x[v].y), "f"(x[v + 1].x), "f"(x[v + 1].y), "r"((int)on) : "memory");
+        }
+    }
+}
+template <bool GLOBAL, int VPT> __device__ __forceinline__ void st_vec(double2 *d, const double2 (&x)[VPT], bool on)
+{
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+        if constexpr (GLOBAL)
+            asm volatile("{.reg .pred p; setp.ne.s32 p, %3, 0; @p st.global.v2.f64 [%0], {%1, %2};}" ::"l"(d + v), "d"(x[v].x), "d"(x[v].y), "r"((int)on) : "memory");
+        else
+            asm volatile("{.reg .pred p; setp.ne.s32 p, %3, 0; @p st.shared.v2.f64 [%0], {%1, %2};}" ::"r"(smem_addr(d + v)), "d"(x[v].x), "d"(x[v].y), "r"((int)on) : "memory");
+    }
+}
+// 16-byte cp.async where on
+__device__ __forceinline__ void cp_async16_if(void *s, const void *g, bool on)
+{
+    asm volatile("{.reg .pred p; setp.ne.s32 p, %2, 0; @p cp.async.cg.shared.global [%0], [%1], 16;}" ::"r"(smem_addr(s)), "l"(g), "r"((int)on) : "memory");
+}
+__device__ __forceinline__ void ld_rec7(float (&o)[7], const float *s)
+{
+    const float4 a = reinterpret_cast<const float4 *>(s)[0], b = reinterpret_cast<const float4 *>(s)[1];
+    o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z;
+}
+__device__ __forceinline__ void ld_rec7(double (&o)[7], const double *s)
+{
+    const double2 *q = reinterpret_cast<const double2 *>(s);
+    const double2 a = q[0], b = q[1], c = q[2];
+    o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y; o[4] = c.x; o[5] = c.y; o[6] = s[6];
+}
+
+template <class T, bool FWD, int VPT, int PF, bool SEAM>
+__global__ void __launch_bounds__(512) k_sweep_lines(Launch L)
+{
+    IDG_LOCATE();
+    using T2 = typename V2<T>::t;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    int *flags = (int *)smraw;  // [16] steps done by each warp
+    const bool cols = p.ni <= p.nj;
+    const int nt = cols ? p.ni : p.nj, nw = cols ? p.nj : p.ni, Nv = p.Nv;
+    const int G = p.sweep_g, lw = 32 / G, strips = (nt + lw - 1) / lw, subs = p.sweep_ktv / G;
+    const int wid = threadIdx.x >> 5, sub = wid / strips, strip = wid - sub * strips;
+    // step s of the block's clock: the lane of line tt is at its cell
+    // ww = s - tt - strip * kSweepBlock; a warp runs from its first line's first
+    // cell to its last line's last one
+    const int s_beg = (strip * (lw + kSweepBlock)) & ~(kSweepBlock - 1);
+    const int s_end = strip * (lw + kSweepBlock) + nw + lw - 1;
+    if ((threadIdx.x & 31) == 0) flags[wid] = s_beg;
+    __syncthreads();
+    if (sub >= subs) return;  // a smaller instance of a batch
+    const int lane = threadIdx.x & 31, l = lane / G, g = lane - l * G;
+    const int tt = strip * lw + l;  // line in sweep order
+    const int tc = min(tt, nt - 1);
+    const int k0 = ((blk * subs + sub) * G + g) * VPT;
+    const bool line = tt < nt && k0 < Nv, has_adj = tt > 0;
+    const int kk = k0 < Nv ? k0 : 0;
+    T ux[VPT], uy[VPT];
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+        ux[v] = vx<T>(p, kk + v);
+        uy[v] = vy<T>(p, kk + v);
+    }
+    // cell of (tt, ww): c0 + ww * cs, ww counted from the end the sweep starts at
+    const int t = FWD ? tc : nt - 1 - tc;
+    const int cs = (FWD ? 1 : -1) * (cols ? p.ni : 1);
+    const int c0 = (cols ? t : t * p.ni) + (FWD ? 0 : (nw - 1) * (cols ? p.ni : 1));
+    const int sv = cs * Nv, sg = cs * 8;
+    T2 *ds = (T2 *)p.dst + (ptrdiff_t)c0 * Nv + kk;
+    T2 *fs = (T2 *)p.f + (ptrdiff_t)c0 * Nv + kk;
+    const T *geo = (const T *)p.sgeo + (FWD ? 0 : (ptrdiff_t)p.N * 8) + (ptrdiff_t)c0 * 8;
+    const unsigned nwl = line ? nw : 0;
+    const int start = tt + strip * kSweepBlock;
+    const bool seam_t = SEAM && (cols ? p.per_i : p.per_j) && nt > 1;
+    const bool seam_w = SEAM && (cols ? p.per_j : p.per_i) && nw > 1;
+    // shared memory: flags, border rings [warp][ring][G * VPT], stages
+    // [warp][PF] of {R or Delta*, f~ (backward), cell records}
+    const int ring = p.sweep_ring, xs = G * VPT, nwarp = subs * strips;
+    T2 *xw = (T2 *)(smraw + 64) + (size_t)wid * ring * xs + g * VPT;
+    const T2 *xr = strip > 0 ? xw - (size_t)ring * xs : xw;  // the strip before's
+    const bool edge = l == 0 && strip > 0, border = l == lw - 1 && strip + 1 < strips;
+    constexpr int RB = 32 * VPT * sizeof(T2), FB = FWD ? 0 : RB, CB = 8 * sizeof(T);
+    const int SB = RB + FB + lw * CB;
+    unsigned char *stage = smraw + 64 + (size_t)nwarp * ring * xs * sizeof(T2) + (size_t)wid * PF * SB;
+
+    // every lane copies at every step (lanes without a cell their line's end
+    // cells, or an existing line's): no branch in the step
+    auto issue = [&](int s) {
+        const int wc = min(max(s - start, 0), nw - 1);
+        unsigned char *st = stage + (s & (PF - 1)) * SB;
+        constexpr int B = VPT * sizeof(T2), CH = B < 16 ? B : 16;
+        const char *gr = (const char *)(ds + (ptrdiff_t)wc * sv);
+#pragma unroll
+        for (int o = 0; o < B; o += CH) cp_async_b<CH>(st + lane * B + o, gr + o);
+        if (!FWD) {
+            const char *gf = (const char *)(fs + (ptrdiff_t)wc * sv);
+#pragma unroll
+            for (int o = 0; o < B; o += CH) cp_async_b<CH>(st + RB + lane * B + o, gf + o);
+        }
+        // the line's record, spread over its lanes
+        const char *gg = (const char *)(geo + (ptrdiff_t)wc * sg);
+#pragma unroll
+        for (int q = 0; q < CB / 16; ++q)
+            cp_async16_if(st + RB + FB + l * CB + 16 * (g + q * G), gg + 16 * (g + q * G), 16 * (g + q * G) < CB);
+        cp_commit();
+    };
+    for (int u = 0; u < PF; ++u) issue(s_beg + u);
+    // (xi.n) S of the line's end face, outward from its first cell (0 where
+    // the cell is its own neighbour)
+    T end[VPT];
+    {
+        const int wm = (cols ? 2 : 0) + (FWD ? 0 : 1);
+        const bool self = nw == 1 && (cols ? p.per_j : p.per_i);
+        const T *e = (const T *)p.cslotT + 8 * (ptrdiff_t)c0 + 2 * wm;
+#pragma unroll
+        for (int v = 0; v < VPT; ++v) end[v] = self ? (T)0 : xi_dot_n<T>(ux[v], uy[v], e[0], e[1]);
+    }
+    T2 prev[VPT], first[VPT];
+    // a step's coefficients, formed one step ahead of their use so that only
+    // the increments are left on the chain from step to step: (xi.n) S inflow
+    // from the adjacent line and from the own one, 1 / D, and the two faces
+    // that a seam can lie on
+    T cl[VPT], co[VPT], iD[VPT], ca[VPT], cu[VPT], ahead[VPT];
+    auto coef = [&](int s) {
+        const int ww = s - start;
+        T q[7];
+        ld_rec7(q, (const T *)(stage + (s & (PF - 1)) * SB + RB + FB + l * CB));
+#pragma unroll
+        for (int v = 0; v < VPT; ++v) {
+            const T own = ww > 0 ? -ahead[v] : end[v];  // the face ahead of the cell before
+            ahead[v] = xi_dot_n<T>(ux[v], uy[v], q[0], q[1]);
+            const T low = xi_dot_n<T>(ux[v], uy[v], q[2], q[3]);
+            const T upp = xi_dot_n<T>(ux[v], uy[v], q[4], q[5]);
+            // D = base + sum of the outflow (xi.n) S: half the sum of all
+            // |xi.n| S, the cell's outward normals summing to zero
+            const T D = q[6] + (T)0.5 * ((fabs(own) + fabs(ahead[v])) + (fabs(low) + fabs(upp)));
+            iD[v] = rcp_nr(D);
+            cl[v] = low < (T)0 && has_adj ? -low : (T)0;
+            co[v] = own < (T)0 && ww > 0 ? -own : (T)0;
+            if (SEAM) {
+                ca[v] = seam_w && ww == nw - 1 && ahead[v] < (T)0 ? -ahead[v] : (T)0;
+                cu[v] = seam_t && tt == nt - 1 && upp < (T)0 ? -upp : (T)0;
+            }
+        }
+    };
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+        prev[v].x = prev[v].y = first[v].x = first[v].y = (T)0;
+        ahead[v] = (T)0;
+    }
+    cp_wait<PF - 1>();
+    __syncwarp();
+    coef(s_beg);
+    int seen_r = 0, seen_w = 0;
+
+    for (int s0 = s_beg; s0 < s_end; s0 += kSweepBlock) {
+        if (strips > 1) {
+            // reads what the strip before wrote in steps < s0; overwrites what the
+            // strip after reads in steps <= s0 + 2 kSweepBlock - ring
+            if (strip > 0) flag_wait(flags + wid - 1, s0, seen_r, p.status);
+            if (strip + 1 < strips) flag_wait(flags + wid + 1, s0 + 2 * kSweepBlock + 1 - ring, seen_w, p.status);
+        }
+#pragma unroll
+        for (int b = 0; b < kSweepBlock; ++b) {
+            const int s = s0 + b, ww = s - start;
+            cp_wait<PF - 2>();  // the copies of this step and the next one's records
+            __syncwarp();
+            const bool on = (unsigned)ww < nwl;
+            const unsigned char *st = stage + (s & (PF - 1)) * SB;
+            T2 ev[VPT], out[VPT], r[VPT], f[VPT];
+            ld_vec<VPT>(ev, xr + (ww & (ring - 1)) * xs);
+            ld_vec<VPT>(r, (const T2 *)st + lane * VPT);
+            if (!FWD) ld_vec<VPT>(f, (const T2 *)(st + RB) + lane * VPT);
+#pragma unroll
+            for (int v = 0; v < VPT; ++v) {
+                T2 adj;
+                adj.x = __shfl_up_sync(0xffffffffu, prev[v].x, G);
+                adj.y = __shfl_up_sync(0xffffffffu, prev[v].y, G);
+                adj.x = edge ? ev[v].x : adj.x;
+                adj.y = edge ? ev[v].y : adj.y;
+                // inflow from the swept side adds |xi.n| S Delta_nb
+                T ag = co[v] * prev[v].x, ah = co[v] * prev[v].y;
+                ag += cl[v] * adj.x;
+                ah += cl[v] * adj.y;
+                if (SEAM) {
+                    if (ca[v] > (T)0) {
+                        ag += ca[v] * first[v].x;
+                        ah += ca[v] * first[v].y;
+                    }
+                    if (on && cu[v] > (T)0) {
+                        const int nb = (FWD ? 0 : nt - 1) - t;  // lines to the first line of the sweep
+                        const T2 dn = ds[(ptrdiff_t)ww * sv + (ptrdiff_t)nb * (cols ? 1 : p.ni) * Nv + v];
+                        ag += cu[v] * dn.x;
+                        ah += cu[v] * dn.y;
+                    }
+                }
+                if (FWD) {
+                    out[v].x = (r[v].x + ag) * iD[v];
+                    out[v].y = (r[v].y + ah) * iD[v];
+                } else {
+                    out[v].x = r[v].x + ag * iD[v];
+                    out[v].y = r[v].y + ah * iD[v];
+                    f[v].x += out[v].x;
+                    f[v].y += out[v].y;
+                }
+                prev[v] = out[v];
+                if (SEAM && ww == 0) first[v] = out[v];
+            }
+            coef(s + 1);
+            if (FWD || SEAM) st_vec<true, VPT>(ds + (ptrdiff_t)ww * sv, out, on && (FWD || (seam_t && tt == 0)));
+            if (!FWD) st_vec<true, VPT>(fs + (ptrdiff_t)ww * sv, f, on);
+            st_vec<false, VPT>(xw + (ww & (ring - 1)) * xs, out, on && border);
+            issue(s + PF);
+        }
+        if (strips > 1) {
+            __syncwarp();
+            if (lane == 0) flag_store(flags + wid, s0 + kSweepBlock);
+        }
+    }
+    cp_wait<0>();
+    if (strips > 1) {
+        __syncwarp();
+        if (lane == 0) flag_store(flags + wid, 0x7fffffff);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2409,19 +2697,61 @@ template <class T> static size_t macro_smem_bytes(const KParams &p, int nt, int 
     return (size_t)stages * (nt / 2) * (kMRec + 4) * sizeof(T) + (size_t)2 * (nt / 2) * kMRing * sizeof(T);
 }
 
-template <class T, int S> static size_t sweep_bytes_s(const KParams &p, bool withF)
+// shared memory of the scheduled micro sweeps (a 4-step prefetch)
+template <class T> static size_t sched_sweep_bytes(const KParams &p, bool withF)
 {
     switch (p.sweep_vpt) {
-    case 4: return sweep_smem_bytes<T, S, 4>(p.sweep_pc, p.sweep_tv, withF);
-    case 2: return sweep_smem_bytes<T, S, 2>(p.sweep_pc, p.sweep_tv, withF);
-    default: return sweep_smem_bytes<T, S, 1>(p.sweep_pc, p.sweep_tv, withF);
+    case 4: return sweep_smem_bytes<T, 4, 4>(p.sweep_pc, p.sweep_tv, withF);
+    case 2: return sweep_smem_bytes<T, 4, 2>(p.sweep_pc, p.sweep_tv, withF);
+    default: return sweep_smem_bytes<T, 4, 1>(p.sweep_pc, p.sweep_tv, withF);
     }
 }
 
-template <class T> static size_t sweep_bytes(const KParams &p, bool withF, int stages)
+// warps of a line-sweep block, and its shared memory
+static int sweep_line_warps(const KParams &p)
 {
-    return stages == 8 ? sweep_bytes_s<T, 8>(p, withF)
-         : stages == 2 ? sweep_bytes_s<T, 2>(p, withF) : sweep_bytes_s<T, 4>(p, withF);
+    const int lw = 32 / p.sweep_g;
+    return p.sweep_ktv / p.sweep_g * ((p.sweep_pc + lw - 1) / lw);
+}
+static size_t sweep_line_bytes(const KParams &p, bool fp64, bool withF, int stages)
+{
+    const size_t T2 = fp64 ? 16 : 8, v = p.sweep_kvpt, g = p.sweep_g;
+    return 64 + sweep_line_warps(p) * (p.sweep_ring * g * v * T2 + stages * (32 * v * T2 * (withF ? 2 : 1) + 32 / g * 4 * T2));
+}
+
+constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory of a block
+
+void sweep_shape(KParams &p, bool fp64, int vpt)
+{
+    p.sweep_ktv = p.sweep_tv;
+    p.sweep_kvpt = vpt ? vpt : p.sweep_vpt;
+    if (p.sched) return;
+    // at most eight velocity groups in a warp, so that it keeps at least four
+    // lines in step, but none of its lanes goes to lines a narrow block lacks
+    int lines = 1;
+    while (lines < p.sweep_pc && lines < 32) lines *= 2;
+    if (!p.sweep_tuned) {
+        // four groups (eight lines a warp) where the block has that many lines,
+        // more on a narrow one
+        p.sweep_ktv = std::max(4, 128 / lines > 32 ? 32 : 128 / lines);
+        while (p.sweep_ktv * p.sweep_pc > 512) p.sweep_ktv /= 2;
+        // two velocities per thread (16-byte copies); one where that leaves
+        // fewer than a warp for each scheduler; four where the warps are many
+        // waves (float64 is bound by its arithmetic pipe: one)
+        if (!vpt) {
+            const int lw = 32 / std::min(p.sweep_ktv, std::max(8, 32 / lines));
+            const int warps = (p.sweep_pc + lw - 1) / lw * (p.Nv / (2 * std::min(p.sweep_ktv, 32 / lw)));
+            p.sweep_kvpt = fp64 || warps < 4 * 152 ? 1 : warps > 32 * 152 ? 4 : 2;
+        }
+    }
+    // 32 ring entries let neighbouring strips drift a few blocks of steps apart
+    // (at least 2 blocks + 5 are needed); a tile too wide for shared memory at
+    // the shallowest prefetch is halved
+    p.sweep_ring = 32;
+    for (;; p.sweep_ktv /= 2) {
+        p.sweep_g = std::min(p.sweep_ktv, std::max(8, 32 / lines));
+        if (p.sweep_ktv == 1 || sweep_line_bytes(p, fp64, true, 2) <= kMaxSmem) return;
+    }
 }
 
 void blocks_per_instance(const KParams &p, int out[KT_COUNT])
@@ -2438,17 +2768,17 @@ void blocks_per_instance(const KParams &p, int out[KT_COUNT])
     out[KT_MACRO_SWEEP] = 1;
     out[KT_MACRO_POST] = nblk(p.N, 32);
     out[KT_MICRO_RES] = p.N * nvb;
-    out[KT_SWEEP] = nblk(p.Nv, p.sweep_tv * p.sweep_vpt);
+    out[KT_SWEEP] = nblk(p.Nv, p.sweep_ktv * p.sweep_kvpt);
 }
 
 // block shape, shared memory and prefetch depth common to all instances of
 // a plan (the maxima of the instances; the deepest pipeline that fits all)
 int plan_shapes(const KParams *hp, int n, bool fp64, Plan &pl)
 {
-    const size_t lim = 227 * 1024;
+    const size_t lim = kMaxSmem;
     pl.macro_threads = pl.sweep_threads = 0;
     pl.limiter_any = 0;
-    pl.sweep_vpt = hp[0].sweep_vpt;
+    pl.sweep_vpt = hp[0].sweep_kvpt;
     pl.relax_sweeps = hp[0].relax_sweeps;
     pl.sched = hp[0].sched != nullptr;
     pl.sched_smem = 0;
@@ -2457,9 +2787,9 @@ int plan_shapes(const KParams *hp, int n, bool fp64, Plan &pl)
         pl.sched_smem = std::max(pl.sched_smem, (size_t)hp[i].N * 4 * (fp64 ? 8 : 4));
         if (hp[i].relax_sweeps != pl.relax_sweeps) return (int)cudaErrorInvalidValue;
         pl.macro_threads = std::max(pl.macro_threads, macro_threads(hp[i]));
-        pl.sweep_threads = std::max(pl.sweep_threads, hp[i].sweep_tv * hp[i].sweep_pc);
+        pl.sweep_threads = std::max(pl.sweep_threads, pl.sched ? hp[i].sweep_tv * hp[i].sweep_pc : 32 * sweep_line_warps(hp[i]));
         pl.limiter_any |= hp[i].limiter;
-        if (hp[i].sweep_vpt != pl.sweep_vpt) return (int)cudaErrorInvalidValue;
+        if (hp[i].sweep_vpt != hp[0].sweep_vpt || hp[i].sweep_kvpt != pl.sweep_vpt) return (int)cudaErrorInvalidValue;
     }
     if (!pl.sched || pl.sched_smem > 200 * 1024) pl.sched_smem = 0;
     pl.any_seam = 0;
@@ -2500,52 +2830,53 @@ int plan_shapes(const KParams *hp, int n, bool fp64, Plan &pl)
         if (m <= lim) break;
     }
     }
-    for (int stages : {pl.sched ? 4 : std::min(hp[0].sweep_stages, 8), 4}) {
-        size_t f = 0, b = 0;
-        for (int i = 0; i < n; ++i) {
-            f = std::max(f, fp64 ? sweep_bytes<double>(hp[i], false, stages) : sweep_bytes<float>(hp[i], false, stages));
-            b = std::max(b, fp64 ? sweep_bytes<double>(hp[i], true, stages) : sweep_bytes<float>(hp[i], true, stages));
-        }
+    for (int stages : {pl.sched ? 4 : std::min(hp[0].sweep_stages, 8), 4, 2}) {
         pl.sweep_stages = stages;
-        pl.fwd_smem = f;
-        pl.bwd_smem = b;
-        if (b <= lim) break;
+        pl.fwd_smem = pl.bwd_smem = 0;
+        for (int i = 0; i < n; ++i) {
+            auto bytes = [&](bool withF) {
+                return !pl.sched ? sweep_line_bytes(hp[i], fp64, withF, stages)
+                                 : fp64 ? sched_sweep_bytes<double>(hp[i], withF) : sched_sweep_bytes<float>(hp[i], withF);
+            };
+            pl.fwd_smem = std::max(pl.fwd_smem, bytes(false));
+            pl.bwd_smem = std::max(pl.bwd_smem, bytes(true));
+        }
+        if (pl.bwd_smem <= lim || pl.sched) break;
     }
     if (pl.macro_smem > lim || pl.bwd_smem > lim) return (int)cudaErrorInvalidValue;
     return 0;
 }
 
-template <class T, bool FWD, int S>
-static void launch_sweep_s(const Plan &pl, cudaStream_t st, const Launch &L)
+// every instantiation of the micro sweeps, by the plan's shape: visit(kernel)
+template <class T, bool FWD, class F> static void sweep_kernel(const Plan &pl, F visit)
 {
-    const size_t sm = FWD ? pl.fwd_smem : pl.bwd_smem;
-    const int nb = pl.nblocks[KT_SWEEP], nt = pl.sweep_threads;
-    switch (pl.sweep_vpt) {
-    case 4: k_sweep<T, FWD, S, 4><<<nb, nt, sm, st>>>(L); break;
-    case 2: k_sweep<T, FWD, S, 2><<<nb, nt, sm, st>>>(L); break;
-    default: k_sweep<T, FWD, S, 1><<<nb, nt, sm, st>>>(L); break;
+    const int v = pl.sweep_vpt;
+    if (pl.sched) {
+        if (v == 4) visit(k_sweep<T, FWD, 4, 4>);
+        else if (v == 2) visit(k_sweep<T, FWD, 4, 2>);
+        else visit(k_sweep<T, FWD, 4, 1>);
+        return;
     }
-}
-
-// unstructured meshes: the scheduled sweeps (always a 4-step prefetch)
-template <class T, bool FWD>
-static void launch_sweep_sched(const Plan &pl, cudaStream_t st, const Launch &L)
-{
-    const size_t sm = FWD ? pl.fwd_smem : pl.bwd_smem;
-    const int nb = pl.nblocks[KT_SWEEP], nt = pl.sweep_threads;
-    switch (pl.sweep_vpt) {
-    case 4: k_sweep<T, FWD, 4, 4, true><<<nb, nt, sm, st>>>(L); break;
-    case 2: k_sweep<T, FWD, 4, 2, true><<<nb, nt, sm, st>>>(L); break;
-    default: k_sweep<T, FWD, 4, 1, true><<<nb, nt, sm, st>>>(L); break;
-    }
+    auto lines = [&](auto seam) {
+        constexpr bool SEAM = decltype(seam)::value;
+        auto depth = [&](auto stages) {
+            constexpr int PF = decltype(stages)::value;
+            if (v == 4) visit(k_sweep_lines<T, FWD, 4, PF, SEAM>);
+            else if (v == 2) visit(k_sweep_lines<T, FWD, 2, PF, SEAM>);
+            else visit(k_sweep_lines<T, FWD, 1, PF, SEAM>);
+        };
+        if (pl.sweep_stages == 8) depth(std::integral_constant<int, 8>{});
+        else if (pl.sweep_stages == 4) depth(std::integral_constant<int, 4>{});
+        else depth(std::integral_constant<int, 2>{});
+    };
+    if (pl.any_seam) lines(std::true_type{});
+    else lines(std::false_type{});
 }
 
 template <class T, bool FWD> static void launch_sweep(const Plan &pl, cudaStream_t st, const Launch &L)
 {
-    if (pl.sched) launch_sweep_sched<T, FWD>(pl, st, L);
-    else if (pl.sweep_stages == 8) launch_sweep_s<T, FWD, 8>(pl, st, L);
-    else if (pl.sweep_stages == 2) launch_sweep_s<T, FWD, 2>(pl, st, L);
-    else launch_sweep_s<T, FWD, 4>(pl, st, L);
+    const size_t sm = FWD ? pl.fwd_smem : pl.bwd_smem;
+    sweep_kernel<T, FWD>(pl, [&](auto k) { k<<<pl.nblocks[KT_SWEEP], pl.sweep_threads, sm, st>>>(L); });
 }
 
 template <class T> static Launch launch_of(const Plan &pl, int kt)
@@ -2647,7 +2978,7 @@ static int iteration_t(const Plan &pl, cudaStream_t st, void **events)
 // opt the wavefront kernels in to the largest dynamic shared memory once
 template <class T> static int configure_t()
 {
-    const int lim = 227 * 1024;
+    const int lim = (int)kMaxSmem;
     cudaError_t e = cudaSuccess;
     auto opt = [&](const void *fn) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
@@ -2662,31 +2993,24 @@ template <class T> static int configure_t()
     opt((const void *)k_macro_sweep<T, 8>);
     opt((const void *)k_macro_sweep<T, 4>);
     opt((const void *)k_macro_sweep<T, 2>);
-    opt((const void *)k_sweep<T, true, 4, 1, true>);
-    opt((const void *)k_sweep<T, false, 4, 1, true>);
-    opt((const void *)k_sweep<T, true, 4, 2, true>);
-    opt((const void *)k_sweep<T, false, 4, 2, true>);
-    opt((const void *)k_sweep<T, true, 4, 4, true>);
-    opt((const void *)k_sweep<T, false, 4, 4, true>);
-    opt((const void *)k_sweep<T, true, 2, 1>);
-    opt((const void *)k_sweep<T, false, 2, 1>);
-    opt((const void *)k_sweep<T, true, 2, 2>);
-    opt((const void *)k_sweep<T, false, 2, 2>);
-    opt((const void *)k_sweep<T, true, 2, 4>);
-    opt((const void *)k_sweep<T, false, 2, 4>);
-    opt((const void *)k_sweep<T, true, 8, 1>);
-    opt((const void *)k_sweep<T, false, 8, 1>);
-    opt((const void *)k_sweep<T, true, 4, 1>);
-    opt((const void *)k_sweep<T, false, 4, 1>);
-    opt((const void *)k_sweep<T, true, 8, 2>);
-    opt((const void *)k_sweep<T, false, 8, 2>);
-    opt((const void *)k_sweep<T, true, 4, 2>);
-    opt((const void *)k_sweep<T, false, 4, 2>);
-    opt((const void *)k_sweep<T, true, 8, 4>);
-    opt((const void *)k_sweep<T, false, 8, 4>);
-    opt((const void *)k_sweep<T, true, 4, 4>);
-    opt((const void *)k_sweep<T, false, 4, 4>);
     return (int)e;
+}
+
+// the plan's two micro-sweep kernels likewise
+template <class T> static int configure_sweeps_t(const Plan &pl)
+{
+    cudaError_t e = cudaSuccess;
+    auto opt = [&](auto k) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    };
+    sweep_kernel<T, true>(pl, opt);
+    sweep_kernel<T, false>(pl, opt);
+    return (int)e;
+}
+
+int configure_sweeps(const Plan &pl, bool fp64)
+{
+    return fp64 ? configure_sweeps_t<double>(pl) : configure_sweeps_t<float>(pl);
 }
 
 int configure_kernels(bool fp64) { return fp64 ? configure_t<double>() : configure_t<float>(); }

@@ -120,18 +120,14 @@ class Solver:
         keys = {"sweep_tv": B.IDG_TUNE_SWEEP_TV, "sweep_stages": B.IDG_TUNE_SWEEP_STAGES,
                 "macro_stages": B.IDG_TUNE_MACRO_STAGES, "graph": B.IDG_TUNE_GRAPH,
                 "sweep_vpt": B.IDG_TUNE_SWEEP_VPT, "macro_kind": B.IDG_TUNE_MACRO_KIND}
-        cur = self.tuning()
-        # shrink shared-memory use first so that every intermediate shape fits
-        if any(k in kw for k in ("sweep_tv", "sweep_vpt", "sweep_stages", "macro_stages", "macro_kind")):
-            B.idg_set_tuning(self.ctx, keys["sweep_stages"], 4)
-            B.idg_set_tuning(self.ctx, keys["macro_stages"], 2)
+        # only the given keys are set: the untouched ones keep the library's own choice.
+        # A wider tile is set with one velocity per thread first, so that it fits on the way
+        if "sweep_tv" in kw and "sweep_vpt" in kw:
             B.idg_set_tuning(self.ctx, keys["sweep_vpt"], 1)
-            B.idg_set_tuning(self.ctx, keys["sweep_tv"], 1)
+        # (a macro_kind re-derives the macroscopic depth: macro_stages comes after it)
         for k in ("graph", "macro_kind", "sweep_tv", "sweep_vpt", "sweep_stages", "macro_stages"):
-            if k == "macro_stages" and "macro_kind" in kw and k not in kw:
-                continue  # the library re-derives the depth for the chosen kernel
-            v = kw.get(k, cur[k])
-            B.idg_set_tuning(self.ctx, keys[k], int(v))
+            if k in kw:
+                B.idg_set_tuning(self.ctx, keys[k], int(kw[k]))
 
     def tuning(self) -> dict:
         return {"sweep_tv": B.idg_get_tuning(self.ctx, B.IDG_TUNE_SWEEP_TV),
