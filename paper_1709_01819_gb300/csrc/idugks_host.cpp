@@ -646,7 +646,10 @@ size_t layout(idg_ctx *c, char *base, KParams *kp)
     k.phi = L.take<double>(32 * nf);
     k.rw = L.take<double>(32 * N);
     k.mrec = L.take<char>(24 * ts * N);
-    k.mdW = L.take<char>(4 * ts * N);
+    // hyperplane by hyperplane, each as long as the shorter axis (k_macro_lines)
+    const size_t nslot = c->unstr ? N : (size_t)std::min(c->ni, c->nj) * (c->ni + c->nj - 1);
+    k.mline = c->unstr ? nullptr : L.take<char>(24 * ts * nslot);
+    k.mdW = L.take<char>(4 * ts * nslot);
     k.mdW2 = c->relax_sweeps > 0 ? L.take<char>(4 * ts * N) : nullptr;
     k.wallS = c->implicit_wall ? L.take<double>(8 * nf) : nullptr;
     k.walldrg = c->implicit_wall ? L.take<double>(8 * nf) : nullptr;

@@ -75,7 +75,8 @@ struct KParams {
     double *rw;     // [N][4]
     // macroscopic LU-SGS work (T = storage precision of the sweep)
     void *mrec;     // [N][24] T: R, 1/D, own base state, per slot (S/2) n_out, (omega/2) Lambda
-    void *mdW;      // [N][4] T increments (Delta W* then Delta W)
+    void *mline;    // [6][nslot][4] T: the record as k_macro_lines reads it (null if unstructured), cell slots by line_slot()
+    void *mdW;      // [N][4] T increments (Delta W* then Delta W); k_macro_lines: [nslot][4]
     void *mdW2;     // [N][4] T second increment buffer of the point relaxation (else null)
     double *mpart;  // [ceil(N/256)] block partial sums of ||R/Omega||^2
     double *res;    // [kMaxHist] absolute residual per iteration

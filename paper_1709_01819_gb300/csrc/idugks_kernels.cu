@@ -1295,7 +1295,91 @@ template <> __device__ __forceinline__ void cp_async_b<16>(void *s, const void *
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
+// Wavefronts over lines of cells (k_macro_lines, k_sweep_lines): the warps of a
+// block run kSweepBlock steps between two looks at their neighbours' progress.
+constexpr int kSweepBlock = 4;
+
+// progress flags between the warps of one block
+__device__ __forceinline__ void flag_store(int *f, int v)
+{
+    asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(smem_addr(f)), "r"(v) : "memory");
+}
+__device__ __forceinline__ int flag_load(const int *f)
+{
+    int v;
+    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_addr(f)) : "memory");
+    return v;
+}
+// waits until *f >= need (seen: what the last poll found).  The warps of a block
+// run at the same time, so the wait ends; should it not (2^22 polls), the status
+// word is raised and the sweep goes on.
+__device__ __forceinline__ void flag_wait(const int *f, int need, int &seen, int *status)
+{
+    for (int n = 0; seen < need; ++n) {
+        seen = flag_load(f);
+        if (n > (1 << 22)) {
+            *status = 6;
+            seen = 0x7fffffff;
+        }
+    }
+}
+
+// four storage scalars, 16-byte aligned
+__device__ __forceinline__ void ld4(float (&o)[4], const float *s)
+{
+    const float4 v = *reinterpret_cast<const float4 *>(s);
+    o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+}
+__device__ __forceinline__ void ld4(double (&o)[4], const double *s)
+{
+    const double2 a = reinterpret_cast<const double2 *>(s)[0], b = reinterpret_cast<const double2 *>(s)[1];
+    o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
+}
+__device__ __forceinline__ void st4(float *d, const float *x)
+{
+    *reinterpret_cast<float4 *>(d) = make_float4(x[0], x[1], x[2], x[3]);
+}
+__device__ __forceinline__ void st4(double *d, const double *x)
+{
+    reinterpret_cast<double2 *>(d)[0] = make_double2(x[0], x[1]);
+    reinterpret_cast<double2 *>(d)[1] = make_double2(x[2], x[3]);
+}
+
+// where on, without a branch, to global (GLOBAL) or shared memory
+template <bool GLOBAL> __device__ __forceinline__ void st4_if(float *d, const float *x, bool on)
+{
+    if constexpr (GLOBAL)
+        asm volatile("{.reg .pred p; setp.ne.s32 p, %5, 0; @p st.global.v4.f32 [%0], {%1, %2, %3, %4};}" ::"l"(d), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "r"((int)on) : "memory");
+    else
+        asm volatile("{.reg .pred p; setp.ne.s32 p, %5, 0; @p st.shared.v4.f32 [%0], {%1, %2, %3, %4};}" ::"r"(smem_addr(d)), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "r"((int)on) : "memory");
+}
+template <bool GLOBAL> __device__ __forceinline__ void st4_if(double *d, const double *x, bool on)
+{
+#pragma unroll
+    for (int q = 0; q < 4; q += 2) {
+        if constexpr (GLOBAL)
+            asm volatile("{.reg .pred p; setp.ne.s32 p, %3, 0; @p st.global.v2.f64 [%0], {%1, %2};}" ::"l"(d + q), "d"(x[q]), "d"(x[q + 1]), "r"((int)on) : "memory");
+        else
+            asm volatile("{.reg .pred p; setp.ne.s32 p, %3, 0; @p st.shared.v2.f64 [%0], {%1, %2};}" ::"r"(smem_addr(d + q)), "d"(x[q]), "d"(x[q + 1]), "r"((int)on) : "memory");
+    }
+}
+template <class T> __device__ __forceinline__ void st4(T *d, T a, T b, T c, T e)
+{
+    const T x[4] = {a, b, c, e};
+    st4(d, x);
+}
+
 constexpr int kMRec = 24;  // macroscopic sweep record: R[4], 1/D, pad, own base[6], 4 x (n S/2 [2], omega Lambda/2)
+// structured blocks, k_macro_lines: cell c = (t, w), t on the shorter axis, by
+// its hyperplane t + w and its line t, so that the lines a warp marches along
+// read and write consecutive slots at every step; six vectors of four (line_rec)
+__device__ __forceinline__ bool by_lines(const KParams &p) { return p.macro_kind == 1 && !p.sched && p.relax_sweeps == 0; }
+__device__ __forceinline__ int line_slot(const KParams &p, int c)
+{
+    const int j = c / p.ni, i = c - j * p.ni, d = i + j;
+    return p.ni <= p.nj ? d * p.ni + i : d * p.nj + j;
+}
+__device__ __forceinline__ size_t line_slots(const KParams &p) { return (size_t)min(p.ni, p.nj) * (p.ni + p.nj - 1); }
 constexpr int kMRing = 12; // ring entry per cell: increment[4], base state[6], pad[2]
 
 // per cell: R_W, ||R_W/Omega||^2 partials, and the record of the macroscopic
@@ -1309,7 +1393,7 @@ __global__ void __launch_bounds__(32) k_macro_pre(Launch L)
     const int c = blk * blockDim.x + threadIdx.x;
     double part[1] = {0.0};
     if (c < p.N) {
-        T *rec = (T *)p.mrec + (size_t)kMRec * c;
+        T rec[kMRec];
         double acc[4] = {0, 0, 0, 0};
         for (int m = 0; m < 4; ++m) {
             double s = p.csign[4 * c + m];
@@ -1337,22 +1421,45 @@ __global__ void __launch_bounds__(32) k_macro_pre(Launch L)
         rec[4] = (T)(1.0 / d);
         rec[5] = (T)0;
         base_state<T>(p, p.W + 4 * c, rec + 6);
+        if (by_lines(p)) {
+            // R | 1/D, rho, m_x, m_y | per sweep: 1/rho, E + p, omega/2 Lambda of
+            // the faces ahead on the own line and towards the next line | their S/2 n
+            const size_t M = line_slots(p);
+            T *o = (T *)p.mline + 4 * (size_t)line_slot(p, c);
+            const bool cols = p.ni <= p.nj;
+            const T ir = rcp_rn(rec[6]);
+            st4(o, rec);
+            st4(o + 4 * M, rec[4], rec[6], rec[7], rec[8]);
+            for (int dir = 0; dir < 2; ++dir) {
+                // slots (west 0, east 1, south 2, north 3): forward w + 1, t + 1; backward w - 1, t - 1
+                const T *cw = rec + 12 + 3 * ((cols ? 2 : 0) + 1 - dir), *ct = rec + 12 + 3 * ((cols ? 0 : 2) + 1 - dir);
+                st4(o + (8 + 8 * dir) * M, ir, rec[11], cw[2], ct[2]);
+                st4(o + (12 + 8 * dir) * M, cw[0], cw[1], ct[0], ct[1]);
+            }
+        } else {
+            T *o = (T *)p.mrec + (size_t)kMRec * c;
+            for (int q = 0; q < kMRec; ++q) o[q] = rec[q];
+        }
     }
     block_sum<1>(part, sm);
     if (threadIdx.x == 0) p.mpart[blk] = part[0];
 }
 
 // ||R_W/Omega||_2 of this iteration from k_macro_pre's partials (fixed
-// order) into the residual ring; a non-finite value raises the status word
+// order) into the residual ring, by the 32 lanes of one warp; a non-finite
+// value raises the status word.  One thread alone took 9 us for the 128
+// partials of a 64 x 64 block, a load latency per few of them.
 __device__ __forceinline__ void record_residual(const KParams &p)
 {
+    const int lane = threadIdx.x & 31, nb = (p.N + 31) / 32;
     double s = 0.0;
-    const int nb = (p.N + 31) / 32;
-    for (int q = 0; q < nb; ++q) s += p.mpart[q];
-    const int it = *p.iter;
-    const double r = sqrt(s);
-    p.res[it & (kMaxHist - 1)] = r;
-    if (!isfinite(r)) *p.status = 5;
+    for (int q = lane; q < nb; q += 32) s += p.mpart[q];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+        const double r = sqrt(s);
+        p.res[*p.iter & (kMaxHist - 1)] = r;
+        if (!isfinite(r)) *p.status = 5;
+    }
 }
 
 // Exact increment F_n(W + dW) - F_n(W) of the Euler flux, written so that no
@@ -1398,7 +1505,7 @@ __global__ void __launch_bounds__(512) k_macro_sweep(Launch L)
     T *srec = (T *)smraw;                               // [kStages][ncs][kMRec]
     T *sdw = srec + (size_t)kStages * ncs * kMRec;      // [kStages][ncs][4] own dW* (backward)
     T *ring = sdw + (size_t)kStages * ncs * 4;          // [2][ncs][kMRing]
-    if (tid == 0) record_residual(p);
+    if (tid < 32) record_residual(p);
     const T gm1 = (T)(p.gam - 1.0);
     T *dWg = (T *)p.mdW;
     const T *mrec = (const T *)p.mrec;
@@ -1508,270 +1615,215 @@ __global__ void __launch_bounds__(512) k_macro_sweep(Launch L)
 
 // The same sweeps with one thread per line of cells.  The lines run along
 // the longer axis (w), one thread per line of the shorter axis (t: columns,
-// t = i, when ni <= nj, else rows, t = j), so at step d thread t owns cell
-// (t, w = d - t) of the i+j hyperplane d -- the lexicographic dependency order
-// as above.  Of a cell's lower neighbours (forward; upper ones backward) the
-// one on the same line is the thread's own result of the previous step, kept
-// in registers; the one on the adjacent line is the neighbouring lane's result
-// of the previous step, taken by a warp shuffle (across a warp boundary from a
-// two-slot shared-memory exchange behind the step's barrier).  Across a
-// periodic seam along the lines the neighbour is the thread's own first cell
-// (registers); across a seam between the last and the first line it is kept
-// in shared memory by the line that computed it.  Each thread prefetches its
-// cell records (and, backward, its dW*) kStages-1 steps ahead with cp.async
-// into its own stage slots.  One thread owns all four components of its
-// cell: no pair shuffle, no hyperplane ring.
-constexpr int kLRec = kMRec + 4;  // stage entry: the record, then dW* (backward)
-
-template <class T> struct LineNb {
-    T dw[4], b[6];
-};
+// t = i, when ni <= nj, else rows, t = j); a thread marches along its line one
+// step behind the line before it, so at every step the lines stand on an i+j
+// hyperplane.  A cell's two already swept neighbours are the thread's own last
+// cell and the last cell of the line before, and both enter a cell's equation
+// only through the terms 1/2 (dF S - omega Lambda dW): each thread forms, from
+// its new increment, the two terms that its own next cell and the next line's
+// cell will need (half of their arithmetic is common) and passes the latter on
+// by a warp shuffle -- four values and no base state.  Warps of 32 lines run as
+// the strips of the micro sweeps do (see there): border terms in a ring, flags
+// every kSweepBlock steps, no block barrier inside a sweep.  The cells' records
+// and increments lie hyperplane by hyperplane (line_slot), so that the lines of
+// a warp copy consecutive vectors, by cp.async kStages steps ahead into the
+// thread's own slots (cell by cell each copy touched 32 cache lines, 670 cycles
+// a step).  A line's first
+// cell keeps its term across a seam along the lines in registers; the first
+// line's terms across a seam to the last one lie in shared memory.
+// Bound by the latency of a step, 140 instructions of one warp per scheduler.
+// One barrier per step, base states passed along, both terms formed by the
+// receiver and one thread adding up the residual took 62 us on 64 x 64 cells,
+// 213 us on 128 x 128 and 39 us on 48 x 40; this 40, 85 and 30 us.
+constexpr int kLRing = 32;        // border-ring entries (see sweep_shape)
 
 template <class T> static size_t macro_lines_smem_bytes(int nlines, int stages, int nw, bool seam)
 {
-    return ((size_t)stages * nlines * kLRec + 2 * 32 * 12 + (seam ? (size_t)nw * 10 : 0)) * sizeof(T);
+    return 64 + ((size_t)stages * nlines * 24 + (size_t)nlines / 32 * kLRing * 4 + (seam ? (size_t)nw * 4 : 0)) * sizeof(T);
 }
 
-// what every step of k_macro_lines reads that does not change
+// The part of the exact Euler-flux increment F_n(W + dW) - F_n(W) that does not
+// depend on the normal, every term an increment times a base quantity:
+// ir = 1 / (rho + drho), the pressure increment through
+// d(|m|^2 / rho) = ((2 m + dm) . dm - (|m|^2 / rho) drho) ir.
+template <class T> struct LineInc {
+    T rho, mx, my, u, v, H, ir, dp;
+    T dW[4];
+};
+// b: 1/D, rho, m_x, m_y; c: 1/rho, E + p
+template <class T> __device__ __forceinline__ void line_inc(LineInc<T> &x, T gm1, const T (&b)[4], const T (&c)[4])
+{
+    x.rho = b[1]; x.mx = b[2]; x.my = b[3]; x.u = x.mx * c[0]; x.v = x.my * c[0]; x.H = c[1];
+    x.ir = rcp_line(x.rho + x.dW[0]);
+    const T k = x.mx * x.u + x.my * x.v;
+    const T q = ((T)2 * x.mx + x.dW[1]) * x.dW[1] + (((T)2 * x.my + x.dW[2]) * x.dW[2] - k * x.dW[0]);
+    x.dp = gm1 * x.dW[3] - ((T)0.5 * gm1 * q) * x.ir;
+}
+// the term 1/2 (dF S - omega Lambda dW) of this cell's increment in the
+// equation of the neighbour across the face with S/2 n out of this cell
+// (ox, oy) and omega/2 Lambda = ol: the neighbour's normal is the opposite one
+template <class T> __device__ __forceinline__ void line_term(const LineInc<T> &x, T ox, T oy, T ol, T (&o)[4])
+{
+    const T nx = -ox, ny = -oy;
+    const T vn = x.u * nx + x.v * ny;
+    const T dm = x.dW[1] * nx + x.dW[2] * ny;
+    const T dvn = (dm - vn * x.dW[0]) * x.ir, vn1 = vn + dvn;
+    o[0] = dm - ol * x.dW[0];
+    o[1] = x.dW[1] * vn1 + (x.mx * dvn + (x.dp * nx - ol * x.dW[1]));
+    o[2] = x.dW[2] * vn1 + (x.my * dvn + (x.dp * ny - ol * x.dW[2]));
+    o[3] = (x.dW[3] + x.dp) * vn1 + (x.H * dvn - ol * x.dW[3]);
+}
+
+// what a sweep of k_macro_lines reads that does not change
 template <class T> struct LineCtx {
-    T *stage, *xb, *seam, *dWg;
-    const T *mrec;
+    T *stage, *ring, *seam, *dWg;
+    int *flags, *status;
+    const T *rec;
+    size_t M;  // slots
     T gm1;
-    int ni, nt, nw, nh, nthr, t, lane, wid, nwarp, s_tm, s_tp, s_wm, s_wp;
-    bool cols, line, per_t, per_w;
-    __device__ __forceinline__ int cell_of(int w) const { return cols ? w * ni + t : t * ni + w; }
+    int nt, nw, nthr, lane, wid, strips;
+    bool per_t, per_w;
 };
 
-// 16-byte cp.async that copies nothing and zero-fills its destination when
-// !valid (the source must still be a valid address)
-__device__ __forceinline__ void cp_async16_zfill(void *s, const void *g, bool valid)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_addr(s)), "l"(g), "r"(valid ? 16 : 0)
-                 : "memory");
-}
-
-// the record's first 12 entries (R[4], 1/D, pad, base state[6]) by 16-byte
-// shared-memory loads (the stage slots are 16-byte aligned)
-__device__ __forceinline__ void ld_rec12(const float *rec, float (&o)[12])
-{
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const float4 v = reinterpret_cast<const float4 *>(rec)[q];
-        o[4 * q] = v.x, o[4 * q + 1] = v.y, o[4 * q + 2] = v.z, o[4 * q + 3] = v.w;
-    }
-}
-__device__ __forceinline__ void ld_rec12(const double *rec, double (&o)[12])
-{
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        const double2 v = reinterpret_cast<const double2 *>(rec)[q];
-        o[2 * q] = v.x, o[2 * q + 1] = v.y;
-    }
-}
-
-
-// acc += 1/2 (dF S - omega Lambda dW_nb) of one neighbour through the slot
-// whose coefficients start at cf (euler_dflux with rcp_line)
-template <class T>
-__device__ __forceinline__ void line_term2(T gm1, const T *cf, const LineNb<T> &nb, T (&acc)[4])
-{
-    const T nx = cf[0], ny = cf[1], ol = cf[2];
-    const T *b = nb.b, *dW = nb.dw;
-    T rho = b[0], mx = b[1], my = b[2], u = b[3], v = b[4], H = b[5];
-    T ir1 = rcp_line(rho + dW[0]);
-    T du = (dW[1] - u * dW[0]) * ir1, dv = (dW[2] - v * dW[0]) * ir1;
-    T vn = u * nx + v * ny, dvn = du * nx + dv * ny, vn1 = vn + dvn;
-    T dmu = dW[1] * (u + du) + dW[2] * (v + dv) + mx * du + my * dv;
-    T dp = gm1 * (dW[3] - (T)0.5 * dmu);
-    acc[0] += dW[0] * vn1 + rho * dvn - ol * dW[0];
-    acc[1] += dW[1] * vn1 + mx * dvn + dp * nx - ol * dW[1];
-    acc[2] += dW[2] * vn1 + my * dvn + dp * ny - ol * dW[2];
-    acc[3] += (dW[3] + dp) * vn1 + H * dvn - ol * dW[3];
-}
-
-// one direction of k_macro_lines (the direction a template parameter: one
-// shuffle direction, one set of slots; SEAM: the block has a periodic seam).
-// The step is written without branches on the common path so that the
-// compiler can interleave the prefetch, the record loads and the stores with
-// the dependent flux arithmetic: every thread issues its copies each step
-// (zero-filling the slot where its line has no cell at that step), evaluates
-// the step on whatever the slot holds, and keeps the result only where the
-// line has a cell.  A neighbour that does not exist enters with a zero
-// increment on a unit-density base state: its flux increment is exactly
-// zero, so no term needs a branch.
+// one direction of k_macro_lines (SEAM: the block has a periodic seam); lines
+// and cells are numbered from the corner the sweep starts at (tt, ww)
 template <class T, int kStages, bool FWD, bool SEAM> __device__ __forceinline__ void line_sweep(const LineCtx<T> &x)
 {
-    constexpr int RC = kMRec * sizeof(T) / 16, DC = 4 * sizeof(T) / 16;
-    auto step_d = [&](int s) { return FWD ? s : x.nh - 1 - s; };
+    constexpr int VC = 4 * sizeof(T) / 16;  // 16-byte chunks of a vector
+    const int tt = x.wid * 32 + x.lane, tc = min(tt, x.nt - 1), t = FWD ? tc : x.nt - 1 - tc;
+    // slot of (tt, ww): e0 + ww * es
+    const int es = FWD ? x.nt : -x.nt, e0 = (FWD ? t : t + x.nw - 1) * x.nt + t;
+    const unsigned nwl = tt < x.nt ? x.nw : 0;
+    const int s_beg = x.wid * (32 + kSweepBlock);
+    const int s_end = s_beg + x.nw + min(32, x.nt - x.wid * 32) - 1;
+    const int start = tt + x.wid * kSweepBlock;
+    // stage slots [kStages][6][nthr][4]: R or dW*, then the record's vectors (the
+    // other sweep's faces, which a seam needs, last)
+    T *stage = x.stage + 4 * (x.wid * 32 + x.lane);
+    const size_t vec = (size_t)4 * x.nthr, slot = 6 * vec;
+    const T *g0 = (FWD ? x.rec : x.dWg), *g1 = x.rec + 4 * x.M, *g2 = x.rec + (FWD ? 8 : 16) * x.M,
+            *g3 = g2 + 4 * x.M, *g4 = x.rec + (FWD ? 16 : 8) * x.M, *g5 = g4 + 4 * x.M;
     auto issue = [&](int s) {
-        const int w = step_d(s) - x.t;
-        const bool valid = s < x.nh && x.line && (unsigned)w < (unsigned)x.nw;
-        const int c = valid ? x.cell_of(w) : 0;
-        T *dst = x.stage + ((size_t)(s & (kStages - 1)) * x.nthr + x.t) * kLRec;
+        const ptrdiff_t e = 4 * (ptrdiff_t)(e0 + min(max(s - start, 0), x.nw - 1) * es);
+        T *dst = stage + (s & (kStages - 1)) * slot;
 #pragma unroll
-        for (int q = 0; q < RC; ++q)
-            cp_async16_zfill((char *)dst + 16 * q, (const char *)(x.mrec + (size_t)kMRec * c) + 16 * q, valid);
-        if (!FWD)
-#pragma unroll
-            for (int q = 0; q < DC; ++q)
-                cp_async16_zfill((char *)(dst + kMRec) + 16 * q, (const char *)(x.dWg + 4 * (size_t)c) + 16 * q, valid);
+        for (int q = 0; q < VC; ++q) {
+            constexpr int E = 16 / sizeof(T);
+            cp_async16(dst + E * q, g0 + e + E * q);
+            cp_async16(dst + vec + E * q, g1 + e + E * q);
+            cp_async16(dst + 2 * vec + E * q, g2 + e + E * q);
+            cp_async16(dst + 3 * vec + E * q, g3 + e + E * q);
+            if (SEAM) {
+                cp_async16(dst + 4 * vec + E * q, g4 + e + E * q);
+                cp_async16(dst + 5 * vec + E * q, g5 + e + E * q);
+            }
+        }
         cp_commit();
     };
-    for (int s = 0; s < kStages - 1; ++s) issue(s);
-    LineNb<T> prev, first;  // this line's result of the previous step / of its first cell
-#pragma unroll
-    for (int q = 0; q < 4; ++q) prev.dw[q] = first.dw[q] = (T)0;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) prev.b[q] = first.b[q] = q == 0 ? (T)1 : (T)0;
-    const int s_adj = FWD ? x.s_tm : x.s_tp, s_own = FWD ? x.s_wm : x.s_wp;
-    const int s_seam_t = FWD ? x.s_tp : x.s_tm, s_seam_w = FWD ? x.s_wp : x.s_wm;
-    const bool has_adj = FWD ? x.t >= 1 : x.t + 1 < x.nt;
-    const bool seam_t_reader = SEAM && x.per_t && x.t == (FWD ? x.nt - 1 : 0);
-    const bool seam_t_writer = SEAM && x.per_t && x.t == (FWD ? 0 : x.nt - 1);
-    const bool edge_reader = FWD ? (x.lane == 0 && x.wid > 0) : (x.lane == 31 && x.wid + 1 < x.nwarp);
-    const bool edge_writer = FWD ? x.lane == 31 : x.lane == 0;
-    // the exchange entry this thread may read (a valid one for every thread)
-    const int edge_src = edge_reader ? (FWD ? x.wid - 1 : x.wid + 1) : 0;
-    for (int s = 0; s < x.nh; ++s) {
-        cp_wait<kStages - 2>();
-        __syncthreads();  // the step's records and the exchange entries of the previous step are written
-        issue(s + kStages - 1);
-        const int w = step_d(s) - x.t;
-        const bool on = x.line && (unsigned)w < (unsigned)x.nw;
-        const T *rec = x.stage + ((size_t)(s & (kStages - 1)) * x.nthr + x.t) * kLRec;
-        T r12[12];
-        ld_rec12(rec, r12);
-        // the adjacent line's result of the previous step, at this thread's w
-        T ev[12];
-        ld_rec12(x.xb + ((size_t)((s + 1) & 1) * 32 + edge_src) * 12, ev);
-        LineNb<T> adj;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const T sh = FWD ? __shfl_up_sync(0xffffffffu, prev.dw[q], 1) : __shfl_down_sync(0xffffffffu, prev.dw[q], 1);
-            adj.dw[q] = has_adj ? (edge_reader ? ev[q] : sh) : (T)0;
+    for (int u = 0; u < kStages; ++u) issue(s_beg + u);
+    const bool edge = x.lane == 0 && x.wid > 0, border = x.lane == 31 && x.wid + 1 < x.strips;
+    T *xw = x.ring + (size_t)x.wid * kLRing * 4;
+    const T *xr = x.wid > 0 ? xw - kLRing * 4 : xw;
+    T to_w[4] = {0, 0, 0, 0}, to_t[4] = {0, 0, 0, 0}, first[4] = {0, 0, 0, 0};
+    int seen_r = 0, seen_w = 0;
+    for (int s0 = s_beg; s0 < s_end; s0 += kSweepBlock) {
+        if (x.strips > 1) {
+            if (x.wid > 0) flag_wait(x.flags + x.wid - 1, s0, seen_r, x.status);
+            if (x.wid + 1 < x.strips) flag_wait(x.flags + x.wid + 1, s0 + 2 * kSweepBlock + 1 - kLRing, seen_w, x.status);
         }
 #pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            const T sh = FWD ? __shfl_up_sync(0xffffffffu, prev.b[q], 1) : __shfl_down_sync(0xffffffffu, prev.b[q], 1);
-            adj.b[q] = edge_reader ? ev[4 + q] : sh;
-        }
-        T acc[4] = {0, 0, 0, 0};
-        line_term2<T>(x.gm1, rec + 12 + 3 * s_adj, adj, acc);
-        // prev is the zero-increment initial state at the line's first cell
-        line_term2<T>(x.gm1, rec + 12 + 3 * s_own, prev, acc);
-        if (SEAM && on) {
-            if (seam_t_reader) {
-                LineNb<T> sn;
-                const T *e = x.seam + (size_t)w * 10;
+        for (int b = 0; b < kSweepBlock; ++b) {
+            const int s = s0 + b, ww = s - start;
+            cp_wait<kStages - 1>();
+            if (SEAM) __syncwarp();
+            const T *rec = stage + (s & (kStages - 1)) * slot;
+            T r[4], rb[4], rc[4], rd[4], e[4];
+            ld4(r, rec);
+            ld4(rb, rec + vec);
+            ld4(rc, rec + 2 * vec);
+            ld4(rd, rec + 3 * vec);
+            ld4(e, xr + (ww & (kLRing - 1)) * 4);
+            LineInc<T> inc;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) sn.dw[q] = e[q];
-#pragma unroll
-                for (int q = 0; q < 6; ++q) sn.b[q] = e[4 + q];
-                line_term2<T>(x.gm1, rec + 12 + 3 * s_seam_t, sn, acc);
+            for (int q = 0; q < 4; ++q) {
+                const T sh = __shfl_up_sync(0xffffffffu, to_t[q], 1);
+                const T adj = tt > 0 ? (edge ? e[q] : sh) : (T)0;
+                T acc = adj + (ww > 0 ? to_w[q] : (T)0);
+                if (SEAM && x.per_w && ww == x.nw - 1) acc += first[q];
+                if (SEAM && x.per_t && tt == x.nt - 1 && (unsigned)ww < nwl) acc += x.seam[4 * ww + q];
+                // forward: dW*_c = (R_c - sum_lower) / D_c;  backward: dW_c = dW*_c - sum_upper / D_c
+                inc.dW[q] = FWD ? (r[q] - acc) * rb[0] : r[q] - acc * rb[0];
             }
-            if (x.per_w && w == (FWD ? x.nw - 1 : 0)) line_term2<T>(x.gm1, rec + 12 + 3 * s_seam_w, first, acc);
-        }
-        // forward: dW*_c = (R_c - sum_lower) / D_c;  backward: dW_c = dW*_c - sum_upper / D_c
-        const T iD = r12[4];
-        LineNb<T> out;
-        if (FWD) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) out.dw[q] = (r12[q] - acc[q]) * iD;
-        } else {
-            T ds[4];
-            if (sizeof(T) == 4) {
-                const float4 v = *reinterpret_cast<const float4 *>(rec + kMRec);
-                ds[0] = v.x, ds[1] = v.y, ds[2] = v.z, ds[3] = v.w;
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) ds[q] = rec[kMRec + q];
+            line_inc<T>(inc, x.gm1, rb, rc);
+            line_term<T>(inc, rd[0], rd[1], rc[2], to_w);
+            line_term<T>(inc, rd[2], rd[3], rc[3], to_t);
+            const bool on = (unsigned)ww < nwl;
+            st4_if<true>(x.dWg + 4 * (ptrdiff_t)(e0 + ww * es), inc.dW, on);
+            st4_if<false>(xw + (ww & (kLRing - 1)) * 4, to_t, on && border);
+            if (SEAM && on) {
+                const T *oc = rec + 4 * vec, *od = rec + 5 * vec;  // the faces behind
+                if (x.per_w && ww == 0) line_term<T>(inc, od[0], od[1], oc[2], first);
+                if (x.per_t && tt == 0) {
+                    T st[4];
+                    line_term<T>(inc, od[2], od[3], oc[3], st);
+                    st4(x.seam + 4 * ww, st);
+                }
             }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) out.dw[q] = ds[q] - acc[q] * iD;
+            issue(s + kStages);
         }
-#pragma unroll
-        for (int q = 0; q < 6; ++q) out.b[q] = r12[6 + q];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) prev.dw[q] = on ? out.dw[q] : prev.dw[q];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) prev.b[q] = on ? out.b[q] : prev.b[q];
-        if (on) {
-            T *g = x.dWg + 4 * (size_t)x.cell_of(w);
-            if (sizeof(T) == 4) {
-                *reinterpret_cast<float4 *>(g) = make_float4(out.dw[0], out.dw[1], out.dw[2], out.dw[3]);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) g[q] = out.dw[q];
-            }
-        }
-        if (SEAM && on) {
-            // the cell a later cell of this line meets across the seam along the line
-            if (x.per_w && w == (FWD ? 0 : x.nw - 1)) first = out;
-            // the seam line's cells for the line across the seam between lines
-            if (seam_t_writer) {
-                T *e = x.seam + (size_t)w * 10;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) e[q] = out.dw[q];
-#pragma unroll
-                for (int q = 0; q < 6; ++q) e[4 + q] = out.b[q];
-            }
-        }
-        // the warp-boundary lane's result for the next warp's edge lane
-        // (its line's current state; a line without a cell leaves it as it was)
-        if (edge_writer) {
-            T *e = x.xb + ((size_t)(s & 1) * 32 + x.wid) * 12;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) e[q] = prev.dw[q];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) e[4 + q] = prev.b[q];
+        if (x.strips > 1) {
+            __syncwarp();
+            if (x.lane == 0) flag_store(x.flags + x.wid, s0 + kSweepBlock);
         }
     }
     cp_wait<0>();
-    __syncthreads();
+    if (x.strips > 1) {
+        __syncwarp();
+        if (x.lane == 0) flag_store(x.flags + x.wid, 0x7fffffff);
+    }
 }
 
+// 32 threads per strip and one more warp that records the residual meanwhile
 template <class T, int kStages, bool SEAM>
-__global__ void __launch_bounds__(256, 1) k_macro_lines(Launch L)
+__global__ void __launch_bounds__(288, 1) k_macro_lines(Launch L)
 {
     IDG_LOCATE();
     (void)blk;
     extern __shared__ __align__(16) unsigned char smraw[];
     LineCtx<T> x;
-    x.ni = p.ni;
-    x.cols = p.ni <= p.nj;
-    x.nt = x.cols ? p.ni : p.nj;
-    x.nw = x.cols ? p.nj : p.ni;
-    x.nh = x.nt + x.nw - 1;
-    x.nthr = blockDim.x;
-    x.t = threadIdx.x;
-    x.lane = x.t & 31;
-    x.wid = x.t >> 5;
-    x.nwarp = blockDim.x >> 5;
-    x.line = x.t < x.nt;
+    const bool cols = p.ni <= p.nj;
+    x.nt = cols ? p.ni : p.nj;
+    x.nw = cols ? p.nj : p.ni;
+    x.strips = (x.nt + 31) / 32;
+    x.lane = threadIdx.x & 31;
+    x.wid = threadIdx.x >> 5;
+    x.nthr = x.strips * 32;
     // periodic between the last and the first line / along the lines; a
     // direction one cell wide wraps onto the cell itself (no term)
-    x.per_t = (x.cols ? p.per_i : p.per_j) && x.nt > 1;
-    x.per_w = (x.cols ? p.per_j : p.per_i) && x.nw > 1;
-    // slots (west 0, east 1, south 2, north 3) towards line t-1 / t+1 and
-    // towards w-1 / w+1
-    x.s_tm = x.cols ? 0 : 2;
-    x.s_tp = x.cols ? 1 : 3;
-    x.s_wm = x.cols ? 2 : 0;
-    x.s_wp = x.cols ? 3 : 1;
-    x.stage = (T *)smraw;                                     // [kStages][nthr][kLRec]
-    x.xb = x.stage + (size_t)kStages * x.nthr * kLRec;        // [2][32 warps][12] warp-boundary exchange
-    x.seam = x.xb + 2 * 32 * 12;                              // [nw][10] the seam line's cells (per_t)
+    x.per_t = (cols ? p.per_i : p.per_j) && x.nt > 1;
+    x.per_w = (cols ? p.per_j : p.per_i) && x.nw > 1;
+    x.flags = (int *)smraw;                           // [8] steps done by each strip
+    x.ring = (T *)(smraw + 64);                       // [strips][kLRing][4]
+    x.stage = x.ring + (size_t)x.strips * kLRing * 4; // [kStages][6][nthr][4]
+    x.seam = x.stage + (size_t)kStages * x.nthr * 24; // [nw][4] the first line's terms (per_t)
+    x.status = p.status;
     x.dWg = (T *)p.mdW;
-    x.mrec = (const T *)p.mrec;
+    x.rec = (const T *)p.mline;
+    x.M = line_slots(p);
     x.gm1 = (T)(p.gam - 1.0);
-    // exchange entries never written read as benign neighbours (zero
-    // increment, unit density)
-    for (int q = x.t; q < 2 * 32 * 12; q += x.nthr) x.xb[q] = (q % 12 == 4) ? (T)1 : (T)0;
-    if (x.t == 0) record_residual(p);
-    __syncthreads();
-    line_sweep<T, kStages, true, SEAM>(x);
-    line_sweep<T, kStages, false, SEAM>(x);
-    if (x.t == 0) *p.iter += 1;
+    const bool sweeps = x.wid < x.strips;
+    auto arm = [&] {
+        if (sweeps && x.lane == 0) x.flags[x.wid] = x.wid * (32 + kSweepBlock);
+        __syncthreads();
+    };
+    arm();
+    if (sweeps) line_sweep<T, kStages, true, SEAM>(x);
+    else if (x.wid == x.strips) record_residual(p);
+    __syncthreads();  // dW* of every line is written, the flags are free
+    arm();
+    if (sweeps) line_sweep<T, kStages, false, SEAM>(x);
+    __syncthreads();  // the residual went to this iteration's slot
+    if (threadIdx.x == 0) *p.iter += 1;
 }
 
 // The macroscopic LU-SGS sweeps on an unstructured mesh: one CTA walks the
@@ -1821,7 +1873,7 @@ __global__ void __launch_bounds__(256) k_macro_sweep_sched(Launch L)
     IDG_LOCATE();
     (void)blk;
     extern __shared__ __align__(16) unsigned char smraw[];
-    if (threadIdx.x == 0) record_residual(p);
+    if (threadIdx.x < 32) record_residual(p);
     const T gm1 = (T)(p.gam - 1.0);
     T *dWg = (T *)p.mdW;
     T *dw = SMEM ? (T *)smraw : dWg;  // [N][4]
@@ -1868,7 +1920,7 @@ __global__ void __launch_bounds__(32) k_macro_post(Launch L)
     const int c = blk * blockDim.x + threadIdx.x;
     if (c >= p.N) return;
     double *W = p.W + 4 * c;
-    const T *dW = (const T *)p.mdW + 4 * c;
+    const T *dW = (const T *)p.mdW + 4 * (by_lines(p) ? line_slot(p, c) : c);
     for (int q = 0; q < 4; ++q) W[q] += (double)dW[q];
     double rho = W[0], U = W[1] / rho, V = W[2] / rho;
     double RT = (2.0 * W[3] / rho - U * U - V * V) / (p.K + 2);
@@ -1951,10 +2003,8 @@ __global__ void __launch_bounds__(32) k_record_residual(Launch L)
 {
     IDG_LOCATE();
     (void)blk;
-    if (threadIdx.x == 0) {
-        record_residual(p);
-        *p.iter += 1;
-    }
+    record_residual(p);
+    if (threadIdx.x == 0) *p.iter += 1;
 }
 
 template <class T>
@@ -2320,33 +2370,6 @@ __global__ void __launch_bounds__(512) k_sweep(Launch L)
 // 462 + 467 -> 355 + 355 us.  Loads into registers instead of cp.async took
 // 53 + 51 us on 64 x 64, a warp running through the steps before its first and
 // after its last cell 57 + 61 us.
-constexpr int kSweepBlock = 4;
-
-// progress flags between the warps of one block
-__device__ __forceinline__ void flag_store(int *f, int v)
-{
-    asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(smem_addr(f)), "r"(v) : "memory");
-}
-__device__ __forceinline__ int flag_load(const int *f)
-{
-    int v;
-    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_addr(f)) : "memory");
-    return v;
-}
-// waits until *f >= need (seen: what the last poll found).  The warps of a block
-// run at the same time, so the wait ends; should it not (2^22 polls), the status
-// word is raised and the sweep goes on.
-__device__ __forceinline__ void flag_wait(const int *f, int need, int &seen, int *status)
-{
-    for (int n = 0; seen < need; ++n) {
-        seen = flag_load(f);
-        if (n > (1 << 22)) {
-            *status = 6;
-            seen = 0x7fffffff;
-        }
-    }
-}
-
 // 1 / x to within an ulp in float32 (one Newton step on the approximation; x is
 // a positive sum of areas and rates, far from the ends of the range), correctly
 // rounded in float64
@@ -2437,7 +2460,7 @@ __global__ void __launch_bounds__(512) k_sweep_lines(Launch L)
     // ww = s - tt - strip * kSweepBlock; a warp runs from its first line's first
     // cell to its last line's last one
     const int s_beg = (strip * (lw + kSweepBlock)) & ~(kSweepBlock - 1);
-    const int s_end = strip * (lw + kSweepBlock) + nw + lw - 1;
+    const int s_end = strip * (lw + kSweepBlock) + nw + min(lw, nt - strip * lw) - 1;
     if ((threadIdx.x & 31) == 0) flags[wid] = s_beg;
     __syncthreads();
     if (sub >= subs) return;  // a smaller instance of a batch
@@ -2802,8 +2825,8 @@ int plan_shapes(const KParams *hp, int n, bool fp64, Plan &pl)
         // walk axis' cells when the lines wrap around (a periodic shorter axis)
         int ntmax = 0;
         for (int i = 0; i < n; ++i) ntmax = std::max(ntmax, std::min(hp[i].ni, hp[i].nj));
-        pl.macro_threads = ((ntmax + 31) / 32) * 32;
-        const int nlines = pl.macro_threads;
+        const int nlines = ((ntmax + 31) / 32) * 32;
+        pl.macro_threads = nlines + 32;  // and the residual's warp
         for (int stages : {std::min(hp[0].macro_stages, 8), 4, 2}) {
             size_t m = 0;
             for (int i = 0; i < n; ++i) {
