@@ -40,6 +40,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     def compile_one(src):
         obj = os.path.join(LIBDIR, os.path.splitext(src)[0] + f".{os.getpid()}.o")
         cmd = [NVCC] + common + ["-c", os.path.join(CSRC, src), "-o", obj]
+        if src == "idugks_kernels.cu":
+            # its kernels exist for one problem and for a batch and have to round alike:
+            # they fuse multiply-adds where they say so, the compiler nowhere else
+            cmd += ["-fmad=false"]
         if src.endswith(".cu"):
             cmd += ["-Xptxas", "-v"] if verbose else []
         r = subprocess.run(cmd, capture_output=True, text=True)

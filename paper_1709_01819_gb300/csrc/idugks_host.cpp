@@ -598,11 +598,13 @@ size_t layout(idg_ctx *c, char *base, KParams *kp)
     KParams k{};
     k.area = L.take<double>(8 * N);
     k.dtimp = L.take<double>(8 * N);
+    k.adt = L.take<double>(8 * N);
     k.cface = L.take<int>(16 * N);
     k.cnb = L.take<int>(16 * N);
     k.csign = L.take<int>(16 * N);
     k.crT = L.take<char>(8 * ts * N);
     k.clsgT = L.take<char>(8 * ts * N);
+    k.cnT = L.take<char>(8 * ts * N);
     k.cslotT = L.take<char>(8 * ts * N);
     k.scode = c->unstr ? L.take<int>(32 * N) : nullptr;
     k.sgeo = c->unstr ? nullptr : L.take<char>(16 * ts * N);
@@ -627,17 +629,16 @@ size_t layout(idg_ctx *c, char *base, KParams *kp)
     k.bdevH = L.take<char>(4 * ts * Nv);
     k.f = L.take<char>(t2 * N * Nv);
     k.fbp = L.take<char>(t2 * N * Nv);
-    k.grad = c->limiter ? L.take<char>(4 * ts * N * Nv) : nullptr;
     k.dst = L.take<char>(t2 * N * Nv);
     // the face-flux buffer doubles as the float64 staging area of
     // idg_set_state / idg_get_state (G and H of every cell): on an unstructured
     // mesh (about 1.5 faces per cell for triangles) that can be the larger need
     k.F = L.take<char>(std::max(t2 * nf * Nv, 16 * N * Nv));
+    k.ftie = L.take<char>(t2 * nf * std::max(c->nvx, c->nvy));
     k.W = L.take<double>(32 * N);
     k.cellraw = L.take<char>(8 * idg::kRaw * N);
     k.cellA = L.take<char>(ts * idg::kCellP * N);
     k.cellq = L.take<double>(16 * N);
-    k.cellp = L.take<double>(8 * idg::kCellP * N);
     k.cellpT = L.take<char>(ts * idg::kCellP * N);
     k.faceraw = L.take<char>(8 * 12 * nf);
     k.facerw = L.take<double>(8 * nf);
@@ -693,6 +694,8 @@ void reference_tables(idg_ctx *c, std::vector<double> &gref, KParams &k)
     k.U_r = c->ref_u;
     k.V_r = c->ref_v;
     k.RT_r = RTr;
+    k.iRT_r = 1.0 / RTr;
+    k.iAref = 2.0 * RTr / c->ref_rho;
 }
 
 template <class T> cudaError_t up(T *dst, const std::vector<T> &src)
@@ -838,6 +841,7 @@ idg_status launch_chunk_graph(idg_ctx *c, cudaStream_t st, int n)
 idg_status refresh_plan(idg_ctx *c)
 {
     idg::Plan pl{};
+    pl.hparams = &c->kp;
     pl.dparams = c->kp_dev;
     pl.doff = nullptr;
     pl.dactive = nullptr;
@@ -1103,13 +1107,16 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
     c->ws_bytes = bytes;
     KParams &k = c->kp;
     layout(c, c->ws, &k);
-    k.N = c->N; k.Nv = c->Nv; k.nf = c->nf; k.ni = c->ni; k.nj = c->nj; k.nvx = c->nvx;
+    k.N = c->N; k.Nv = c->Nv; k.nf = c->nf; k.ni = c->ni; k.nj = c->nj; k.nvx = c->nvx; k.nvy = c->nvy;
     k.K = c->K; k.shakhov = c->model == IDG_SHAKHOV; k.limiter = c->limiter;
     k.venkat_k3 = c->venkat_k * c->venkat_k * c->venkat_k;
     k.per_i = c->bc_kind[IDG_IMIN] == IDG_BC_PERIODIC;
     k.per_j = c->bc_kind[IDG_JMIN] == IDG_BC_PERIODIC;
     k.dt = c->dt; k.h = 0.5 * c->dt; k.mu_ref = c->mu_ref; k.RT_ref = c->RT_ref; k.omega = c->omega;
     k.Pr = c->Pr; k.gam = (double)(c->K + 4) / (double)(c->K + 2); k.lusgs_omega = c->lusgs_omega;
+    k.iRT_ref = 1.0 / c->RT_ref;
+    k.iK2 = 1.0 / (c->K + 2);
+    k.pc0 = (1.0 - c->Pr) / (c->K + 4);
     k.relax_sweeps = c->relax_sweeps;
     k.implicit_wall = c->implicit_wall;
     if (c->unstr) {
@@ -1136,9 +1143,11 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
     // step's float64 chain); float32 storage: one thread per line of cells
     k.macro_kind = c->precision == IDG_FP64 ? 0 : 1;
     // uploads
+    std::vector<double> adt(c->N);
+    for (int q = 0; q < c->N; ++q) adt[q] = c->area[q] / c->dtimp[q];
     std::vector<float> uxf(c->ux.begin(), c->ux.end()), uyf(c->uy.begin(), c->uy.end()),
         wf(c->w.begin(), c->w.end());
-    std::vector<double> fgeo8((size_t)8 * c->nf, 0.0), cslot((size_t)8 * c->N, 0.0);
+    std::vector<double> fgeo8((size_t)8 * c->nf, 0.0), cslot((size_t)8 * c->N, 0.0), cnrm((size_t)8 * c->N, 0.0);
     // scheduled micro sweeps: the role of each slot's neighbour in the forward
     // (dir +1) and backward (dir -1) sweep: -2 a ghost or not yet swept,
     // -4 - nb the neighbour nb, already swept
@@ -1157,6 +1166,8 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
         for (int m = 0; m < 4; ++m) {
             int fi = c->cface[4 * q + m];
             double s = c->csign[4 * q + m], S = c->fgeo[(size_t)7 * fi + 2];
+            cnrm[8 * q + 2 * m] = s * c->fgeo[(size_t)7 * fi];
+            cnrm[8 * q + 2 * m + 1] = s * c->fgeo[(size_t)7 * fi + 1];
             cslot[8 * q + 2 * m] = s * c->fgeo[(size_t)7 * fi] * S;
             cslot[8 * q + 2 * m + 1] = s * c->fgeo[(size_t)7 * fi + 1] * S;
         }
@@ -1179,9 +1190,9 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
             }
     }
     cudaError_t errs[] = {
-        up((double *)k.area, c->area), up((double *)k.dtimp, c->dtimp), up((int *)k.cface, c->cface),
+        up((double *)k.area, c->area), up((double *)k.dtimp, c->dtimp), up((double *)k.adt, adt), up((int *)k.cface, c->cface),
         up((int *)k.cnb, c->cnb), up((int *)k.csign, c->csign), up_storage(c, k.crT, c->cr),
-        up_storage(c, k.clsgT, c->clsg), up_storage(c, k.cslotT, cslot),
+        up_storage(c, k.clsgT, c->clsg), up_storage(c, k.cslotT, cslot), up_storage(c, k.cnT, cnrm),
         c->unstr ? up((int *)k.scode, scode) : up_storage(c, k.sgeo, sgeo), up((int *)k.fL, c->fL),
         up((int *)k.fR, c->fR), up((double *)k.fgeo, c->fgeo), up_storage(c, k.fgeoT, fgeo8),
         up((int *)k.fbc, c->fbc), up((int *)k.fside, c->fside),

@@ -20,17 +20,19 @@ constexpr int kNoAllocMaxCells = 16384;  // cell limit of idg_get_moments_noallo
 // relative to one reference Maxwellian M_ref (f = M_ref + dev).
 struct KParams {
     // sizes
-    int N, Nv, nf, ni, nj, nvx;
+    int N, Nv, nf, ni, nj, nvx, nvy;
     int K, shakhov, limiter;
     int per_i, per_j;
     // cells
     const double *area;    // [N]
     const double *dtimp;   // [N]
+    const double *adt;     // [N] area / dtimp
     const int *cface;      // [N][4] faces in slots west, east, south, north
     const int *cnb;        // [N][4] neighbour across the slot (-1 ghost)
     const int *csign;      // [N][4] +1 if the cell is the L side of that face
     const void *crT;       // [N][8] T: face midpoint minus centroid, per slot
     const void *clsgT;     // [N][8] T: least-squares weight vector per slot
+    const void *cnT;       // [N][4][2] T: outward normal per slot, sign*nx, sign*ny
     const void *cslotT;    // [N][4][2] T: sign*nx*S, sign*ny*S per slot (micro sweeps)
     const int *scode;      // [2][N][4] forward, backward: role of each slot's neighbour in that micro sweep
                            // (scheduled sweeps of an unstructured mesh; null on a structured block)
@@ -53,20 +55,21 @@ struct KParams {
     double venkat_k3;  // cube of the limiter's smoothing constant: eps^2 = venkat_k3 * area^(3/2)
     // reference Maxwellian parameters and its discrete moments
     double rho_r, U_r, V_r, RT_r;
+    double iRT_r, iAref;     // 1 / RT_r, 2 RT_r / rho_r (one over rho_r lambda_r)
+    double iRT_ref, iK2, pc0; // 1 / RT_ref, 1 / (K + 2), (1 - Pr) / (K + 4)
     double mref_raw[kRaw];     // raw moments: G: 1,x,y,xx,xy,yy,x|xi|^2,y|xi|^2; H: 1,x,y
     double mref_flux[4][2];    // sum w psi xi_a M_ref, psi = 1, xi_x, xi_y, energy
     // state and work (T2 = {G, H} deviation pairs of the storage type)
     void *f;        // [N][Nv] T2 state f~ - M_ref
     void *fbp;      // [N][Nv] T2 fb+ - M_ref
-    void *grad;     // [N][Nv][4] T limited gradients phi sigma of G and H (limiter on; else null)
-    void *F;        // [nf][Nv] T2 flux of (f_face - M_ref)
+    void *F;        // [nf][Nv] T2 fb at the face (minus M_ref), then the flux of (f_face - M_ref)
+    void *ftie;     // [nf][max(nvx, nvy)] T2 interior faces: fb from the R side at velocities along the face (tie_slot())
     void *dst;      // [N][Nv] T2 Delta* then Delta
     double *W;      // [N][4]
     void *cellraw;  // [N][kRaw] acc raw moments of f~ - M_ref
     void *cellA;    // [N][16] T: equilibrium at W^n (14), c1, c2 of fb+
     double *cellq;  // [N][2]  heat flux of f at cells (from f~^n)
-    double *cellp;  // [N][16] post-predictor cell coefficients (float64)
-    void *cellpT;   // [N][16] T copy of cellp for the sweeps
+    void *cellpT;   // [N][16] T: equilibrium at the predicted state (14), collision rate, micro diagonal base
     void *faceraw;  // [nf][12] acc raw moments of fb - M_ref, wall outgoing sum
     double *facerw; // [nf] wall density rho_w (1 elsewhere)
     void *faceA;    // [nf][16] T: face equilibrium (14), a, b of Eq. (18)
@@ -122,6 +125,7 @@ enum KType {
 // (null for a single instance), activity flags (null: all active), and the
 // block shapes common to all instances.
 struct Plan {
+    const KParams *hparams;  // a single instance: its parameters on the host, passed by value; null for a batch
     const KParams *dparams;
     const int *doff;     // [KT_COUNT][ninst + 1]
     const int *dactive;  // [ninst]

@@ -25,13 +25,12 @@
 //   k_cell_params    thread per cell: heat flux (q of Eq. 20), tau,
 //                    equilibrium at W^n, coefficients of fb+ (Eq. 10, 12)
 //   k_fbp            per (cell, velocity): fb+ = c1 f~ + c2 f^S
-//   k_cell_grad      (limiter on) per (cell, velocity): least-squares gradient
-//                    (Eq. 14-15) and limiter (Eq. 16-17), stored as phi sigma
-//   k_face_moments   warp per face: characteristic reconstruction of fb at the
-//                    half step (Eq. 11, 13) with the gradient (computed in
-//                    place when the limiter is off), wall density (Eq. 35),
-//                    raw moments of fb; with the linearised wall the ghost
-//                    density increment of Eq. (35)                     [a2-a3]
+//   k_cell_recon     per (cell, velocity): least-squares gradient (Eq. 14-15),
+//                    limiter (Eq. 16-17) and fb at the half step (Eq. 11, 13)
+//                    at the faces the velocity leaves the cell by          [a2]
+//   k_face_moments   warp per face: wall density (Eq. 35) and the incoming
+//                    part at boundary faces, raw moments of fb; with the
+//                    linearised wall the ghost density increment of Eq. (35) [a3]
 //   k_face_params    thread per face: face state, tau, q, equilibrium, and
 //                    the weights of Eq. (18)                              [a4]
 //   k_face_flux      warp per face: f at the face (Eq. 18), flux (Eq. 19),
@@ -71,6 +70,11 @@ __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, 
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+// a b + c in one rounding.  This file is compiled without contraction
+// (-fmad=false) and says where it fuses: a kernel's instances for one problem
+// and for a batch then round alike, whatever the compiler makes of each.
+__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 // correctly rounded reciprocals: the same value as 1 / x in IEEE division,
 // without the general division routine
 __device__ __forceinline__ float rcp_rn(float x) { return __frcp_rn(x); }
@@ -86,8 +90,42 @@ __device__ __forceinline__ float rcp_line(float x)
     return r;
 }
 __device__ __forceinline__ double rcp_line(double x) { return __drcp_rn(x); }
-__device__ __forceinline__ float t_expm1(float x) { return expm1f(x); }
-__device__ __forceinline__ double t_expm1(double x) { return expm1(x); }
+// e^x - 1 for |x| < 1/2 by its Taylor series in Horner form (every x^k / k! up
+// to k = 9 in float32, 15 in float64: the remainder is below 5.4e-10 and 1.5e-18
+// of x, the rounding of the last two operations within an ulp): half the
+// instructions of the general function, which reduces the range first.  (Taking
+// it up to |x| = 1 raised the float32 residual floor of a Ma 5 flow by half: the
+// exponent difference carries the rounding of its large terms.)
+__device__ __forceinline__ float expm1_near(float x)
+{
+    float q = 1.0f / 362880.0f;
+    q = fmaf(q, x, 1.0f / 40320.0f);
+    q = fmaf(q, x, 1.0f / 5040.0f);
+    q = fmaf(q, x, 1.0f / 720.0f);
+    q = fmaf(q, x, 1.0f / 120.0f);
+    q = fmaf(q, x, 1.0f / 24.0f);
+    q = fmaf(q, x, 1.0f / 6.0f);
+    q = fmaf(q, x, 0.5f);
+    return fmaf(x * x, q, x);
+}
+__device__ __forceinline__ double expm1_near(double x)
+{
+    double q = 1.0 / 1307674368000.0;
+    q = fma(q, x, 1.0 / 87178291200.0);
+    q = fma(q, x, 1.0 / 6227020800.0);
+    q = fma(q, x, 1.0 / 479001600.0);
+    q = fma(q, x, 1.0 / 39916800.0);
+    q = fma(q, x, 1.0 / 3628800.0);
+    q = fma(q, x, 1.0 / 362880.0);
+    q = fma(q, x, 1.0 / 40320.0);
+    q = fma(q, x, 1.0 / 5040.0);
+    q = fma(q, x, 1.0 / 720.0);
+    q = fma(q, x, 1.0 / 120.0);
+    q = fma(q, x, 1.0 / 24.0);
+    q = fma(q, x, 1.0 / 6.0);
+    q = fma(q, x, 0.5);
+    return fma(x * x, q, x);
+}
 __device__ __forceinline__ float t_exp(float x) { return expf(x); }
 __device__ __forceinline__ double t_exp(double x) { return exp(x); }
 
@@ -137,7 +175,13 @@ template <class T> struct Acc;
 template <> struct Acc<float> {
     FF v;
     __device__ __forceinline__ void zero() { v = {0.f, 0.f}; }
-    __device__ __forceinline__ void add(float x) { v = ff_add(v, FF{x, 0.f}); }
+    // (the error terms collect in lo: renormalised once, by warp_sum)
+    __device__ __forceinline__ void add(float x)
+    {
+        const FF s = two_sum(v.hi, x);
+        v.hi = s.hi;
+        v.lo += s.lo;
+    }
     __device__ __forceinline__ void warp_sum()
     {
         for (int o = 16; o > 0; o >>= 1) {
@@ -159,6 +203,51 @@ template <> struct Acc<double> {
     __device__ __forceinline__ void store(void *base, size_t i) const { ((double *)base)[i] = v; }
     __device__ __forceinline__ double value() const { return v; }
 };
+
+// Sums of NA <= 16 accumulators over the 32 lanes, stored at base[q], q < NA.
+// Lanes halve the set of sums they carry at each exchange (16, 8, 4, 2, 1 lanes
+// apart), so that 16 sums take 16 exchanges instead of 16 x 5; lane pairs meet
+// in the same order as in warp_sum.
+__device__ __forceinline__ FF shfl_xor_acc(FF a, int o)
+{
+    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ double shfl_xor_acc(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ FF sum_acc(FF a, FF b) { return ff_add(a, b); }
+__device__ __forceinline__ double sum_acc(double a, double b) { return a + b; }
+template <int NA, class T> __device__ __forceinline__ void warp_sum_store(const Acc<T> (&acc)[NA], int lane, void *base, size_t i0)
+{
+    constexpr int NP = NA <= 4 ? 4 : 16;  // sums carried, the ones past NA zero
+    decltype(acc[0].v) x[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+        if (q < NA) x[q] = acc[q].v;
+        else x[q] = decltype(acc[0].v){};
+    }
+    int mine = 0;
+#pragma unroll
+    for (int o = 16, n = NP; o > 0; o >>= 1) {
+        if (n > 1) {
+            // the upper lane of a pair keeps the upper half of the sums
+            n >>= 1;
+            const bool up = lane & o;
+#pragma unroll
+            for (int q = 0; q < n; ++q) {
+                const auto keep = up ? x[q + n] : x[q], give = up ? x[q] : x[q + n];
+                x[q] = sum_acc(keep, shfl_xor_acc(give, o));
+            }
+            if (up) mine += n;
+        } else {
+            x[0] = sum_acc(x[0], shfl_xor_acc(x[0], o));
+        }
+    }
+    // lanes that differ in the last log2(32 / NP) bits carry the same sum
+    if ((lane & (32 / NP - 1)) == 0 && mine < NA) {
+        Acc<T> a;
+        a.v = x[0];
+        a.store(base, i0 + mine);
+    }
+}
 
 // an accumulator entry widened to float64
 template <class T> __device__ __forceinline__ double acc_load(const void *base, size_t i);
@@ -226,6 +315,18 @@ __device__ __forceinline__ bool locate(const Launch &L, const KParams *&pp, int 
     return !L.active || L.active[inst];
 }
 
+// one instance's launch: its parameters by value (the kernel's constant bank),
+// which saves every block a chain of dependent loads before its first data
+struct LaunchOne {
+    KParams p;
+};
+__device__ __forceinline__ bool locate(const LaunchOne &L, const KParams *&pp, int &blk)
+{
+    pp = &L.p;
+    blk = blockIdx.x;
+    return true;
+}
+
 #define IDG_LOCATE()                                   \
     const KParams *pp_;                                \
     int blk;                                           \
@@ -237,7 +338,7 @@ __device__ __forceinline__ bool locate(const Launch &L, const KParams *&pp, int 
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double viscosity(const KParams &p, double RT)
 {
-    return p.mu_ref * pow(RT / p.RT_ref, p.omega);
+    return p.mu_ref * pow(RT * p.iRT_ref, p.omega);
 }
 
 // The power law of the viscosity for tau in the iteration's kernels: with
@@ -251,7 +352,7 @@ template <> __device__ __forceinline__ double viscosity_t<double>(const KParams 
 }
 template <> __device__ __forceinline__ double viscosity_t<float>(const KParams &p, double RT)
 {
-    return p.mu_ref * (double)powf((float)(RT / p.RT_ref), (float)p.omega);
+    return p.mu_ref * (double)powf((float)(RT * p.iRT_ref), (float)p.omega);
 }
 
 // heat flux q = 1/2 sum w c (c^2 G + H) about (U, V) from raw moments
@@ -259,23 +360,26 @@ template <> __device__ __forceinline__ double viscosity_t<float>(const KParams &
 __device__ __forceinline__ void raw_heat_flux(const double *r, double U, double V, double &qx,
                                               double &qy)
 {
-    double U2 = U * U + V * V;
-    double sx = r[6] - 2.0 * U * r[3] - 2.0 * V * r[4] + U2 * r[1] - U * (r[3] + r[5]) +
-                2.0 * U * U * r[1] + 2.0 * U * V * r[2] - U * U2 * r[0];
-    double sy = r[7] - 2.0 * U * r[4] - 2.0 * V * r[5] + U2 * r[2] - V * (r[3] + r[5]) +
-                2.0 * U * V * r[1] + 2.0 * V * V * r[2] - V * U2 * r[0];
-    qx = 0.5 * (sx + r[9] - U * r[8]);
-    qy = 0.5 * (sy + r[10] - V * r[8]);
+    const double U2 = mad(U, U, V * V), e = r[3] + r[5] + r[8];
+    // the energy-weighted sums less U e, plus 2 U (U . m) and U2 (m - U rho), where
+    // m = (r1, r2), less the shear part 2 (r3, r4; r4, r5) U
+    const double um = mad(U, r[1], V * r[2]);
+    const double cx = mad(-U, r[0], r[1]), cy = mad(-V, r[0], r[2]);
+    const double sx = mad(U2, cx, mad(2.0 * U, um, mad(-U, e, r[6] + r[9])));
+    const double sy = mad(U2, cy, mad(2.0 * V, um, mad(-V, e, r[7] + r[10])));
+    qx = 0.5 * mad(-2.0, mad(U, r[3], V * r[4]), sx);
+    qy = 0.5 * mad(-2.0, mad(U, r[4], V * r[5]), sy);
 }
 
-__device__ void raw_to_state(const double *r, int K, double &rho, double &U, double &V,
-                             double &RT, double &qx, double &qy)
+__device__ __forceinline__ void raw_to_state(const KParams &p, const double *r, double &rho, double &irho, double &U,
+                                             double &V, double &RT, double &qx, double &qy)
 {
     rho = r[0];
-    U = r[1] / rho;
-    V = r[2] / rho;
-    double rhoE = 0.5 * (r[3] + r[5] + r[8]);
-    RT = (2.0 * rhoE / rho - U * U - V * V) / (K + 2);
+    irho = rcp_rn(rho);
+    U = r[1] * irho;
+    V = r[2] * irho;
+    const double rhoE2 = r[3] + r[5] + r[8];  // twice the energy density
+    RT = mad(-V, V, mad(-U, U, rhoE2 * irho)) * p.iK2;
     raw_heat_flux(r, U, V, qx, qy);
 }
 
@@ -286,30 +390,32 @@ struct EqD {
     double e0, ex, ey, e2, U, V, invRT, pqx, pqy, rr, rrm1, kRT, A, lam;
 };
 
-__device__ EqD make_eq(const KParams &p, double rho, double U, double V, double RT, double qx,
-                       double qy)
+// (irho, ir: 1 / rho and 1 / RT; the float64 pipe issues a warp's operation in
+// 16 cycles and a division is a dozen of them, so that every division is taken
+// once and by its reciprocal, the reference's on the host)
+__device__ __forceinline__ EqD make_eq(const KParams &p, double rho, double irho, double U, double V, double RT,
+                                       double ir, double qx, double qy)
 {
     EqD e;
-    double lam = 0.5 / RT, lamr = 0.5 / p.RT_r;
+    const double lam = 0.5 * ir, lamr = 0.5 * p.iRT_r;
     e.e2 = lamr - lam;
-    e.ex = 2.0 * (lam * U - lamr * p.U_r);
-    e.ey = 2.0 * (lam * V - lamr * p.V_r);
+    e.ex = 2.0 * mad(lam, U, -lamr * p.U_r);
+    e.ey = 2.0 * mad(lam, V, -lamr * p.V_r);
     // a non-positive density (a transient state, e.g. an evacuated wall
     // face after an impulsive start) has no logarithm: e0 then sends every
     // velocity to the direct branch, which takes the signed amplitude A
-    e.e0 = rho > 0.0 ? log(rho * lam / (p.rho_r * lamr)) - lam * (U * U + V * V) +
-                           lamr * (p.U_r * p.U_r + p.V_r * p.V_r)
+    e.e0 = rho > 0.0 ? mad(-lam, mad(U, U, V * V), log(rho * lam * p.iAref)) + lamr * mad(p.U_r, p.U_r, p.V_r * p.V_r)
                      : 1e30;
     e.U = U;
     e.V = V;
-    e.invRT = 1.0 / RT;
-    double pc = p.shakhov && rho != 0.0 ? (1.0 - p.Pr) / ((p.K + 4) * rho * RT * RT) : 0.0;
+    e.invRT = ir;
+    const double pc = p.shakhov && rho != 0.0 ? p.pc0 * irho * (ir * ir) : 0.0;
     e.pqx = pc * qx;
     e.pqy = pc * qy;
-    e.rr = RT / p.RT_r;
-    e.rrm1 = (RT - p.RT_r) / p.RT_r;
+    e.rr = RT * p.iRT_r;
+    e.rrm1 = (RT - p.RT_r) * p.iRT_r;
     e.kRT = p.K * RT;
-    e.A = rho * lam / M_PI;
+    e.A = rho * lam * (1.0 / M_PI);
     e.lam = lam;
     return e;
 }
@@ -324,8 +430,6 @@ template <class T> __device__ __forceinline__ void eq_storeT(T *cp, const EqD &e
     cp[5] = (T)e.V; cp[6] = (T)e.invRT; cp[7] = (T)e.pqx; cp[8] = (T)e.pqy; cp[9] = (T)e.rr;
     cp[10] = (T)e.rrm1; cp[11] = (T)e.kRT; cp[12] = (T)e.A; cp[13] = (T)e.lam;
 }
-
-__device__ __forceinline__ void eq_store(double *cp, const EqD &e) { eq_storeT<double>(cp, e); }
 
 template <class T> __device__ __forceinline__ EqT<T> eq_loadT(const T *cp)
 {
@@ -343,22 +447,20 @@ template <class T>
 __device__ __forceinline__ void dev_equilibrium(const EqT<T> &e, T ux, T uy, T gref, T kRTr,
                                                 T &dG, T &dH)
 {
-    T cx = ux - e.U, cy = uy - e.V;
-    T q2 = cx * cx + cy * cy;
-    T t = q2 * e.invRT;
-    T P = e.pqx * cx + e.pqy * cy;
-    T PG = P * (t - (T)4), PH = P * (t - (T)2);
-    T E = e.e0 + e.ex * ux + e.ey * uy + e.e2 * (ux * ux + uy * uy);
-    T href = kRTr * gref;
+    const T cx = ux - e.U, cy = uy - e.V;
+    const T q2 = mad(cx, cx, cy * cy);
+    const T P = mad(e.pqx, cx, e.pqy * cy);
+    const T PG = P * mad(q2, e.invRT, (T)-4), PH = P * mad(q2, e.invRT, (T)-2);
+    const T E = mad(e.e2, mad(ux, ux, uy * uy), mad(e.ex, ux, mad(e.ey, uy, e.e0)));
+    const T href = kRTr * gref;
     if (fabs(E) < (T)0.5) {
-        T em = t_expm1(E);
-        T s = em + PG * ((T)1 + em);
-        dG = gref * s;
-        dH = href * (e.rrm1 + e.rr * (em + PH * ((T)1 + em)));
+        const T em = expm1_near(E), em1 = (T)1 + em;
+        dG = gref * mad(PG, em1, em);
+        dH = href * mad(e.rr, mad(PH, em1, em), e.rrm1);
     } else {
-        T g = e.A * t_exp(-e.lam * q2);
-        dG = g * ((T)1 + PG) - gref;
-        dH = e.kRT * g * ((T)1 + PH) - href;
+        const T g = e.A * t_exp(-e.lam * q2);
+        dG = mad(g, PG, g) - gref;
+        dH = mad(e.kRT * g, (T)1 + PH, -href);
     }
 }
 
@@ -366,10 +468,10 @@ __device__ __forceinline__ void dev_equilibrium(const EqT<T> &e, T ux, T uy, T g
 template <class T>
 __device__ __forceinline__ void raw_terms(T (&a)[kRaw], T w, T ux, T uy, T g, T h)
 {
-    T wg = w * g, wh = w * h, s2 = ux * ux + uy * uy;
-    a[0] += wg; a[1] += wg * ux; a[2] += wg * uy; a[3] += wg * ux * ux; a[4] += wg * ux * uy;
-    a[5] += wg * uy * uy; a[6] += wg * ux * s2; a[7] += wg * uy * s2;
-    a[8] += wh; a[9] += wh * ux; a[10] += wh * uy;
+    const T wg = w * g, wh = w * h, s2 = mad(ux, ux, uy * uy), gx = wg * ux, gy = wg * uy;
+    a[0] += wg; a[1] += gx; a[2] += gy; a[3] = mad(gx, ux, a[3]); a[4] = mad(gx, uy, a[4]);
+    a[5] = mad(gy, uy, a[5]); a[6] = mad(gx, s2, a[6]); a[7] = mad(gy, s2, a[7]);
+    a[8] += wh; a[9] = mad(wh, ux, a[9]); a[10] = mad(wh, uy, a[10]);
 }
 
 // Warp loop over the discrete velocities: lane l takes k = k0 + 32u + l,
@@ -409,9 +511,9 @@ template <class T> __device__ __forceinline__ void load_pair(const void *base, s
 // k, k + 1 with k = k0 + 64u + 2l, u < 4, for chunks of 256 velocities (the
 // stored velocity count is a multiple of 4, so pairs are whole and start on
 // 16-byte boundaries); each chunk's per-lane partial sums (at most 8 terms)
-// are folded into the accumulators as in vel_loop.
-template <int NA, class T, class Body>
-__device__ __forceinline__ void vel_loop2(int Nv, int lane, Acc<T> (&acc)[NA], Body body)
+// are folded into the accumulators as in vel_loop.  fold(a) takes them.
+template <int NA, class T, class Body, class Fold>
+__device__ __forceinline__ void vel_loop2(int Nv, int lane, Body body, Fold fold)
 {
     int k0 = 0;
     for (; k0 + 256 <= Nv; k0 += 256) {
@@ -420,8 +522,7 @@ __device__ __forceinline__ void vel_loop2(int Nv, int lane, Acc<T> (&acc)[NA], B
         for (int q = 0; q < NA; ++q) a[q] = (T)0;
 #pragma unroll 2
         for (int u = 0; u < 4; ++u) body(k0 + 64 * u + 2 * lane, a);
-#pragma unroll
-        for (int q = 0; q < NA; ++q) acc[q].add(a[q]);
+        fold(a);
     }
     if (k0 < Nv) {
         T a[NA];
@@ -431,9 +532,39 @@ __device__ __forceinline__ void vel_loop2(int Nv, int lane, Acc<T> (&acc)[NA], B
             int k = k0 + 64 * u + 2 * lane;
             if (k < Nv) body(k, a);
         }
+        fold(a);
+    }
+}
+template <int NA, class T, class Body>
+__device__ __forceinline__ void vel_loop2(int Nv, int lane, Acc<T> (&acc)[NA], Body body)
+{
+    vel_loop2<NA, T>(Nv, lane, body, [&](const T(&a)[NA]) {
 #pragma unroll
         for (int q = 0; q < NA; ++q) acc[q].add(a[q]);
-    }
+    });
+}
+
+// The same with each thread's float-float accumulators held in shared memory
+// (sacc[q * blockDim.x + threadIdx.x]) between chunks, which leaves a
+// 64-register thread room for its loads in flight.
+template <int NA, class Body>
+__device__ __forceinline__ void vel_loop2_sm(int Nv, int lane, Acc<float> (&acc)[NA], FF *sacc, Body body)
+{
+    FF *s = sacc + threadIdx.x;
+    const int nt = blockDim.x;
+#pragma unroll
+    for (int q = 0; q < NA; ++q) s[q * nt] = FF{0.f, 0.f};
+    vel_loop2<NA, float>(Nv, lane, body, [&](const float(&a)[NA]) {
+#pragma unroll
+        for (int q = 0; q < NA; ++q) {
+            Acc<float> x;
+            x.v = s[q * nt];
+            x.add(a[q]);
+            s[q * nt] = x.v;
+        }
+    });
+#pragma unroll
+    for (int q = 0; q < NA; ++q) acc[q].v = s[q * nt];
 }
 
 // store of two consecutive velocities' {G, H} (see load_pair)
@@ -448,6 +579,19 @@ template <> __device__ __forceinline__ void store_pair<double>(void *base, size_
     ((double2 *)base)[i + 1] = make_double2(g[1], h[1]);
 }
 
+// the same where on[v], without branches
+__device__ __forceinline__ void st_pair_if(float2 *d, const float (&g)[2], const float (&h)[2], const bool (&on)[2])
+{
+    asm volatile("{.reg .pred p, q, r; setp.ne.s32 p, %5, 0; setp.ne.s32 q, %6, 0; and.pred r, p, q; xor.pred p, p, r; xor.pred q, q, r; "
+                 "@r st.global.v4.f32 [%0], {%1, %2, %3, %4}; @p st.global.v2.f32 [%0], {%1, %2}; @q st.global.v2.f32 [%0+8], {%3, %4};}"
+                 ::"l"(d), "f"(g[0]), "f"(h[0]), "f"(g[1]), "f"(h[1]), "r"((int)on[0]), "r"((int)on[1]) : "memory");
+}
+__device__ __forceinline__ void st_pair_if(double2 *d, const double (&g)[2], const double (&h)[2], const bool (&on)[2])
+{
+    if (on[0]) d[0] = make_double2(g[0], h[0]);
+    if (on[1]) d[1] = make_double2(g[1], h[1]);
+}
+
 // velocity table entries k, k + 1 (k even)
 template <class T> __device__ __forceinline__ void vtab2(const float *tf, const double *td, int k, T (&o)[2]);
 template <> __device__ __forceinline__ void vtab2<float>(const float *tf, const double *, int k, float (&o)[2])
@@ -459,73 +603,6 @@ template <> __device__ __forceinline__ void vtab2<double>(const float *, const d
 {
     const double2 v = ((const double2 *)td)[k >> 1];
     o[0] = v.x; o[1] = v.y;
-}
-
-// The same loop with each thread's float-float accumulators held in shared
-// memory (sacc[q * blockDim.x + threadIdx.x]) between chunks: the arithmetic is
-// that of vel_loop, while the registers of a 64-register thread stay free for
-// the loads in flight.  Float storage only; the float64 path keeps vel_loop.
-template <int NA, class Body>
-__device__ __forceinline__ void vel_loop_sm(int Nv, int lane, FF *sacc, Body body)
-{
-    const int t = threadIdx.x, nt = blockDim.x;
-#pragma unroll
-    for (int q = 0; q < NA; ++q) sacc[q * nt + t] = FF{0.f, 0.f};
-    auto fold = [&](const float(&a)[NA]) {
-#pragma unroll
-        for (int q = 0; q < NA; ++q) sacc[q * nt + t] = ff_add(sacc[q * nt + t], FF{a[q], 0.f});
-    };
-    int k0 = 0;
-    for (; k0 + 256 <= Nv; k0 += 256) {
-        float a[NA];
-#pragma unroll
-        for (int q = 0; q < NA; ++q) a[q] = 0.f;
-#pragma unroll 4
-        for (int u = 0; u < 8; ++u) body(k0 + 32 * u + lane, a);
-        fold(a);
-    }
-    if (k0 < Nv) {
-        float a[NA];
-#pragma unroll
-        for (int q = 0; q < NA; ++q) a[q] = 0.f;
-        for (int u = 0; u < 8; ++u) {
-            int k = k0 + 32 * u + lane;
-            if (k < Nv) body(k, a);
-        }
-        fold(a);
-    }
-}
-
-// vel_loop2 with the accumulators of vel_loop_sm
-template <int NA, class Body>
-__device__ __forceinline__ void vel_loop2_sm(int Nv, int lane, FF *sacc, Body body)
-{
-    const int t = threadIdx.x, nt = blockDim.x;
-#pragma unroll
-    for (int q = 0; q < NA; ++q) sacc[q * nt + t] = FF{0.f, 0.f};
-    auto fold = [&](const float(&a)[NA]) {
-#pragma unroll
-        for (int q = 0; q < NA; ++q) sacc[q * nt + t] = ff_add(sacc[q * nt + t], FF{a[q], 0.f});
-    };
-    int k0 = 0;
-    for (; k0 + 256 <= Nv; k0 += 256) {
-        float a[NA];
-#pragma unroll
-        for (int q = 0; q < NA; ++q) a[q] = 0.f;
-#pragma unroll 2
-        for (int u = 0; u < 4; ++u) body(k0 + 64 * u + 2 * lane, a);
-        fold(a);
-    }
-    if (k0 < Nv) {
-        float a[NA];
-#pragma unroll
-        for (int q = 0; q < NA; ++q) a[q] = 0.f;
-        for (int u = 0; u < 4; ++u) {
-            int k = k0 + 64 * u + 2 * lane;
-            if (k < Nv) body(k, a);
-        }
-        fold(a);
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -542,7 +619,7 @@ __device__ __forceinline__ void cell_moments_body(const KParams &__restrict__ p,
     Acc<T> acc[kRaw];
 #pragma unroll
     for (int q = 0; q < kRaw; ++q) acc[q].zero();
-    vel_loop2<kRaw, T>(p.Nv, lane, acc, [&](int k, T(&a)[kRaw]) {
+    auto body = [&](int k, T(&a)[kRaw]) {
         T ux[2], uy[2], w[2], g[2], h[2];
         vtab2<T>(p.uxf, p.ux, k, ux);
         vtab2<T>(p.uyf, p.uy, k, uy);
@@ -550,16 +627,18 @@ __device__ __forceinline__ void cell_moments_body(const KParams &__restrict__ p,
         load_pair<T>(f, k, g, h);
         raw_terms<T>(a, w[0], ux[0], uy[0], g[0], h[0]);
         raw_terms<T>(a, w[1], ux[1], uy[1], g[1], h[1]);
-    });
-#pragma unroll
-    for (int q = 0; q < kRaw; ++q) acc[q].warp_sum();
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < kRaw; ++q) acc[q].store(p.cellraw, (size_t)c * kRaw + q);
+    };
+    if constexpr (sizeof(T) == 4) {
+        __shared__ FF sacc[kRaw * 256];
+        vel_loop2_sm<kRaw>(p.Nv, lane, acc, sacc, body);
+    } else {
+        vel_loop2<kRaw, T>(p.Nv, lane, acc, body);
+    }
+    warp_sum_store<kRaw, T>(acc, lane, p.cellraw, (size_t)c * kRaw);
 }
 
-template <class T>
-__global__ void __launch_bounds__(256) k_cell_moments(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_cell_moments(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     cell_moments_body<T>(p, blk);
@@ -574,8 +653,8 @@ __global__ void __launch_bounds__(256) k_cell_moments_v(KParams p)
 
 // per cell: heat flux of f from f~ (about U of W), tau, equilibrium at W^n,
 // and the two coefficients of fb+ = (2tau-h)/(2tau+dt) f~ + 3h/(2tau+dt) f^S
-template <class T>
-__global__ void __launch_bounds__(32) k_cell_params(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(32) k_cell_params(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     const int c = blk * blockDim.x + threadIdx.x;
@@ -583,26 +662,26 @@ __global__ void __launch_bounds__(32) k_cell_params(Launch L)
     double r[kRaw];
     for (int q = 0; q < kRaw; ++q) r[q] = acc_load<T>(p.cellraw, (size_t)c * kRaw + q) + p.mref_raw[q];
     const double *W = p.W + 4 * c;
-    double rho = W[0], U = W[1] / rho, V = W[2] / rho;
-    double RT = (2.0 * W[3] / rho - U * U - V * V) / (p.K + 2);
-    double tau = viscosity_t<T>(p, RT) / (rho * RT);
+    const double rho = W[0], irho = rcp_rn(rho), U = W[1] * irho, V = W[2] * irho;
+    const double RT = mad(-V, V, mad(-U, U, 2.0 * W[3] * irho)) * p.iK2, ir = rcp_rn(RT);
+    const double tau2 = 2.0 * viscosity_t<T>(p, RT) * (irho * ir);  // 2 tau
     double qtx, qty;
     raw_heat_flux(r, U, V, qtx, qty);
-    double Pr = p.shakhov ? p.Pr : 1.0;
-    double qx = 2.0 * tau * qtx / (2.0 * tau + p.dt * Pr);
-    double qy = 2.0 * tau * qty / (2.0 * tau + p.dt * Pr);
+    const double Pr = p.shakhov ? p.Pr : 1.0, fq = tau2 * rcp_rn(tau2 + p.dt * Pr);
+    const double qx = fq * qtx, qy = fq * qty;
     p.cellq[2 * c] = qx;
     p.cellq[2 * c + 1] = qy;
     T *cA = (T *)p.cellA + kCellP * c;
-    eq_storeT<T>(cA, make_eq(p, rho, U, V, RT, qx, qy));
-    cA[14] = (T)((2.0 * tau - p.h) / (2.0 * tau + p.dt));
-    cA[15] = (T)(3.0 * p.h / (2.0 * tau + p.dt));
+    eq_storeT<T>(cA, make_eq(p, rho, irho, U, V, RT, ir, qx, qy));
+    const double fd = rcp_rn(tau2 + p.dt);
+    cA[14] = (T)((tau2 - p.h) * fd);
+    cA[15] = (T)(3.0 * p.h * fd);
 }
 
 // per (cell, pair of velocities): fb+ = c1 f~ + c2 f^S; 128-thread blocks,
 // each over 256 velocities of one cell
-template <class T>
-__global__ void __launch_bounds__(128) k_fbp(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(128) k_fbp(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     const int nvb = (p.Nv + 255) / 256;
@@ -622,8 +701,8 @@ __global__ void __launch_bounds__(128) k_fbp(Launch L)
     for (int v = 0; v < 2; ++v) {
         T dG, dH;
         dev_equilibrium<T>(e, ux[v], uy[v], gr[v], kRTr, dG, dH);
-        g[v] = c1 * g[v] + c2 * dG;
-        h[v] = c1 * h[v] + c2 * dH;
+        g[v] = mad(c1, g[v], c2 * dG);
+        h[v] = mad(c1, h[v], c2 * dH);
     }
     store_pair<T>(p.fbp, ck, g, h);
 }
@@ -632,39 +711,13 @@ __global__ void __launch_bounds__(128) k_fbp(Launch L)
 // faces: reconstruction from one cell along the characteristic (Eq. 11,
 // 13-17), moments, face equilibrium and flux (Eq. 18-19)            [a2-a4]
 // ---------------------------------------------------------------------------
-template <class T> struct SideRec {
-    int c;
-    int nb[4];
-    T gx[4], gy[4];    // least-squares weights: sigma = sum_m g_m (phi_nb - phi_c)
-    T rx, ry;          // face midpoint minus centroid for the face being built
-    T frx[4], fry[4];  // all four face offsets of the cell (limiter)
-};
-
-template <class T>
-__device__ __forceinline__ void load_side(const KParams &p, int c, T rx, T ry, SideRec<T> &r)
-{
-    const T *g = (const T *)p.clsgT + 8 * c;
-    const T *o = (const T *)p.crT + 8 * c;
-    r.c = c;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        r.nb[m] = p.cnb[4 * c + m];
-        r.gx[m] = g[2 * m];
-        r.gy[m] = g[2 * m + 1];
-        r.frx[m] = o[2 * m];
-        r.fry[m] = o[2 * m + 1];
-    }
-    r.rx = rx;
-    r.ry = ry;
-}
-
 // Divisions of the limiter: exact in float64 (the oracle's rounding up to
 // order); in float32 storage the approximate quotient (2 ulp) of the fast
 // reciprocal path, the limiter being a smooth function of its ratios
 __device__ __forceinline__ float lim_div(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double lim_div(double a, double b) { return a / b; }
 
-template <class T> __device__ __forceinline__ T venkat(T x) { return lim_div(x * x + (T)2 * x, x * x + x + (T)2); }
+template <class T> __device__ __forceinline__ T venkat(T x) { return lim_div(mad(x, x, (T)2 * x), mad(x, x, x + (T)2)); }
 
 // G and H of two consecutive velocities k, k + 1 (k even: 16-byte aligned
 // because the stored velocity count is a multiple of 4)
@@ -680,17 +733,7 @@ template <> __device__ __forceinline__ void load_pair<double>(const void *base, 
     g[0] = a.x; h[0] = a.y; g[1] = b.x; h[1] = b.y;
 }
 
-// four storage scalars (one velocity's limited gradients), 16- or 32-byte aligned
-template <class T> __device__ __forceinline__ void store4(T *d, T a, T b, T c, T e);
-template <> __device__ __forceinline__ void store4<float>(float *d, float a, float b, float c, float e)
-{
-    *(float4 *)d = make_float4(a, b, c, e);
-}
-template <> __device__ __forceinline__ void store4<double>(double *d, double a, double b, double c, double e)
-{
-    ((double2 *)d)[0] = make_double2(a, b);
-    ((double2 *)d)[1] = make_double2(c, e);
-}
+// four storage scalars, 16- or 32-byte aligned
 template <class T> __device__ __forceinline__ void load4(const T *s, T &a, T &b, T &c, T &e);
 template <> __device__ __forceinline__ void load4<float>(const float *s, float &a, float &b, float &c, float &e)
 {
@@ -723,9 +766,9 @@ __device__ __forceinline__ T limit_scalar_sel(const T (&frx)[4], const T (&fry)[
         T phi = (T)1;
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            const T d = sx * frx[m] + sy * fry[m];
-            const T P = (d > (T)0 ? vmax : vmin) - v0;
-            const T t = lim_div(P * P + e2 + (T)2 * d * P, P * P + (T)2 * d * d + P * d + e2);
+            const T d = mad(sx, frx[m], sy * fry[m]);
+            const T P = (d > (T)0 ? vmax : vmin) - v0, q = mad(P, P, e2);
+            const T t = lim_div(mad((T)2 * d, P, q), mad((T)2 * d, d, mad(P, d, q)));
             phi = (d != (T)0 && t < phi) ? t : phi;
         }
         return phi;
@@ -733,38 +776,62 @@ __device__ __forceinline__ T limit_scalar_sel(const T (&frx)[4], const T (&fry)[
     T xm = (T)2;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-        const T d = sx * frx[m] + sy * fry[m];
+        const T d = mad(sx, frx[m], sy * fry[m]);
         const T x = lim_div((d > (T)0 ? vmax : vmin) - v0, d);
         xm = (d != (T)0 && x < xm) ? x : xm;
     }
     return venkat<T>(xm);
 }
 
-// per (cell, pair of velocities), limiter on: least-squares gradients of fb+
-// (Eq. 14-15) and the Venkatakrishnan limiter (Eq. 16-17) of G and H, stored
-// as the limited gradients phi sigma for the reconstructions at the cell's
-// faces.  128-thread blocks, each over 256 velocities of one cell; the cell's
-// stencil record is read by every thread (one broadcast per load).
-template <class T>
-__global__ void __launch_bounds__(128) k_cell_grad(Launch L)
+// slot of velocity k among those along a face (xi.n = 0 in the storage type):
+// the velocity grid is a tensor product, so every row (or column) of it, taken
+// across the normal's larger component, holds at most one such velocity
+template <class T> __device__ __forceinline__ int tie_slot(const KParams &p, int k, T nx, T ny)
+{
+    return fabs(nx) >= fabs(ny) ? k / p.nvx : k % p.nvx;
+}
+
+// Per (cell, pair of velocities): the least-squares gradient of fb+ (Eq. 14-15),
+// LIM: the Venkatakrishnan limiter (Eq. 16-17), and fb at the half step
+// (Eq. 11, 13) at those of the cell's faces that the velocity leaves it by --
+// fb+_c + phi sigma_c . (x_f - xi h - x_c) -- into the face buffer.  The
+// limiter ratios and the gradients only involve differences of fb+ between
+// cells at one velocity, so the M_ref offset cancels and deviations serve as
+// is.  An interior face gets each velocity from the one cell that is upwind of
+// it; at a velocity along the face (s = 0) both sides count half, the L side
+// going to the face buffer and the R side to the tie buffer (k_face_moments
+// takes the mean).  Boundary faces get the outgoing velocities and the ties.
+// 128-thread blocks, each over 256 velocities of one cell; the cell's stencil
+// record is read by every thread (one broadcast per load).
+// Bound by the face buffer's bytes and the issue of the stencil arithmetic.
+// Gathering at the faces instead formed every gradient twice (once per face a
+// velocity leaves by) with one warp walking a face: LIMTXT
+template <class T, bool LIM, class LT>
+__global__ void __launch_bounds__(128) k_cell_recon(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
-    if (!p.limiter) return;
+    using T2 = typename V2<T>::t;
     const int nvb = (p.Nv + 255) / 256;
     const int c = blk / nvb;
     const int k = 2 * ((blk - c * nvb) * 128 + threadIdx.x);
     if (k >= p.Nv) return;
-    int nb[4];
-    T gx[4], gy[4], frx[4], fry[4];
+    int nb[4], fc[4], sg[4];
+    T gx[4], gy[4], frx[4], fry[4], nx[4], ny[4];
     {
-        const int4 n4 = *(const int4 *)(p.cnb + 4 * c);
+        const int4 n4 = *(const int4 *)(p.cnb + 4 * c), f4 = *(const int4 *)(p.cface + 4 * c),
+                   s4 = *(const int4 *)(p.csign + 4 * c);
         nb[0] = n4.x; nb[1] = n4.y; nb[2] = n4.z; nb[3] = n4.w;
+        fc[0] = f4.x; fc[1] = f4.y; fc[2] = f4.z; fc[3] = f4.w;
+        sg[0] = s4.x; sg[1] = s4.y; sg[2] = s4.z; sg[3] = s4.w;
         const T *g = (const T *)p.clsgT + 8 * c;
         const T *o = (const T *)p.crT + 8 * c;
+        const T *n = (const T *)p.cnT + 8 * c;
         load4<T>(g, gx[0], gy[0], gx[1], gy[1]);
         load4<T>(g + 4, gx[2], gy[2], gx[3], gy[3]);
         load4<T>(o, frx[0], fry[0], frx[1], fry[1]);
         load4<T>(o + 4, frx[2], fry[2], frx[3], fry[3]);
+        load4<T>(n, nx[0], ny[0], nx[1], ny[1]);
+        load4<T>(n + 4, nx[2], ny[2], nx[3], ny[3]);
     }
     T g0[2], h0[2];
     load_pair<T>(p.fbp, (size_t)c * p.Nv + k, g0, h0);
@@ -778,170 +845,70 @@ __global__ void __launch_bounds__(128) k_cell_grad(Launch L)
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
             const T dg = gn[v] - g0[v], dh = hn[v] - h0[v];
-            sgx[v] += gx[m] * dg; sgy[v] += gy[m] * dg;
-            shx[v] += gx[m] * dh; shy[v] += gy[m] * dh;
-            gmax[v] = gn[v] > gmax[v] ? gn[v] : gmax[v]; gmin[v] = gn[v] < gmin[v] ? gn[v] : gmin[v];
-            hmax[v] = hn[v] > hmax[v] ? hn[v] : hmax[v]; hmin[v] = hn[v] < hmin[v] ? hn[v] : hmin[v];
+            sgx[v] = mad(gx[m], dg, sgx[v]); sgy[v] = mad(gy[m], dg, sgy[v]);
+            shx[v] = mad(gx[m], dh, shx[v]); shy[v] = mad(gy[m], dh, shy[v]);
+            if (LIM) {
+                gmax[v] = gn[v] > gmax[v] ? gn[v] : gmax[v]; gmin[v] = gn[v] < gmin[v] ? gn[v] : gmin[v];
+                hmax[v] = hn[v] > hmax[v] ? hn[v] : hmax[v]; hmin[v] = hn[v] < hmin[v] ? hn[v] : hmin[v];
+            }
         }
     }
-    T *gout = (T *)p.grad + 4 * ((size_t)c * p.Nv + k);
-    // the smoothing constant's eps^2 = (K h)^3, h = sqrt(area) (0: Eq. 16-17)
-    T e2 = (T)0;
-    if (p.venkat_k3 > 0.0) {
-        const double a = p.area[c];
-        e2 = (T)(p.venkat_k3 * a * sqrt(a));
-    }
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        const T pg = limit_scalar_sel<T>(frx, fry, g0[v], gmax[v], gmin[v], sgx[v], sgy[v], e2);
-        const T ph = limit_scalar_sel<T>(frx, fry, h0[v], hmax[v], hmin[v], shx[v], shy[v], e2);
-        store4<T>(gout + 4 * v, pg * sgx[v], pg * sgy[v], ph * shx[v], ph * shy[v]);
-    }
-}
-
-// fb at the face from side r: fb+_c + phi sigma_c . (x_f - xi h - x_c).  The
-// limiter ratios only involve differences of fb+ between cells at one
-// velocity, so the M_ref offset cancels and deviations serve as is.
-template <class T, bool LIM>
-__device__ __forceinline__ typename V2<T>::t reconstruct(const KParams &p, const SideRec<T> &r,
-                                                         int k, T ux, T uy, T h)
-{
-    using T2 = typename V2<T>::t;
-    const T2 *fb = (const T2 *)p.fbp;
-    T2 f0 = fb[(size_t)r.c * p.Nv + k];
     if (LIM && p.limiter) {
-        // limited gradients phi sigma of G and H, stored once per (cell,
-        // velocity) by k_cell_grad
-        T g0, g1, g2, g3;
-        load4<T>((const T *)p.grad + 4 * ((size_t)r.c * p.Nv + k), g0, g1, g2, g3);
-        const T ax = r.rx - ux * h, ay = r.ry - uy * h;
-        T2 o;
-        o.x = f0.x + (g0 * ax + g1 * ay);
-        o.y = f0.y + (g2 * ax + g3 * ay);
-        return o;
-    }
-    // limiter off: the unlimited least-squares gradient in place
-    T sgx = 0, sgy = 0, shx = 0, shy = 0;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        if (r.nb[m] < 0) continue;
-        T2 fn = fb[(size_t)r.nb[m] * p.Nv + k];
-        T dg = fn.x - f0.x, dh = fn.y - f0.y;
-        sgx += r.gx[m] * dg; sgy += r.gy[m] * dg;
-        shx += r.gx[m] * dh; shy += r.gy[m] * dh;
-    }
-    T ax = r.rx - ux * h, ay = r.ry - uy * h;
-    T2 o;
-    o.x = f0.x + (sgx * ax + sgy * ay);
-    o.y = f0.y + (shx * ax + shy * ay);
-    return o;
-}
-
-// reconstruct for the velocity pair k, k + 1 from one side
-template <class T, bool LIM>
-__device__ __forceinline__ void reconstruct2(const KParams &p, const SideRec<T> &r, int k, const T (&ux)[2],
-                                             const T (&uy)[2], T h, T (&og)[2], T (&oh)[2])
-{
-    T g0[2], h0[2];
-    load_pair<T>(p.fbp, (size_t)r.c * p.Nv + k, g0, h0);
-    if (LIM) {
-        const T *gp = (const T *)p.grad + 4 * ((size_t)r.c * p.Nv + k);
+        // the smoothing constant's eps^2 = (K h)^3, h = sqrt(area) (0: Eq. 16-17)
+        T e2 = (T)0;
+        if (p.venkat_k3 > 0.0) {
+            const double a = p.area[c];
+            e2 = (T)(p.venkat_k3 * a * sqrt(a));
+        }
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
-            T a0, a1, a2, a3;
-            load4<T>(gp + 4 * v, a0, a1, a2, a3);
-            const T ax = r.rx - ux[v] * h, ay = r.ry - uy[v] * h;
-            og[v] = g0[v] + (a0 * ax + a1 * ay);
-            oh[v] = h0[v] + (a2 * ax + a3 * ay);
-        }
-        return;
-    }
-    T sgx[2] = {0, 0}, sgy[2] = {0, 0}, shx[2] = {0, 0}, shy[2] = {0, 0};
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        if (r.nb[m] < 0) continue;
-        T gn[2], hn[2];
-        load_pair<T>(p.fbp, (size_t)r.nb[m] * p.Nv + k, gn, hn);
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-            const T dg = gn[v] - g0[v], dh = hn[v] - h0[v];
-            sgx[v] += r.gx[m] * dg; sgy[v] += r.gy[m] * dg;
-            shx[v] += r.gx[m] * dh; shy[v] += r.gy[m] * dh;
+            const T pg = limit_scalar_sel<T>(frx, fry, g0[v], gmax[v], gmin[v], sgx[v], sgy[v], e2);
+            const T ph = limit_scalar_sel<T>(frx, fry, h0[v], hmax[v], hmin[v], shx[v], shy[v], e2);
+            sgx[v] *= pg; sgy[v] *= pg;
+            shx[v] *= ph; shy[v] *= ph;
         }
     }
+    T ux[2], uy[2];
+    vtab2<T>(p.uxf, p.ux, k, ux);
+    vtab2<T>(p.uyf, p.uy, k, uy);
+    const T h = (T)p.h;
+    // back along the characteristic first, then to each face's midpoint
+    T bg[2], bh[2];
 #pragma unroll
     for (int v = 0; v < 2; ++v) {
-        const T ax = r.rx - ux[v] * h, ay = r.ry - uy[v] * h;
-        og[v] = g0[v] + (sgx[v] * ax + sgy[v] * ay);
-        oh[v] = h0[v] + (shx[v] * ax + shy[v] * ay);
+        bg[v] = mad(-h, mad(sgx[v], ux[v], sgy[v] * uy[v]), g0[v]);
+        bh[v] = mad(-h, mad(shx[v], ux[v], shy[v] * uy[v]), h0[v]);
     }
-}
-
-// The two side records live in shared memory (one pair per warp) so the
-// per-lane choice of the upwind side is an indexed shared-memory read.
-template <class T> struct FaceCtx {
-    int kind;          // -1 interior, 1 wall, 2 far field
-    int side;
-    T nx, ny, S, on;   // normal L->R, length; boundary: +1 if the interior cell is L
-    const SideRec<T> *rec;  // [2]: L, R (boundary faces: [0] is the interior cell)
-};
-
-template <class T>
-__device__ __forceinline__ void load_face(const KParams &p, int f, SideRec<T> *srec, FaceCtx<T> &fc)
-{
-    const int lane = threadIdx.x & 31;
-    const T *g = (const T *)p.fgeoT + 8 * f;
-    fc.nx = g[0];
-    fc.ny = g[1];
-    fc.S = g[2];
-    fc.kind = p.fbc[f];
-    fc.side = p.fside[f];
-    const int L = p.fL[f], R = p.fR[f];
-    fc.on = (fc.kind < 0 || L >= 0) ? (T)1 : (T)-1;
-    if (lane == 0) {
-        if (L >= 0) load_side<T>(p, L, g[3], g[4], srec[0]);
-        else load_side<T>(p, R, g[5], g[6], srec[0]);
-    } else if (lane == 1 && fc.kind < 0) {
-        load_side<T>(p, R, g[5], g[6], srec[1]);
-    }
-    __syncwarp();
-    fc.rec = srec;
-}
-
-// fb - M_ref at velocity k.  Interior: upwind side by sign(xi.n), average at
-// a tie.  Boundary: outgoing from the interior cell; incoming from the wall
-// Maxwellian rho_w M_w (rho_w - 1 passed as rwm1) or the far-field state.
-template <class T, bool LIM>
-__device__ __forceinline__ typename V2<T>::t face_fbar(const KParams &p, const FaceCtx<T> &fc, int k,
-                                                       T ux, T uy, T s, T rhow, T rwm1)
-{
-    using T2 = typename V2<T>::t;
-    const T h = (T)p.h;
-    if (fc.kind < 0) {
-        T2 fb = reconstruct<T, LIM>(p, fc.rec[s > (T)0 ? 0 : 1], k, ux, uy, h);
-        if (s == (T)0) {
-            T2 o = reconstruct<T, LIM>(p, fc.rec[0], k, ux, uy, h);
-            fb.x = (T)0.5 * (o.x + fb.x);
-            fb.y = (T)0.5 * (o.y + fb.y);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        if (sg[m] == 0) continue;  // a triangle's unused slot
+        T og[2], oh[2], s[2];
+        bool out[2];
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            s[v] = xi_dot_n<T>(ux[v], uy[v], nx[m], ny[m]);
+            out[v] = s[v] > (T)0;
+            og[v] = bg[v] + mad(sgx[v], frx[m], sgy[v] * fry[m]);
+            oh[v] = bh[v] + mad(shx[v], frx[m], shy[v] * fry[m]);
         }
-        return fb;
+        if (s[0] == (T)0 || s[1] == (T)0) {
+            // along the face: the L side (of a boundary face the only one) to the
+            // face buffer, the R side to the tie buffer
+            const bool own = sg[m] > 0 || nb[m] < 0;
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+                if (s[v] == (T)0) {
+                    out[v] = own;
+                    if (!own && k + v < p.nvx * p.nvy) {  // (the ghost velocities have no slot)
+                        T2 o;
+                        o.x = og[v];
+                        o.y = oh[v];
+                        ((T2 *)p.ftie)[(size_t)fc[m] * max(p.nvx, p.nvy) + tie_slot<T>(p, k + v, nx[m], ny[m])] = o;
+                    }
+                }
+        }
+        st_pair_if((T2 *)p.F + ((size_t)fc[m] * p.Nv + k), og, oh, out);
     }
-    T so = fc.on * s;
-    T2 in;
-    if (so <= (T)0) {
-        const T *bG = (const T *)p.bdevG + (size_t)fc.side * p.Nv;
-        const T *bH = (const T *)p.bdevH + (size_t)fc.side * p.Nv;
-        T gref = vgref<T>(p, k);
-        in.x = rhow * bG[k] + rwm1 * gref;
-        in.y = rhow * bH[k] + rwm1 * (T)(p.K * p.RT_r) * gref;
-        if (so < (T)0) return in;
-    }
-    T2 fb = reconstruct<T, LIM>(p, fc.rec[0], k, ux, uy, h);
-    if (so == (T)0) {
-        fb.x = (T)0.5 * (fb.x + in.x);
-        fb.y = (T)0.5 * (fb.y + in.y);
-    }
-    return fb;
 }
 
 // Linearised wall (Eq. 33-35), at a wall face f: the outgoing sum
@@ -963,7 +930,7 @@ __device__ __noinline__ void wall_ghost_density(const KParams &p, int f, int lan
     a[0].zero();
     vel_loop<1, T>(p.Nv, lane, a, [&](int k, T(&q)[1]) {
         const T so = on * xi_dot_n<T>(vx<T>(p, k), vy<T>(p, k), nx, ny);
-        if (so > (T)0) q[0] += vw<T>(p, k) * so * fc0[k].x;
+        if (so > (T)0) q[0] = mad(vw<T>(p, k) * so, fc0[k].x, q[0]);
     });
     a[0].warp_sum();
     const double sn = __shfl_sync(0xffffffffu, a[0].value(), 0);
@@ -973,94 +940,95 @@ __device__ __noinline__ void wall_ghost_density(const KParams &p, int f, int lan
     }
 }
 
-// raw moments of fb - M_ref at every face (plus the wall density, Eq. 35).
-// float32: the kernel is bound by the latency of its stencil loads, so
-// occupancy decides: four 256-thread blocks per SM (64 registers, the lanes'
-// float-float accumulators in shared memory, two velocities per lane); three
-// or two blocks without spills, or five, six and eight with more, were slower
-template <class T, bool LIM>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_moments(Launch L)
+// raw moments of fb - M_ref at every face (plus the wall density, Eq. 35), a
+// warp per face.  k_cell_recon left fb in the face buffer, except what enters
+// through a boundary face -- the wall Maxwellian rho_w M_w or the far-field
+// state, formed and stored here -- and the R side of the ties.
+template <class T, class LT>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_moments(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     using T2 = typename V2<T>::t;
-    __shared__ SideRec<T> srec[8][2];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int f = blk * 8 + wid;
     if (f >= p.nf) return;  // whole warp
-    FaceCtx<T> fc;
-    load_face<T>(p, f, srec[wid], fc);
-    const T h = (T)p.h;
-    T rhow = (T)1, rwm1 = (T)0;
-    double rw = 1.0;
+    const T *geo = (const T *)p.fgeoT + 8 * f;
+    const T nx = geo[0], ny = geo[1];
+    const int kind = p.fbc[f];  // -1 interior, 1 wall, 2 far field
+    T2 *Fo = (T2 *)p.F + (size_t)f * p.Nv;
     Acc<T> outsum[1];
     outsum[0].zero();
-    if (fc.kind == 1) {
-        // zero net mass flux: rho_w sum_in w |xi.n| G_w = sum_out w (xi.n) fb
-        vel_loop<1, T>(p.Nv, lane, outsum, [&](int k, T(&a)[1]) {
-            T ux = vx<T>(p, k), uy = vy<T>(p, k);
-            T so = fc.on * xi_dot_n<T>(ux, uy, fc.nx, fc.ny);
-            if (so > (T)0) {
-                T2 fb = reconstruct<T, LIM>(p, fc.rec[0], k, ux, uy, h);
-                a[0] += vw<T>(p, k) * so * fb.x;
-            }
-        });
-        outsum[0].warp_sum();
-        double o = __shfl_sync(0xffffffffu, outsum[0].value(), 0);
-        const double *bc = p.bconst + 2 * f;
-        rw = (bc[0] + o) / bc[1];
-        rhow = (T)rw;
-        rwm1 = (T)((bc[0] - bc[1] + o) / bc[1]);
-        if (p.implicit_wall) wall_ghost_density<T>(p, f, lane, fc.rec[0].c, fc.on, fc.nx, fc.ny, bc[1]);
-    }
-    // fb - M_ref is kept in the face-flux buffer for k_face_flux
-    T2 *Fo = (T2 *)p.F + (size_t)f * p.Nv;
+    double rw = 1.0;
     Acc<T> acc[kRaw];
-    auto body = [&](int k, T(&a)[kRaw]) {
-        T ux = vx<T>(p, k), uy = vy<T>(p, k);
-        T s = xi_dot_n<T>(ux, uy, fc.nx, fc.ny);
-        T2 fb = face_fbar<T, LIM>(p, fc, k, ux, uy, s, rhow, rwm1);
-        Fo[k] = fb;
-        raw_terms<T>(a, vw<T>(p, k), ux, uy, fb.x, fb.y);
-    };
-    // velocity pairs: at an interior face whose two velocities are upwind
-    // from the same side (no tie) one pair reconstruction; else per velocity
-    auto body2 = [&](int k, T(&a)[kRaw]) {
-        T ux[2], uy[2], w[2], s[2], g[2], hh[2];
-        vtab2<T>(p.uxf, p.ux, k, ux);
-        vtab2<T>(p.uyf, p.uy, k, uy);
-        vtab2<T>(p.wf, p.w, k, w);
-        s[0] = xi_dot_n<T>(ux[0], uy[0], fc.nx, fc.ny);
-        s[1] = xi_dot_n<T>(ux[1], uy[1], fc.nx, fc.ny);
-        const bool up0 = s[0] > (T)0, up1 = s[1] > (T)0;
-        if (fc.kind < 0 && up0 == up1 && s[0] != (T)0 && s[1] != (T)0) {
-            reconstruct2<T, LIM>(p, fc.rec[up0 ? 0 : 1], k, ux, uy, h, g, hh);
-        } else {
+#pragma unroll
+    for (int q = 0; q < kRaw; ++q) acc[q].zero();
+    if (kind < 0) {
+        const T2 *tb = (const T2 *)p.ftie + (size_t)f * max(p.nvx, p.nvy);
+        auto body = [&](int k, T(&a)[kRaw]) {
+            T ux[2], uy[2], w[2], g[2], h[2];
+            vtab2<T>(p.uxf, p.ux, k, ux);
+            vtab2<T>(p.uyf, p.uy, k, uy);
+            vtab2<T>(p.wf, p.w, k, w);
+            load_pair<T>(Fo, k, g, h);
 #pragma unroll
             for (int v = 0; v < 2; ++v) {
-                const T2 fb = face_fbar<T, LIM>(p, fc, k + v, ux[v], uy[v], s[v], rhow, rwm1);
-                g[v] = fb.x;
-                hh[v] = fb.y;
+                if (xi_dot_n<T>(ux[v], uy[v], nx, ny) == (T)0 && k + v < p.nvx * p.nvy) {
+                    // average of both sides (the flux there is zero: fb itself is not needed again)
+                    const T2 r = tb[tie_slot<T>(p, k + v, nx, ny)];
+                    g[v] = (T)0.5 * (g[v] + r.x);
+                    h[v] = (T)0.5 * (h[v] + r.y);
+                }
+                raw_terms<T>(a, w[v], ux[v], uy[v], g[v], h[v]);
             }
+        };
+        if constexpr (sizeof(T) == 4) {
+            __shared__ FF sacc[kRaw * 256];
+            vel_loop2_sm<kRaw>(p.Nv, lane, acc, sacc, body);
+        } else {
+            vel_loop2<kRaw, T>(p.Nv, lane, acc, body);
         }
-        store_pair<T>(Fo, k, g, hh);
-        raw_terms<T>(a, w[0], ux[0], uy[0], g[0], hh[0]);
-        raw_terms<T>(a, w[1], ux[1], uy[1], g[1], hh[1]);
-    };
-    if constexpr (sizeof(T) == 4) {
-        __shared__ FF sacc[kRaw * 256];
-        vel_loop2_sm<kRaw>(p.Nv, lane, sacc, body2);
-#pragma unroll
-        for (int q = 0; q < kRaw; ++q) acc[q].v = sacc[q * blockDim.x + threadIdx.x];
     } else {
-#pragma unroll
-        for (int q = 0; q < kRaw; ++q) acc[q].zero();
-        vel_loop<kRaw, T>(p.Nv, lane, acc, body);
+        const int lc = p.fL[f], c = lc >= 0 ? lc : p.fR[f], side = p.fside[f];
+        const T on = lc >= 0 ? (T)1 : (T)-1;
+        T rhow = (T)1, rwm1 = (T)0;
+        if (kind == 1) {
+            // zero net mass flux: rho_w sum_in w |xi.n| G_w = sum_out w (xi.n) fb
+            vel_loop<1, T>(p.Nv, lane, outsum, [&](int k, T(&a)[1]) {
+                const T so = on * xi_dot_n<T>(vx<T>(p, k), vy<T>(p, k), nx, ny);
+                if (so > (T)0) a[0] = mad(vw<T>(p, k) * so, Fo[k].x, a[0]);
+            });
+            outsum[0].warp_sum();
+            const double o = __shfl_sync(0xffffffffu, outsum[0].value(), 0);
+            const double *bc = p.bconst + 2 * f;
+            rw = (bc[0] + o) / bc[1];
+            rhow = (T)rw;
+            rwm1 = (T)((bc[0] - bc[1] + o) / bc[1]);
+            if (p.implicit_wall) wall_ghost_density<T>(p, f, lane, c, on, nx, ny, bc[1]);
+        }
+        const T *bG = (const T *)p.bdevG + (size_t)side * p.Nv, *bH = (const T *)p.bdevH + (size_t)side * p.Nv;
+        const T kRTr = (T)(p.K * p.RT_r);
+        vel_loop<kRaw, T>(p.Nv, lane, acc, [&](int k, T(&a)[kRaw]) {
+            const T ux = vx<T>(p, k), uy = vy<T>(p, k), so = on * xi_dot_n<T>(ux, uy, nx, ny);
+            T2 fb;
+            if (so >= (T)0) fb = Fo[k];
+            if (so <= (T)0) {
+                const T gref = vgref<T>(p, k);
+                T2 in;
+                in.x = mad(rhow, bG[k], rwm1 * gref);
+                in.y = mad(rhow, bH[k], rwm1 * (kRTr * gref));
+                if (so < (T)0) {
+                    fb = in;
+                } else {
+                    fb.x = (T)0.5 * (fb.x + in.x);
+                    fb.y = (T)0.5 * (fb.y + in.y);
+                }
+                Fo[k] = fb;
+            }
+            raw_terms<T>(a, vw<T>(p, k), ux, uy, fb.x, fb.y);
+        });
     }
-#pragma unroll
-    for (int q = 0; q < kRaw; ++q) acc[q].warp_sum();
+    warp_sum_store<kRaw, T>(acc, lane, p.faceraw, (size_t)f * 12);
     if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < kRaw; ++q) acc[q].store(p.faceraw, (size_t)f * 12 + q);
         outsum[0].store(p.faceraw, (size_t)f * 12 + 11);
         p.facerw[f] = rw;
     }
@@ -1068,16 +1036,16 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_moments(La
 
 // per face: state from the moments of fb, tau, q = 2 tau qbar/(2 tau + h Pr),
 // equilibrium, and the weights a, b of f = a fb + b f^S (Eq. 18)
-template <class T>
-__global__ void __launch_bounds__(32) k_face_params(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(32) k_face_params(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     const int f = blk * blockDim.x + threadIdx.x;
     if (f >= p.nf) return;
     double r[kRaw];
     for (int q = 0; q < kRaw; ++q) r[q] = acc_load<T>(p.faceraw, (size_t)f * 12 + q) + p.mref_raw[q];
-    double rho, U, V, RT, qbx, qby;
-    raw_to_state(r, p.K, rho, U, V, RT, qbx, qby);
+    double rho, irho, U, V, RT, qbx, qby;
+    raw_to_state(p, r, rho, irho, U, V, RT, qbx, qby);
     T *fA = (T *)p.faceA + kCellP * f;
     // float32 storage keeps fb relative to the reference Maxwellian, so a
     // face that an impulsive start evacuates (density ~1e-18 of the reference
@@ -1086,24 +1054,23 @@ __global__ void __launch_bounds__(32) k_face_params(Launch L)
     // or temperature such a face takes the vacuum limit of Eq. (18):
     // tau -> infinity, f = fb (free transport), no equilibrium part.
     if (sizeof(T) == 4 && !(rho > 1e-6 * p.rho_r && RT > 1e-6 * p.RT_r)) {
-        eq_storeT<T>(fA, make_eq(p, 0.0, p.U_r, p.V_r, p.RT_r, 0.0, 0.0));
+        eq_storeT<T>(fA, make_eq(p, 0.0, 0.0, p.U_r, p.V_r, p.RT_r, p.iRT_r, 0.0, 0.0));
         fA[14] = (T)1;
         fA[15] = (T)0;
         return;
     }
-    double tau = viscosity_t<T>(p, RT) / (rho * RT);
-    double Pr = p.shakhov ? p.Pr : 1.0;
-    double qx = 2.0 * tau * qbx / (2.0 * tau + p.h * Pr);
-    double qy = 2.0 * tau * qby / (2.0 * tau + p.h * Pr);
-    eq_storeT<T>(fA, make_eq(p, rho, U, V, RT, qx, qy));
-    fA[14] = (T)(2.0 * tau / (2.0 * tau + p.h));
-    fA[15] = (T)(p.h / (2.0 * tau + p.h));
+    const double ir = rcp_rn(RT), tau2 = 2.0 * viscosity_t<T>(p, RT) * (irho * ir);  // 2 tau
+    const double Pr = p.shakhov ? p.Pr : 1.0, fq = tau2 * rcp_rn(tau2 + p.h * Pr);
+    eq_storeT<T>(fA, make_eq(p, rho, irho, U, V, RT, ir, fq * qbx, fq * qby));
+    const double fd = rcp_rn(tau2 + p.h);
+    fA[14] = (T)(tau2 * fd);
+    fA[15] = (T)(p.h * fd);
 }
 
 // face flux of (f_face - M_ref), Eq. (18)-(19), and its moments; fb - M_ref
 // comes from k_face_moments through the same buffer and is overwritten
-template <class T>
-__global__ void __launch_bounds__(256) k_face_flux(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_flux(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     using T2 = typename V2<T>::t;
@@ -1132,21 +1099,17 @@ __global__ void __launch_bounds__(256) k_face_flux(Launch L)
             T dG, dH;
             dev_equilibrium<T>(e, ux[v], uy[v], gr[v], kRTr, dG, dH);
             T sS = s * S;
-            fg[v] = sS * (wa * fg[v] + wb * dG);
-            fh[v] = sS * (wa * fh[v] + wb * dH);
+            fg[v] = sS * mad(wa, fg[v], wb * dG);
+            fh[v] = sS * mad(wa, fh[v], wb * dH);
             T wg = w[v] * fg[v];
             a[0] += wg;
-            a[1] += wg * ux[v];
-            a[2] += wg * uy[v];
-            a[3] += (T)0.5 * w[v] * ((ux[v] * ux[v] + uy[v] * uy[v]) * fg[v] + fh[v]);
+            a[1] = mad(wg, ux[v], a[1]);
+            a[2] = mad(wg, uy[v], a[2]);
+            a[3] = mad((T)0.5 * w[v], mad(mad(ux[v], ux[v], uy[v] * uy[v]), fg[v], fh[v]), a[3]);
         }
         store_pair<T>(Fo, k, fg, fh);
     });
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[q].warp_sum();
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q].store(p.phiraw, (size_t)f * 4 + q);
+    warp_sum_store<4, T>(acc, lane, p.phiraw, (size_t)f * 4);
     if (p.implicit_wall && p.fbc[f] == 1) {
         // linearised wall (Eq. 33-35): the ghost increment drho_g M_w of the
         // incoming velocities enters the micro sweeps as the upwind term
@@ -1163,8 +1126,8 @@ __global__ void __launch_bounds__(256) k_face_flux(Launch L)
                 if (on * sn < (T)0) {
                     const T a = sn * SD, gr = vgref<T>(p, k);
                     T2 v = Fo[k];
-                    v.x += a * (bG[k] + gr);
-                    v.y += a * (bH[k] + kRTr * gr);
+                    v.x = mad(a, bG[k] + gr, v.x);
+                    v.y = mad(a, mad(kRTr, gr, bH[k]), v.y);
                     Fo[k] = v;
                 }
             }
@@ -1174,8 +1137,8 @@ __global__ void __launch_bounds__(256) k_face_flux(Launch L)
 
 // Phi_f = sum_k w psi F_k (Eq. 27): deviation part plus the flux of M_ref;
 // the mass flux through an impermeable wall is exactly zero
-template <class T>
-__global__ void __launch_bounds__(256) k_face_phi(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(256) k_face_phi(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     const int f = blk * blockDim.x + threadIdx.x;
@@ -1200,59 +1163,23 @@ __global__ void __launch_bounds__(256) k_face_phi(Launch L)
 //   k_macro_post   (all cells): W^{n+1} = W + dW (Eq. 32) in float64 and the
 //                  micro coefficients at the predicted state
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void prim_uvc(const KParams &p, const double *W, double &u, double &v,
-                                         double &cs)
+// velocity and sound speed of a cell for the face spectral radii.  In float32
+// storage the spectral radius and the neighbours' base states only enter the
+// float32 wavefront (R_W, the diagonal's sum and W^{n+1} stay float64), so they
+// are evaluated in float32; float64 storage evaluates them in float64.
+__device__ __forceinline__ void prim_uvc(const KParams &p, const double *W, double &u, double &v, double &cs)
 {
-    double rho = W[0];
-    u = W[1] / rho;
-    v = W[2] / rho;
-    double RT = (2.0 * W[3] / rho - u * u - v * v) / (p.K + 2);
-    cs = sqrt(p.gam * RT);
+    const double irho = rcp_rn(W[0]);
+    u = W[1] * irho;
+    v = W[2] * irho;
+    cs = sqrt(p.gam * ((2.0 * W[3] * irho - u * u - v * v) * p.iK2));
 }
-
-__device__ __forceinline__ double face_lambda(const KParams &p, int fi)
+__device__ __forceinline__ void prim_uvc(const KParams &p, const double *W, float &u, float &v, float &cs)
 {
-    int L = p.fL[fi], R = p.fR[fi];
-    const double *g = p.fgeo + 7 * fi;
-    double u, v, cs;
-    if (L >= 0 && R >= 0) {
-        double u1, v1, c1, u2, v2, c2;
-        prim_uvc(p, p.W + 4 * L, u1, v1, c1);
-        prim_uvc(p, p.W + 4 * R, u2, v2, c2);
-        u = 0.5 * (u1 + u2); v = 0.5 * (v1 + v2); cs = 0.5 * (c1 + c2);
-    } else {
-        prim_uvc(p, p.W + 4 * (L >= 0 ? L : R), u, v, cs);
-    }
-    return (fabs(u * g[0] + v * g[1]) + cs) * g[2];
-}
-
-// Preconditioner coefficients of the macroscopic LU-SGS: in float32 storage
-// the spectral radius and the neighbours' base states only enter the float32
-// wavefront (R_W, the diagonal's sum and W^{n+1} stay float64), so they are
-// evaluated in float32; float64 storage evaluates them in float64.
-template <class T> __device__ __forceinline__ double face_lambda_t(const KParams &p, int fi);
-template <> __device__ __forceinline__ double face_lambda_t<double>(const KParams &p, int fi)
-{
-    return face_lambda(p, fi);
-}
-template <> __device__ __forceinline__ double face_lambda_t<float>(const KParams &p, int fi)
-{
-    const int L = p.fL[fi], R = p.fR[fi];
-    const double *g = p.fgeo + 7 * fi;
-    const float gam = (float)p.gam, k2 = 1.0f / (float)(p.K + 2);
-    float u = 0.f, v = 0.f, cs = 0.f;
-    int nc = 0;
-    for (int side = 0; side < 2; ++side) {
-        const int c = side ? R : L;
-        if (c < 0) continue;
-        const double *W = p.W + 4 * c;
-        const float rho = (float)W[0], ir = 1.0f / rho, uc = (float)W[1] * ir, vc = (float)W[2] * ir;
-        const float RT = (2.0f * (float)W[3] * ir - uc * uc - vc * vc) * k2;
-        u += uc; v += vc; cs += sqrtf(gam * RT);
-        ++nc;
-    }
-    if (nc == 2) { u *= 0.5f; v *= 0.5f; cs *= 0.5f; }
-    return (double)((fabsf(u * (float)g[0] + v * (float)g[1]) + cs) * (float)g[2]);
+    const float ir = rcp_rn((float)W[0]);
+    u = (float)W[1] * ir;
+    v = (float)W[2] * ir;
+    cs = sqrtf((float)p.gam * ((2.0f * (float)W[3] * ir - u * u - v * v) * (float)p.iK2));
 }
 
 // base state (rho, m_x, m_y, u, v, E + p) of a neighbour for the flux increments
@@ -1267,7 +1194,7 @@ template <> __device__ __forceinline__ void base_state<double>(const KParams &p,
 template <> __device__ __forceinline__ void base_state<float>(const KParams &p, const double *W, float *o)
 {
     const float rho = (float)W[0], mx = (float)W[1], my = (float)W[2], E = (float)W[3];
-    const float ir = 1.0f / rho, u = mx * ir, v = my * ir;
+    const float ir = rcp_rn(rho), u = mx * ir, v = my * ir;
     const float pr = (float)(p.gam - 1.0) * (E - 0.5f * rho * (u * u + v * v));
     o[0] = rho; o[1] = mx; o[2] = my;
     o[3] = u; o[4] = v; o[5] = E + pr;
@@ -1385,8 +1312,8 @@ constexpr int kMRing = 12; // ring entry per cell: increment[4], base state[6], 
 // per cell: R_W, ||R_W/Omega||^2 partials, and the record of the macroscopic
 // sweep (inverse diagonal, the cell's own base state for its neighbours'
 // flux increments, per-slot face coefficients)
-template <class T>
-__global__ void __launch_bounds__(32) k_macro_pre(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(32) k_macro_pre(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     __shared__ double sm[32];
@@ -1400,25 +1327,38 @@ __global__ void __launch_bounds__(32) k_macro_pre(Launch L)
             const double *ph = p.phi + 4 * p.cface[4 * c + m];
             for (int q = 0; q < 4; ++q) acc[q] -= s * ph[q];
         }
+        const double iA = rcp_rn(p.area[c]);
         for (int q = 0; q < 4; ++q) {
             p.rw[4 * c + q] = acc[q];
             rec[q] = (T)acc[q];
-            double rr = acc[q] / p.area[c];
+            const double rr = acc[q] * iA;
             part[0] += rr * rr;
         }
-        double d = p.area[c] / p.dtimp[c];
+        double d = p.adt[c];
+        T u0, v0, c0;
+        prim_uvc(p, p.W + 4 * c, u0, v0, c0);
         for (int m = 0; m < 4; ++m) {
-            int fi = p.cface[4 * c + m];
-            double lam = face_lambda_t<T>(p, fi);
+            // spectral radius (|V.n| + c) S of Eq. (31) at the average of the
+            // face's cells (at a boundary the inner one)
+            const int nb = p.cnb[4 * c + m];
+            const double *g = p.fgeo + 7 * p.cface[4 * c + m];
+            const T nx = (T)g[0], ny = (T)g[1], S = (T)g[2];
+            T u = u0, v = v0, cs = c0;
+            if (nb >= 0) {
+                prim_uvc(p, p.W + 4 * nb, u, v, cs);
+                u = (T)0.5 * (u0 + u);
+                v = (T)0.5 * (v0 + v);
+                cs = (T)0.5 * (c0 + cs);
+            }
+            const double lam = (double)((fabs(u * nx + v * ny) + cs) * S);
             double s = p.csign[4 * c + m];  // 0: a triangle's unused slot
-            if (s != 0.0 && p.fL[fi] != p.fR[fi]) d += 0.5 * p.lusgs_omega * lam;
-            const double *g = p.fgeo + 7 * fi;
+            if (s != 0.0 && nb != c) d += 0.5 * p.lusgs_omega * lam;
             T *o = rec + 12 + 3 * m;
             o[0] = (T)(0.5 * g[2] * s * g[0]);
             o[1] = (T)(0.5 * g[2] * s * g[1]);
             o[2] = (T)(0.5 * p.lusgs_omega * lam);
         }
-        rec[4] = (T)(1.0 / d);
+        rec[4] = (T)rcp_rn(d);
         rec[5] = (T)0;
         base_state<T>(p, p.W + 4 * c, rec + 6);
         if (by_lines(p)) {
@@ -1468,16 +1408,16 @@ __device__ __forceinline__ void record_residual(const KParams &p)
 template <class T>
 __device__ __forceinline__ void euler_dflux(T gm1, const T *b, const T *dW, T nx, T ny, T *dF)
 {
-    T rho = b[0], mx = b[1], my = b[2], u = b[3], v = b[4], H = b[5];
-    T ir1 = rcp_rn(rho + dW[0]);
-    T du = (dW[1] - u * dW[0]) * ir1, dv = (dW[2] - v * dW[0]) * ir1;
-    T vn = u * nx + v * ny, dvn = du * nx + dv * ny, vn1 = vn + dvn;
-    T dmu = dW[1] * (u + du) + dW[2] * (v + dv) + mx * du + my * dv;
-    T dp = gm1 * (dW[3] - (T)0.5 * dmu);
-    dF[0] = dW[0] * vn1 + rho * dvn;
-    dF[1] = dW[1] * vn1 + mx * dvn + dp * nx;
-    dF[2] = dW[2] * vn1 + my * dvn + dp * ny;
-    dF[3] = (dW[3] + dp) * vn1 + H * dvn;
+    const T rho = b[0], mx = b[1], my = b[2], u = b[3], v = b[4], H = b[5];
+    const T ir1 = rcp_rn(rho + dW[0]);
+    const T du = mad(-u, dW[0], dW[1]) * ir1, dv = mad(-v, dW[0], dW[2]) * ir1;
+    const T dvn = mad(du, nx, dv * ny), vn1 = mad(u, nx, v * ny) + dvn;
+    const T dmu = mad(dW[1], u + du, mad(dW[2], v + dv, mad(mx, du, my * dv)));
+    const T dp = gm1 * mad((T)-0.5, dmu, dW[3]);
+    dF[0] = mad(dW[0], vn1, rho * dvn);
+    dF[1] = mad(dW[1], vn1, mad(mx, dvn, dp * nx));
+    dF[2] = mad(dW[2], vn1, mad(my, dvn, dp * ny));
+    dF[3] = mad(dW[3] + dp, vn1, H * dvn);
 }
 
 // One CTA: forward then backward sweep over the i+j hyperplanes (the
@@ -1573,10 +1513,10 @@ __global__ void __launch_bounds__(512) k_macro_sweep(Launch L)
                     const T *cf = rec + 12 + 3 * m;
                     T dF[4];
                     euler_dflux<T>(gm1, base, dn, cf[0], cf[1], dF);
-                    acc0 += dF[0] - cf[2] * dn[0];
-                    acc1 += dF[1] - cf[2] * dn[1];
-                    acc2 += dF[2] - cf[2] * dn[2];
-                    acc3 += dF[3] - cf[2] * dn[3];
+                    acc0 += mad(-cf[2], dn[0], dF[0]);
+                    acc1 += mad(-cf[2], dn[1], dF[1]);
+                    acc2 += mad(-cf[2], dn[2], dF[2]);
+                    acc3 += mad(-cf[2], dn[3], dF[3]);
                 }
             }
             // sum over the two slot pairs of the cell
@@ -1594,8 +1534,8 @@ __global__ void __launch_bounds__(512) k_macro_sweep(Launch L)
                     x0 = (rec[q0] - a0) * iD;
                     x1 = (rec[q0 + 1] - a1) * iD;
                 } else {
-                    x0 = sdw[e * 4 + q0] - a0 * iD;
-                    x1 = sdw[e * 4 + q0 + 1] - a1 * iD;
+                    x0 = mad(-a0, iD, sdw[e * 4 + q0]);
+                    x1 = mad(-a1, iD, sdw[e * 4 + q0 + 1]);
                 }
                 T *r = ring + ((size_t)(s & 1) * ncs + cs) * kMRing;
                 r[q0] = x0;
@@ -1655,9 +1595,9 @@ template <class T> __device__ __forceinline__ void line_inc(LineInc<T> &x, T gm1
 {
     x.rho = b[1]; x.mx = b[2]; x.my = b[3]; x.u = x.mx * c[0]; x.v = x.my * c[0]; x.H = c[1];
     x.ir = rcp_line(x.rho + x.dW[0]);
-    const T k = x.mx * x.u + x.my * x.v;
-    const T q = ((T)2 * x.mx + x.dW[1]) * x.dW[1] + (((T)2 * x.my + x.dW[2]) * x.dW[2] - k * x.dW[0]);
-    x.dp = gm1 * x.dW[3] - ((T)0.5 * gm1 * q) * x.ir;
+    const T k = mad(x.mx, x.u, x.my * x.v);
+    const T q = mad(mad((T)2, x.mx, x.dW[1]), x.dW[1], mad(mad((T)2, x.my, x.dW[2]), x.dW[2], -k * x.dW[0]));
+    x.dp = mad((T)-0.5 * gm1 * q, x.ir, gm1 * x.dW[3]);
 }
 // the term 1/2 (dF S - omega Lambda dW) of this cell's increment in the
 // equation of the neighbour across the face with S/2 n out of this cell
@@ -1665,13 +1605,13 @@ template <class T> __device__ __forceinline__ void line_inc(LineInc<T> &x, T gm1
 template <class T> __device__ __forceinline__ void line_term(const LineInc<T> &x, T ox, T oy, T ol, T (&o)[4])
 {
     const T nx = -ox, ny = -oy;
-    const T vn = x.u * nx + x.v * ny;
-    const T dm = x.dW[1] * nx + x.dW[2] * ny;
-    const T dvn = (dm - vn * x.dW[0]) * x.ir, vn1 = vn + dvn;
-    o[0] = dm - ol * x.dW[0];
-    o[1] = x.dW[1] * vn1 + (x.mx * dvn + (x.dp * nx - ol * x.dW[1]));
-    o[2] = x.dW[2] * vn1 + (x.my * dvn + (x.dp * ny - ol * x.dW[2]));
-    o[3] = (x.dW[3] + x.dp) * vn1 + (x.H * dvn - ol * x.dW[3]);
+    const T vn = mad(x.u, nx, x.v * ny);
+    const T dm = mad(x.dW[1], nx, x.dW[2] * ny);
+    const T dvn = mad(-vn, x.dW[0], dm) * x.ir, vn1 = vn + dvn;
+    o[0] = mad(-ol, x.dW[0], dm);
+    o[1] = mad(x.dW[1], vn1, mad(x.mx, dvn, mad(x.dp, nx, -ol * x.dW[1])));
+    o[2] = mad(x.dW[2], vn1, mad(x.my, dvn, mad(x.dp, ny, -ol * x.dW[2])));
+    o[3] = mad(x.dW[3] + x.dp, vn1, mad(x.H, dvn, -ol * x.dW[3]));
 }
 
 // what a sweep of k_macro_lines reads that does not change
@@ -1752,7 +1692,7 @@ template <class T, int kStages, bool FWD, bool SEAM> __device__ __forceinline__ 
                 if (SEAM && x.per_w && ww == x.nw - 1) acc += first[q];
                 if (SEAM && x.per_t && tt == x.nt - 1 && (unsigned)ww < nwl) acc += x.seam[4 * ww + q];
                 // forward: dW*_c = (R_c - sum_lower) / D_c;  backward: dW_c = dW*_c - sum_upper / D_c
-                inc.dW[q] = FWD ? (r[q] - acc) * rb[0] : r[q] - acc * rb[0];
+                inc.dW[q] = FWD ? (r[q] - acc) * rb[0] : mad(-acc, rb[0], r[q]);
             }
             line_inc<T>(inc, x.gm1, rb, rc);
             line_term<T>(inc, rd[0], rd[1], rc[2], to_w);
@@ -1897,12 +1837,12 @@ __global__ void __launch_bounds__(256) k_macro_sweep_sched(Launch L)
                     T dF[4];
                     euler_dflux<T>(gm1, cur.base[m], dn, cur.cf[3 * m], cur.cf[3 * m + 1], dF);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) acc[q] += dF[q] - cur.cf[3 * m + 2] * dn[q];
+                    for (int q = 0; q < 4; ++q) acc[q] += mad(-cur.cf[3 * m + 2], dn[q], dF[q]);
                 }
                 // forward: dW*_c = (R_c - sum_lower) / D_c;  backward: dW_c = dW*_c - sum_upper / D_c
                 T *o = dw + 4 * (size_t)cur.c;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) o[q] = dir > 0 ? (cur.r[q] - acc[q]) * cur.iD : o[q] - acc[q] * cur.iD;
+                for (int q = 0; q < 4; ++q) o[q] = dir > 0 ? (cur.r[q] - acc[q]) * cur.iD : mad(-acc[q], cur.iD, o[q]);
             }
             cur = nxt;
         }
@@ -1913,8 +1853,8 @@ __global__ void __launch_bounds__(256) k_macro_sweep_sched(Launch L)
     if (threadIdx.x == 0) *p.iter += 1;
 }
 
-template <class T>
-__global__ void __launch_bounds__(32) k_macro_post(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(32) k_macro_post(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     const int c = blk * blockDim.x + threadIdx.x;
@@ -1922,22 +1862,20 @@ __global__ void __launch_bounds__(32) k_macro_post(Launch L)
     double *W = p.W + 4 * c;
     const T *dW = (const T *)p.mdW + 4 * (by_lines(p) ? line_slot(p, c) : c);
     for (int q = 0; q < 4; ++q) W[q] += (double)dW[q];
-    double rho = W[0], U = W[1] / rho, V = W[2] / rho;
-    double RT = (2.0 * W[3] / rho - U * U - V * V) / (p.K + 2);
-    double taup = viscosity_t<T>(p, RT) / (rho * RT);
-    EqD e = make_eq(p, rho, U, V, RT, p.cellq[2 * c], p.cellq[2 * c + 1]);
-    double *cp = p.cellp + kCellP * c;
-    eq_store(cp, e);
-    double cq = 2.0 * p.area[c] / (2.0 * taup + p.dt);
-    cp[14] = cq;
-    cp[15] = p.area[c] / p.dtimp[c] + cq;
+    const double rho = W[0], irho = rcp_rn(rho), U = W[1] * irho, V = W[2] * irho;
+    const double RT = mad(-V, V, mad(-U, U, 2.0 * W[3] * irho)) * p.iK2, ir = rcp_rn(RT);
+    const double tau2 = 2.0 * viscosity_t<T>(p, RT) * (irho * ir);  // 2 tau'
     T *ct = (T *)p.cellpT + kCellP * c;
-    for (int q = 0; q < kCellP; ++q) ct[q] = (T)cp[q];
+    eq_storeT<T>(ct, make_eq(p, rho, irho, U, V, RT, ir, p.cellq[2 * c], p.cellq[2 * c + 1]));
+    const double cq = 2.0 * p.area[c] * rcp_rn(tau2 + p.dt);
+    const T D0 = (T)(p.adt[c] + cq);  // diagonal base of Eq. (26)
+    ct[14] = (T)cq;
+    ct[15] = D0;
     if (p.sgeo) {
-        // the diagonal base where both line sweeps read it
+        // where both line sweeps read it
         T *sg = (T *)p.sgeo + 8 * (size_t)c + 6;
-        sg[0] = (T)cp[15];
-        sg[8 * (size_t)p.N] = (T)cp[15];
+        sg[0] = D0;
+        sg[8 * (size_t)p.N] = D0;
     }
 }
 
@@ -1949,8 +1887,8 @@ __global__ void __launch_bounds__(32) k_macro_post(Launch L)
 // last one leaves dW in mdW for k_macro_post; sweep 1 gives dW = R / D.  The
 // record of k_macro_pre holds R, 1/D, the cell's base state and per slot
 // (S/2) n_out and (omega/2) Lambda, as for the sweeps.
-template <class T>
-__global__ void __launch_bounds__(32) k_macro_relax(Launch L, int sweep, int nsweeps)
+template <class T, class LT>
+__global__ void __launch_bounds__(32) k_macro_relax(const __grid_constant__ LT L, int sweep, int nsweeps)
 {
     IDG_LOCATE();
     const int c = blk * blockDim.x + threadIdx.x;
@@ -1973,7 +1911,7 @@ __global__ void __launch_bounds__(32) k_macro_relax(Launch L, int sweep, int nsw
             T dF[4];
             euler_dflux<T>(gm1, mrec + (size_t)kMRec * nb + 6, dn, cf[0], cf[1], dF);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += dF[q] - cf[2] * dn[q];
+            for (int q = 0; q < 4; ++q) acc[q] += mad(-cf[2], dn[q], dF[q]);
         }
     }
     const T iD = rec[4];
@@ -1998,8 +1936,8 @@ __global__ void __launch_bounds__(32) k_macro_relax(Launch L, int sweep, int nsw
 
 // one thread per instance: the residual of this iteration from the block
 // partials of the kernel before it into the ring, and the iteration count
-template <class T>
-__global__ void __launch_bounds__(32) k_record_residual(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(32) k_record_residual(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     (void)blk;
@@ -2007,8 +1945,8 @@ __global__ void __launch_bounds__(32) k_record_residual(Launch L)
     if (threadIdx.x == 0) *p.iter += 1;
 }
 
-template <class T>
-__global__ void __launch_bounds__(128) k_explicit_update(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(128) k_explicit_update(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     const int nvb = (p.Nv + 255) / 256;
@@ -2032,8 +1970,8 @@ __global__ void __launch_bounds__(128) k_explicit_update(Launch L)
         const T sg = (T)p.csign[4 * c + m];
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
-            sg_[v] += sg * fg[v];
-            sh_[v] += sg * fh[v];
+            sg_[v] = mad(sg, fg[v], sg_[v]);
+            sh_[v] = mad(sg, fh[v], sh_[v]);
         }
     }
     const size_t ck = (size_t)c * p.Nv + k;
@@ -2043,16 +1981,16 @@ __global__ void __launch_bounds__(128) k_explicit_update(Launch L)
     for (int v = 0; v < 2; ++v) {
         T dG, dH;
         dev_equilibrium<T>(e, ux[v], uy[v], gr[v], kRTr, dG, dH);
-        g[v] = a * g[v] + b * dG - dto * sg_[v];
-        h[v] = a * h[v] + b * dH - dto * sh_[v];
+        g[v] = mad(-dto, sg_[v], mad(a, g[v], b * dG));
+        h[v] = mad(-dto, sh_[v], mad(a, h[v], b * dH));
     }
     store_pair<T>(p.f, ck, g, h);
 }
 
 // W = (rho, rho U, rho V, rho E) of f~ from its raw moments (Eq. 4), and
 // block partials of ||(W_new - W_old)/dt||^2 (fixed order)
-template <class T>
-__global__ void __launch_bounds__(32) k_explicit_w(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(32) k_explicit_w(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     __shared__ double sm[32];
@@ -2086,8 +2024,8 @@ __global__ void __launch_bounds__(32) k_explicit_w(Launch L)
 // tile of sweep_tv velocities, a thread per (cell of the step, velocity),
 // everything but the neighbours' increments copied kStages-1 steps ahead).
 // ---------------------------------------------------------------------------
-template <class T>
-__global__ void __launch_bounds__(128) k_micro_residual(Launch L)
+template <class T, class LT>
+__global__ void __launch_bounds__(128) k_micro_residual(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     const int nvb = (p.Nv + 255) / 256;
@@ -2118,8 +2056,8 @@ __global__ void __launch_bounds__(128) k_micro_residual(Launch L)
         const T sg = (T)p.csign[4 * c + m];
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
-            rg[v] -= sg * fg[v];
-            rh[v] -= sg * fh[v];
+            rg[v] = mad(-sg, fg[v], rg[v]);
+            rh[v] = mad(-sg, fh[v], rh[v]);
         }
     }
     store_pair<T>(p.dst, ck, rg, rh);
@@ -2318,8 +2256,8 @@ __global__ void __launch_bounds__(512) k_sweep(Launch L)
             T ag = 0, ah = 0;
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
-                ag -= aS[m] * dn[m].x;
-                ah -= aS[m] * dn[m].y;
+                ag = mad(-aS[m], dn[m].x, ag);
+                ah = mad(-aS[m], dn[m].y, ah);
             }
             const T2 r = sm.R[rbase + v];
             const T iD = rcp_rn(D);
@@ -2328,8 +2266,8 @@ __global__ void __launch_bounds__(512) k_sweep(Launch L)
                 o.x = (r.x + ag) * iD;
                 o.y = (r.y + ah) * iD;
             } else {
-                o.x = r.x + ag * iD;
-                o.y = r.y + ah * iD;
+                o.x = mad(ag, iD, r.x);
+                o.y = mad(ah, iD, r.y);
                 T2 fv = sm.F[rbase + v];
                 fv.x += o.x;
                 fv.y += o.y;
@@ -2548,7 +2486,7 @@ __global__ void __launch_bounds__(512) k_sweep_lines(Launch L)
             const T upp = xi_dot_n<T>(ux[v], uy[v], q[4], q[5]);
             // D = base + sum of the outflow (xi.n) S: half the sum of all
             // |xi.n| S, the cell's outward normals summing to zero
-            const T D = q[6] + (T)0.5 * ((fabs(own) + fabs(ahead[v])) + (fabs(low) + fabs(upp)));
+            const T D = mad((T)0.5, (fabs(own) + fabs(ahead[v])) + (fabs(low) + fabs(upp)), q[6]);
             iD[v] = rcp_nr(D);
             cl[v] = low < (T)0 && has_adj ? -low : (T)0;
             co[v] = own < (T)0 && ww > 0 ? -own : (T)0;
@@ -2595,26 +2533,26 @@ __global__ void __launch_bounds__(512) k_sweep_lines(Launch L)
                 adj.y = edge ? ev[v].y : adj.y;
                 // inflow from the swept side adds |xi.n| S Delta_nb
                 T ag = co[v] * prev[v].x, ah = co[v] * prev[v].y;
-                ag += cl[v] * adj.x;
-                ah += cl[v] * adj.y;
+                ag = mad(cl[v], adj.x, ag);
+                ah = mad(cl[v], adj.y, ah);
                 if (SEAM) {
                     if (ca[v] > (T)0) {
-                        ag += ca[v] * first[v].x;
-                        ah += ca[v] * first[v].y;
+                        ag = mad(ca[v], first[v].x, ag);
+                        ah = mad(ca[v], first[v].y, ah);
                     }
                     if (on && cu[v] > (T)0) {
                         const int nb = (FWD ? 0 : nt - 1) - t;  // lines to the first line of the sweep
                         const T2 dn = ds[(ptrdiff_t)ww * sv + (ptrdiff_t)nb * (cols ? 1 : p.ni) * Nv + v];
-                        ag += cu[v] * dn.x;
-                        ah += cu[v] * dn.y;
+                        ag = mad(cu[v], dn.x, ag);
+                        ah = mad(cu[v], dn.y, ah);
                     }
                 }
                 if (FWD) {
                     out[v].x = (r[v].x + ag) * iD[v];
                     out[v].y = (r[v].y + ah) * iD[v];
                 } else {
-                    out[v].x = r[v].x + ag * iD[v];
-                    out[v].y = r[v].y + ah * iD[v];
+                    out[v].x = mad(ag, iD[v], r[v].x);
+                    out[v].y = mad(ah, iD[v], r[v].y);
                     f[v].x += out[v].x;
                     f[v].y += out[v].y;
                 }
@@ -2694,18 +2632,18 @@ __global__ void __launch_bounds__(256) k_moments_out(KParams p, double *out6)
     double r[kRaw];
     for (int q = 0; q < kRaw; ++q) r[q] = acc_load<T>(p.cellraw, (size_t)c * kRaw + q) + p.mref_raw[q];
     const double *W = p.W + 4 * c;
-    double rho = W[0], U = W[1] / rho, V = W[2] / rho;
-    double RT = (2.0 * W[3] / rho - U * U - V * V) / (p.K + 2);
-    double tau = viscosity_t<T>(p, RT) / (rho * RT);
+    const double rho = W[0], irho = rcp_rn(rho), U = W[1] * irho, V = W[2] * irho;
+    const double RT = mad(-V, V, mad(-U, U, 2.0 * W[3] * irho)) * p.iK2;
+    const double tau2 = 2.0 * viscosity_t<T>(p, RT) * (irho * rcp_rn(RT));  // 2 tau
     double qtx, qty;
     raw_heat_flux(r, U, V, qtx, qty);
-    double Pr = p.shakhov ? p.Pr : 1.0;
+    const double Pr = p.shakhov ? p.Pr : 1.0, fq = tau2 * rcp_rn(tau2 + p.dt * Pr);
     out6[6 * c + 0] = rho;
     out6[6 * c + 1] = U;
     out6[6 * c + 2] = V;
-    out6[6 * c + 3] = RT / p.RT_ref;
-    out6[6 * c + 4] = 2.0 * tau * qtx / (2.0 * tau + p.dt * Pr);
-    out6[6 * c + 5] = 2.0 * tau * qty / (2.0 * tau + p.dt * Pr);
+    out6[6 * c + 3] = RT * p.iRT_ref;
+    out6[6 * c + 4] = fq * qtx;
+    out6[6 * c + 5] = fq * qty;
 }
 
 // ---------------------------------------------------------------------------
@@ -2912,6 +2850,14 @@ template <class T> static Launch launch_of(const Plan &pl, int kt)
     return L;
 }
 
+// run(launch, blocks) of kernel type kt, for one instance by value, for a batch
+// through its tables
+template <class F> static void run_plan(const Plan &pl, int kt, F launch)
+{
+    if (pl.hparams) launch(LaunchOne{*pl.hparams}, pl.nblocks[kt]);
+    else launch(launch_of<void>(pl, kt), pl.nblocks[kt]);
+}
+
 // events (optional): kProfiled+1 cudaEvent_t recorded between the six groups
 // cell prep | face moments+params | face flux+phi | macro | residual+fwd | bwd
 template <class T>
@@ -2921,49 +2867,50 @@ static int iteration_t(const Plan &pl, cudaStream_t st, void **events)
         if (events) cudaEventRecord((cudaEvent_t)events[q], st);
     };
     auto L = [&](int kt) { return launch_of<T>(pl, kt); };
+    auto run = [&](int kt, auto launch) { run_plan(pl, kt, launch); };
     const int *nb = pl.nblocks;
     if (pl.explicit_dugks) {
         // W^n and the raw moments of f~^n are left by the previous step (or
         // by launch_explicit_prologue)
         mark(0);
-        k_cell_params<T><<<nb[KT_CELL_PAR], 32, 0, st>>>(L(KT_CELL_PAR));
-        k_fbp<T><<<nb[KT_FBP], 128, 0, st>>>(L(KT_FBP));
+        run(KT_CELL_PAR, [&](const auto &l, int nb) { k_cell_params<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
+        run(KT_FBP, [&](const auto &l, int nb) { k_fbp<T, std::decay_t<decltype(l)>><<<nb, 128, 0, st>>>(l); });
         mark(1);
-        if (pl.limiter_any) k_cell_grad<T><<<nb[KT_FBP], 128, 0, st>>>(L(KT_FBP));
-        if (pl.limiter_any) k_face_moments<T, true><<<nb[KT_FACE_MOM], 256, 0, st>>>(L(KT_FACE_MOM));
-        else k_face_moments<T, false><<<nb[KT_FACE_MOM], 256, 0, st>>>(L(KT_FACE_MOM));
-        k_face_params<T><<<nb[KT_FACE_PAR], 32, 0, st>>>(L(KT_FACE_PAR));
+        if (pl.limiter_any) run(KT_FBP, [&](const auto &l, int nb) { k_cell_recon<T, true, std::decay_t<decltype(l)>><<<nb, 128, 0, st>>>(l); });
+        else run(KT_FBP, [&](const auto &l, int nb) { k_cell_recon<T, false, std::decay_t<decltype(l)>><<<nb, 128, 0, st>>>(l); });
+        run(KT_FACE_MOM, [&](const auto &l, int nb) { k_face_moments<T, std::decay_t<decltype(l)>><<<nb, 256, 0, st>>>(l); });
+        run(KT_FACE_PAR, [&](const auto &l, int nb) { k_face_params<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
         mark(2);
-        k_face_flux<T><<<nb[KT_FACE_FLUX], 256, 0, st>>>(L(KT_FACE_FLUX));
-        k_face_phi<T><<<nb[KT_FACE_PHI], 64, 0, st>>>(L(KT_FACE_PHI));
+        run(KT_FACE_FLUX, [&](const auto &l, int nb) { k_face_flux<T, std::decay_t<decltype(l)>><<<nb, 256, 0, st>>>(l); });
+        run(KT_FACE_PHI, [&](const auto &l, int nb) { k_face_phi<T, std::decay_t<decltype(l)>><<<nb, 64, 0, st>>>(l); });
         mark(3);
         mark(4);
-        k_explicit_update<T><<<nb[KT_MICRO_RES], 128, 0, st>>>(L(KT_MICRO_RES));
-        k_cell_moments<T><<<nb[KT_CELL_MOM], 256, 0, st>>>(L(KT_CELL_MOM));
-        k_explicit_w<T><<<nb[KT_CELL_PAR], 32, 0, st>>>(L(KT_CELL_PAR));
-        k_record_residual<T><<<nb[KT_MACRO_SWEEP], 32, 0, st>>>(L(KT_MACRO_SWEEP));
+        run(KT_MICRO_RES, [&](const auto &l, int nb) { k_explicit_update<T, std::decay_t<decltype(l)>><<<nb, 128, 0, st>>>(l); });
+        run(KT_CELL_MOM, [&](const auto &l, int nb) { k_cell_moments<T, std::decay_t<decltype(l)>><<<nb, 256, 0, st>>>(l); });
+        run(KT_CELL_PAR, [&](const auto &l, int nb) { k_explicit_w<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
+        run(KT_MACRO_SWEEP, [&](const auto &l, int nb) { k_record_residual<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
         mark(5);
         mark(6);
         return (int)cudaGetLastError();
     }
     mark(0);
-    k_cell_moments<T><<<nb[KT_CELL_MOM], 256, 0, st>>>(L(KT_CELL_MOM));
-    k_cell_params<T><<<nb[KT_CELL_PAR], 32, 0, st>>>(L(KT_CELL_PAR));
-    k_fbp<T><<<nb[KT_FBP], 128, 0, st>>>(L(KT_FBP));
+    run(KT_CELL_MOM, [&](const auto &l, int nb) { k_cell_moments<T, std::decay_t<decltype(l)>><<<nb, 256, 0, st>>>(l); });
+    run(KT_CELL_PAR, [&](const auto &l, int nb) { k_cell_params<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
+    run(KT_FBP, [&](const auto &l, int nb) { k_fbp<T, std::decay_t<decltype(l)>><<<nb, 128, 0, st>>>(l); });
     mark(1);
-    if (pl.limiter_any) k_cell_grad<T><<<nb[KT_FBP], 128, 0, st>>>(L(KT_FBP));
-    if (pl.limiter_any) k_face_moments<T, true><<<nb[KT_FACE_MOM], 256, 0, st>>>(L(KT_FACE_MOM));
-    else k_face_moments<T, false><<<nb[KT_FACE_MOM], 256, 0, st>>>(L(KT_FACE_MOM));
-    k_face_params<T><<<nb[KT_FACE_PAR], 32, 0, st>>>(L(KT_FACE_PAR));
+    if (pl.limiter_any) run(KT_FBP, [&](const auto &l, int nb) { k_cell_recon<T, true, std::decay_t<decltype(l)>><<<nb, 128, 0, st>>>(l); });
+    else run(KT_FBP, [&](const auto &l, int nb) { k_cell_recon<T, false, std::decay_t<decltype(l)>><<<nb, 128, 0, st>>>(l); });
+    run(KT_FACE_MOM, [&](const auto &l, int nb) { k_face_moments<T, std::decay_t<decltype(l)>><<<nb, 256, 0, st>>>(l); });
+    run(KT_FACE_PAR, [&](const auto &l, int nb) { k_face_params<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
     mark(2);
-    k_face_flux<T><<<nb[KT_FACE_FLUX], 256, 0, st>>>(L(KT_FACE_FLUX));
-    k_face_phi<T><<<nb[KT_FACE_PHI], 64, 0, st>>>(L(KT_FACE_PHI));
+    run(KT_FACE_FLUX, [&](const auto &l, int nb) { k_face_flux<T, std::decay_t<decltype(l)>><<<nb, 256, 0, st>>>(l); });
+    run(KT_FACE_PHI, [&](const auto &l, int nb) { k_face_phi<T, std::decay_t<decltype(l)>><<<nb, 64, 0, st>>>(l); });
     mark(3);
-    k_macro_pre<T><<<nb[KT_MACRO_PRE], 32, 0, st>>>(L(KT_MACRO_PRE));
+    run(KT_MACRO_PRE, [&](const auto &l, int nb) { k_macro_pre<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
     if (pl.relax_sweeps > 0) {
-        k_record_residual<T><<<nb[KT_MACRO_SWEEP], 32, 0, st>>>(L(KT_MACRO_SWEEP));
+        run(KT_MACRO_SWEEP, [&](const auto &l, int nb) { k_record_residual<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
         for (int k = 1; k <= pl.relax_sweeps; ++k)
-            k_macro_relax<T><<<nb[KT_MACRO_PRE], 32, 0, st>>>(L(KT_MACRO_PRE), k, pl.relax_sweeps);
+            run(KT_MACRO_PRE, [&](const auto &l, int nb) { k_macro_relax<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l, k, pl.relax_sweeps); });
     } else if (pl.sched) {
         if (pl.sched_smem)
             k_macro_sweep_sched<T, true><<<nb[KT_MACRO_SWEEP], 256, pl.sched_smem, st>>>(L(KT_MACRO_SWEEP));
@@ -2988,9 +2935,9 @@ static int iteration_t(const Plan &pl, cudaStream_t st, void **events)
         k_macro_sweep<T, 4><<<nb[KT_MACRO_SWEEP], pl.macro_threads, pl.macro_smem, st>>>(L(KT_MACRO_SWEEP));
     else
         k_macro_sweep<T, 2><<<nb[KT_MACRO_SWEEP], pl.macro_threads, pl.macro_smem, st>>>(L(KT_MACRO_SWEEP));
-    k_macro_post<T><<<nb[KT_MACRO_POST], 32, 0, st>>>(L(KT_MACRO_POST));
+    run(KT_MACRO_POST, [&](const auto &l, int nb) { k_macro_post<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
     mark(4);
-    k_micro_residual<T><<<nb[KT_MICRO_RES], 128, 0, st>>>(L(KT_MICRO_RES));
+    run(KT_MICRO_RES, [&](const auto &l, int nb) { k_micro_residual<T, std::decay_t<decltype(l)>><<<nb, 128, 0, st>>>(l); });
     launch_sweep<T, true>(pl, st, L(KT_SWEEP));
     mark(5);
     launch_sweep<T, false>(pl, st, L(KT_SWEEP));
@@ -3046,9 +2993,9 @@ int launch_iteration(const Plan &pl, bool fp64, void *stream, void **events)
 
 template <class T> static int explicit_prologue_t(const Plan &pl, cudaStream_t st)
 {
-    auto L = [&](int kt) { return launch_of<T>(pl, kt); };
-    k_cell_moments<T><<<pl.nblocks[KT_CELL_MOM], 256, 0, st>>>(L(KT_CELL_MOM));
-    k_explicit_w<T><<<pl.nblocks[KT_CELL_PAR], 32, 0, st>>>(L(KT_CELL_PAR));
+    auto run = [&](int kt, auto launch) { run_plan(pl, kt, launch); };
+    run(KT_CELL_MOM, [&](const auto &l, int nb) { k_cell_moments<T, std::decay_t<decltype(l)>><<<nb, 256, 0, st>>>(l); });
+    run(KT_CELL_PAR, [&](const auto &l, int nb) { k_explicit_w<T, std::decay_t<decltype(l)>><<<nb, 32, 0, st>>>(l); });
     return (int)cudaGetLastError();
 }
 
