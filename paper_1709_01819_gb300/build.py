@@ -17,7 +17,7 @@ LIBDIR = os.path.join(PKG, "lib")
 LIB = os.path.join(LIBDIR, "libidugks.so")
 SOURCES = ["idugks_host.cpp", "idugks_kernels.cu", "idugks_adjoint.cu"]
 HEADERS = [os.path.join(ROOT, "include", "idugks.h")] + [
-    os.path.join(CSRC, h) for h in ("idugks_internal.h", "idugks_adjoint.h", "adjoint_math.h")]
+    os.path.join(CSRC, h) for h in ("idugks_internal.h", "idugks_adjoint.h", "adjoint_math.h", "wavefront.cuh")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")
 

@@ -26,6 +26,7 @@ enum { FP_RHO, FP_U, FP_V, FP_RT, FP_TAU, FP_QBX, FP_QBY, FP_QX, FP_QY, FP_A, FP
 struct AParams {
     // sizes and model
     int N, Nv, nf, ni, nj, K, shakhov, limiter;
+    int per_i, per_j;
     int lim_frozen;    // 1: the limiter factor is held at its linearisation value (no derivative)
     double venkat_k3;  // cube of the limiter's smoothing constant (0: Eq. 16-17)
     double dt, h, mu_ref, RT_ref, omega, Pr, gam, lusgs_omega, kappa;
@@ -53,6 +54,8 @@ struct AParams {
     double *fpar;      // [nf][kFP]
     double *fbarG, *fbarH;  // [nf][Nv]
     double *DW;        // [N] macroscopic LU-SGS diagonal
+    double *MW;        // [N][4][16] per slot the transposed macroscopic block over DW (0: no coupling)
+    double *sgeo;      // [2][N][8] ascending, descending: what the micro sweeps read of a cell (k_adj_lines)
     // adjoint iteration
     double *lamG, *lamH, *lamW;  // [N][Nv], [N][Nv], [N][4]
     double *bbG, *bbH;           // [N][Nv] P_f^-T lambda_f
@@ -66,6 +69,7 @@ struct AParams {
     double *cpp;                 // [N][2]  Kn partials of the cell (collision, cell prep)
     double *rpart;               // [N] squared increment of lambda_f per cell
     double *res;                 // [kMaxHist] ||increment of lambda_f|| per adjoint iteration
+    int *status;                 // status word of the context (a bounded wait that ran out)
     double *dlamW;               // [N][4] increment of lambda_W of the last iteration
 };
 

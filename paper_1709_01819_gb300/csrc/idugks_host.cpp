@@ -1124,6 +1124,10 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
         k.nsteps_f = c->nsteps_f;
         k.nsteps_b = c->nsteps_b;
     }
+    // per-(cell, velocity) kernels: four cells a block once that leaves every SM
+    // its eight resident blocks, two or one below
+    const long long nblocks = (long long)c->N * ((c->Nv + 255) / 256);
+    k.cpb = nblocks >= 4 * 8 * 152 ? 4 : nblocks >= 2 * 8 * 152 ? 2 : 1;
     // sweep launch shape: cell slots cover the longest hyperplane up to 64
     // micro sweeps: one thread per cell of the longest hyperplane (of the
     // longest schedule step on an unstructured mesh) and tv velocities per
@@ -2038,6 +2042,8 @@ idg::AParams adjoint_shape(const idg_ctx *c)
 {
     idg::AParams a{};
     a.N = c->N; a.Nv = c->Nv; a.nf = c->nf; a.ni = c->ni; a.nj = c->nj;
+    a.per_i = c->bc_kind[IDG_IMIN] == IDG_BC_PERIODIC;
+    a.per_j = c->bc_kind[IDG_JMIN] == IDG_BC_PERIODIC;
     return a;
 }
 
@@ -2147,7 +2153,7 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
     base.kappa = base.shakhov ? (1.0 - c->Pr) / (c->K + 4) : 0.0;
     base.area = k.area; base.dtimp = k.dtimp; base.fgeo = k.fgeo; base.ux = k.ux; base.uy = k.uy; base.w = k.w;
     base.cface = k.cface; base.cnb = k.cnb; base.csign = k.csign; base.fL = k.fL; base.fR = k.fR;
-    base.fbc = k.fbc; base.fside = k.fside; base.W = k.W;
+    base.fbc = k.fbc; base.fside = k.fside; base.W = k.W; base.status = k.status;
     for (int sd = 0; sd < 4; ++sd) {
         base.b_kind[sd] = c->bc_kind[sd];
         base.b_rho[sd] = c->bc_kind[sd] == IDG_BC_WALL ? 1.0 : c->bc_rho[sd];

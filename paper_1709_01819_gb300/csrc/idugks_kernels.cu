@@ -49,6 +49,7 @@
 // Data are laid out per cell in four face slots (a triangle's fourth slot is
 // unused: sign 0, no neighbour, no geometry).
 #include "idugks_internal.h"
+#include "wavefront.cuh"
 
 #include <cuda_runtime.h>
 #include <math.h>
@@ -678,33 +679,48 @@ __global__ void __launch_bounds__(32) k_cell_params(const __grid_constant__ LT L
     cA[15] = (T)(3.0 * p.h * fd);
 }
 
-// per (cell, pair of velocities): fb+ = c1 f~ + c2 f^S; 128-thread blocks,
-// each over 256 velocities of one cell
+// The per-(cell, velocity) kernels: 128-thread blocks, each over 256 velocities
+// (a pair per thread) of p.cpb consecutive cells.  Several cells a block where
+// there are enough of them: the block's parameters and velocity tables are read
+// once, and the next cell's loads overlap the current one's arithmetic (16
+// cavities of 32 to 96 cells a side, one cell a block before: k_fbp 272 ->
+// 208 us, k_micro_residual 453 -> 349 us).
+// body(c) for the block's cells, k the thread's first velocity.
+template <class Body> __device__ __forceinline__ void for_cells(const KParams &p, int blk, int &k, Body body)
+{
+    const int nvb = (p.Nv + 255) / 256;
+    const int b = blk / nvb;
+    k = 2 * ((blk - b * nvb) * 128 + threadIdx.x);
+    if (k >= p.Nv) return;
+    const int c0 = b * p.cpb, c1 = min(c0 + p.cpb, p.N);
+    for (int c = c0; c < c1; ++c) body(c);
+}
+
+// per (cell, pair of velocities): fb+ = c1 f~ + c2 f^S
 template <class T, class LT>
 __global__ void __launch_bounds__(128) k_fbp(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
-    const int nvb = (p.Nv + 255) / 256;
-    const int c = blk / nvb;
-    const int k = 2 * ((blk - c * nvb) * 128 + threadIdx.x);
-    if (k >= p.Nv) return;
-    const T *cA = (const T *)p.cellA + kCellP * c;
-    const EqT<T> e = eq_loadT<T>(cA);
-    const T c1 = cA[14], c2 = cA[15], kRTr = (T)(p.K * p.RT_r);
-    const size_t ck = (size_t)c * p.Nv + k;
-    T ux[2], uy[2], gr[2], g[2], h[2];
-    vtab2<T>(p.uxf, p.ux, k, ux);
-    vtab2<T>(p.uyf, p.uy, k, uy);
-    vtab2<T>(p.greff, p.gref, k, gr);
-    load_pair<T>(p.f, ck, g, h);
+    int k;
+    for_cells(p, blk, k, [&](int c) {
+        const T *cA = (const T *)p.cellA + kCellP * c;
+        const EqT<T> e = eq_loadT<T>(cA);
+        const T c1 = cA[14], c2 = cA[15], kRTr = (T)(p.K * p.RT_r);
+        const size_t ck = (size_t)c * p.Nv + k;
+        T ux[2], uy[2], gr[2], g[2], h[2];
+        vtab2<T>(p.uxf, p.ux, k, ux);
+        vtab2<T>(p.uyf, p.uy, k, uy);
+        vtab2<T>(p.greff, p.gref, k, gr);
+        load_pair<T>(p.f, ck, g, h);
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        T dG, dH;
-        dev_equilibrium<T>(e, ux[v], uy[v], gr[v], kRTr, dG, dH);
-        g[v] = mad(c1, g[v], c2 * dG);
-        h[v] = mad(c1, h[v], c2 * dH);
-    }
-    store_pair<T>(p.fbp, ck, g, h);
+        for (int v = 0; v < 2; ++v) {
+            T dG, dH;
+            dev_equilibrium<T>(e, ux[v], uy[v], gr[v], kRTr, dG, dH);
+            g[v] = mad(c1, g[v], c2 * dG);
+            h[v] = mad(c1, h[v], c2 * dH);
+        }
+        store_pair<T>(p.fbp, ck, g, h);
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -801,20 +817,20 @@ template <class T> __device__ __forceinline__ int tie_slot(const KParams &p, int
 // it; at a velocity along the face (s = 0) both sides count half, the L side
 // going to the face buffer and the R side to the tie buffer (k_face_moments
 // takes the mean).  Boundary faces get the outgoing velocities and the ties.
-// 128-thread blocks, each over 256 velocities of one cell; the cell's stencil
-// record is read by every thread (one broadcast per load).
-// Bound by the face buffer's bytes and the issue of the stencil arithmetic.
-// Gathering at the faces instead formed every gradient twice (once per face a
-// velocity leaves by) with one warp walking a face: LIMTXT
+// The cell's stencil record is read by every thread (one broadcast per load).
+// Bound by the latency of the stencil's loads and the face buffer's bytes.
+// Gathering at the faces instead formed an unlimited gradient once per face a
+// velocity leaves by, or stored the limited ones in a second pass; with the
+// moments of a face (k_face_moments) it took, float32, 81 us on 64 x 64 cells
+// x 1024 velocities, 259 us on 128 x 128 x 784 and, limited, 1952 us on
+// 121 x 81 x 7921; this 32 + 35, 107 + 101 and 908 + 464 us.
 template <class T, bool LIM, class LT>
 __global__ void __launch_bounds__(128) k_cell_recon(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
     using T2 = typename V2<T>::t;
-    const int nvb = (p.Nv + 255) / 256;
-    const int c = blk / nvb;
-    const int k = 2 * ((blk - c * nvb) * 128 + threadIdx.x);
-    if (k >= p.Nv) return;
+    int k;
+    for_cells(p, blk, k, [&](int c) {
     int nb[4], fc[4], sg[4];
     T gx[4], gy[4], frx[4], fry[4], nx[4], ny[4];
     {
@@ -909,6 +925,7 @@ __global__ void __launch_bounds__(128) k_cell_recon(const __grid_constant__ LT L
         }
         st_pair_if((T2 *)p.F + ((size_t)fc[m] * p.Nv + k), og, oh, out);
     }
+    });
 }
 
 // Linearised wall (Eq. 33-35), at a wall face f: the outgoing sum
@@ -962,70 +979,64 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_moments(co
     Acc<T> acc[kRaw];
 #pragma unroll
     for (int q = 0; q < kRaw; ++q) acc[q].zero();
-    if (kind < 0) {
-        const T2 *tb = (const T2 *)p.ftie + (size_t)f * max(p.nvx, p.nvy);
-        auto body = [&](int k, T(&a)[kRaw]) {
-            T ux[2], uy[2], w[2], g[2], h[2];
-            vtab2<T>(p.uxf, p.ux, k, ux);
-            vtab2<T>(p.uyf, p.uy, k, uy);
-            vtab2<T>(p.wf, p.w, k, w);
-            load_pair<T>(Fo, k, g, h);
+    const int lc = p.fL[f], side = p.fside[f];
+    const T on = kind < 0 || lc >= 0 ? (T)1 : (T)-1;
+    T rhow = (T)1, rwm1 = (T)0;
+    if (kind == 1) {
+        // zero net mass flux: rho_w sum_in w |xi.n| G_w = sum_out w (xi.n) fb
+        vel_loop<1, T>(p.Nv, lane, outsum, [&](int k, T(&a)[1]) {
+            const T so = on * xi_dot_n<T>(vx<T>(p, k), vy<T>(p, k), nx, ny);
+            if (so > (T)0) a[0] = mad(vw<T>(p, k) * so, Fo[k].x, a[0]);
+        });
+        outsum[0].warp_sum();
+        const double o = __shfl_sync(0xffffffffu, outsum[0].value(), 0);
+        const double *bc = p.bconst + 2 * f;
+        rw = (bc[0] + o) / bc[1];
+        rhow = (T)rw;
+        rwm1 = (T)((bc[0] - bc[1] + o) / bc[1]);
+        if (p.implicit_wall) wall_ghost_density<T>(p, f, lane, lc >= 0 ? lc : p.fR[f], on, nx, ny, bc[1]);
+    }
+    auto body = [&](int k, T(&a)[kRaw]) {
+        T ux[2], uy[2], w[2], s[2], g[2], h[2];
+        vtab2<T>(p.uxf, p.ux, k, ux);
+        vtab2<T>(p.uyf, p.uy, k, uy);
+        vtab2<T>(p.wf, p.w, k, w);
+        load_pair<T>(Fo, k, g, h);
+        bool cut = kind >= 0;
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            s[v] = on * xi_dot_n<T>(ux[v], uy[v], nx, ny);
+            cut |= s[v] == (T)0;
+        }
+        if (cut) {
+            const T2 *tb = (const T2 *)p.ftie + (size_t)f * max(p.nvx, p.nvy);
 #pragma unroll
             for (int v = 0; v < 2; ++v) {
-                if (xi_dot_n<T>(ux[v], uy[v], nx, ny) == (T)0 && k + v < p.nvx * p.nvy) {
-                    // average of both sides (the flux there is zero: fb itself is not needed again)
-                    const T2 r = tb[tie_slot<T>(p, k + v, nx, ny)];
-                    g[v] = (T)0.5 * (g[v] + r.x);
-                    h[v] = (T)0.5 * (h[v] + r.y);
-                }
-                raw_terms<T>(a, w[v], ux[v], uy[v], g[v], h[v]);
-            }
-        };
-        if constexpr (sizeof(T) == 4) {
-            __shared__ FF sacc[kRaw * 256];
-            vel_loop2_sm<kRaw>(p.Nv, lane, acc, sacc, body);
-        } else {
-            vel_loop2<kRaw, T>(p.Nv, lane, acc, body);
-        }
-    } else {
-        const int lc = p.fL[f], c = lc >= 0 ? lc : p.fR[f], side = p.fside[f];
-        const T on = lc >= 0 ? (T)1 : (T)-1;
-        T rhow = (T)1, rwm1 = (T)0;
-        if (kind == 1) {
-            // zero net mass flux: rho_w sum_in w |xi.n| G_w = sum_out w (xi.n) fb
-            vel_loop<1, T>(p.Nv, lane, outsum, [&](int k, T(&a)[1]) {
-                const T so = on * xi_dot_n<T>(vx<T>(p, k), vy<T>(p, k), nx, ny);
-                if (so > (T)0) a[0] = mad(vw<T>(p, k) * so, Fo[k].x, a[0]);
-            });
-            outsum[0].warp_sum();
-            const double o = __shfl_sync(0xffffffffu, outsum[0].value(), 0);
-            const double *bc = p.bconst + 2 * f;
-            rw = (bc[0] + o) / bc[1];
-            rhow = (T)rw;
-            rwm1 = (T)((bc[0] - bc[1] + o) / bc[1]);
-            if (p.implicit_wall) wall_ghost_density<T>(p, f, lane, c, on, nx, ny, bc[1]);
-        }
-        const T *bG = (const T *)p.bdevG + (size_t)side * p.Nv, *bH = (const T *)p.bdevH + (size_t)side * p.Nv;
-        const T kRTr = (T)(p.K * p.RT_r);
-        vel_loop<kRaw, T>(p.Nv, lane, acc, [&](int k, T(&a)[kRaw]) {
-            const T ux = vx<T>(p, k), uy = vy<T>(p, k), so = on * xi_dot_n<T>(ux, uy, nx, ny);
-            T2 fb;
-            if (so >= (T)0) fb = Fo[k];
-            if (so <= (T)0) {
-                const T gref = vgref<T>(p, k);
+                if (s[v] > (T)0 || (kind < 0 && (s[v] < (T)0 || k + v >= p.nvx * p.nvy))) continue;
                 T2 in;
-                in.x = mad(rhow, bG[k], rwm1 * gref);
-                in.y = mad(rhow, bH[k], rwm1 * (kRTr * gref));
-                if (so < (T)0) {
-                    fb = in;
+                if (kind < 0) {
+                    in = tb[tie_slot<T>(p, k + v, nx, ny)];
                 } else {
-                    fb.x = (T)0.5 * (fb.x + in.x);
-                    fb.y = (T)0.5 * (fb.y + in.y);
+                    const T *bG = (const T *)p.bdevG + (size_t)side * p.Nv, *bH = (const T *)p.bdevH + (size_t)side * p.Nv;
+                    const T gref = vgref<T>(p, k + v);
+                    in.x = mad(rhow, bG[k + v], rwm1 * gref);
+                    in.y = mad(rhow, bH[k + v], rwm1 * ((T)(p.K * p.RT_r) * gref));
                 }
-                Fo[k] = fb;
+                // along the face the mean of both sides (at an interior face the
+                // flux there is zero: the mean is not stored)
+                g[v] = s[v] < (T)0 ? in.x : (T)0.5 * (g[v] + in.x);
+                h[v] = s[v] < (T)0 ? in.y : (T)0.5 * (h[v] + in.y);
             }
-            raw_terms<T>(a, vw<T>(p, k), ux, uy, fb.x, fb.y);
-        });
+            if (kind >= 0) store_pair<T>(Fo, k, g, h);
+        }
+        raw_terms<T>(a, w[0], ux[0], uy[0], g[0], h[0]);
+        raw_terms<T>(a, w[1], ux[1], uy[1], g[1], h[1]);
+    };
+    if constexpr (sizeof(T) == 4) {
+        __shared__ FF sacc[kRaw * 256];
+        vel_loop2_sm<kRaw>(p.Nv, lane, acc, sacc, body);
+    } else {
+        vel_loop2<kRaw, T>(p.Nv, lane, acc, body);
     }
     warp_sum_store<kRaw, T>(acc, lane, p.faceraw, (size_t)f * 12);
     if (lane == 0) {
@@ -1198,57 +1209,6 @@ template <> __device__ __forceinline__ void base_state<float>(const KParams &p, 
     const float pr = (float)(p.gam - 1.0) * (E - 0.5f * rho * (u * u + v * v));
     o[0] = rho; o[1] = mx; o[2] = my;
     o[3] = u; o[4] = v; o[5] = E + pr;
-}
-
-// cp.async helpers: asynchronous global -> shared copies used to prefetch
-// the next hyperplanes of a wavefront while the current one is computed
-__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cp_async16(void *s, const void *g)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void *s, const void *g)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void *s, const void *g)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(s)), "l"(g) : "memory");
-}
-template <int B> __device__ __forceinline__ void cp_async_b(void *s, const void *g);
-template <> __device__ __forceinline__ void cp_async_b<4>(void *s, const void *g) { cp_async4(s, g); }
-template <> __device__ __forceinline__ void cp_async_b<8>(void *s, const void *g) { cp_async8(s, g); }
-template <> __device__ __forceinline__ void cp_async_b<16>(void *s, const void *g) { cp_async16(s, g); }
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-// Wavefronts over lines of cells (k_macro_lines, k_sweep_lines): the warps of a
-// block run kSweepBlock steps between two looks at their neighbours' progress.
-constexpr int kSweepBlock = 4;
-
-// progress flags between the warps of one block
-__device__ __forceinline__ void flag_store(int *f, int v)
-{
-    asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(smem_addr(f)), "r"(v) : "memory");
-}
-__device__ __forceinline__ int flag_load(const int *f)
-{
-    int v;
-    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_addr(f)) : "memory");
-    return v;
-}
-// waits until *f >= need (seen: what the last poll found).  The warps of a block
-// run at the same time, so the wait ends; should it not (2^22 polls), the status
-// word is raised and the sweep goes on.
-__device__ __forceinline__ void flag_wait(const int *f, int need, int &seen, int *status)
-{
-    for (int n = 0; seen < need; ++n) {
-        seen = flag_load(f);
-        if (n > (1 << 22)) {
-            *status = 6;
-            seen = 0x7fffffff;
-        }
-    }
 }
 
 // four storage scalars, 16-byte aligned
@@ -1949,10 +1909,8 @@ template <class T, class LT>
 __global__ void __launch_bounds__(128) k_explicit_update(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
-    const int nvb = (p.Nv + 255) / 256;
-    const int c = blk / nvb;
-    const int k = 2 * ((blk - c * nvb) * 128 + threadIdx.x);
-    if (k >= p.Nv) return;
+    int k;
+    for_cells(p, blk, k, [&](int c) {
     const T *cA = (const T *)p.cellA + kCellP * c;
     const EqT<T> e = eq_loadT<T>(cA);
     // k_cell_params stores c2 = 3h/(2tau+dt) = (3/4) 2dt/(2tau+dt) (h = dt/2)
@@ -1985,6 +1943,7 @@ __global__ void __launch_bounds__(128) k_explicit_update(const __grid_constant__
         h[v] = mad(-dto, sh_[v], mad(a, h[v], b * dH));
     }
     store_pair<T>(p.f, ck, g, h);
+    });
 }
 
 // W = (rho, rho U, rho V, rho E) of f~ from its raw moments (Eq. 4), and
@@ -2028,10 +1987,8 @@ template <class T, class LT>
 __global__ void __launch_bounds__(128) k_micro_residual(const __grid_constant__ LT L)
 {
     IDG_LOCATE();
-    const int nvb = (p.Nv + 255) / 256;
-    const int c = blk / nvb;
-    const int k = 2 * ((blk - c * nvb) * 128 + threadIdx.x);
-    if (k >= p.Nv) return;
+    int k;
+    for_cells(p, blk, k, [&](int c) {
     const T *cp = (const T *)p.cellpT + kCellP * c;
     const EqT<T> e = eq_loadT<T>(cp);
     const T cq = cp[14], kRTr = (T)(p.K * p.RT_r);
@@ -2061,6 +2018,7 @@ __global__ void __launch_bounds__(128) k_micro_residual(const __grid_constant__ 
         }
     }
     store_pair<T>(p.dst, ck, rg, rh);
+    });
 }
 
 // 16 storage scalars from 16-byte-aligned shared memory
@@ -2720,7 +2678,7 @@ void blocks_per_instance(const KParams &p, int out[KT_COUNT])
     const int nvb = nblk(p.Nv, 256);
     out[KT_CELL_MOM] = nblk(p.N, 8);
     out[KT_CELL_PAR] = nblk(p.N, 32);
-    out[KT_FBP] = p.N * nvb;
+    out[KT_FBP] = nblk(p.N, p.cpb) * nvb;
     out[KT_FACE_MOM] = nblk(p.nf, 8);
     out[KT_FACE_PAR] = nblk(p.nf, 32);
     out[KT_FACE_FLUX] = nblk(p.nf, 8);
@@ -2728,7 +2686,7 @@ void blocks_per_instance(const KParams &p, int out[KT_COUNT])
     out[KT_MACRO_PRE] = nblk(p.N, 32);
     out[KT_MACRO_SWEEP] = 1;
     out[KT_MACRO_POST] = nblk(p.N, 32);
-    out[KT_MICRO_RES] = p.N * nvb;
+    out[KT_MICRO_RES] = nblk(p.N, p.cpb) * nvb;
     out[KT_SWEEP] = nblk(p.Nv, p.sweep_ktv * p.sweep_kvpt);
 }
 
