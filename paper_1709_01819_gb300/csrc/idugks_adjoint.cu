@@ -14,9 +14,9 @@
 //     dJ/dp = dJ/dp|_u + bar_a^T dR_W/dp + bar_b^T dR_f/dp
 // with bar_b = P_f^-T lambda_f and bar_a = P_W^-T (lambda_W + (dR_f/dW')^T bar_b).
 // One adjoint iteration, in launch order:
-//   k_adj_micro_asc, k_adj_micro_desc   bar_b = P_f^-T lambda_f: the transposed
-//       factors of Eq. (26) couple each cell to its downwind neighbours; the
-//       lower transposed factor runs last, over the hyperplanes in descending order
+//   k_adj_lines     bar_b = P_f^-T lambda_f, ascending then descending: the
+//       transposed factors of Eq. (26) couple each cell to its downwind neighbours;
+//       the lower transposed factor runs last, over the cells in descending order
 //   k_adj_wprime    (dR_f/dW')^T bar_b: collision term at the predicted state
 //   k_adj_macro     bar_a = P_W^-T (...): transposed block LU-SGS with the Euler
 //       flux Jacobians of the own cell, ascending then descending hyperplanes
@@ -33,9 +33,12 @@
 
 #include "adjoint_math.h"
 #include "idugks.h"
+#include "wavefront.cuh"
 
 #include <cuda_runtime.h>
 #include <math.h>
+
+#include <algorithm>
 
 namespace idg {
 namespace {
@@ -337,92 +340,203 @@ __global__ void __launch_bounds__(kTB) k_adj_face_lin(AParams a)
     if (threadIdx.x < kFP) a.fpar[(size_t)kFP * f + threadIdx.x] = fp[threadIdx.x];
 }
 
-// per cell: diagonal of the macroscopic LU-SGS, Omega/dt_imp + (omega/2) sum Lambda
+// per cell: diagonal of the macroscopic LU-SGS, Omega/dt_imp + (omega/2) sum
+// Lambda, and the transposed blocks towards its neighbours,
+// (1/2)(S A(W_c; n_out)^T + omega Lambda I), A the Euler flux Jacobian, over that
+// diagonal (they stay what they are through the iteration); the record of the
+// micro sweeps: per direction the scaled outward normals of the own line's next
+// face and of the faces towards the adjacent lines, the swept side first (0 where
+// a cell is its own neighbour), and Omega/dt_imp + cq
 __global__ void k_adj_macro_lin(AParams a)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= a.N) return;
     double d = a.area[c] / a.dtimp[c];
+    const double D0 = d + a.cpar[(size_t)kCP * c + CP_CQ];
     for (int m = 0; m < 4; ++m) {
         const int f = a.cface[4 * c + m];
         if (a.fL[f] == a.fR[f]) continue;
         d += 0.5 * a.lusgs_omega * a.fpar[(size_t)kFP * f + FP_LAM];
     }
     a.DW[c] = d;
+    const bool cols = a.ni <= a.nj;
+    for (int m = 0; m < 4; ++m) {
+        const int f = a.cface[4 * c + m], nb = a.cnb[4 * c + m];
+        const bool self = a.fL[f] == a.fR[f];
+        const double *g = a.fgeo + 7 * f;
+        const double sgn = a.csign[4 * c + m], nx = sgn * g[0], ny = sgn * g[1];
+        double *M = a.MW + 16 * (4 * (size_t)c + m);
+        for (int q = 0; q < 4; ++q) {
+            double y[4] = {0, 0, 0, 0}, t[4] = {0, 0, 0, 0};
+            y[q] = 1.0;
+            if (nb >= 0 && !self) adj::euler_jacT(a.W + 4 * c, a.gam, nx, ny, y, t);
+            for (int r = 0; r < 4; ++r)
+                M[4 * r + q] = nb >= 0 && !self ? 0.5 * (g[2] * t[r] + (r == q ? a.lusgs_omega * a.fpar[(size_t)kFP * f + FP_LAM] : 0.0)) / d : 0.0;
+        }
+        // slots (west 0, east 1, south 2, north 3) -> entry of the two records
+        const bool own = cols ? m >= 2 : m < 2, up = m & 1;
+        for (int dir = 0; dir < 2; ++dir) {
+            double *o = a.sgeo + 8 * ((size_t)dir * a.N + c);
+            const int e = own ? (up != (dir == 1) ? 0 : -1) : (up != (dir == 1) ? 4 : 2);
+            if (e < 0) continue;
+            o[e] = self ? 0.0 : nx * g[2];
+            o[e + 1] = self ? 0.0 : ny * g[2];
+        }
+    }
+    a.sgeo[8 * (size_t)c + 6] = a.sgeo[8 * ((size_t)a.N + c) + 6] = D0;
 }
 
 // ---------------------------------------------------------------------------
 // adjoint iteration
 // ---------------------------------------------------------------------------
 
-// micro LU-SGS diagonal of Eq. (26) and the cell range of hyperplane d
-__device__ __forceinline__ double micro_diag(const AParams &a, int c, int k)
+// The transposed micro sweeps, D of Eq. (26): ascending
+//     y_c = (lambda_c + sum_{lower nb} (xi.n)^+ S y_nb) / D_c,
+// descending, in place, y_c += sum_{upper nb} (xi.n)^+ S y_nb / D_c.  A warp
+// marches along 32 / G neighbouring lines of the longer axis at G neighbouring
+// velocities, one step behind one another, exactly as the forward sweeps of a
+// structured block do (k_sweep_lines: registers along the line, shuffles across,
+// rings and flags between the strips of a block, copies kAdjAhead steps ahead);
+// a thread carries both components.  Bound by the float64 pipe and the latency of
+// a step.  A hyperplane per barrier with the geometry re-derived at every face
+// took 400 + 461 us on 24 x 24 cells x 256 velocities, this 14 + 15 us.
+constexpr int kAdjAhead = 4, kAdjRing = 32;
+
+struct AdjShape {
+    int G, strips;
+    size_t smem;
+};
+AdjShape adj_shape(const AParams &a)
 {
-    double d = a.area[c] / a.dtimp[c] + a.cpar[(size_t)kCP * c + CP_CQ];
-    for (int m = 0; m < 4; ++m) {
-        const int f = a.cface[4 * c + m];
-        if (a.fL[f] == a.fR[f]) continue;
-        const double *g = a.fgeo + 7 * f;
-        const double so = a.csign[4 * c + m] * xdn(a.ux[k], a.uy[k], g[0], g[1]);
-        if (so > 0) d += so * g[2];
-    }
-    return d;
+    const int nt = a.ni < a.nj ? a.ni : a.nj;
+    AdjShape s;
+    // as many velocities side by side as leave every SM a block, at most 8; at
+    // most 16 strips a block
+    s.G = 8;
+    while (s.G > 1 && (a.Nv / s.G < 152 || (nt + 32 / s.G - 1) / (32 / s.G) > 16)) s.G /= 2;
+    const int lw = 32 / s.G;
+    s.strips = (nt + lw - 1) / lw;
+    s.smem = 64 + (size_t)s.strips * (kAdjRing * s.G * 16 + kAdjAhead * (32 * 16 + lw * 64));
+    return s;
 }
 
-// sum over neighbours nb (lower: nb < c, else nb > c) of (xi.n_out)^+ S y_nb
-template <bool LOWER>
-__device__ __forceinline__ double micro_couple(const AParams &a, const double *y, int c, int k)
+template <bool ASC> __global__ void __launch_bounds__(512) k_adj_lines(AParams a, AdjShape sh, int *status)
 {
-    double acc = 0.0;
-    for (int m = 0; m < 4; ++m) {
-        const int nb = a.cnb[4 * c + m];
-        if (nb < 0 || nb == c || (LOWER ? nb > c : nb < c)) continue;
-        const int f = a.cface[4 * c + m];
-        if (a.fL[f] == a.fR[f]) continue;
-        const double *g = a.fgeo + 7 * f;
-        const double so = a.csign[4 * c + m] * xdn(a.ux[k], a.uy[k], g[0], g[1]);
-        if (so > 0) acc += so * g[2] * y[(size_t)nb * a.Nv + k];
+    extern __shared__ __align__(16) unsigned char smraw[];
+    int *flags = (int *)smraw;
+    const bool cols = a.ni <= a.nj;
+    const int nt = cols ? a.ni : a.nj, nw = cols ? a.nj : a.ni, Nv = a.Nv;
+    const int G = sh.G, lw = 32 / G, strips = sh.strips;
+    const int strip = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane / G, g = lane - l * G;
+    // step s of the block's clock: line tt is at its cell ww = s - tt - strip * kSweepBlock
+    const int s_beg = (strip * (lw + kSweepBlock)) & ~(kSweepBlock - 1);
+    const int s_end = strip * (lw + kSweepBlock) + nw + min(lw, nt - strip * lw) - 1;
+    if (lane == 0) flags[strip] = s_beg;
+    __syncthreads();
+    const int tt = strip * lw + l, tc = min(tt, nt - 1);
+    const int k0 = blockIdx.x * G + g, k = k0 < Nv ? k0 : 0;
+    const double ux = a.ux[k], uy = a.uy[k];
+    const int t = ASC ? tc : nt - 1 - tc;
+    const int cs = (ASC ? 1 : -1) * (cols ? a.ni : 1);
+    const int c0 = (cols ? t : t * a.ni) + (ASC ? 0 : (nw - 1) * (cols ? a.ni : 1));
+    const ptrdiff_t base = (ptrdiff_t)c0 * Nv + k;
+    const int sv = cs * Nv, sg = cs * 8;
+    const double *xG = (ASC ? a.lamG : a.bbG) + base, *xH = (ASC ? a.lamH : a.bbH) + base;
+    double *yG = a.bbG + base, *yH = a.bbH + base;
+    const double *geo = a.sgeo + (ASC ? 0 : (ptrdiff_t)a.N * 8) + (ptrdiff_t)c0 * 8;
+    const unsigned nwl = tt < nt && k0 < Nv ? nw : 0;
+    const int start = tt + strip * kSweepBlock;
+    const bool seam_t = (cols ? a.per_i : a.per_j) && nt > 1, seam_w = (cols ? a.per_j : a.per_i) && nw > 1;
+    const bool edge = l == 0 && strip > 0, border = l == lw - 1 && strip + 1 < strips;
+    double2 *xw = (double2 *)(smraw + 64) + (size_t)strip * kAdjRing * G + g;
+    const double2 *xr = strip > 0 ? xw - (size_t)kAdjRing * G : xw;
+    const int SB = 32 * 16 + lw * 64;
+    unsigned char *stage = smraw + 64 + (size_t)strips * kAdjRing * G * 16 + (size_t)strip * kAdjAhead * SB;
+    auto issue = [&](int s) {
+        const int wc = min(max(s - start, 0), nw - 1);
+        unsigned char *st = stage + (s & (kAdjAhead - 1)) * SB;
+        cp_async8(st + lane * 16, xG + (ptrdiff_t)wc * sv);
+        cp_async8(st + lane * 16 + 8, xH + (ptrdiff_t)wc * sv);
+        const char *gg = (const char *)(geo + (ptrdiff_t)wc * sg);
+        for (int q = g; q < 4; q += G) cp_async16(st + 512 + l * 64 + 16 * q, gg + 16 * q);
+        cp_commit();
+    };
+    for (int u = 0; u < kAdjAhead; ++u) issue(s_beg + u);
+    // (xi.n) S of the line's end face, outward from its first cell
+    double end = 0.0;
+    {
+        const int m = (cols ? 2 : 0) + (ASC ? 0 : 1), f = a.cface[4 * c0 + m];
+        if (a.fL[f] != a.fR[f]) {
+            const double *q = a.fgeo + 7 * f, sgn = a.csign[4 * c0 + m];
+            end = xdn(ux, uy, sgn * q[0] * q[2], sgn * q[1] * q[2]);
+        }
     }
-    return acc;
-}
-
-// y = (D - U~^T)^-1 lambda_f: ascending hyperplanes.  Block = 32 velocities x
-// 8 warps; blockIdx.y = component.  Dependencies stay inside the block.
-__global__ void __launch_bounds__(kTB) k_adj_micro_asc(AParams a)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int k = blockIdx.x * 32 + lane;
-    const double *x = blockIdx.y ? a.lamH : a.lamG;
-    double *y = blockIdx.y ? a.bbH : a.bbG;
-    const int ni = a.ni, nj = a.nj;
-    for (int d = 0; d <= ni + nj - 2; ++d) {
-        const int i0 = max(0, d - nj + 1), i1 = min(d, ni - 1);
-        if (k < a.Nv)
-            for (int i = i0 + wid; i <= i1; i += nw) {
-                const int c = (d - i) * ni + i;
-                const double acc = x[(size_t)c * a.Nv + k] + micro_couple<true>(a, y, c, k);
-                y[(size_t)c * a.Nv + k] = acc / micro_diag(a, c, k);
+    double2 prev = make_double2(0, 0), first = make_double2(0, 0);
+    double cl, co, ca, cu, iD, ahead = 0.0;
+    auto coef = [&](int s) {
+        const int ww = s - start;
+        const double *q = (const double *)(stage + (s & (kAdjAhead - 1)) * SB + 512 + l * 64);
+        const double own = ww > 0 ? -ahead : end;
+        ahead = xdn(ux, uy, q[0], q[1]);
+        const double low = xdn(ux, uy, q[2], q[3]), upp = xdn(ux, uy, q[4], q[5]);
+        // half the sum of all |xi.n| S is the outflow: the normals sum to zero
+        iD = __drcp_rn(fma(0.5, (fabs(own) + fabs(ahead)) + (fabs(low) + fabs(upp)), q[6]));
+        cl = low > 0.0 && tt > 0 ? low : 0.0;
+        co = own > 0.0 && ww > 0 ? own : 0.0;
+        ca = seam_w && ww == nw - 1 && ahead > 0.0 ? ahead : 0.0;
+        cu = seam_t && tt == nt - 1 && upp > 0.0 ? upp : 0.0;
+    };
+    cp_wait<kAdjAhead - 1>();
+    __syncwarp();
+    coef(s_beg);
+    int seen_r = 0, seen_w = 0;
+    for (int s0 = s_beg; s0 < s_end; s0 += kSweepBlock) {
+        if (strips > 1) {
+            if (strip > 0) flag_wait(flags + strip - 1, s0, seen_r, status);
+            if (strip + 1 < strips) flag_wait(flags + strip + 1, s0 + 2 * kSweepBlock + 1 - kAdjRing, seen_w, status);
+        }
+#pragma unroll
+        for (int b = 0; b < kSweepBlock; ++b) {
+            const int s = s0 + b, ww = s - start;
+            cp_wait<kAdjAhead - 2>();
+            __syncwarp();
+            const bool on = (unsigned)ww < nwl;
+            const double2 x = *(const double2 *)(stage + (s & (kAdjAhead - 1)) * SB + lane * 16);
+            const double2 ev = xr[(ww & (kAdjRing - 1)) * G];
+            double2 adj;
+            adj.x = __shfl_up_sync(0xffffffffu, prev.x, G);
+            adj.y = __shfl_up_sync(0xffffffffu, prev.y, G);
+            if (edge) adj = ev;
+            double ag = fma(cl, adj.x, co * prev.x), ah = fma(cl, adj.y, co * prev.y);
+            if (ca > 0.0) {
+                ag = fma(ca, first.x, ag);
+                ah = fma(ca, first.y, ah);
             }
-        __syncthreads();
-    }
-}
-
-// w = (D - L~^T)^-1 D y: descending hyperplanes, in place
-__global__ void __launch_bounds__(kTB) k_adj_micro_desc(AParams a)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int k = blockIdx.x * 32 + lane;
-    double *y = blockIdx.y ? a.bbH : a.bbG;
-    const int ni = a.ni, nj = a.nj;
-    for (int d = ni + nj - 2; d >= 0; --d) {
-        const int i0 = max(0, d - nj + 1), i1 = min(d, ni - 1);
-        if (k < a.Nv)
-            for (int i = i0 + wid; i <= i1; i += nw) {
-                const int c = (d - i) * ni + i;
-                const double up = micro_couple<false>(a, y, c, k);
-                y[(size_t)c * a.Nv + k] += up / micro_diag(a, c, k);
+            if (on && cu > 0.0) {
+                const ptrdiff_t o = (ptrdiff_t)ww * sv + (ptrdiff_t)((ASC ? 0 : nt - 1) - t) * (cols ? 1 : a.ni) * Nv;
+                ag = fma(cu, yG[o], ag);
+                ah = fma(cu, yH[o], ah);
             }
-        __syncthreads();
+            prev.x = ASC ? (x.x + ag) * iD : fma(ag, iD, x.x);
+            prev.y = ASC ? (x.y + ah) * iD : fma(ah, iD, x.y);
+            if (ww == 0) first = prev;
+            coef(s + 1);
+            if (on) {
+                yG[(ptrdiff_t)ww * sv] = prev.x;
+                yH[(ptrdiff_t)ww * sv] = prev.y;
+                if (border) xw[(ww & (kAdjRing - 1)) * G] = prev;
+            }
+            issue(s + kAdjAhead);
+        }
+        if (strips > 1) {
+            __syncwarp();
+            if (lane == 0) flag_store(flags + strip, s0 + kSweepBlock);
+        }
+    }
+    cp_wait<0>();
+    if (strips > 1) {
+        __syncwarp();
+        if (lane == 0) flag_store(flags + strip, 0x7fffffff);
     }
 }
 
@@ -460,50 +574,65 @@ __global__ void __launch_bounds__(kTB) k_adj_wprime(AParams a)
     }
 }
 
-// bar_a = P_W^-T bwp: (D + U^T)^-1 ascending, times D, (D + L^T)^-1 descending.
-// The transposed blocks of cell c toward neighbour nb are
-// -(1/2)(S A(W_c; n_out)^T + omega Lambda I), A the Euler flux Jacobian.
-__device__ __forceinline__ void macro_couple(const AParams &a, int c, bool lower, double *acc)
+// bar_a = P_W^-T bwp: (D + U^T)^-1 ascending, times D, (D + L^T)^-1 descending,
+// one block over the hyperplanes, four threads (components) per cell.  The
+// transposed blocks over the diagonal come ready (MW), and a step's are loaded
+// before the barrier that opens it, so that after it only the neighbours'
+// increments are read -- from shared memory where all cells' fit (SMEM).
+// Re-deriving the Jacobians at every face took 767 us on 24 x 24 cells, this
+// 22 us.
+struct AdjMacroCell {
+    int c, nb[4];
+    double b, m[4][4];
+};
+template <bool SMEM, int NT>
+__global__ void __launch_bounds__(NT) k_adj_macro(AParams a)
 {
-    const double *Wc = a.W + 4 * c;
-    for (int m = 0; m < 4; ++m) {
-        const int nb = a.cnb[4 * c + m];
-        if (nb < 0 || nb == c || (lower ? nb > c : nb < c)) continue;
-        const int f = a.cface[4 * c + m];
-        if (a.fL[f] == a.fR[f]) continue;
-        const double *g = a.fgeo + 7 * f;
-        const double sgn = a.csign[4 * c + m];
-        const double lam = a.fpar[(size_t)kFP * f + FP_LAM];
-        const double *y = a.ba + 4 * nb;
-        double t[4];
-        adj::euler_jacT(Wc, a.gam, sgn * g[0], sgn * g[1], y, t);
-        for (int q = 0; q < 4; ++q) acc[q] += 0.5 * (g[2] * t[q] + a.lusgs_omega * lam * y[q]);
-    }
-}
-
-__global__ void __launch_bounds__(kTB) k_adj_macro(AParams a)
-{
-    const int ni = a.ni, nj = a.nj;
-    for (int d = 0; d <= ni + nj - 2; ++d) {
-        const int i0 = max(0, d - nj + 1), i1 = min(d, ni - 1);
-        for (int i = i0 + threadIdx.x; i <= i1; i += blockDim.x) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double *y = SMEM ? (double *)smraw : a.ba;  // [N][4]
+    const int ni = a.ni, nj = a.nj, nd = ni + nj - 1;
+    const int q = threadIdx.x & 3, slot = threadIdx.x >> 2;
+    for (int pass = 0; pass < 2; ++pass) {
+        auto load = [&](int step, AdjMacroCell &x) {
+            x.c = -1;
+            if (step >= nd) return;
+            const int d = pass ? nd - 1 - step : step;
+            const int i = max(0, d - nj + 1) + slot;
+            if (i > min(d, ni - 1)) return;
             const int c = (d - i) * ni + i;
-            double acc[4] = {a.bwp[4 * c], a.bwp[4 * c + 1], a.bwp[4 * c + 2], a.bwp[4 * c + 3]};
-            macro_couple(a, c, true, acc);
-            for (int q = 0; q < 4; ++q) a.ba[4 * c + q] = acc[q] / a.DW[c];
+            x.c = c;
+            if (!pass) x.b = a.bwp[4 * c + q] / a.DW[c];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int nb = a.cnb[4 * c + m];
+                x.nb[m] = nb >= 0 && nb != c && (pass ? nb > c : nb < c) ? nb : -1;
+                if (x.nb[m] < 0) continue;
+                const double2 *M = (const double2 *)(a.MW + 16 * (4 * (size_t)c + m) + 4 * q);
+                const double2 u = M[0], v = M[1];
+                x.m[m][0] = u.x; x.m[m][1] = u.y; x.m[m][2] = v.x; x.m[m][3] = v.y;
+            }
+        };
+        AdjMacroCell cur, nxt;
+        load(0, cur);
+        for (int step = 0; step < nd; ++step) {
+            load(step + 1, nxt);
+            __syncthreads();
+            if (cur.c >= 0) {
+                double acc = pass ? y[4 * cur.c + q] : cur.b;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    if (cur.nb[m] < 0) continue;
+                    const double *z = y + 4 * cur.nb[m];
+                    acc += fma(cur.m[m][0], z[0], cur.m[m][1] * z[1]) + fma(cur.m[m][2], z[2], cur.m[m][3] * z[3]);
+                }
+                y[4 * cur.c + q] = acc;
+            }
+            cur = nxt;
         }
         __syncthreads();
     }
-    for (int d = ni + nj - 2; d >= 0; --d) {
-        const int i0 = max(0, d - nj + 1), i1 = min(d, ni - 1);
-        for (int i = i0 + threadIdx.x; i <= i1; i += blockDim.x) {
-            const int c = (d - i) * ni + i;
-            double acc[4] = {0, 0, 0, 0};
-            macro_couple(a, c, false, acc);
-            for (int q = 0; q < 4; ++q) a.ba[4 * c + q] += acc[q] / a.DW[c];
-        }
-        __syncthreads();
-    }
+    if (SMEM)
+        for (int i = threadIdx.x; i < 4 * a.N; i += blockDim.x) a.ba[i] = y[i];
 }
 
 // per face: seeds bar F (from bar_b of the two cells), bar Phi (from bar_a and
@@ -813,6 +942,8 @@ size_t adjoint_layout(const AParams &s, int nrhs, char *base, AParams *out)
     a.fbarG = (double *)take(nf * Nv * d);
     a.fbarH = (double *)take(nf * Nv * d);
     a.DW = (double *)take(N * d);
+    a.MW = (double *)take(64 * N * d);
+    a.sgeo = (double *)take(16 * N * d);
     for (int r = 0; r < nrhs; ++r) {
         a.seed = r;
         a.lamG = (double *)take(NNv * d);
@@ -837,9 +968,15 @@ size_t adjoint_layout(const AParams &s, int nrhs, char *base, AParams *out)
     return off + 256;
 }
 
+constexpr size_t kAdjSmem = 224 * 1024;  // dynamic shared memory the sweeps may ask for
+
 int launch_adjoint_setup(const AParams &a, void *stream)
 {
     cudaStream_t st = (cudaStream_t)stream;
+    for (const void *k : {(const void *)k_adj_lines<true>, (const void *)k_adj_lines<false>, (const void *)k_adj_macro<true, 512>, (const void *)k_adj_macro<true, 1024>}) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAdjSmem);
+        if (e != cudaSuccess) return (int)e;
+    }
     const size_t NNv = (size_t)a.N * a.Nv;
     k_adj_cell_lin<<<a.N, kTB, 0, st>>>(a);
     k_adj_grad_lin<<<nblk(2 * NNv, 256), 256, 0, st>>>(a);
@@ -905,11 +1042,16 @@ int launch_adjoint_iteration(const AParams &a, int it, void *stream)
 {
     cudaStream_t st = (cudaStream_t)stream;
     const size_t NNv = (size_t)a.N * a.Nv;
-    const dim3 sweep_grid(nblk(a.Nv, 32), 2);
-    k_adj_micro_asc<<<sweep_grid, kTB, 0, st>>>(a);
-    k_adj_micro_desc<<<sweep_grid, kTB, 0, st>>>(a);
+    const AdjShape sh = adj_shape(a);
+    k_adj_lines<true><<<nblk(a.Nv, sh.G), 32 * sh.strips, sh.smem, st>>>(a, sh, a.status);
+    k_adj_lines<false><<<nblk(a.Nv, sh.G), 32 * sh.strips, sh.smem, st>>>(a, sh, a.status);
     k_adj_wprime<<<a.N, kTB, 0, st>>>(a);
-    k_adj_macro<<<1, kTB, 0, st>>>(a);
+    const int mt = std::min(1024, (4 * std::min(a.ni, a.nj) + 31) / 32 * 32);
+    const size_t ysm = (size_t)32 * a.N;
+    // (more than 128 lines leave a thread 64 registers, too few for two steps' blocks)
+    if (ysm > kAdjSmem) k_adj_macro<false, 1024><<<1, mt, 0, st>>>(a);
+    else if (mt <= 512) k_adj_macro<true, 512><<<1, mt, ysm, st>>>(a);
+    else k_adj_macro<true, 1024><<<1, mt, ysm, st>>>(a);
     k_adj_face<<<a.nf, kTB, 0, st>>>(a);
     k_adj_gather<<<nblk(2 * NNv, 256), 256, 0, st>>>(a);
     k_adj_cell<<<a.N, kTB, 0, st>>>(a);
