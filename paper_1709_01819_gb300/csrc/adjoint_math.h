@@ -79,24 +79,35 @@ struct Eq {
 // reciprocal of the cell's or boundary's own numbers: a loop over velocities
 // takes each reciprocal once, and a float64 division costs a dozen operations
 // of a pipe that issues one per 16 cycles.)
-IDG_AD void eq_eval(const Eq &e, double ux, double uy, double &G, double &H)
+// E, the reduced Maxwellian (the only part with an exponential)
+IDG_AD double eq_maxwell(const Eq &e, double ux, double uy)
 {
-    const double iRT = 1.0 / e.RT, lam = 0.5 * iRT, A = e.rho * lam * (1.0 / M_PI);
+    const double lam = 0.5 / e.RT, A = e.rho * lam * (1.0 / M_PI);
+    const double cx = ux - e.U, cy = uy - e.V;
+    return A * exp(-(cx * cx + cy * cy) * lam);
+}
+
+// the equilibrium from its Maxwellian E
+IDG_AD void eq_eval_at(const Eq &e, double E, double ux, double uy, double &G, double &H)
+{
+    const double iRT = 1.0 / e.RT;
     const double r2 = e.kappa * iRT * iRT / e.rho, px = r2 * e.qx, py = r2 * e.qy, kRT = e.K * e.RT;
-    const double cx = ux - e.U, cy = uy - e.V, c2 = cx * cx + cy * cy;
-    const double E = A * exp(-c2 * lam);
-    const double P = cx * px + cy * py, t = c2 * iRT;
+    const double cx = ux - e.U, cy = uy - e.V;
+    const double P = cx * px + cy * py, t = (cx * cx + cy * cy) * iRT;
     G = E * (1.0 + P * (t - 4.0));
     H = kRT * E * (1.0 + P * (t - 2.0));
 }
-
-// b[0..5] += (d(G,H)/d(rho, U, V, RT, qx, qy))^T (bG, bH) at one velocity
-IDG_AD void eq_vjp(const Eq &e, double ux, double uy, double bG, double bH, double *b)
+IDG_AD void eq_eval(const Eq &e, double ux, double uy, double &G, double &H)
 {
-    const double iRT = 1.0 / e.RT, irho = 1.0 / e.rho, lam = 0.5 * iRT, A = e.rho * lam * (1.0 / M_PI);
+    eq_eval_at(e, eq_maxwell(e, ux, uy), ux, uy, G, H);
+}
+
+// b[0..5] += (d(G,H)/d(rho, U, V, RT, qx, qy))^T (bG, bH) at one velocity, from E
+IDG_AD void eq_vjp_at(const Eq &e, double E, double ux, double uy, double bG, double bH, double *b)
+{
+    const double iRT = 1.0 / e.RT, irho = 1.0 / e.rho;
     const double r2 = e.kappa * irho * iRT * iRT, px = r2 * e.qx, py = r2 * e.qy, kRT = e.K * e.RT;
-    const double cx = ux - e.U, cy = uy - e.V, c2 = cx * cx + cy * cy, t = c2 * iRT;
-    const double E = A * exp(-c2 * lam);
+    const double cx = ux - e.U, cy = uy - e.V, t = (cx * cx + cy * cy) * iRT;
     const double P = cx * px + cy * py, sG = t - 4.0, sH = t - 2.0;
     const double gH = bH * (1.0 + P * sH), bHk = bH * kRT;
     const double bE = (bG * (1.0 + P * sG) + kRT * gH) * E;  // (weight of E) E
@@ -109,6 +120,10 @@ IDG_AD void eq_vjp(const Eq &e, double ux, double uy, double bG, double bH, doub
     b[3] += (bE * (0.5 * t - 1.0) - 2.0 * bP * P - bs * t) * iRT + e.K * E * gH;
     b[4] += bP * r2 * cx;
     b[5] += bP * r2 * cy;
+}
+IDG_AD void eq_vjp(const Eq &e, double ux, double uy, double bG, double bH, double *b)
+{
+    eq_vjp_at(e, eq_maxwell(e, ux, uy), ux, uy, bG, bH, b);
 }
 
 // Maxwellian of a boundary (q = 0): (G, H) and their derivatives with

@@ -143,7 +143,9 @@ __global__ void __launch_bounds__(kTB) k_adj_cell_lin(AParams a)
     const adj::Eq e = cell_eq(a, cp);
     for (int k = threadIdx.x; k < Nv; k += blockDim.x) {
         double eg, eh;
-        adj::eq_eval(e, a.ux[k], a.uy[k], eg, eh);
+        const double E = adj::eq_maxwell(e, a.ux[k], a.uy[k]);
+        a.Ec[(size_t)c * Nv + k] = E;
+        adj::eq_eval_at(e, E, a.ux[k], a.uy[k], eg, eh);
         a.fbG[(size_t)c * Nv + k] = cp[CP_C1] * G[k] + cp[CP_C2] * eg;
         a.fbH[(size_t)c * Nv + k] = cp[CP_C1] * H[k] + cp[CP_C2] * eh;
     }
@@ -311,7 +313,9 @@ __global__ void __launch_bounds__(kTB) k_adj_face_lin(AParams a)
     double ph[4] = {0, 0, 0, 0};
     for (int k = threadIdx.x; k < Nv; k += blockDim.x) {
         double eg, eh;
-        adj::eq_eval(e, a.ux[k], a.uy[k], eg, eh);
+        const double E = adj::eq_maxwell(e, a.ux[k], a.uy[k]);
+        a.Ef[(size_t)f * Nv + k] = E;
+        adj::eq_eval_at(e, E, a.ux[k], a.uy[k], eg, eh);
         const double sn = xdn(a.ux[k], a.uy[k], nx, ny);
         const double Fg = sn * S * (fp[FP_A] * a.fbarG[(size_t)f * Nv + k] + fp[FP_B] * eg);
         const double Fh = sn * S * (fp[FP_A] * a.fbarH[(size_t)f * Nv + k] + fp[FP_B] * eh);
@@ -340,50 +344,65 @@ __global__ void __launch_bounds__(kTB) k_adj_face_lin(AParams a)
     if (threadIdx.x < kFP) a.fpar[(size_t)kFP * f + threadIdx.x] = fp[threadIdx.x];
 }
 
-// per cell: diagonal of the macroscopic LU-SGS, Omega/dt_imp + (omega/2) sum
-// Lambda, and the transposed blocks towards its neighbours,
-// (1/2)(S A(W_c; n_out)^T + omega Lambda I), A the Euler flux Jacobian, over that
-// diagonal (they stay what they are through the iteration); the record of the
-// micro sweeps: per direction the scaled outward normals of the own line's next
-// face and of the faces towards the adjacent lines, the swept side first (0 where
-// a cell is its own neighbour), and Omega/dt_imp + cq
+// per cell: one over the diagonal of the macroscopic LU-SGS, Omega/dt_imp +
+// (omega/2) sum Lambda, and over it the transposed blocks towards the neighbours,
+// (1/2)(S A(W_c; n_out)^T + omega Lambda I), A the Euler flux Jacobian (they stay
+// what they are through the iteration)
 __global__ void k_adj_macro_lin(AParams a)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= a.N) return;
     double d = a.area[c] / a.dtimp[c];
-    const double D0 = d + a.cpar[(size_t)kCP * c + CP_CQ];
     for (int m = 0; m < 4; ++m) {
         const int f = a.cface[4 * c + m];
         if (a.fL[f] == a.fR[f]) continue;
         d += 0.5 * a.lusgs_omega * a.fpar[(size_t)kFP * f + FP_LAM];
     }
-    a.DW[c] = d;
-    const bool cols = a.ni <= a.nj;
+    const double id = 1.0 / d;
+    a.iDW[c] = id;
     for (int m = 0; m < 4; ++m) {
         const int f = a.cface[4 * c + m], nb = a.cnb[4 * c + m];
-        const bool self = a.fL[f] == a.fR[f];
+        const bool couples = nb >= 0 && a.fL[f] != a.fR[f];
         const double *g = a.fgeo + 7 * f;
-        const double sgn = a.csign[4 * c + m], nx = sgn * g[0], ny = sgn * g[1];
+        const double sgn = a.csign[4 * c + m], lam = a.lusgs_omega * a.fpar[(size_t)kFP * f + FP_LAM];
         double *M = a.MW + 16 * (4 * (size_t)c + m);
         for (int q = 0; q < 4; ++q) {
             double y[4] = {0, 0, 0, 0}, t[4] = {0, 0, 0, 0};
             y[q] = 1.0;
-            if (nb >= 0 && !self) adj::euler_jacT(a.W + 4 * c, a.gam, nx, ny, y, t);
-            for (int r = 0; r < 4; ++r)
-                M[4 * r + q] = nb >= 0 && !self ? 0.5 * (g[2] * t[r] + (r == q ? a.lusgs_omega * a.fpar[(size_t)kFP * f + FP_LAM] : 0.0)) / d : 0.0;
-        }
-        // slots (west 0, east 1, south 2, north 3) -> entry of the two records
-        const bool own = cols ? m >= 2 : m < 2, up = m & 1;
-        for (int dir = 0; dir < 2; ++dir) {
-            double *o = a.sgeo + 8 * ((size_t)dir * a.N + c);
-            const int e = own ? (up != (dir == 1) ? 0 : -1) : (up != (dir == 1) ? 4 : 2);
-            if (e < 0) continue;
-            o[e] = self ? 0.0 : nx * g[2];
-            o[e + 1] = self ? 0.0 : ny * g[2];
+            if (couples) adj::euler_jacT(a.W + 4 * c, a.gam, sgn * g[0], sgn * g[1], y, t);
+            for (int r = 0; r < 4; ++r) M[4 * r + q] = couples ? 0.5 * id * (g[2] * t[r] + (r == q ? lam : 0.0)) : 0.0;
         }
     }
-    a.sgeo[8 * (size_t)c + 6] = a.sgeo[8 * ((size_t)a.N + c) + 6] = D0;
+}
+
+// (xi.n)^+ S through slot m of cell c, outward (0 where the cell is its own neighbour)
+__device__ __forceinline__ double outflow(const AParams &a, int c, int m, double ux, double uy)
+{
+    const int f = a.cface[4 * c + m];
+    if (a.fL[f] == a.fR[f]) return 0.0;
+    const double *g = a.fgeo + 7 * f;
+    const double so = a.csign[4 * c + m] * xdn(ux, uy, g[0], g[1]);
+    return so > 0 ? so * g[2] : 0.0;
+}
+
+// per (cell, velocity): one over the micro LU-SGS diagonal of Eq. (26) and over it
+// the couplings of the transposed sweeps to the two neighbours already swept away
+// from a seam (constant through the iteration; both components share them)
+__global__ void k_adj_micro_lin(AParams a)
+{
+    const size_t NNv = (size_t)a.N * a.Nv, ck = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (ck >= NNv) return;
+    const int c = (int)(ck / a.Nv), k = (int)(ck % a.Nv), j = c / a.ni, i = c - j * a.ni;
+    double so[4], d = a.area[c] / a.dtimp[c] + a.cpar[(size_t)kCP * c + CP_CQ];
+    for (int m = 0; m < 4; ++m) d += so[m] = outflow(a, c, m, a.ux[k], a.uy[k]);
+    const double id = 1.0 / d;
+    a.iDm[ck] = id;
+    // neighbours that exist without crossing a seam: west, east, south, north
+    const bool in[4] = {i > 0, i + 1 < a.ni, j > 0, j + 1 < a.nj};
+    const int w = a.ni <= a.nj ? 2 : 0, t = 2 - w;  // slots along the own line, across
+    double2 *o = (double2 *)a.cm;
+    for (int dir = 0; dir < 2; ++dir)
+        o[dir * NNv + ck] = make_double2(in[w + dir] ? so[w + dir] * id : 0.0, in[t + dir] ? so[t + dir] * id : 0.0);
 }
 
 // ---------------------------------------------------------------------------
@@ -397,9 +416,12 @@ __global__ void k_adj_macro_lin(AParams a)
 // velocities, one step behind one another, exactly as the forward sweeps of a
 // structured block do (k_sweep_lines: registers along the line, shuffles across,
 // rings and flags between the strips of a block, copies kAdjAhead steps ahead);
-// a thread carries both components.  Bound by the float64 pipe and the latency of
-// a step.  A hyperplane per barrier with the geometry re-derived at every face
-// took 400 + 461 us on 24 x 24 cells x 256 velocities, this 14 + 15 us.
+// a thread carries both components, and the couplings come from
+// k_adj_micro_lin: the float64 pipe takes 64 cycles per warp instruction of a
+// scheduler, and forming them in the step was 60 such instructions, using them
+// is 6.  A hyperplane per barrier with the geometry re-derived at every face
+// took 400 + 461 us on 24 x 24 cells x 256 velocities, lines with the couplings
+// formed in the step 129 + 129 us, this 25 + 29 us.
 constexpr int kAdjAhead = 4, kAdjRing = 32;
 
 struct AdjShape {
@@ -416,11 +438,11 @@ AdjShape adj_shape(const AParams &a)
     while (s.G > 1 && (a.Nv / s.G < 152 || (nt + 32 / s.G - 1) / (32 / s.G) > 16)) s.G /= 2;
     const int lw = 32 / s.G;
     s.strips = (nt + lw - 1) / lw;
-    s.smem = 64 + (size_t)s.strips * (kAdjRing * s.G * 16 + kAdjAhead * (32 * 16 + lw * 64));
+    s.smem = 64 + (size_t)s.strips * (kAdjRing * s.G * 16 + kAdjAhead * 32 * 40);
     return s;
 }
 
-template <bool ASC> __global__ void __launch_bounds__(512) k_adj_lines(AParams a, AdjShape sh, int *status)
+template <bool ASC> __global__ void __launch_bounds__(512) k_adj_lines(AParams a, AdjShape sh)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     int *flags = (int *)smraw;
@@ -435,96 +457,87 @@ template <bool ASC> __global__ void __launch_bounds__(512) k_adj_lines(AParams a
     __syncthreads();
     const int tt = strip * lw + l, tc = min(tt, nt - 1);
     const int k0 = blockIdx.x * G + g, k = k0 < Nv ? k0 : 0;
-    const double ux = a.ux[k], uy = a.uy[k];
     const int t = ASC ? tc : nt - 1 - tc;
     const int cs = (ASC ? 1 : -1) * (cols ? a.ni : 1);
     const int c0 = (cols ? t : t * a.ni) + (ASC ? 0 : (nw - 1) * (cols ? a.ni : 1));
     const ptrdiff_t base = (ptrdiff_t)c0 * Nv + k;
-    const int sv = cs * Nv, sg = cs * 8;
-    const double *xG = (ASC ? a.lamG : a.bbG) + base, *xH = (ASC ? a.lamH : a.bbH) + base;
+    const int sv = cs * Nv;
+    const double *xG = (ASC ? a.lamG : a.bbG) + base, *xH = (ASC ? a.lamH : a.bbH) + base, *iD = a.iDm + base;
+    const double2 *cm = (const double2 *)a.cm + (ASC ? 0 : (ptrdiff_t)a.N * Nv) + base;
     double *yG = a.bbG + base, *yH = a.bbH + base;
-    const double *geo = a.sgeo + (ASC ? 0 : (ptrdiff_t)a.N * 8) + (ptrdiff_t)c0 * 8;
     const unsigned nwl = tt < nt && k0 < Nv ? nw : 0;
     const int start = tt + strip * kSweepBlock;
     const bool seam_t = (cols ? a.per_i : a.per_j) && nt > 1, seam_w = (cols ? a.per_j : a.per_i) && nw > 1;
+    const int m_w = (cols ? 2 : 0) + (ASC ? 1 : 0), m_t = (cols ? 0 : 2) + (ASC ? 1 : 0);  // slots ahead
     const bool edge = l == 0 && strip > 0, border = l == lw - 1 && strip + 1 < strips;
     double2 *xw = (double2 *)(smraw + 64) + (size_t)strip * kAdjRing * G + g;
     const double2 *xr = strip > 0 ? xw - (size_t)kAdjRing * G : xw;
-    const int SB = 32 * 16 + lw * 64;
+    // stages [kAdjAhead] of {couplings, x_G and x_H, 1/D (ascending)} per lane
+    constexpr int SB = 32 * 40;
     unsigned char *stage = smraw + 64 + (size_t)strips * kAdjRing * G * 16 + (size_t)strip * kAdjAhead * SB;
     auto issue = [&](int s) {
-        const int wc = min(max(s - start, 0), nw - 1);
+        const ptrdiff_t o = (ptrdiff_t)min(max(s - start, 0), nw - 1) * sv;
         unsigned char *st = stage + (s & (kAdjAhead - 1)) * SB;
-        cp_async8(st + lane * 16, xG + (ptrdiff_t)wc * sv);
-        cp_async8(st + lane * 16 + 8, xH + (ptrdiff_t)wc * sv);
-        const char *gg = (const char *)(geo + (ptrdiff_t)wc * sg);
-        for (int q = g; q < 4; q += G) cp_async16(st + 512 + l * 64 + 16 * q, gg + 16 * q);
+        cp_async16(st + lane * 16, cm + o);
+        cp_async8(st + 512 + lane * 16, xG + o);
+        cp_async8(st + 512 + lane * 16 + 8, xH + o);
+        if (ASC) cp_async8(st + 1024 + lane * 8, iD + o);
         cp_commit();
     };
     for (int u = 0; u < kAdjAhead; ++u) issue(s_beg + u);
-    // (xi.n) S of the line's end face, outward from its first cell
-    double end = 0.0;
-    {
-        const int m = (cols ? 2 : 0) + (ASC ? 0 : 1), f = a.cface[4 * c0 + m];
-        if (a.fL[f] != a.fR[f]) {
-            const double *q = a.fgeo + 7 * f, sgn = a.csign[4 * c0 + m];
-            end = xdn(ux, uy, sgn * q[0] * q[2], sgn * q[1] * q[2]);
-        }
-    }
     double2 prev = make_double2(0, 0), first = make_double2(0, 0);
-    double cl, co, ca, cu, iD, ahead = 0.0;
-    auto coef = [&](int s) {
-        const int ww = s - start;
-        const double *q = (const double *)(stage + (s & (kAdjAhead - 1)) * SB + 512 + l * 64);
-        const double own = ww > 0 ? -ahead : end;
-        ahead = xdn(ux, uy, q[0], q[1]);
-        const double low = xdn(ux, uy, q[2], q[3]), upp = xdn(ux, uy, q[4], q[5]);
-        // half the sum of all |xi.n| S is the outflow: the normals sum to zero
-        iD = __drcp_rn(fma(0.5, (fabs(own) + fabs(ahead)) + (fabs(low) + fabs(upp)), q[6]));
-        cl = low > 0.0 && tt > 0 ? low : 0.0;
-        co = own > 0.0 && ww > 0 ? own : 0.0;
-        ca = seam_w && ww == nw - 1 && ahead > 0.0 ? ahead : 0.0;
-        cu = seam_t && tt == nt - 1 && upp > 0.0 ? upp : 0.0;
-    };
-    cp_wait<kAdjAhead - 1>();
-    __syncwarp();
-    coef(s_beg);
     int seen_r = 0, seen_w = 0;
     for (int s0 = s_beg; s0 < s_end; s0 += kSweepBlock) {
         if (strips > 1) {
-            if (strip > 0) flag_wait(flags + strip - 1, s0, seen_r, status);
-            if (strip + 1 < strips) flag_wait(flags + strip + 1, s0 + 2 * kSweepBlock + 1 - kAdjRing, seen_w, status);
+            if (strip > 0) flag_wait(flags + strip - 1, s0, seen_r, a.status);
+            if (strip + 1 < strips) flag_wait(flags + strip + 1, s0 + 2 * kSweepBlock + 1 - kAdjRing, seen_w, a.status);
         }
 #pragma unroll
         for (int b = 0; b < kSweepBlock; ++b) {
             const int s = s0 + b, ww = s - start;
-            cp_wait<kAdjAhead - 2>();
+            cp_wait<kAdjAhead - 1>();
             __syncwarp();
             const bool on = (unsigned)ww < nwl;
-            const double2 x = *(const double2 *)(stage + (s & (kAdjAhead - 1)) * SB + lane * 16);
+            const unsigned char *st = stage + (s & (kAdjAhead - 1)) * SB;
+            const double2 cf = *(const double2 *)(st + lane * 16);
+            const double2 x = *(const double2 *)(st + 512 + lane * 16);
             const double2 ev = xr[(ww & (kAdjRing - 1)) * G];
             double2 adj;
             adj.x = __shfl_up_sync(0xffffffffu, prev.x, G);
             adj.y = __shfl_up_sync(0xffffffffu, prev.y, G);
             if (edge) adj = ev;
-            double ag = fma(cl, adj.x, co * prev.x), ah = fma(cl, adj.y, co * prev.y);
-            if (ca > 0.0) {
-                ag = fma(ca, first.x, ag);
-                ah = fma(ca, first.y, ah);
+            double2 y = x;
+            if (ASC) {
+                const double d = *(const double *)(st + 1024 + lane * 8);
+                y.x *= d;
+                y.y *= d;
             }
-            if (on && cu > 0.0) {
-                const ptrdiff_t o = (ptrdiff_t)ww * sv + (ptrdiff_t)((ASC ? 0 : nt - 1) - t) * (cols ? 1 : a.ni) * Nv;
-                ag = fma(cu, yG[o], ag);
-                ah = fma(cu, yH[o], ah);
+            // (a line's first cell and the first line couple to nothing behind them)
+            y.x = fma(cf.y, adj.x, fma(cf.x, prev.x, y.x));
+            y.y = fma(cf.y, adj.y, fma(cf.x, prev.y, y.y));
+            // across a seam: the line's own first cell, the first line's cell
+            if (on && ((seam_w && ww == nw - 1) || (seam_t && tt == nt - 1))) {
+                const int c = c0 + ww * cs;
+                const double d = iD[(ptrdiff_t)ww * sv];
+                if (seam_w && ww == nw - 1) {
+                    const double ca = d * outflow(a, c, m_w, a.ux[k], a.uy[k]);
+                    y.x = fma(ca, first.x, y.x);
+                    y.y = fma(ca, first.y, y.y);
+                }
+                if (seam_t && tt == nt - 1) {
+                    const double cu = d * outflow(a, c, m_t, a.ux[k], a.uy[k]);
+                    const ptrdiff_t o = (ptrdiff_t)ww * sv + (ptrdiff_t)((ASC ? 0 : nt - 1) - t) * (cols ? 1 : a.ni) * Nv;
+                    y.x = fma(cu, yG[o], y.x);
+                    y.y = fma(cu, yH[o], y.y);
+                }
             }
-            prev.x = ASC ? (x.x + ag) * iD : fma(ag, iD, x.x);
-            prev.y = ASC ? (x.y + ah) * iD : fma(ah, iD, x.y);
-            if (ww == 0) first = prev;
-            coef(s + 1);
+            // (lanes without a cell copy an existing one: their results are finite and unused)
+            prev = y;
+            if (ww == 0) first = y;
             if (on) {
-                yG[(ptrdiff_t)ww * sv] = prev.x;
-                yH[(ptrdiff_t)ww * sv] = prev.y;
-                if (border) xw[(ww & (kAdjRing - 1)) * G] = prev;
+                yG[(ptrdiff_t)ww * sv] = y.x;
+                yH[(ptrdiff_t)ww * sv] = y.y;
+                if (border) xw[(ww & (kAdjRing - 1)) * G] = y;
             }
             issue(s + kAdjAhead);
         }
@@ -555,9 +568,10 @@ __global__ void __launch_bounds__(kTB) k_adj_wprime(AParams a)
     double s[7] = {0, 0, 0, 0, 0, 0, 0};
     for (int k = threadIdx.x; k < Nv; k += blockDim.x) {
         double eg, eh;
-        adj::eq_eval(e, a.ux[k], a.uy[k], eg, eh);
-        s[6] -= bG[k] * (G[k] - eg) + bH[k] * (H[k] - eh);
-        adj::eq_vjp(e, a.ux[k], a.uy[k], cq * bG[k], cq * bH[k], s);
+        const double E = a.Ec[(size_t)c * Nv + k], x = a.ux[k], y = a.uy[k], bg = bG[k], bh = bH[k];
+        adj::eq_eval_at(e, E, x, y, eg, eh);
+        s[6] -= bg * (G[k] - eg) + bh * (H[k] - eh);
+        adj::eq_vjp_at(e, E, x, y, cq * bg, cq * bh, s);
     }
     bsum<7>(s, sm);
     if (threadIdx.x == 0) {
@@ -580,7 +594,7 @@ __global__ void __launch_bounds__(kTB) k_adj_wprime(AParams a)
 // before the barrier that opens it, so that after it only the neighbours'
 // increments are read -- from shared memory where all cells' fit (SMEM).
 // Re-deriving the Jacobians at every face took 767 us on 24 x 24 cells, this
-// 22 us.
+// 84 us (float64 operations of a few warps, 64 cycles each).
 struct AdjMacroCell {
     int c, nb[4];
     double b, m[4][4];
@@ -601,7 +615,7 @@ __global__ void __launch_bounds__(NT) k_adj_macro(AParams a)
             if (i > min(d, ni - 1)) return;
             const int c = (d - i) * ni + i;
             x.c = c;
-            if (!pass) x.b = a.bwp[4 * c + q] / a.DW[c];
+            if (!pass) x.b = a.bwp[4 * c + q] * a.iDW[c];
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 const int nb = a.cnb[4 * c + m];
@@ -675,11 +689,12 @@ __global__ void __launch_bounds__(kTB) k_adj_face(AParams a)
     for (int k = threadIdx.x; k < Nv; k += blockDim.x) {
         double bg, bh, eg, eh;
         barF(k, bg, bh);
-        adj::eq_eval(e, a.ux[k], a.uy[k], eg, eh);
+        const double E = a.Ef[(size_t)f * Nv + k];
+        adj::eq_eval_at(e, E, a.ux[k], a.uy[k], eg, eh);
         const double snS = xdn(a.ux[k], a.uy[k], nx, ny) * S;
         s[6] += snS * (fbG[k] * bg + fbH[k] * bh);
         s[7] += snS * (eg * bg + eh * bh);
-        adj::eq_vjp(e, a.ux[k], a.uy[k], snS * Bc * bg, snS * Bc * bh, s);
+        adj::eq_vjp_at(e, E, a.ux[k], a.uy[k], snS * Bc * bg, snS * Bc * bh, s);
     }
     bsum<8>(s, sm);
     if (threadIdx.x == 0) {
@@ -859,10 +874,11 @@ __global__ void __launch_bounds__(kTB) k_adj_cell(AParams a)
         a.bfb[(size_t)c * Nv + k] = b[0];
         a.bfb[NNv + (size_t)c * Nv + k] = b[1];
         double eg, eh;
-        adj::eq_eval(e, a.ux[k], a.uy[k], eg, eh);
+        const double E = a.Ec[(size_t)c * Nv + k], x = a.ux[k], y = a.uy[k];
+        adj::eq_eval_at(e, E, x, y, eg, eh);
         s[6] += G[k] * b[0] + H[k] * b[1];
         s[7] += eg * b[0] + eh * b[1];
-        adj::eq_vjp(e, a.ux[k], a.uy[k], c2 * b[0], c2 * b[1], s);
+        adj::eq_vjp_at(e, E, x, y, c2 * b[0], c2 * b[1], s);
     }
     bsum<8>(s, sm);
     if (threadIdx.x == 0) {
@@ -941,9 +957,12 @@ size_t adjoint_layout(const AParams &s, int nrhs, char *base, AParams *out)
     a.fpar = (double *)take(kFP * nf * d);
     a.fbarG = (double *)take(nf * Nv * d);
     a.fbarH = (double *)take(nf * Nv * d);
-    a.DW = (double *)take(N * d);
+    a.iDW = (double *)take(N * d);
     a.MW = (double *)take(64 * N * d);
-    a.sgeo = (double *)take(16 * N * d);
+    a.Ec = (double *)take(NNv * d);
+    a.Ef = (double *)take(nf * Nv * d);
+    a.iDm = (double *)take(NNv * d);
+    a.cm = (double *)take(4 * NNv * d);
     for (int r = 0; r < nrhs; ++r) {
         a.seed = r;
         a.lamG = (double *)take(NNv * d);
@@ -981,7 +1000,8 @@ int launch_adjoint_setup(const AParams &a, void *stream)
     k_adj_cell_lin<<<a.N, kTB, 0, st>>>(a);
     k_adj_grad_lin<<<nblk(2 * NNv, 256), 256, 0, st>>>(a);
     k_adj_face_lin<<<a.nf, kTB, 0, st>>>(a);
-    k_adj_macro_lin<<<nblk(a.N, 128), 128, 0, st>>>(a);
+    k_adj_macro_lin<<<nblk(a.N, 32), 32, 0, st>>>(a);
+    k_adj_micro_lin<<<nblk(NNv, 256), 256, 0, st>>>(a);
     return (int)cudaGetLastError();
 }
 
@@ -1043,8 +1063,8 @@ int launch_adjoint_iteration(const AParams &a, int it, void *stream)
     cudaStream_t st = (cudaStream_t)stream;
     const size_t NNv = (size_t)a.N * a.Nv;
     const AdjShape sh = adj_shape(a);
-    k_adj_lines<true><<<nblk(a.Nv, sh.G), 32 * sh.strips, sh.smem, st>>>(a, sh, a.status);
-    k_adj_lines<false><<<nblk(a.Nv, sh.G), 32 * sh.strips, sh.smem, st>>>(a, sh, a.status);
+    k_adj_lines<true><<<nblk(a.Nv, sh.G), 32 * sh.strips, sh.smem, st>>>(a, sh);
+    k_adj_lines<false><<<nblk(a.Nv, sh.G), 32 * sh.strips, sh.smem, st>>>(a, sh);
     k_adj_wprime<<<a.N, kTB, 0, st>>>(a);
     const int mt = std::min(1024, (4 * std::min(a.ni, a.nj) + 31) / 32 * 32);
     const size_t ysm = (size_t)32 * a.N;

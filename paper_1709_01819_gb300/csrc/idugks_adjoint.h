@@ -53,9 +53,12 @@ struct AParams {
     signed char *lsl;  // [2][N][Nv][2] limiter: binding face slot, extreme-neighbour slot (-1: self)
     double *fpar;      // [nf][kFP]
     double *fbarG, *fbarH;  // [nf][Nv]
-    double *DW;        // [N] macroscopic LU-SGS diagonal
+    double *Ec, *Ef;   // [N][Nv], [nf][Nv] reduced Maxwellian of the cell's / face's equilibrium
+    double *iDm;       // [N][Nv] one over the micro LU-SGS diagonal
+    double *cm;        // [2][N][Nv][2] ascending, descending: micro couplings over the diagonal, towards
+                       // the cell behind on the own line and the swept adjacent line
+    double *iDW;       // [N] one over the macroscopic LU-SGS diagonal
     double *MW;        // [N][4][16] per slot the transposed macroscopic block over DW (0: no coupling)
-    double *sgeo;      // [2][N][8] ascending, descending: what the micro sweeps read of a cell (k_adj_lines)
     // adjoint iteration
     double *lamG, *lamH, *lamW;  // [N][Nv], [N][Nv], [N][4]
     double *bbG, *bbH;           // [N][Nv] P_f^-T lambda_f
