@@ -609,6 +609,7 @@ size_t layout(idg_ctx *c, char *base, KParams *kp)
     k.scode = c->unstr ? L.take<int>(32 * N) : nullptr;
     k.sgeo = c->unstr ? nullptr : L.take<char>(16 * ts * N);
     k.sched = c->unstr ? L.take<int>(4 * c->sched.size()) : nullptr;
+    k.snb = c->unstr ? L.take<int>(32 * N) : nullptr;
     k.sptr = c->unstr ? L.take<int>(4 * c->sptr.size()) : nullptr;
     k.fL = L.take<int>(4 * nf);
     k.fR = L.take<int>(4 * nf);
@@ -1193,6 +1194,15 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
                             sgeo[8 * ((size_t)dir * c->N + q) + 2 * m + x] = cslot[8 * q + 2 * slot[m] + x];
             }
     }
+    std::vector<int> snb(c->unstr ? (size_t)8 * c->N : 0, -1);
+    for (size_t q = 0; q < snb.size() / 4; ++q) {
+        const int cell = c->sched[q];
+        const bool fwd = q < (size_t)c->N;
+        for (int m = 0; m < 4; ++m) {
+            const int nb = c->cnb[4 * cell + m];
+            if (nb >= 0 && (fwd ? nb < cell : nb > cell)) snb[4 * q + m] = nb;
+        }
+    }
     cudaError_t errs[] = {
         up((double *)k.area, c->area), up((double *)k.dtimp, c->dtimp), up((double *)k.adt, adt), up((int *)k.cface, c->cface),
         up((int *)k.cnb, c->cnb), up((int *)k.csign, c->csign), up_storage(c, k.crT, c->cr),
@@ -1203,7 +1213,7 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
         up((double *)k.ux, c->ux), up((double *)k.uy, c->uy), up((double *)k.w, c->w),
         up((float *)k.uxf, uxf), up((float *)k.uyf, uyf), up((float *)k.wf, wf),
         cudaMemset(k.iter, 0, 256), cudaMemset(k.phi, 0, 32 * (size_t)c->nf),
-        c->unstr ? up((int *)k.sched, c->sched) : cudaSuccess, c->unstr ? up((int *)k.sptr, c->sptr) : cudaSuccess};
+        c->unstr ? up((int *)k.snb, snb) : cudaSuccess, c->unstr ? up((int *)k.sched, c->sched) : cudaSuccess, c->unstr ? up((int *)k.sptr, c->sptr) : cudaSuccess};
     for (cudaError_t x : errs)
         if (x != cudaSuccess) return cuda_fail(c, x, "workspace upload");
     int rcfg = idg::configure_kernels(c->precision == IDG_FP64);

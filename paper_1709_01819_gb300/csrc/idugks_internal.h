@@ -104,6 +104,7 @@ struct KParams {
     // into each ([nsteps_f + 1] then [nsteps_b + 1]); the cells of one step
     // depend on none of each other
     const int *sched, *sptr;
+    const int *snb;  // [2][N][4] in the order of sched: the cell's neighbours already swept, by slot (else -1)
     int nsteps_f, nsteps_b;
     // linearised diffuse wall of the micro sweeps (Eq. 33-35), implicit_wall
     // = 1: per face, wallS the inner cell's outgoing sum sum_out w (xi.n_out)
