@@ -1505,11 +1505,11 @@ idg_status idg_iterate(idg_ctx *c, int max_iter, double tol, void *stream, int *
         done += n;
         // residuals of this chunk from the device ring
         cudaError_t e;
-        for (int q = 0; q < n; ++q) {
-            long long slot = (it0 + q) & (idg::kMaxHist - 1);
-            e = cudaMemcpyAsync(&buf[q], c->kp.res + slot, 8, cudaMemcpyDeviceToHost, st);
-            if (e != cudaSuccess) return cuda_fail(c, e, "D2H residual");
-        }
+        // (one copy, two across the ring's end)
+        const int slot = (int)(it0 & (idg::kMaxHist - 1)), n1 = std::min(n, idg::kMaxHist - slot);
+        if ((e = cudaMemcpyAsync(buf.data(), c->kp.res + slot, (size_t)n1 * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+            (n1 < n && (e = cudaMemcpyAsync(buf.data() + n1, c->kp.res, (size_t)(n - n1) * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess))
+            return cuda_fail(c, e, "D2H residual");
         if ((e = cudaMemcpyAsync(&status, c->kp.status, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
             return cuda_fail(c, e, "D2H status");
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(c, e, "iteration");
