@@ -1125,6 +1125,13 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
         k.nsteps_f = c->nsteps_f;
         k.nsteps_b = c->nsteps_b;
     }
+    // k_cell_moments: a warp a cell, two or four from the length on that leaves each
+    // about four chunks of 256 velocities or more; the cells of such a problem are
+    // few thousands and fill few waves of warps (121 x 81 cells x 7921 velocities:
+    // 2.02 waves, 221 us; four warps a cell 173 us.  The face rows, twice as many,
+    // took 464 + 584 us at one warp and 454 + 565 us at four there, but 201 and
+    // 213 us on 128 x 128 x 784 with the code for several in them: they stay at one)
+    k.row_warps = c->Nv >= 4096 ? 4 : c->Nv >= 2048 ? 2 : 1;
     // per-(cell, velocity) kernels: four cells a block once that leaves every SM
     // its eight resident blocks, two or one below
     const long long nblocks = (long long)c->N * ((c->Nv + 255) / 256);

@@ -88,6 +88,7 @@ struct KParams {
     // launch shape of the wavefront kernels: velocities per CTA and cell
     // slots of the micro sweeps, prefetch depths (hyperplanes; 4 or 8)
     int sweep_tv, sweep_pc, sweep_stages, macro_stages;
+    int row_warps;   // warps per cell of k_cell_moments (1, 2, 4)
     int cpb;         // cells per block of the per-(cell, velocity) kernels
     int sweep_tuned; // 1: sweep_tv or sweep_vpt was set by the caller
     // line micro sweeps (sweep_shape()): threads per cell of a block and

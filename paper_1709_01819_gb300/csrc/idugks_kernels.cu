@@ -173,7 +173,7 @@ __device__ __forceinline__ FF ff_add(FF a, FF b)
 }
 
 template <class T> struct Acc;
-template <> struct Acc<float> {
+template <> struct alignas(8) Acc<float> {
     FF v;
     __device__ __forceinline__ void zero() { v = {0.f, 0.f}; }
     // (the error terms collect in lo: renormalised once, by warp_sum)
@@ -216,7 +216,27 @@ __device__ __forceinline__ FF shfl_xor_acc(FF a, int o)
 __device__ __forceinline__ double shfl_xor_acc(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
 __device__ __forceinline__ FF sum_acc(FF a, FF b) { return ff_add(a, b); }
 __device__ __forceinline__ double sum_acc(double a, double b) { return a + b; }
-template <int NA, class T> __device__ __forceinline__ void warp_sum_store(const Acc<T> (&acc)[NA], int lane, void *base, size_t i0)
+// One to four warps share a row (row_warps): with more than one their sums meet
+// in shared memory behind a barrier of those warps and are added in order.
+constexpr int kRowSums = 8 * 16;  // shared sums of a 256-thread block
+struct Row {
+    int sub, warps;  // this warp of the row's warps
+};
+__device__ __forceinline__ Row row_of(const KParams &p, int blk, int &row)
+{
+    Row r;
+    r.warps = p.row_warps;
+    const int w = threadIdx.x >> 5;
+    row = blk * (8 / r.warps) + w / r.warps;
+    r.sub = w & (r.warps - 1);
+    return r;
+}
+__device__ __forceinline__ void row_barrier(const Row &r)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x >> 5) / r.warps), "r"(32 * r.warps) : "memory");
+}
+template <int NA, class T>
+__device__ __forceinline__ void row_sum_store(const Acc<T> (&acc)[NA], int lane, const Row &r, Acc<T> *sums, void *base, size_t i0)
 {
     constexpr int NP = NA <= 4 ? 4 : 16;  // sums carried, the ones past NA zero
     decltype(acc[0].v) x[NP];
@@ -243,11 +263,18 @@ template <int NA, class T> __device__ __forceinline__ void warp_sum_store(const 
         }
     }
     // lanes that differ in the last log2(32 / NP) bits carry the same sum
-    if ((lane & (32 / NP - 1)) == 0 && mine < NA) {
-        Acc<T> a;
-        a.v = x[0];
-        a.store(base, i0 + mine);
+    const bool owner = (lane & (32 / NP - 1)) == 0 && mine < NA;
+    Acc<T> a;
+    a.v = x[0];
+    if (r.warps > 1) {
+        Acc<T> *s = sums + 16 * (threadIdx.x >> 5) + mine;
+        if (owner) *s = a;
+        row_barrier(r);
+        if (r.sub > 0) return;
+        if (owner)
+            for (int w = 1; w < r.warps; ++w) a.v = sum_acc(a.v, s[16 * w].v);
     }
+    if (owner) a.store(base, i0 + mine);
 }
 
 // an accumulator entry widened to float64
@@ -512,12 +539,13 @@ template <class T> __device__ __forceinline__ void load_pair(const void *base, s
 // k, k + 1 with k = k0 + 64u + 2l, u < 4, for chunks of 256 velocities (the
 // stored velocity count is a multiple of 4, so pairs are whole and start on
 // 16-byte boundaries); each chunk's per-lane partial sums (at most 8 terms)
-// are folded into the accumulators as in vel_loop.  fold(a) takes them.
+// are folded into the accumulators as in vel_loop.  fold(a) takes them.  The warps
+// of a row take its chunks in turn.
 template <int NA, class T, class Body, class Fold>
-__device__ __forceinline__ void vel_loop2(int Nv, int lane, Body body, Fold fold)
+__device__ __forceinline__ void vel_loop2(int Nv, int lane, const Row &row, Body body, Fold fold)
 {
-    int k0 = 0;
-    for (; k0 + 256 <= Nv; k0 += 256) {
+    int k0 = 256 * row.sub;
+    for (; k0 + 256 <= Nv; k0 += 256 * row.warps) {
         T a[NA];
 #pragma unroll
         for (int q = 0; q < NA; ++q) a[q] = (T)0;
@@ -537,9 +565,9 @@ __device__ __forceinline__ void vel_loop2(int Nv, int lane, Body body, Fold fold
     }
 }
 template <int NA, class T, class Body>
-__device__ __forceinline__ void vel_loop2(int Nv, int lane, Acc<T> (&acc)[NA], Body body)
+__device__ __forceinline__ void vel_loop2(int Nv, int lane, const Row &row, Acc<T> (&acc)[NA], Body body)
 {
-    vel_loop2<NA, T>(Nv, lane, body, [&](const T(&a)[NA]) {
+    vel_loop2<NA, T>(Nv, lane, row, body, [&](const T(&a)[NA]) {
 #pragma unroll
         for (int q = 0; q < NA; ++q) acc[q].add(a[q]);
     });
@@ -549,13 +577,13 @@ __device__ __forceinline__ void vel_loop2(int Nv, int lane, Acc<T> (&acc)[NA], B
 // (sacc[q * blockDim.x + threadIdx.x]) between chunks, which leaves a
 // 64-register thread room for its loads in flight.
 template <int NA, class Body>
-__device__ __forceinline__ void vel_loop2_sm(int Nv, int lane, Acc<float> (&acc)[NA], FF *sacc, Body body)
+__device__ __forceinline__ void vel_loop2_sm(int Nv, int lane, const Row &row, Acc<float> (&acc)[NA], FF *sacc, Body body)
 {
     FF *s = sacc + threadIdx.x;
     const int nt = blockDim.x;
 #pragma unroll
     for (int q = 0; q < NA; ++q) s[q * nt] = FF{0.f, 0.f};
-    vel_loop2<NA, float>(Nv, lane, body, [&](const float(&a)[NA]) {
+    vel_loop2<NA, float>(Nv, lane, row, body, [&](const float(&a)[NA]) {
 #pragma unroll
         for (int q = 0; q < NA; ++q) {
             Acc<float> x;
@@ -614,8 +642,10 @@ __device__ __forceinline__ void cell_moments_body(const KParams &__restrict__ p,
 {
     using T2 = typename V2<T>::t;
     const int lane = threadIdx.x & 31;
-    const int c = blk * 8 + (threadIdx.x >> 5);
-    if (c >= p.N) return;  // whole warp
+    int c;
+    const Row row = row_of(p, blk, c);
+    if (c >= p.N) return;  // all warps of a row
+    __shared__ Acc<T> sums[kRowSums];
     const T2 *f = (const T2 *)p.f + (size_t)c * p.Nv;
     Acc<T> acc[kRaw];
 #pragma unroll
@@ -631,11 +661,11 @@ __device__ __forceinline__ void cell_moments_body(const KParams &__restrict__ p,
     };
     if constexpr (sizeof(T) == 4) {
         __shared__ FF sacc[kRaw * 256];
-        vel_loop2_sm<kRaw>(p.Nv, lane, acc, sacc, body);
+        vel_loop2_sm<kRaw>(p.Nv, lane, row, acc, sacc, body);
     } else {
-        vel_loop2<kRaw, T>(p.Nv, lane, acc, body);
+        vel_loop2<kRaw, T>(p.Nv, lane, row, acc, body);
     }
-    warp_sum_store<kRaw, T>(acc, lane, p.cellraw, (size_t)c * kRaw);
+    row_sum_store<kRaw, T>(acc, lane, row, sums, p.cellraw, (size_t)c * kRaw);
 }
 
 template <class T, class LT>
@@ -966,9 +996,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_moments(co
 {
     IDG_LOCATE();
     using T2 = typename V2<T>::t;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int f = blk * 8 + wid;
+    const int lane = threadIdx.x & 31;
+    const int f = blk * 8 + (threadIdx.x >> 5);
     if (f >= p.nf) return;  // whole warp
+    constexpr Row row{0, 1};
     const T *geo = (const T *)p.fgeoT + 8 * f;
     const T nx = geo[0], ny = geo[1];
     const int kind = p.fbc[f];  // -1 interior, 1 wall, 2 far field
@@ -1034,11 +1065,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_moments(co
     };
     if constexpr (sizeof(T) == 4) {
         __shared__ FF sacc[kRaw * 256];
-        vel_loop2_sm<kRaw>(p.Nv, lane, acc, sacc, body);
+        vel_loop2_sm<kRaw>(p.Nv, lane, row, acc, sacc, body);
     } else {
-        vel_loop2<kRaw, T>(p.Nv, lane, acc, body);
+        vel_loop2<kRaw, T>(p.Nv, lane, row, acc, body);
     }
-    warp_sum_store<kRaw, T>(acc, lane, p.faceraw, (size_t)f * 12);
+    row_sum_store<kRaw, T>(acc, lane, row, nullptr, p.faceraw, (size_t)f * 12);
     if (lane == 0) {
         outsum[0].store(p.faceraw, (size_t)f * 12 + 11);
         p.facerw[f] = rw;
@@ -1085,9 +1116,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_flux(const
 {
     IDG_LOCATE();
     using T2 = typename V2<T>::t;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int f = blk * 8 + wid;
+    const int lane = threadIdx.x & 31;
+    const int f = blk * 8 + (threadIdx.x >> 5);
     if (f >= p.nf) return;  // whole warp
+    constexpr Row row{0, 1};
     const T *g = (const T *)p.fgeoT + 8 * f;
     const T nx = g[0], ny = g[1], S = g[2];
     const T *fA = (const T *)p.faceA + kCellP * f;
@@ -1097,7 +1129,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_flux(const
     Acc<T> acc[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[q].zero();
-    vel_loop2<4, T>(p.Nv, lane, acc, [&](int k, T(&a)[4]) {
+    vel_loop2<4, T>(p.Nv, lane, row, acc, [&](int k, T(&a)[4]) {
         T ux[2], uy[2], w[2], gr[2], fg[2], fh[2];
         vtab2<T>(p.uxf, p.ux, k, ux);
         vtab2<T>(p.uyf, p.uy, k, uy);
@@ -1120,7 +1152,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_face_flux(const
         }
         store_pair<T>(Fo, k, fg, fh);
     });
-    warp_sum_store<4, T>(acc, lane, p.phiraw, (size_t)f * 4);
+    row_sum_store<4, T>(acc, lane, row, nullptr, p.phiraw, (size_t)f * 4);
     if (p.implicit_wall && p.fbc[f] == 1) {
         // linearised wall (Eq. 33-35): the ghost increment drho_g M_w of the
         // incoming velocities enters the micro sweeps as the upwind term
@@ -2017,8 +2049,8 @@ __global__ void __launch_bounds__(32) k_explicit_w(const __grid_constant__ LT L)
 //   k_micro_residual  per (cell, velocity), fully parallel:
 //                     R = -sum_faces F - (2 Omega/(2 tau' + dt)) (f~ - f^S(W^{n+1})),
 //                     written into the increment buffer
-//   k_sweep_fwd       Delta*_c = (R_c + sum_{lower inflow nb} |xi.n| S Delta*_nb) / D_c
-//   k_sweep_bwd       Delta_c = Delta*_c + sum_{upper inflow nb} |xi.n| S Delta_nb / D_c,
+//   forward sweep     Delta*_c = (R_c + sum_{lower inflow nb} |xi.n| S Delta*_nb) / D_c
+//   backward sweep    Delta_c = Delta*_c + sum_{upper inflow nb} |xi.n| S Delta_nb / D_c,
 //                     f~ += Delta (Eq. 32)
 // with D = Omega/dt_imp + sum_{outflow} xi.n S + 2 Omega/(2 tau' + dt).
 // A structured block's sweeps run lines of cells (k_sweep_lines), an
@@ -2719,7 +2751,7 @@ void sweep_shape(KParams &p, bool fp64, int vpt)
 void blocks_per_instance(const KParams &p, int out[KT_COUNT])
 {
     const int nvb = nblk(p.Nv, 256);
-    out[KT_CELL_MOM] = nblk(p.N, 8);
+    out[KT_CELL_MOM] = nblk(p.N, 8 / p.row_warps);
     out[KT_CELL_PAR] = nblk(p.N, 32);
     out[KT_FBP] = nblk(p.N, p.cpb) * nvb;
     out[KT_FACE_MOM] = nblk(p.nf, 8);
@@ -3010,10 +3042,10 @@ int launch_cell_moments(const KParams &p, bool fp64, double *out6_dev, void *str
 {
     cudaStream_t st = (cudaStream_t)stream;
     if (fp64) {
-        k_cell_moments_v<double><<<nblk(p.N, 8), 256, 0, st>>>(p);
+        k_cell_moments_v<double><<<nblk(p.N, 8 / p.row_warps), 256, 0, st>>>(p);
         k_moments_out<double><<<nblk(p.N, 256), 256, 0, st>>>(p, out6_dev);
     } else {
-        k_cell_moments_v<float><<<nblk(p.N, 8), 256, 0, st>>>(p);
+        k_cell_moments_v<float><<<nblk(p.N, 8 / p.row_warps), 256, 0, st>>>(p);
         k_moments_out<float><<<nblk(p.N, 256), 256, 0, st>>>(p, out6_dev);
     }
     return (int)cudaGetLastError();
@@ -3065,10 +3097,10 @@ int launch_cell_moments_noalloc(const KParams &p0, bool fp64, int device, double
     p.cellraw = scratch;
     cudaStream_t st = (cudaStream_t)stream;
     if (fp64) {
-        k_cell_moments_v<double><<<nblk(p.N, 8), 256, 0, st>>>(p);
+        k_cell_moments_v<double><<<nblk(p.N, 8 / p.row_warps), 256, 0, st>>>(p);
         k_moments_out<double><<<nblk(p.N, 256), 256, 0, st>>>(p, out6_dev);
     } else {
-        k_cell_moments_v<float><<<nblk(p.N, 8), 256, 0, st>>>(p);
+        k_cell_moments_v<float><<<nblk(p.N, 8 / p.row_warps), 256, 0, st>>>(p);
         k_moments_out<float><<<nblk(p.N, 256), 256, 0, st>>>(p, out6_dev);
     }
     return (int)cudaGetLastError();

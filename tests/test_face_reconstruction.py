@@ -42,6 +42,9 @@ def _cases():
          "triangles_limited": dataclasses.replace(I.tri_cavity(4, Kn=0.1, nv=9, cfl_imp=10.0), limiter=1),
          # four cells a block from 4864 blocks of 256 velocities on, two from 2432
          "cells_4_per_block_ragged": I.cavity(71, Kn=0.1, nv=16, cfl_imp=50.0),
+         # a row of velocities shared by two and by four warps (2116, 4225 velocities)
+         "rows_2_warps": dataclasses.replace(I.cavity(4, Kn=0.1, nv=46, cfl_imp=50.0), implicit_wall=1),
+         "rows_4_warps": dataclasses.replace(I.cavity(4, Kn=0.1, nv=65, cfl_imp=50.0), implicit_wall=1),
          "cells_2_per_block_ragged": I.cavity(51, Kn=0.1, nv=16, cfl_imp=50.0)}
     p = c["axis_ties"]
     c["unequal_rows_and_columns"] = dataclasses.replace(p, nvx=11, nvy=7)
