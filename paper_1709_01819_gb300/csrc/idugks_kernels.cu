@@ -2178,24 +2178,16 @@ struct SweepArgs {
     int nsteps;               // steps of the sweep
 };
 
-// the cell of slot `slot` at the d-th step of the schedule, -1 past the step's end
-__device__ __forceinline__ int sweep_cell(const SweepArgs &p, int d, int slot)
-{
-    const int b = p.sptr[d];
-    return slot < p.sptr[d + 1] - b ? p.sched[b + slot] : -1;
-}
-
 // asynchronous copy of one step's data for the thread's cell: its VPT
 // consecutive velocities of R (or Delta*, f~), and the cell's slot geometry
 // and diagonal base spread over the cell's tv threads
 template <class T, int kStages, int VPT>
-__device__ __forceinline__ void sweep_issue(const SweepArgs &p, const SweepSmem<T, kStages, VPT> &sm, int s,
+__device__ __forceinline__ void sweep_issue(const SweepArgs &p, const SweepSmem<T, kStages, VPT> &sm, int s, int c,
                                             int slot, int t, int k0, bool act, bool withF)
 {
     using T2 = typename V2<T>::t;
     const int tv = p.tv, pc = p.pc;
-    if (s < p.nsteps) {
-        const int c = sweep_cell(p, s, slot);
+    {
         if (c >= 0) {
             int st = s & (kStages - 1);
             size_t e = ((size_t)st * pc + slot);
@@ -2225,10 +2217,55 @@ __device__ __forceinline__ void sweep_issue(const SweepArgs &p, const SweepSmem<
     cp_commit();
 }
 
-// unstructured meshes: the sweeps walk the steps of the level schedule
+// A step's coefficients at one cell, of its VPT velocities: |xi.n| S of the
+// inflow slots from already-swept cells (bits of `in`; zero elsewhere), their
+// cells, 1/D.
+template <class T, int VPT> struct SweepCoef {
+    T w[VPT][4], iD[VPT];
+    int nb[4];
+    unsigned in;  // a bit: in float64 a comparison costs the pipe as much as a sum
+    __device__ __forceinline__ void load(const T *geo, const int *codes, T D0, const T (&ux)[VPT], const T (&uy)[VPT])
+    {
+        T g[8];
+        load8<T>(g, geo);
+        const int4 cd = *(const int4 *)codes;
+        const int code[4] = {cd.x, cd.y, cd.z, cd.w};
+#pragma unroll
+        for (int m = 0; m < 4; ++m) nb[m] = kSeam - code[m];
+        in = 0;
+#pragma unroll
+        for (int v = 0; v < VPT; ++v) {
+            // outflow adds (xi.n) S to D
+            T D = D0;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const T aS = add_rn(mul_rn(ux[v], g[2 * m]), mul_rn(uy[v], g[2 * m + 1]));
+                D += aS > (T)0 ? aS : (T)0;
+                const bool i = aS < (T)0 && nb[m] >= 0;
+                w[v][m] = i ? -aS : (T)0;
+                in |= i ? 1u << (4 * v + m) : 0u;
+            }
+            iD[v] = rcp_rn(D);
+        }
+    }
+};
+
+// Unstructured meshes: the sweeps walk the steps of the level schedule, a block
+// barrier between them.  Bound by the latency of a step, whose chain is the
+// barrier, the neighbours' increments from L2 and the update: the cells are
+// read from the schedule a step before their copies are issued, and a step's
+// coefficients are formed in the step before it, while that one's increments
+// are on their way (float32 with one velocity per thread: more would take the
+// registers of a second block, and float64 is bound by its arithmetic pipe).
+// Forward + backward, float32, 64 x 64 squares of two triangles with 1024
+// velocities: 178 + 159 us with the cells read and the coefficients formed
+// behind the step's own barrier, 104 + 95 us this way; float64 488 + 488 and
+// 500 + 500 us (48 x 48 with 576).
 template <class T, bool FWD, int kStages, int VPT>
 __global__ void __launch_bounds__(512) k_sweep(Launch L)
 {
+    static_assert(kStages >= 3, "the next step's records are read a step ahead");
+    constexpr bool kAhead = VPT == 1 && sizeof(T) == 4;
     IDG_LOCATE();
     using T2 = typename V2<T>::t;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -2250,64 +2287,83 @@ __global__ void __launch_bounds__(512) k_sweep(Launch L)
     T2 *ds = (T2 *)a.dst;
     T2 *f = (T2 *)a.f;
     const int nh = a.nsteps;
-    const size_t w = (size_t)tv * VPT;
-    for (int s = 0; s < kStages - 1; ++s) sweep_issue<T, kStages, VPT>(a, sm, s, slot, t, k0, act, !FWD);
-    for (int s = 0; s < nh; ++s) {
-        cp_wait<kStages - 2>();
-        __syncthreads();
-        sweep_issue<T, kStages, VPT>(a, sm, s + kStages - 1, slot, t, k0, act, !FWD);
-        const int c = sweep_cell(a, s, slot);
-        if (c < 0 || !act) continue;
+    // cells of the steps s .. s + kStages - 1 (-1: none), the bounds of the next one
+    int cell[kStages];
+    int b0 = a.sptr[0], b1 = a.sptr[min(1, nh)];
+#pragma unroll
+    for (int q = 0; q < kStages; ++q) {
+        cell[q] = slot < b1 - b0 ? a.sched[b0 + slot] : -1;
+        b0 = b1;
+        b1 = a.sptr[min(q + 2, nh)];
+    }
+#pragma unroll
+    for (int q = 0; q < kStages - 1; ++q) sweep_issue<T, kStages, VPT>(a, sm, q, cell[q], slot, t, k0, act, !FWD);
+    SweepCoef<T, VPT> cf;
+    cp_wait<kStages - 2>();
+    __syncthreads();
+    auto coef = [&](int s, int c) {
         const size_t e = (size_t)(s & (kStages - 1)) * pc + slot;
-        T g[8];
-        load8<T>(g, sm.geo + e * 8);
-        const int4 cd = *(const int4 *)(sm.code + e * 4);
-        const int code[4] = {cd.x, cd.y, cd.z, cd.w};
-        const T D0 = sm.D0[e];
-        const size_t ck = (size_t)c * Nv + k0;
-        const size_t rbase = e * w + (size_t)t * VPT;
-#pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            // slot terms, branch-free: outflow adds (xi.n) S to D, inflow
-            // from the already-swept side adds |xi.n| S Delta_nb
-            T D = D0;
-            T aS[4];
-            bool in[4];
+        if (c >= 0) cf.load(sm.geo + e * 8, sm.code + e * 4, sm.D0[e], ux, uy);
+    };
+    if (kAhead) coef(0, cell[0]);
+    for (int s = 0; s < nh; ++s) {
+        cp_wait<kStages - (kAhead ? 3 : 2)>();
+        __syncthreads();
+        const bool on = cell[0] >= 0 && act;
+        if (!kAhead) coef(s, cell[0]);
+        T w[4], dg[4], dh[4];
+        auto neighbours = [&](int v) {
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
-                aS[m] = add_rn(mul_rn(ux[v], g[2 * m]), mul_rn(uy[v], g[2 * m + 1]));
-                D += aS[m] > (T)0 ? aS[m] : (T)0;
-                in[m] = aS[m] < (T)0 && code[m] <= kSeam;
+                w[m] = cf.w[v][m];
+                dg[m] = dh[m] = (T)0;
+                if (on && (cf.in >> (4 * v + m) & 1)) {
+                    const T2 x = ds[(size_t)cf.nb[m] * Nv + k0 + v];
+                    dg[m] = x.x;
+                    dh[m] = x.y;
+                }
             }
-            T2 dn[4];
+        };
+        neighbours(0);
+        const int cnext = slot < b1 - b0 ? a.sched[b0 + slot] : -1;
+        b0 = b1;
+        b1 = a.sptr[min(s + kStages + 2, nh)];
+        sweep_issue<T, kStages, VPT>(a, sm, s + kStages - 1, cell[kStages - 1], slot, t, k0, act, !FWD);
+        T iD[VPT];
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                dn[m].x = (T)0;
-                dn[m].y = (T)0;
-                if (in[m]) dn[m] = ds[(size_t)(kSeam - code[m]) * Nv + k0 + v];
-            }
-            T ag = 0, ah = 0;
+        for (int v = 0; v < VPT; ++v) iD[v] = cf.iD[v];
+        if (kAhead) coef(s + 1, cell[1]);
+        if (on) {
+            const size_t ck = (size_t)cell[0] * Nv + k0;
+            const size_t rbase = ((size_t)(s & (kStages - 1)) * pc + slot) * tv * VPT + (size_t)t * VPT;
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                ag = mad(-aS[m], dn[m].x, ag);
-                ah = mad(-aS[m], dn[m].y, ah);
+            for (int v = 0; v < VPT; ++v) {
+                if (v > 0) neighbours(v);
+                T ag = 0, ah = 0;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    ag = mad(w[m], dg[m], ag);
+                    ah = mad(w[m], dh[m], ah);
+                }
+                const T2 r = sm.R[rbase + v];
+                T2 o;
+                if (FWD) {
+                    o.x = (r.x + ag) * iD[v];
+                    o.y = (r.y + ah) * iD[v];
+                } else {
+                    o.x = mad(ag, iD[v], r.x);
+                    o.y = mad(ah, iD[v], r.y);
+                    T2 fv = sm.F[rbase + v];
+                    fv.x += o.x;
+                    fv.y += o.y;
+                    f[ck + v] = fv;
+                }
+                ds[ck + v] = o;
             }
-            const T2 r = sm.R[rbase + v];
-            const T iD = rcp_rn(D);
-            T2 o;
-            if (FWD) {
-                o.x = (r.x + ag) * iD;
-                o.y = (r.y + ah) * iD;
-            } else {
-                o.x = mad(ag, iD, r.x);
-                o.y = mad(ah, iD, r.y);
-                T2 fv = sm.F[rbase + v];
-                fv.x += o.x;
-                fv.y += o.y;
-                f[ck + v] = fv;
-            }
-            ds[ck + v] = o;
         }
+#pragma unroll
+        for (int q = 0; q + 1 < kStages; ++q) cell[q] = cell[q + 1];
+        cell[kStages - 1] = cnext;
     }
     cp_wait<0>();
 }
