@@ -42,8 +42,8 @@ from paper_1709_01819_gb300 import inputs as I  # noqa: E402
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 KERNELS = ["cell_prep", "face_moments", "face_flux", "macro", "k_sweep_fwd", "k_sweep_bwd"]
 # launch groups timed by idg_iterate_profiled: cell_prep = k_cell_moments + k_cell_params + k_fbp;
-# face_moments = k_face_moments + k_face_params; face_flux = k_face_flux + k_face_phi;
-# macro = k_macro_pre + k_macro_sweep + k_macro_post
+# face_moments = k_cell_recon + k_face_moments + k_face_params; face_flux = k_face_flux + k_face_phi;
+# macro = k_macro_pre + the macroscopic sweep + k_macro_post
 
 
 # point-relaxation sweeps per workload for the time-to-residual report (the
