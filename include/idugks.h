@@ -53,7 +53,8 @@ typedef enum {
     IDG_ERR_NONFINITE = 5,     /* the residual became NaN or Inf (sticky until the     */
                                /* next idg_init_uniform or idg_set_state)              */
     IDG_ERR_TIMEOUT = 6,       /* a bounded wait between the warps of one thread block */
-                               /* ran out (no kernel waits on another block)           */
+                               /* ran out (no kernel waits on another block);          */
+                               /* idg_set_wait_limit                                   */
     IDG_ERR_NOT_CONVERGED = 7  /* idg_iterate reached max_iter above tol               */
 } idg_status;
 
@@ -342,6 +343,16 @@ enum { IDG_TUNE_SWEEP_TV = 1, IDG_TUNE_SWEEP_STAGES = 2, IDG_TUNE_MACRO_STAGES =
        IDG_TUNE_SWEEP_VPT = 5, IDG_TUNE_MACRO_KIND = 6 };
 idg_status idg_set_tuning(idg_ctx *ctx, int key, int value);
 idg_status idg_get_tuning(const idg_ctx *ctx, int key, int *value);
+
+/* The polls after the first (default 2^22, seconds) before a wait between the
+ * warps of a sweep kernel's block gives up (after idg_bind_workspace; >= 0).
+ * No such wait runs out unless a warp of the block is lost; one that does
+ * lets its kernel finish on stale values and makes the call that launched it
+ * -- idg_iterate, idg_iterate_profiled, idg_batch_iterate, idg_adjoint --
+ * return IDG_ERR_TIMEOUT.  The iteration's word is sticky like that of
+ * IDG_ERR_NONFINITE; the adjoint has its own, cleared by each call.  A limit
+ * of 0 makes them run out: a way to see one reported. */
+idg_status idg_set_wait_limit(idg_ctx *ctx, int polls);
 
 /* Sizes and host-side tables (valid after the corresponding setters). */
 idg_status idg_get_sizes(const idg_ctx *ctx, int *ncell, int *nvel, int *nface);

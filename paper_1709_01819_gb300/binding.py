@@ -60,6 +60,7 @@ SIGNATURES = [
     ("idg_iterate_profiled", _i, [_vp, _vp, _P(_d)]),
     ("idg_set_tuning", _i, [_vp, _i, _i]),
     ("idg_get_tuning", _i, [_vp, _i, _P(_i)]),
+    ("idg_set_wait_limit", _i, [_vp, _i]),
     ("idg_get_moments", _i, [_vp, _P(_d), _vp]),
     ("idg_get_moments_noalloc", _i, [_vp, _vp, _vp]),
     ("idg_get_residual_history", _i, [_vp, _P(_d), _i, _P(_i)]),
@@ -229,6 +230,10 @@ def idg_iterate_profiled(ctx, stream=None):
 
 def idg_set_tuning(ctx, key, value):
     return check(ctx, lib().idg_set_tuning(ctx, key, value))
+
+
+def idg_set_wait_limit(ctx, polls):
+    return check(ctx, lib().idg_set_wait_limit(ctx, polls))
 
 
 def idg_get_tuning(ctx, key):

@@ -489,8 +489,8 @@ template <bool ASC> __global__ void __launch_bounds__(512) k_adj_lines(AParams a
     int seen_r = 0, seen_w = 0;
     for (int s0 = s_beg; s0 < s_end; s0 += kSweepBlock) {
         if (strips > 1) {
-            if (strip > 0) flag_wait(flags + strip - 1, s0, seen_r, a.status);
-            if (strip + 1 < strips) flag_wait(flags + strip + 1, s0 + 2 * kSweepBlock + 1 - kAdjRing, seen_w, a.status);
+            if (strip > 0) flag_wait(flags + strip - 1, s0, seen_r, a.status, a.wait_polls);
+            if (strip + 1 < strips) flag_wait(flags + strip + 1, s0 + 2 * kSweepBlock + 1 - kAdjRing, seen_w, a.status, a.wait_polls);
         }
 #pragma unroll
         for (int b = 0; b < kSweepBlock; ++b) {
@@ -963,6 +963,7 @@ size_t adjoint_layout(const AParams &s, int nrhs, char *base, AParams *out)
     a.Ef = (double *)take(nf * Nv * d);
     a.iDm = (double *)take(NNv * d);
     a.cm = (double *)take(4 * NNv * d);
+    a.status = (int *)take(256);
     for (int r = 0; r < nrhs; ++r) {
         a.seed = r;
         a.lamG = (double *)take(NNv * d);

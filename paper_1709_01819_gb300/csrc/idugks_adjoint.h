@@ -72,7 +72,8 @@ struct AParams {
     double *cpp;                 // [N][2]  Kn partials of the cell (collision, cell prep)
     double *rpart;               // [N] squared increment of lambda_f per cell
     double *res;                 // [kMaxHist] ||increment of lambda_f|| per adjoint iteration
-    int *status;                 // status word of the context (a bounded wait that ran out)
+    int *status;                 // the adjoint's own status word: a bounded wait of its sweeps that ran out
+    int wait_polls;              // KParams::wait_polls
     double *dlamW;               // [N][4] increment of lambda_W of the last iteration
 };
 

@@ -98,6 +98,13 @@ idg_status fail(idg_ctx *c, idg_status s, const char *fmt, ...)
     return s;
 }
 
+// a device status word that is not zero
+idg_status status_fail(idg_ctx *c, int word, const char *what)
+{
+    if (word == IDG_ERR_TIMEOUT) return fail(c, IDG_ERR_TIMEOUT, "a wait inside a sweep kernel ran out");
+    return fail(c, IDG_ERR_NONFINITE, "%s became non-finite", what);
+}
+
 idg_status cuda_fail(idg_ctx *c, cudaError_t e, const char *where)
 {
     return fail(c, IDG_ERR_CUDA, "%s: %s", where, cudaGetErrorString(e));
@@ -777,6 +784,7 @@ idg_status check_ready(idg_ctx *c)
 }
 
 constexpr int kGraphChunk = 16;
+constexpr int kWaitPolls = 1 << 22;  // default of idg_set_wait_limit: seconds
 
 void drop_graph(idg_ctx *c)
 {
@@ -1120,6 +1128,7 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
     k.pc0 = (1.0 - c->Pr) / (c->K + 4);
     k.relax_sweeps = c->relax_sweeps;
     k.implicit_wall = c->implicit_wall;
+    k.wait_polls = kWaitPolls;
     if (c->unstr) {
         k.per_i = k.per_j = 0;
         k.nsteps_f = c->nsteps_f;
@@ -1523,8 +1532,7 @@ idg_status idg_iterate(idg_ctx *c, int max_iter, double tol, void *stream, int *
         for (int q = 0; q < n; ++q) c->hist.push_back(buf[q]);
         if (status) {
             if (iters_done) *iters_done = done;
-            if (status == IDG_ERR_TIMEOUT) return fail(c, IDG_ERR_TIMEOUT, "a wait inside a sweep kernel ran out");
-            return fail(c, IDG_ERR_NONFINITE, "residual became non-finite");
+            return status_fail(c, status, "residual");
         }
         double r1 = c->hist.front();
         rel = r1 > 0 ? c->hist.back() / r1 : c->hist.back();
@@ -1554,6 +1562,7 @@ idg_status idg_iterate_profiled(idg_ctx *c, void *stream, double *kernel_ms)
     if (!rc) rc = idg::launch_iteration(c->plan, c->precision == IDG_FP64, st, (void **)ev);
     cudaError_t e = rc ? (cudaError_t)rc : cudaStreamSynchronize(st);
     double r = 0.0;
+    int status = 0;
     if (e == cudaSuccess) {
         for (int q = 0; q < 6; ++q) {
             float ms = 0.f;
@@ -1562,11 +1571,14 @@ idg_status idg_iterate_profiled(idg_ctx *c, void *stream, double *kernel_ms)
         }
         long long slot = c->host_iter & (idg::kMaxHist - 1);
         e = cudaMemcpy(&r, c->kp.res + slot, 8, cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess) e = cudaMemcpy(&status, c->kp.status, sizeof(int), cudaMemcpyDeviceToHost);
     }
     for (int q = 0; q < 7; ++q) cudaEventDestroy(ev[q]);
     if (e != cudaSuccess) return cuda_fail(c, e, "profiled iteration");
     c->host_iter += 1;
     c->hist.push_back(r);
+    // (a residual that is not finite stands in the history and is idg_iterate's to report)
+    if (status == IDG_ERR_TIMEOUT) return status_fail(c, status, "residual");
     return IDG_OK;
 }
 
@@ -1632,6 +1644,17 @@ idg_status idg_get_tuning(const idg_ctx *c, int key, int *value)
     else if (key == IDG_TUNE_MACRO_KIND) *value = c->kp.macro_kind;
     else return IDG_ERR_ARG;
     return IDG_OK;
+}
+
+idg_status idg_set_wait_limit(idg_ctx *c, int polls)
+{
+    idg_status s = check_ready(c);
+    if (s) return s;
+    if (polls < 0) return fail(c, IDG_ERR_ARG, "wait limit %d is negative", polls);
+    const int old = c->kp.wait_polls;
+    c->kp.wait_polls = polls;
+    if ((s = refresh_plan(c))) c->kp.wait_polls = old;
+    return s;
 }
 
 idg_status idg_get_moments(idg_ctx *c, double *out6, void *stream)
@@ -2012,8 +2035,8 @@ idg_status idg_batch_iterate(idg_batch *b, int max_iter, double tol, void *strea
             for (int q = 0; q < m; ++q) c->hist.push_back(res[(size_t)i * kGraphChunk + q]);
             c->host_iter += m;
             if (status[i]) {
-                ret = IDG_ERR_NONFINITE;
-                fail(c, IDG_ERR_NONFINITE, "residual became non-finite");
+                const idg_status x = status_fail(c, status[i], "residual");
+                if (ret != IDG_ERR_TIMEOUT) ret = x;
                 b->active[i] = 0;
                 changed = true;
                 continue;
@@ -2043,7 +2066,7 @@ idg_status idg_batch_iterate(idg_batch *b, int max_iter, double tol, void *strea
     }
     if (iters_done) *iters_done = done;
     if (max_residual) *max_residual = worst;
-    if (ret) return bfail(b, ret, "an instance became non-finite");
+    if (ret) return bfail(b, ret, ret == IDG_ERR_TIMEOUT ? "a wait inside a sweep kernel ran out" : "an instance became non-finite");
     if (tol > 0 && !all) return bfail(b, IDG_ERR_NOT_CONVERGED, "largest residual %.3e above tol %.3e", worst, tol);
     return IDG_OK;
 }
@@ -2170,7 +2193,7 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
     base.kappa = base.shakhov ? (1.0 - c->Pr) / (c->K + 4) : 0.0;
     base.area = k.area; base.dtimp = k.dtimp; base.fgeo = k.fgeo; base.ux = k.ux; base.uy = k.uy; base.w = k.w;
     base.cface = k.cface; base.cnb = k.cnb; base.csign = k.csign; base.fL = k.fL; base.fR = k.fR;
-    base.fbc = k.fbc; base.fside = k.fside; base.W = k.W; base.status = k.status;
+    base.fbc = k.fbc; base.fside = k.fside; base.W = k.W; base.wait_polls = k.wait_polls;
     for (int sd = 0; sd < 4; ++sd) {
         base.b_kind[sd] = c->bc_kind[sd];
         base.b_rho[sd] = c->bc_kind[sd] == IDG_BC_WALL ? 1.0 : c->bc_rho[sd];
@@ -2186,8 +2209,15 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
     if ((e = cudaMemcpyAsync(A[0].lsw, c->clsg.data(), c->clsg.size() * 8, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(A[0].crv, c->cr.data(), c->cr.size() * 8, cudaMemcpyHostToDevice, st)) != cudaSuccess)
+        (e = cudaMemcpyAsync(A[0].crv, c->cr.data(), c->cr.size() * 8, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
+        (e = cudaMemsetAsync(A[0].status, 0, sizeof(int), st)) != cudaSuccess)
         return cuda_fail(c, e, "adjoint geometry upload");
+    int status = 0;
+    auto read_status = [&]() { return cudaMemcpyAsync(&status, A[0].status, sizeof(int), cudaMemcpyDeviceToHost, st); };
+    auto timed_out = [&](int done) {
+        if (iters_done) *iters_done = done;
+        return status_fail(c, status, "adjoint");
+    };
     int rc = idg::launch_from_dev(c->kp, c->precision == IDG_FP64, A[0].G, A[0].H, c->Nv, st);
     if (!rc) rc = idg::launch_adjoint_setup(A[0], st);
     for (int r = 0; r < nrhs && !rc; ++r) rc = idg::launch_adjoint_zero(A[r], st);
@@ -2244,6 +2274,7 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
         auto dot = [&](const double *x, const double *y) {
             if (!err) err = idg::launch_vec_dot(x, y, n, dpart, st);
             if (!err) err = (int)cudaMemcpyAsync(part.data(), dpart, nblk * 8, cudaMemcpyDeviceToHost, st);
+            if (!err) err = (int)read_status();
             if (!err) err = (int)cudaStreamSynchronize(st);
             double t = 0.0;
             for (int q = 0; q < nblk; ++q) t += part[q];
@@ -2262,7 +2293,7 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
             axpby(-1.0, xv, 1.0, wv);
             const double r0 = std::sqrt(dot(wv, wv));
             rel = bnorm > 0 ? r0 / bnorm : 0.0;
-            if (!std::isfinite(rel)) break;
+            if (status || !std::isfinite(rel)) break;
             if ((tol > 0 && rel <= tol) || r0 == 0.0) break;
             axpby(1.0 / r0, wv, 0.0, V);
             std::fill(g.begin(), g.end(), 0.0);
@@ -2296,7 +2327,7 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
                 g[j] = cs[j] * g[j];
                 k = j + 1;
                 rel = bnorm > 0 ? std::fabs(g[j + 1]) / bnorm : 0.0;
-                if (!std::isfinite(rel) || (tol > 0 && rel <= tol) || hn == 0.0) break;
+                if (status || !std::isfinite(rel) || (tol > 0 && rel <= tol) || hn == 0.0) break;
             }
             for (int i = k - 1; i >= 0; --i) {  // H y = g, upper triangular
                 double t = g[i];
@@ -2306,6 +2337,7 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
             for (int i = 0; i < k; ++i) axpby(y[i], V + (size_t)i * n, 1.0, xv);
         }
         if (err) return cuda_fail(c, (cudaError_t)err, "adjoint GMRES");
+        if (status) return timed_out(done);
         if (!std::isfinite(rel)) {
             if (iters_done) *iters_done = done;
             return fail(c, IDG_ERR_NONFINITE, "adjoint GMRES residual became non-finite");
@@ -2333,8 +2365,10 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
                 (e = cudaMemcpyAsync(dW[r].data(), A[r].dlamW, N4 * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
                 return cuda_fail(c, e, "adjoint residual");
         }
-        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(c, e, "adjoint iteration");
+        if ((e = read_status()) != cudaSuccess || (e = cudaStreamSynchronize(st)) != cudaSuccess)
+            return cuda_fail(c, e, "adjoint iteration");
         done += n;
+        if (status) return timed_out(done);
         double fnorm = buf[0][n - 1], w2 = 0.0, ww = 0.0, wm = 0.0;
         bool finite = std::isfinite(fnorm);
         if (nrhs == 2) {
@@ -2371,7 +2405,9 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
             (e = cudaMemcpyAsync(cpp[r].data(), A[r].cpp, cpp[r].size() * 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
             return cuda_fail(c, e, "adjoint results");
     }
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(c, e, "adjoint results");
+    if ((e = read_status()) != cudaSuccess || (e = cudaStreamSynchronize(st)) != cudaSuccess)
+        return cuda_fail(c, e, "adjoint results");
+    if (status) return timed_out(done);
     double Jv = 0.0, knsum = 0.0, side_par[4][3] = {};
     for (int f = 0; f < c->nf; ++f) {
         const double *fp = &fpar[(size_t)idg::kFP * f];

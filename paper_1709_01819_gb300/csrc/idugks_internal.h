@@ -95,6 +95,7 @@ struct KParams {
     // velocities per thread, sweep_g of those threads neighbours in one warp,
     // entries of a border ring
     int sweep_ktv, sweep_kvpt, sweep_g, sweep_ring;
+    int wait_polls;  // polls after the first before a wait between warps gives up (idg_set_wait_limit)
     int sweep_vpt;  // consecutive velocities per thread in the micro sweeps (1, 2, 4)
     int macro_kind; // macroscopic LU-SGS on a structured block: 0 hyperplane slots (k_macro_sweep),
                     // 1 one thread per line of cells (k_macro_lines)

@@ -1390,7 +1390,8 @@ __device__ __forceinline__ void record_residual(const KParams &p)
     if (lane == 0) {
         const double r = sqrt(s);
         p.res[*p.iter & (kMaxHist - 1)] = r;
-        if (!isfinite(r)) *p.status = 5;
+        // (a wait that ran out stays the cause that is reported: the sweep then ran on stale values)
+        if (!isfinite(r)) atomicCAS(p.status, 0, 5);
     }
 }
 
@@ -1613,7 +1614,7 @@ template <class T> struct LineCtx {
     const T *rec;
     size_t M;  // slots
     T gm1;
-    int nt, nw, nthr, lane, wid, strips;
+    int nt, nw, nthr, lane, wid, strips, polls;
     bool per_t, per_w;
 };
 
@@ -1660,8 +1661,8 @@ template <class T, int kStages, bool FWD, bool SEAM> __device__ __forceinline__ 
     int seen_r = 0, seen_w = 0;
     for (int s0 = s_beg; s0 < s_end; s0 += kSweepBlock) {
         if (x.strips > 1) {
-            if (x.wid > 0) flag_wait(x.flags + x.wid - 1, s0, seen_r, x.status);
-            if (x.wid + 1 < x.strips) flag_wait(x.flags + x.wid + 1, s0 + 2 * kSweepBlock + 1 - kLRing, seen_w, x.status);
+            if (x.wid > 0) flag_wait(x.flags + x.wid - 1, s0, seen_r, x.status, x.polls);
+            if (x.wid + 1 < x.strips) flag_wait(x.flags + x.wid + 1, s0 + 2 * kSweepBlock + 1 - kLRing, seen_w, x.status, x.polls);
         }
 #pragma unroll
         for (int b = 0; b < kSweepBlock; ++b) {
@@ -1739,6 +1740,7 @@ __global__ void __launch_bounds__(288, 1) k_macro_lines(Launch L)
     x.stage = x.ring + (size_t)x.strips * kLRing * 4; // [kStages][6][nthr][4]
     x.seam = x.stage + (size_t)kStages * x.nthr * 24; // [nw][4] the first line's terms (per_t)
     x.status = p.status;
+    x.polls = p.wait_polls;
     x.dWg = (T *)p.mdW;
     x.rec = (const T *)p.mline;
     x.M = line_slots(p);
@@ -2599,8 +2601,8 @@ __global__ void __launch_bounds__(512) k_sweep_lines(Launch L)
         if (strips > 1) {
             // reads what the strip before wrote in steps < s0; overwrites what the
             // strip after reads in steps <= s0 + 2 kSweepBlock - ring
-            if (strip > 0) flag_wait(flags + wid - 1, s0, seen_r, p.status);
-            if (strip + 1 < strips) flag_wait(flags + wid + 1, s0 + 2 * kSweepBlock + 1 - ring, seen_w, p.status);
+            if (strip > 0) flag_wait(flags + wid - 1, s0, seen_r, p.status, p.wait_polls);
+            if (strip + 1 < strips) flag_wait(flags + wid + 1, s0 + 2 * kSweepBlock + 1 - ring, seen_w, p.status, p.wait_polls);
         }
 #pragma unroll
         for (int b = 0; b < kSweepBlock; ++b) {

@@ -45,13 +45,14 @@ __device__ __forceinline__ int flag_load(const int *f)
     return v;
 }
 // waits until *f >= need (seen: what the last poll found).  The warps of a block
-// run at the same time, so the wait ends; should it not (2^22 polls), the status
-// word is raised and the sweep goes on.
-__device__ __forceinline__ void flag_wait(const int *f, int need, int &seen, int *status)
+// run at the same time, so the wait ends; should it not within limit more polls
+// than the first, the status word takes IDG_ERR_TIMEOUT (over anything else it
+// holds) and the sweep goes on without waiting, on whatever the ring holds.
+__device__ __forceinline__ void flag_wait(const int *f, int need, int &seen, int *status, int limit)
 {
     for (int n = 0; seen < need; ++n) {
         seen = flag_load(f);
-        if (n > (1 << 22)) {
+        if (seen < need && n >= limit) {
             *status = 6;
             seen = 0x7fffffff;
         }
