@@ -314,17 +314,20 @@ idg_status idg_get_wall(idg_ctx *ctx, int side, double *out5, int cap, int *nfac
 idg_status idg_iterate_profiled(idg_ctx *ctx, void *stream, double *kernel_ms);
 
 /* Launch-shape tuning of the wavefront kernels (after idg_bind_workspace;
- * no effect on results).  IDG_TUNE_SWEEP_TV: threads per cell and block of the
- * micro LU-SGS sweeps (power of two, 1..32, times min(ni, nj) at most 512);
- * IDG_TUNE_SWEEP_VPT: consecutive velocities per thread (1, 2 or 4; all
- * instances of a batch must agree).  On a structured block the sweeps take a
- * shape by size until one of the two is set (the values read back before are
- * those of a first setting).  IDG_TUNE_SWEEP_STAGES / IDG_TUNE_MACRO_STAGES:
- * steps prefetched ahead by the micro / macroscopic sweeps (2, 4 or 8, the
- * micro sweeps at most what shared memory holds; the macroscopic sweep takes
- * 2 by default for a float64 block with min(ni, nj) above 213, its records
- * filling shared memory).  Returns IDG_ERR_ARG for a value that is invalid or
- * whose macroscopic records do not fit in shared memory.  Any velocity count
+ * no effect on results).  idg_get_tuning reads the shape that runs: what was
+ * set, and where nothing was the library's choice by size, so that setting what
+ * was read leaves the shape as it is.  IDG_TUNE_SWEEP_TV: threads per cell and
+ * block of the micro LU-SGS sweeps (power of two, 1..32, times min(ni, nj) at
+ * most 512); IDG_TUNE_SWEEP_VPT: consecutive velocities per thread (1, 2 or 4;
+ * all instances of a batch must agree, those of a batch in which none is set
+ * run two, one in float64).  IDG_TUNE_SWEEP_STAGES / IDG_TUNE_MACRO_STAGES:
+ * steps prefetched ahead by the micro / macroscopic sweeps (2, 4 or 8; 4 only
+ * by the micro sweeps of an unstructured mesh).  Where a request fits shared
+ * memory only without the padding of the lines to whole warps, the micro sweeps
+ * run the next shallower depth that fits (the macroscopic sweep takes 2 by
+ * default for a float64 block with min(ni, nj) above 213, its records filling
+ * shared memory).  Returns IDG_ERR_ARG for a value that is invalid or does not
+ * fit in shared memory.  Any velocity count
  * takes all of these: the library stores each cell's velocities rounded up to
  * a multiple of 4, the extra ones being ghost velocities of zero weight at
  * xi = 0 that enter no moment and no flux and never reach the caller.

@@ -1156,10 +1156,10 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
     k.sweep_tv = 8;
     while (k.sweep_tv > 1 && k.sweep_tv * k.sweep_pc > 512) k.sweep_tv /= 2;
     while (k.sweep_tv < 32 && 2 * k.sweep_tv * k.sweep_pc <= 256) k.sweep_tv *= 2;
-    // prefetch depth: 8 hyperplanes where shared memory allows (the plan
-    // falls back to 4)
+    // prefetch depth: 8 hyperplanes where shared memory allows (the plan falls
+    // back to 4, then 2); the scheduled sweeps' is 4
     k.macro_stages = 8;
-    k.sweep_stages = 8;
+    k.sweep_stages = c->unstr || !idg::sweep_request_fits(k, c->precision == IDG_FP64) ? 4 : 8;
     // float64: the hyperplane-slot kernel (two threads per cell halve each
     // step's float64 chain); float32 storage: one thread per line of cells
     k.macro_kind = c->precision == IDG_FP64 ? 0 : 1;
@@ -1596,14 +1596,15 @@ idg_status idg_set_tuning(idg_ctx *c, int key, int value)
         if (value < 1 || value > 32 || (value & (value - 1)) || value * k.sweep_pc > 512)
             return fail(c, IDG_ERR_ARG, "sweep velocities per block %d invalid for %d cell slots", value, k.sweep_pc);
         k.sweep_tv = value;
-        k.sweep_tuned = 1;
+        k.sweep_tuned |= 1;
     } else if (key == IDG_TUNE_SWEEP_VPT) {
         if ((value != 1 && value != 2 && value != 4) || k.Nv % value)
             return fail(c, IDG_ERR_ARG, "velocities per thread %d must be 1, 2 or 4 and divide %d", value, k.Nv);
         k.sweep_vpt = value;
-        k.sweep_tuned = 1;
+        k.sweep_tuned |= 2;
     } else if (key == IDG_TUNE_SWEEP_STAGES) {
         if (value != 2 && value != 4 && value != 8) return fail(c, IDG_ERR_ARG, "sweep stages must be 2, 4 or 8");
+        if (c->unstr && value != 4) return fail(c, IDG_ERR_ARG, "the scheduled sweeps of an unstructured mesh prefetch 4 steps");
         k.sweep_stages = value;
     } else if (key == IDG_TUNE_MACRO_STAGES) {
         if (value != 2 && value != 4 && value != 8) return fail(c, IDG_ERR_ARG, "macro stages must be 2, 4 or 8");
@@ -1621,7 +1622,9 @@ idg_status idg_set_tuning(idg_ctx *c, int key, int value)
     idg::blocks_per_instance(k, trial.nblocks);
     if (key == IDG_TUNE_MACRO_KIND && !idg::plan_shapes(&k, 1, c->precision == IDG_FP64, trial))
         k.macro_stages = trial.macro_stages;
-    if (idg::plan_shapes(&k, 1, c->precision == IDG_FP64, trial) || trial.macro_stages != k.macro_stages)
+    const bool sweeps = key == IDG_TUNE_SWEEP_TV || key == IDG_TUNE_SWEEP_VPT || key == IDG_TUNE_SWEEP_STAGES;
+    if ((sweeps && !idg::sweep_request_fits(k, c->precision == IDG_FP64)) ||
+        idg::plan_shapes(&k, 1, c->precision == IDG_FP64, trial) || trial.macro_stages != k.macro_stages)
         return fail(c, IDG_ERR_ARG, "launch shape does not fit in shared memory");
     KParams old = c->kp;
     c->kp = k;
@@ -1637,9 +1640,9 @@ idg_status idg_get_tuning(const idg_ctx *c, int key, int *value)
     if (!c || !value) return IDG_ERR_ARG;
     if (!c->bound) return IDG_ERR_STATE;
     if (key == IDG_TUNE_GRAPH) *value = c->use_graph;
-    else if (key == IDG_TUNE_SWEEP_TV) *value = c->kp.sweep_tv;
-    else if (key == IDG_TUNE_SWEEP_VPT) *value = c->kp.sweep_vpt;
-    else if (key == IDG_TUNE_SWEEP_STAGES) *value = c->kp.sweep_stages;
+    else if (key == IDG_TUNE_SWEEP_TV) *value = c->kp.sweep_ktv;
+    else if (key == IDG_TUNE_SWEEP_VPT) *value = c->kp.sweep_kvpt;
+    else if (key == IDG_TUNE_SWEEP_STAGES) *value = c->plan.sweep_stages;
     else if (key == IDG_TUNE_MACRO_STAGES) *value = c->plan.macro_stages;
     else if (key == IDG_TUNE_MACRO_KIND) *value = c->kp.macro_kind;
     else return IDG_ERR_ARG;
@@ -1842,12 +1845,12 @@ idg_status batch_refresh(idg_batch *b)
     const int n = (int)b->ctx.size();
     b->hparams.resize(n);
     for (int i = 0; i < n; ++i) b->hparams[i] = b->ctx[i]->kp;
-    // one number of velocities per thread for the whole batch: the tuned one,
-    // or, untuned, the one of an instance with many waves of warps
+    // one number of velocities per thread for the whole batch: the one the caller
+    // set (plan_shapes refuses different ones), otherwise two, in float64 one
     std::vector<KParams> hp = b->hparams;
     int vpt = b->precision == IDG_FP64 ? 1 : 2;
     for (int i = 0; i < n; ++i)
-        if (hp[i].sweep_tuned) vpt = hp[i].sweep_vpt;
+        if (hp[i].sweep_tuned & 2) vpt = hp[i].sweep_vpt;
     for (int i = 0; i < n; ++i) idg::sweep_shape(hp[i], b->precision == IDG_FP64, vpt);
     std::vector<int> off((size_t)idg::KT_COUNT * (n + 1), 0);
     idg::Plan pl{};

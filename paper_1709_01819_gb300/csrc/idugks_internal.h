@@ -90,10 +90,10 @@ struct KParams {
     int sweep_tv, sweep_pc, sweep_stages, macro_stages;
     int row_warps;   // warps per cell of k_cell_moments (1, 2, 4)
     int cpb;         // cells per block of the per-(cell, velocity) kernels
-    int sweep_tuned; // 1: sweep_tv or sweep_vpt was set by the caller
-    // line micro sweeps (sweep_shape()): threads per cell of a block and
-    // velocities per thread, sweep_g of those threads neighbours in one warp,
-    // entries of a border ring
+    int sweep_tuned; // set by the caller: 1 sweep_tv, 2 sweep_vpt
+    // the tile that runs (sweep_shape()): threads per cell of a block and
+    // velocities per thread; line sweeps: sweep_g of those threads neighbours in
+    // one warp, entries of a border ring
     int sweep_ktv, sweep_kvpt, sweep_g, sweep_ring;
     int wait_polls;  // polls after the first before a wait between warps gives up (idg_set_wait_limit)
     int sweep_vpt;  // consecutive velocities per thread in the micro sweeps (1, 2, 4)
@@ -147,9 +147,12 @@ struct Plan {
 };
 
 // launch shape of the micro sweeps: KParams::sweep_ktv, sweep_kvpt, sweep_g,
-// sweep_ring, from the tuned tile or, untuned, by size; vpt > 0 fixes the
+// sweep_ring, what the caller set and the rest by size; vpt > 0 fixes the
 // velocities per thread (one value for all instances of a batch)
 void sweep_shape(KParams &p, bool fp64, int vpt = 0);
+// whether shared memory holds what the caller asks of the micro sweeps: sweep_tv,
+// sweep_vpt and sweep_stages
+bool sweep_request_fits(const KParams &p, bool fp64);
 
 // kernel launchers (idugks_kernels.cu)
 int configure_kernels(bool fp64);

@@ -2773,6 +2773,18 @@ static size_t sweep_line_bytes(const KParams &p, bool fp64, bool withF, int stag
 
 constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory of a block
 
+// What a caller asks of the micro sweeps: the copies of sweep_stages steps of
+// sweep_pc cells (backward: Delta* and f~ of the tile's velocities, a record of
+// twelve scalars) and two steps' borders.  The line sweeps may need more, lines
+// padded to whole warps and rings; they then take the next shallower depth
+// (plan_shapes), which idg_get_tuning reads back: at two steps every tile fits
+// that is accepted here.
+bool sweep_request_fits(const KParams &p, bool fp64)
+{
+    const size_t T = fp64 ? 8 : 4, w = (size_t)p.sweep_tv * p.sweep_vpt * 2 * T, st = p.sweep_stages;
+    return p.sweep_pc * (st * (2 * w + 9 * T + 16) + 2 * w) <= kMaxSmem;
+}
+
 void sweep_shape(KParams &p, bool fp64, int vpt)
 {
     p.sweep_ktv = p.sweep_tv;
@@ -2782,28 +2794,33 @@ void sweep_shape(KParams &p, bool fp64, int vpt)
     // lines in step, but none of its lanes goes to lines a narrow block lacks
     int lines = 1;
     while (lines < p.sweep_pc && lines < 32) lines *= 2;
-    if (!p.sweep_tuned) {
+    if (!(p.sweep_tuned & 1)) {
         // four groups (eight lines a warp) where the block has that many lines,
         // more on a narrow one
         p.sweep_ktv = std::max(4, 128 / lines > 32 ? 32 : 128 / lines);
         while (p.sweep_ktv * p.sweep_pc > 512) p.sweep_ktv /= 2;
+    }
+    if (!(p.sweep_tuned & 2) && !vpt) {
         // two velocities per thread (16-byte copies); one where that leaves
         // fewer than a warp for each scheduler; four where the warps are many
         // waves (float64 is bound by its arithmetic pipe: one)
-        if (!vpt) {
-            const int lw = 32 / std::min(p.sweep_ktv, std::max(8, 32 / lines));
-            const int warps = (p.sweep_pc + lw - 1) / lw * (p.Nv / (2 * std::min(p.sweep_ktv, 32 / lw)));
-            p.sweep_kvpt = fp64 || warps < 4 * 152 ? 1 : warps > 32 * 152 ? 4 : 2;
-        }
+        const int lw = 32 / std::min(p.sweep_ktv, std::max(8, 32 / lines));
+        const int warps = (p.sweep_pc + lw - 1) / lw * (p.Nv / (2 * std::min(p.sweep_ktv, 32 / lw)));
+        p.sweep_kvpt = fp64 || warps < 4 * 152 ? 1 : warps > 32 * 152 ? 4 : 2;
     }
     // 32 ring entries let neighbouring strips drift a few blocks of steps apart
-    // (at least 2 blocks + 5 are needed); a tile too wide for shared memory at
-    // the shallowest prefetch is halved
-    p.sweep_ring = 32;
-    for (;; p.sweep_ktv /= 2) {
-        p.sweep_g = std::min(p.sweep_ktv, std::max(8, 32 / lines));
-        if (p.sweep_ktv == 1 || sweep_line_bytes(p, fp64, true, 2) <= kMaxSmem) return;
-    }
+    // (at least 2 blocks + 5 are needed: 16).  Where shared memory holds neither
+    // that nor 16 -- the library's own tile at the shallowest prefetch, a caller's
+    // at the one asked for, then the shallower ones -- a warp takes more lines:
+    // fewer, longer strips with less border between them, as far as 512 threads
+    // hold the padded lines
+    const int g0 = std::min(p.sweep_ktv, std::max(8, 32 / lines));
+    for (int st = p.sweep_tuned ? p.sweep_stages : 2; st >= 2; st /= 2)
+        for (p.sweep_g = g0; p.sweep_g >= 1 && 16 * p.sweep_g >= p.sweep_ktv; p.sweep_g /= 2)
+            for (p.sweep_ring = 32; p.sweep_ring >= 16; p.sweep_ring /= 2)
+                if (sweep_line_bytes(p, fp64, true, st) <= kMaxSmem) return;
+    p.sweep_g = g0;
+    p.sweep_ring = 32;  // (does not fit: plan_shapes refuses it)
 }
 
 void blocks_per_instance(const KParams &p, int out[KT_COUNT])
@@ -2839,7 +2856,7 @@ int plan_shapes(const KParams *hp, int n, bool fp64, Plan &pl)
         pl.sched_smem = std::max(pl.sched_smem, (size_t)hp[i].N * 4 * (fp64 ? 8 : 4));
         if (hp[i].relax_sweeps != pl.relax_sweeps) return (int)cudaErrorInvalidValue;
         pl.macro_threads = std::max(pl.macro_threads, macro_threads(hp[i]));
-        pl.sweep_threads = std::max(pl.sweep_threads, pl.sched ? hp[i].sweep_tv * hp[i].sweep_pc : 32 * sweep_line_warps(hp[i]));
+        pl.sweep_threads = std::max(pl.sweep_threads, pl.sched ? hp[i].sweep_ktv * hp[i].sweep_pc : 32 * sweep_line_warps(hp[i]));
         pl.limiter_any |= hp[i].limiter;
         if (hp[i].sweep_vpt != hp[0].sweep_vpt || hp[i].sweep_kvpt != pl.sweep_vpt) return (int)cudaErrorInvalidValue;
     }

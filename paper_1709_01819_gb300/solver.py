@@ -121,7 +121,10 @@ class Solver:
                 "macro_stages": B.IDG_TUNE_MACRO_STAGES, "graph": B.IDG_TUNE_GRAPH,
                 "sweep_vpt": B.IDG_TUNE_SWEEP_VPT, "macro_kind": B.IDG_TUNE_MACRO_KIND}
         # only the given keys are set: the untouched ones keep the library's own choice.
-        # A wider tile is set with one velocity per thread first, so that it fits on the way
+        # A shallower prefetch comes first, and a wider tile with one velocity per thread,
+        # so that it fits on the way
+        if "sweep_stages" in kw and int(kw["sweep_stages"]) <= B.idg_get_tuning(self.ctx, keys["sweep_stages"]):
+            B.idg_set_tuning(self.ctx, keys["sweep_stages"], int(kw["sweep_stages"]))
         if "sweep_tv" in kw and "sweep_vpt" in kw:
             B.idg_set_tuning(self.ctx, keys["sweep_vpt"], 1)
         # (a macro_kind re-derives the macroscopic depth: macro_stages comes after it)
@@ -396,7 +399,9 @@ class Autotuner:
         # the micro sweeps' prefetch depth also decides how many velocity
         # tiles fit on the GPU at once (shared memory per block); the
         # macroscopic sweep keeps the deepest prefetch that fits
-        cands = [dict(sweep_tv=tv, sweep_vpt=vpt, sweep_stages=st, macro_stages=8)
+        own = {k: v for k, v in solver.tuning().items() if k != "graph"}  # the library's own choice first
+        cands = [own] if own["sweep_vpt"] in self.candidates_vpt else []
+        cands += [dict(sweep_tv=tv, sweep_vpt=vpt, sweep_stages=st, macro_stages=8)
                  for tv in self.candidates_tv for vpt in self.candidates_vpt for st in (2, 4, 8)]
         for cand in cands:
             try:
