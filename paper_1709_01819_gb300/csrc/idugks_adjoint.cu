@@ -592,15 +592,20 @@ __global__ void __launch_bounds__(kTB) k_adj_wprime(AParams a)
 // one block over the hyperplanes, four threads (components) per cell.  The
 // transposed blocks over the diagonal come ready (MW), and a step's are loaded
 // before the barrier that opens it, so that after it only the neighbours'
-// increments are read -- from shared memory where all cells' fit (SMEM).
+// increments are read -- from shared memory where all cells' fit (SMEM).  NT,
+// the largest block, sets the registers: a warp's float64 operation takes 64
+// cycles of its scheduler, and spills stand in the chain.
 // Re-deriving the Jacobians at every face took 767 us on 24 x 24 cells, this
-// 84 us (float64 operations of a few warps, 64 cycles each).
+// 84 us; a whole pass over 90 x 80 cells x 64 velocities, whose increments do not
+// fit, 3.96 ms with the instance for 1024 threads and 3.30 ms with this one, over
+// 130 x 130 cells, which need 1024, 8.66 ms at the 32 registers the compiler
+// chose and 7.87 ms at 64.
 struct AdjMacroCell {
     int c, nb[4];
     double b, m[4][4];
 };
 template <bool SMEM, int NT>
-__global__ void __launch_bounds__(NT) k_adj_macro(AParams a)
+__global__ void __launch_bounds__(NT, 1) k_adj_macro(AParams a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     double *y = SMEM ? (double *)smraw : a.ba;  // [N][4]
@@ -993,7 +998,7 @@ constexpr size_t kAdjSmem = 224 * 1024;  // dynamic shared memory the sweeps may
 int launch_adjoint_setup(const AParams &a, void *stream)
 {
     cudaStream_t st = (cudaStream_t)stream;
-    for (const void *k : {(const void *)k_adj_lines<true>, (const void *)k_adj_lines<false>, (const void *)k_adj_macro<true, 512>, (const void *)k_adj_macro<true, 1024>}) {
+    for (const void *k : {(const void *)k_adj_lines<true>, (const void *)k_adj_lines<false>, (const void *)k_adj_macro<true, 512>}) {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAdjSmem);
         if (e != cudaSuccess) return (int)e;
     }
@@ -1069,10 +1074,11 @@ int launch_adjoint_iteration(const AParams &a, int it, void *stream)
     k_adj_wprime<<<a.N, kTB, 0, st>>>(a);
     const int mt = std::min(1024, (4 * std::min(a.ni, a.nj) + 31) / 32 * 32);
     const size_t ysm = (size_t)32 * a.N;
-    // (more than 128 lines leave a thread 64 registers, too few for two steps' blocks)
-    if (ysm > kAdjSmem) k_adj_macro<false, 1024><<<1, mt, 0, st>>>(a);
-    else if (mt <= 512) k_adj_macro<true, 512><<<1, mt, ysm, st>>>(a);
-    else k_adj_macro<true, 1024><<<1, mt, ysm, st>>>(a);
+    // more than 128 lines leave a thread 64 registers, too few for two steps' blocks
+    // (such a block has over 16384 cells: their increments never fit shared memory)
+    if (mt > 512) k_adj_macro<false, 1024><<<1, mt, 0, st>>>(a);
+    else if (ysm > kAdjSmem) k_adj_macro<false, 512><<<1, mt, 0, st>>>(a);
+    else k_adj_macro<true, 512><<<1, mt, ysm, st>>>(a);
     k_adj_face<<<a.nf, kTB, 0, st>>>(a);
     k_adj_gather<<<nblk(2 * NNv, 256), 256, 0, st>>>(a);
     k_adj_cell<<<a.N, kTB, 0, st>>>(a);
