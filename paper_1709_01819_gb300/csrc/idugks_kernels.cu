@@ -2468,8 +2468,11 @@ __device__ __forceinline__ void ld_rec7(double (&o)[7], const double *s)
     o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y; o[4] = c.x; o[5] = c.y; o[6] = s[6];
 }
 
+// (Four float64 velocities per thread spill in any case; without the bound of one
+// block the compiler may give them 32 registers: a 64 x 64 block with a periodic
+// seam and 576 velocities then took 1600 us backward, 1000 us with it.)
 template <class T, bool FWD, int VPT, int PF, bool SEAM>
-__global__ void __launch_bounds__(512) k_sweep_lines(Launch L)
+__global__ void __launch_bounds__(512, sizeof(T) == 8 && VPT == 4 ? 1 : 0) k_sweep_lines(Launch L)
 {
     IDG_LOCATE();
     using T2 = typename V2<T>::t;
