@@ -637,7 +637,7 @@ size_t layout(idg_ctx *c, char *base, KParams *kp)
     k.bdevH = L.take<char>(4 * ts * Nv);
     k.f = L.take<char>(t2 * N * Nv);
     k.fbp = L.take<char>(t2 * N * Nv);
-    k.dst = L.take<char>(t2 * N * Nv);
+    k.dst = k.fbp;  // fb+ is dead once the reconstruction has read it, the increments are born after it
     // the face-flux buffer doubles as the float64 staging area of
     // idg_set_state / idg_get_state (G and H of every cell): on an unstructured
     // mesh (about 1.5 faces per cell for triangles) that can be the larger need

@@ -64,7 +64,7 @@ struct KParams {
     void *fbp;      // [N][Nv] T2 fb+ - M_ref
     void *F;        // [nf][Nv] T2 fb at the face (minus M_ref), then the flux of (f_face - M_ref)
     void *ftie;     // [nf][max(nvx, nvy)] T2 interior faces: fb from the R side at velocities along the face (tie_slot())
-    void *dst;      // [N][Nv] T2 Delta* then Delta
+    void *dst;      // [N][Nv] T2 residual, Delta* then Delta (the memory of fbp)
     double *W;      // [N][4]
     void *cellraw;  // [N][kRaw] acc raw moments of f~ - M_ref
     void *cellA;    // [N][16] T: equilibrium at W^n (14), c1, c2 of fb+
