@@ -1043,11 +1043,12 @@ __global__ void __launch_bounds__(kVecThreads) k_vec_dot(const double *x, const 
     }
 }
 
-// y = a x + b y
+// y = a x + b y; with b = 0 y is only written (memory never written before may
+// hold NaN)
 __global__ void k_vec_axpby(double a, const double *x, double b, double *y, size_t n)
 {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        y[i] = a * x[i] + b * y[i];
+        y[i] = b == 0.0 ? a * x[i] : a * x[i] + b * y[i];
 }
 
 int launch_vec_dot(const double *x, const double *y, size_t n, double *dpart, void *stream)
