@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kTB) k_adj_cell_lin(AParams a)
     for (int k = threadIdx.x; k < Nv; k += blockDim.x) {
         double eg, eh;
         const double E = adj::eq_maxwell(e, a.ux[k], a.uy[k]);
-        a.Ec[(size_t)c * Nv + k] = E;
+        if (a.Ec) a.Ec[(size_t)c * Nv + k] = E;
         adj::eq_eval_at(e, E, a.ux[k], a.uy[k], eg, eh);
         a.fbG[(size_t)c * Nv + k] = cp[CP_C1] * G[k] + cp[CP_C2] * eg;
         a.fbH[(size_t)c * Nv + k] = cp[CP_C1] * H[k] + cp[CP_C2] * eh;
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(kTB) k_adj_face_lin(AParams a)
     for (int k = threadIdx.x; k < Nv; k += blockDim.x) {
         double eg, eh;
         const double E = adj::eq_maxwell(e, a.ux[k], a.uy[k]);
-        a.Ef[(size_t)f * Nv + k] = E;
+        if (a.Ef) a.Ef[(size_t)f * Nv + k] = E;
         adj::eq_eval_at(e, E, a.ux[k], a.uy[k], eg, eh);
         const double sn = xdn(a.ux[k], a.uy[k], nx, ny);
         const double Fg = sn * S * (fp[FP_A] * a.fbarG[(size_t)f * Nv + k] + fp[FP_B] * eg);
@@ -387,8 +387,9 @@ __device__ __forceinline__ double outflow(const AParams &a, int c, int m, double
 
 // per (cell, velocity): one over the micro LU-SGS diagonal of Eq. (26) and over it
 // the couplings of the transposed sweeps to the two neighbours already swept away
-// from a seam (constant through the iteration; both components share them)
-__global__ void k_adj_micro_lin(AParams a)
+// from a seam (constant through the iteration; both components share them), of
+// the directions d0 .. d1 - 1 (0 ascending, 1 descending)
+__global__ void k_adj_micro_lin(AParams a, int d0, int d1)
 {
     const size_t NNv = (size_t)a.N * a.Nv, ck = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (ck >= NNv) return;
@@ -401,8 +402,8 @@ __global__ void k_adj_micro_lin(AParams a)
     const bool in[4] = {i > 0, i + 1 < a.ni, j > 0, j + 1 < a.nj};
     const int w = a.ni <= a.nj ? 2 : 0, t = 2 - w;  // slots along the own line, across
     double2 *o = (double2 *)a.cm;
-    for (int dir = 0; dir < 2; ++dir)
-        o[dir * NNv + ck] = make_double2(in[w + dir] ? so[w + dir] * id : 0.0, in[t + dir] ? so[t + dir] * id : 0.0);
+    for (int dir = d0; dir < d1; ++dir)
+        o[(a.compact ? 0 : dir * NNv) + ck] = make_double2(in[w + dir] ? so[w + dir] * id : 0.0, in[t + dir] ? so[t + dir] * id : 0.0);
 }
 
 // ---------------------------------------------------------------------------
@@ -463,7 +464,7 @@ template <bool ASC> __global__ void __launch_bounds__(512) k_adj_lines(AParams a
     const ptrdiff_t base = (ptrdiff_t)c0 * Nv + k;
     const int sv = cs * Nv;
     const double *xG = (ASC ? a.lamG : a.bbG) + base, *xH = (ASC ? a.lamH : a.bbH) + base, *iD = a.iDm + base;
-    const double2 *cm = (const double2 *)a.cm + (ASC ? 0 : (ptrdiff_t)a.N * Nv) + base;
+    const double2 *cm = (const double2 *)a.cm + (ASC || a.compact ? 0 : (ptrdiff_t)a.N * Nv) + base;
     double *yG = a.bbG + base, *yH = a.bbH + base;
     const unsigned nwl = tt < nt && k0 < Nv ? nw : 0;
     const int start = tt + strip * kSweepBlock;
@@ -556,7 +557,7 @@ template <bool ASC> __global__ void __launch_bounds__(512) k_adj_lines(AParams a
 // per cell: bar W' = (dR_f/dW')^T bar_b from the collision term
 // -cq (f~ - f^S(W', q)), cq = 2 Omega/(2 tau' + dt); bar q of the cell from the
 // same term; bwp = lambda_W + bar W'
-__global__ void __launch_bounds__(kTB) k_adj_wprime(AParams a)
+template <bool KEPT> __global__ void __launch_bounds__(kTB) k_adj_wprime(AParams a)
 {
     __shared__ double sm[32 * 7 + 7];
     const int c = blockIdx.x, Nv = a.Nv;
@@ -568,7 +569,8 @@ __global__ void __launch_bounds__(kTB) k_adj_wprime(AParams a)
     double s[7] = {0, 0, 0, 0, 0, 0, 0};
     for (int k = threadIdx.x; k < Nv; k += blockDim.x) {
         double eg, eh;
-        const double E = a.Ec[(size_t)c * Nv + k], x = a.ux[k], y = a.uy[k], bg = bG[k], bh = bH[k];
+        const double x = a.ux[k], y = a.uy[k], bg = bG[k], bh = bH[k];
+        const double E = KEPT ? a.Ec[(size_t)c * Nv + k] : adj::eq_maxwell(e, x, y);
         adj::eq_eval_at(e, E, x, y, eg, eh);
         s[6] -= bg * (G[k] - eg) + bh * (H[k] - eh);
         adj::eq_vjp_at(e, E, x, y, cq * bg, cq * bh, s);
@@ -657,7 +659,7 @@ __global__ void __launch_bounds__(NT, 1) k_adj_macro(AParams a)
 // per face: seeds bar F (from bar_b of the two cells), bar Phi (from bar_a and
 // the objective), then the VJP of Eq. (18)-(20), the face moments and the
 // boundary; writes the adjoint weight of each cell's reconstruction at the face
-__global__ void __launch_bounds__(kTB) k_adj_face(AParams a)
+template <bool KEPT> __global__ void __launch_bounds__(kTB) k_adj_face(AParams a)
 {
     __shared__ double sm[32 * 8 + 8];
     __shared__ double bc_sh[8];
@@ -694,7 +696,7 @@ __global__ void __launch_bounds__(kTB) k_adj_face(AParams a)
     for (int k = threadIdx.x; k < Nv; k += blockDim.x) {
         double bg, bh, eg, eh;
         barF(k, bg, bh);
-        const double E = a.Ef[(size_t)f * Nv + k];
+        const double E = KEPT ? a.Ef[(size_t)f * Nv + k] : adj::eq_maxwell(e, a.ux[k], a.uy[k]);
         adj::eq_eval_at(e, E, a.ux[k], a.uy[k], eg, eh);
         const double snS = xdn(a.ux[k], a.uy[k], nx, ny) * S;
         s[6] += snS * (fbG[k] * bg + fbH[k] * bh);
@@ -841,7 +843,7 @@ __global__ void k_adj_gather(AParams a)
 // per cell: adjoint weight of fb+ (own record plus the neighbours' gradient
 // and limiter terms), VJP of fb+ = c1 f~ + c2 f^S (Eq. 12), of the equilibrium,
 // q (Eq. 20), the heat flux and tau; lambda <- lambda + increment
-__global__ void __launch_bounds__(kTB) k_adj_cell(AParams a)
+template <bool KEPT> __global__ void __launch_bounds__(kTB) k_adj_cell(AParams a)
 {
     __shared__ double sm[32 * 8 + 8];
     __shared__ double bc_sh[2];
@@ -879,7 +881,8 @@ __global__ void __launch_bounds__(kTB) k_adj_cell(AParams a)
         a.bfb[(size_t)c * Nv + k] = b[0];
         a.bfb[NNv + (size_t)c * Nv + k] = b[1];
         double eg, eh;
-        const double E = a.Ec[(size_t)c * Nv + k], x = a.ux[k], y = a.uy[k];
+        const double x = a.ux[k], y = a.uy[k];
+        const double E = KEPT ? a.Ec[(size_t)c * Nv + k] : adj::eq_maxwell(e, x, y);
         adj::eq_eval_at(e, E, x, y, eg, eh);
         s[6] += G[k] * b[0] + H[k] * b[1];
         s[7] += eg * b[0] + eh * b[1];
@@ -937,7 +940,12 @@ unsigned nblk(size_t n, int tb) { return (unsigned)((n + tb - 1) / tb); }
 
 }  // namespace
 
-size_t adjoint_layout(const AParams &s, int nrhs, char *base, AParams *out)
+// What one pass leaves for the next is the multipliers' alone; the solves run one
+// after the other and share the rest.  fb+ of the linearisation lies where the
+// passes keep the reconstruction's weights, a cell's weight of fb+ where the
+// faces' weights were before k_adj_gather took them.  compact leaves out what
+// can be formed again: the Maxwellians, and one direction's micro couplings.
+size_t adjoint_layout(const AParams &s, int nrhs, bool compact, char *base, AParams *out)
 {
     size_t off = 0;
     auto take = [&](size_t bytes) -> char * {
@@ -948,14 +956,13 @@ size_t adjoint_layout(const AParams &s, int nrhs, char *base, AParams *out)
     };
     const size_t N = s.N, Nv = s.Nv, nf = s.nf, NNv = N * Nv, d = sizeof(double);
     AParams a = s;
+    a.compact = compact;
     // linearisation, shared by the solves
     a.lsw = (double *)take(8 * N * d);
     a.crv = (double *)take(8 * N * d);
     a.G = (double *)take(NNv * d);
     a.H = (double *)take(NNv * d);
     a.cpar = (double *)take(kCP * N * d);
-    a.fbG = (double *)take(NNv * d);
-    a.fbH = (double *)take(NNv * d);
     a.sig = (double *)take(4 * NNv * d);
     a.lim = (double *)take(6 * NNv * d);
     a.lsl = (signed char *)take(4 * NNv);
@@ -964,25 +971,28 @@ size_t adjoint_layout(const AParams &s, int nrhs, char *base, AParams *out)
     a.fbarH = (double *)take(nf * Nv * d);
     a.iDW = (double *)take(N * d);
     a.MW = (double *)take(64 * N * d);
-    a.Ec = (double *)take(NNv * d);
-    a.Ef = (double *)take(nf * Nv * d);
+    a.Ec = compact ? nullptr : (double *)take(NNv * d);
+    a.Ef = compact ? nullptr : (double *)take(nf * Nv * d);
     a.iDm = (double *)take(NNv * d);
-    a.cm = (double *)take(4 * NNv * d);
+    a.cm = (double *)take((compact ? 2 : 4) * NNv * d);
+    // scratch of a pass
+    a.bbG = (double *)take(NNv * d);
+    a.bbH = (double *)take(NNv * d);
+    a.bfG = (double *)take(2 * nf * Nv * d);
+    a.bfH = a.bfG + nf * Nv;
+    a.bfb = a.bfG;
+    a.crec = (double *)take(8 * NNv * d);
+    a.fbG = a.crec;
+    a.fbH = a.fbG + NNv;
     a.status = (int *)take(256);
     for (int r = 0; r < nrhs; ++r) {
         a.seed = r;
         a.lamG = (double *)take(NNv * d);
         a.lamH = (double *)take(NNv * d);
         a.lamW = (double *)take(4 * N * d);
-        a.bbG = (double *)take(NNv * d);
-        a.bbH = (double *)take(NNv * d);
         a.bwp = (double *)take(4 * N * d);
         a.ba = (double *)take(4 * N * d);
         a.bqc = (double *)take(2 * N * d);
-        a.bfG = (double *)take(nf * Nv * d);
-        a.bfH = (double *)take(nf * Nv * d);
-        a.crec = (double *)take(8 * NNv * d);
-        a.bfb = (double *)take(2 * NNv * d);
         a.fpp = (double *)take(kFPar * nf * d);
         a.cpp = (double *)take(2 * N * d);
         a.rpart = (double *)take(N * d);
@@ -1007,7 +1017,7 @@ int launch_adjoint_setup(const AParams &a, void *stream)
     k_adj_grad_lin<<<nblk(2 * NNv, 256), 256, 0, st>>>(a);
     k_adj_face_lin<<<a.nf, kTB, 0, st>>>(a);
     k_adj_macro_lin<<<nblk(a.N, 32), 32, 0, st>>>(a);
-    k_adj_micro_lin<<<nblk(NNv, 256), 256, 0, st>>>(a);
+    if (!a.compact) k_adj_micro_lin<<<nblk(NNv, 256), 256, 0, st>>>(a, 0, 2);
     return (int)cudaGetLastError();
 }
 
@@ -1065,14 +1075,16 @@ int launch_vec_axpby(double a, const double *x, double b, double *y, size_t n, v
 
 int vec_dot_blocks() { return kVecBlocks; }
 
-int launch_adjoint_iteration(const AParams &a, int it, void *stream)
+// a pass with the Maxwellians and couplings at hand (KEPT) or formed again
+template <bool KEPT> static int adjoint_iteration(const AParams &a, int it, cudaStream_t st)
 {
-    cudaStream_t st = (cudaStream_t)stream;
     const size_t NNv = (size_t)a.N * a.Nv;
     const AdjShape sh = adj_shape(a);
+    if (!KEPT) k_adj_micro_lin<<<nblk(NNv, 256), 256, 0, st>>>(a, 0, 1);
     k_adj_lines<true><<<nblk(a.Nv, sh.G), 32 * sh.strips, sh.smem, st>>>(a, sh);
+    if (!KEPT) k_adj_micro_lin<<<nblk(NNv, 256), 256, 0, st>>>(a, 1, 2);
     k_adj_lines<false><<<nblk(a.Nv, sh.G), 32 * sh.strips, sh.smem, st>>>(a, sh);
-    k_adj_wprime<<<a.N, kTB, 0, st>>>(a);
+    k_adj_wprime<KEPT><<<a.N, kTB, 0, st>>>(a);
     const int mt = std::min(1024, (4 * std::min(a.ni, a.nj) + 31) / 32 * 32);
     const size_t ysm = (size_t)32 * a.N;
     // more than 128 lines leave a thread 64 registers, too few for two steps' blocks
@@ -1080,11 +1092,17 @@ int launch_adjoint_iteration(const AParams &a, int it, void *stream)
     if (mt > 512) k_adj_macro<false, 1024><<<1, mt, 0, st>>>(a);
     else if (ysm > kAdjSmem) k_adj_macro<false, 512><<<1, mt, 0, st>>>(a);
     else k_adj_macro<true, 512><<<1, mt, ysm, st>>>(a);
-    k_adj_face<<<a.nf, kTB, 0, st>>>(a);
+    k_adj_face<KEPT><<<a.nf, kTB, 0, st>>>(a);
     k_adj_gather<<<nblk(2 * NNv, 256), 256, 0, st>>>(a);
-    k_adj_cell<<<a.N, kTB, 0, st>>>(a);
+    k_adj_cell<KEPT><<<a.N, kTB, 0, st>>>(a);
     k_adj_res<<<1, kTB, 0, st>>>(a, it);
     return (int)cudaGetLastError();
+}
+
+int launch_adjoint_iteration(const AParams &a, int it, void *stream)
+{
+    cudaStream_t st = (cudaStream_t)stream;
+    return a.compact ? adjoint_iteration<false>(a, it, st) : adjoint_iteration<true>(a, it, st);
 }
 
 }  // namespace idg

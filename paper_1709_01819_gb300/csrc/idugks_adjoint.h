@@ -53,6 +53,7 @@ struct AParams {
     signed char *lsl;  // [2][N][Nv][2] limiter: binding face slot, extreme-neighbour slot (-1: self)
     double *fpar;      // [nf][kFP]
     double *fbarG, *fbarH;  // [nf][Nv]
+    int compact;       // 1: no Ec, Ef; cm holds one direction, formed before each sweep
     double *Ec, *Ef;   // [N][Nv], [nf][Nv] reduced Maxwellian of the cell's / face's equilibrium
     double *iDm;       // [N][Nv] one over the micro LU-SGS diagonal
     double *cm;        // [2][N][Nv][2] ascending, descending: micro couplings over the diagonal, towards
@@ -79,7 +80,7 @@ struct AParams {
 
 // Workspace of the linearisation and of nrhs (1 or 2) adjoint solves that
 // share it; out[r] describes solve r.
-size_t adjoint_layout(const AParams &shape, int nrhs, char *base, AParams *out);
+size_t adjoint_layout(const AParams &shape, int nrhs, bool compact, char *base, AParams *out);
 int launch_adjoint_setup(const AParams &a, void *stream);  // linearisation
 int launch_adjoint_zero(const AParams &a, void *stream);   // lambda = 0 of one solve
 int launch_adjoint_iteration(const AParams &a, int it, void *stream);

@@ -82,6 +82,7 @@ struct idg_ctx {
     double venkat_k = 0.0;   // idg_set_limiter_smoothing
     // last idg_adjoint: number of right-hand sides and the mass multiplier
     int adj_nrhs = 0;
+    bool adj_compact = false;
     double adj_beta = 0.0;
 };
 
@@ -2122,7 +2123,7 @@ idg_status idg_adjoint_workspace_size(idg_ctx *c, size_t *bytes)
     if (!c || !bytes) return IDG_ERR_ARG;
     idg_status s = build(c);
     if (s) return s;
-    *bytes = idg::adjoint_layout(adjoint_shape(c), adjoint_rhs(c), nullptr, nullptr) + krylov_bytes(c);
+    *bytes = idg::adjoint_layout(adjoint_shape(c), adjoint_rhs(c), false, nullptr, nullptr) + krylov_bytes(c);
     return IDG_OK;
 }
 
@@ -2182,7 +2183,10 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
     const int nrhs = adjoint_rhs(c);
     if (c->adj_method == IDG_ADJ_GMRES && nrhs != 1)
         return fail(c, IDG_ERR_ARG, "the GMRES adjoint solves one right-hand side: a domain with a far field");
-    const size_t base_need = idg::adjoint_layout(adjoint_shape(c), nrhs, nullptr, nullptr);
+    // the tables that save a pass time, or the smaller layout that forms them again
+    size_t base_need = idg::adjoint_layout(adjoint_shape(c), nrhs, false, nullptr, nullptr);
+    const bool compact = bytes < base_need + krylov_bytes(c);
+    if (compact) base_need = idg::adjoint_layout(adjoint_shape(c), nrhs, true, nullptr, nullptr);
     const size_t need = base_need + krylov_bytes(c);
     if (bytes < need) return fail(c, IDG_ERR_OOM, "adjoint workspace of %zu bytes, need %zu", bytes, need);
 
@@ -2207,7 +2211,7 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
     base.obj_axis = objective == IDG_OBJ_FORCE_X ? 0 : 1;
     base.obj_mask = side_mask;
     idg::AParams A[2];
-    idg::adjoint_layout(base, nrhs, (char *)workspace, A);
+    idg::adjoint_layout(base, nrhs, compact, (char *)workspace, A);
 
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
@@ -2441,6 +2445,7 @@ idg_status idg_adjoint(idg_ctx *c, int objective, int side_mask, const int *para
     }
     c->adj_beta = beta;
     c->adj_nrhs = nrhs;
+    c->adj_compact = compact;
     if (J) *J = Jv;
     if (iters_done) *iters_done = done;
     if (residual) *residual = rel;
@@ -2460,7 +2465,7 @@ idg_status idg_adjoint_state(idg_ctx *c, const void *workspace, int which, doubl
     const double wJ = which == 2 ? 0.0 : 1.0;
     const double wm = which == 0 ? c->adj_beta : (which == 2 ? 1.0 : 0.0);
     idg::AParams A[2];
-    idg::adjoint_layout(adjoint_shape(c), c->adj_nrhs, (char *)workspace, A);
+    idg::adjoint_layout(adjoint_shape(c), c->adj_nrhs, c->adj_compact, (char *)workspace, A);
     cudaStream_t st = (cudaStream_t)stream;
     const size_t n = (size_t)c->N * c->Nv, n4 = (size_t)4 * c->N;
     double *out[3] = {lamG, lamH, lamW};

@@ -1,5 +1,6 @@
 """Workspace sizes (no GPU work): a buffer that held a problem when the
-increments had memory of their own still holds it."""
+increments, or each adjoint solve's scratch, had memory of their own still holds
+it."""
 import json
 
 import pytest
@@ -50,3 +51,16 @@ def test_no_workspace_has_grown(name):
         configure(ctx, PROBLEMS[name]())
         assert B.idg_workspace_size(ctx) <= size
         B.idg_destroy(ctx)
+
+
+# closed domains: two solves
+ADJOINT = {"couette64": 29743616, "couette64_v8": 2909696, "cavity64": 1840644352, "cavity64_v8": 120324352,
+           "cavity128_v28": 5629411584, "long": 117116672}
+
+
+@pytest.mark.parametrize("name", sorted(ADJOINT))
+def test_no_closed_domains_adjoint_workspace_has_grown(name):
+    ctx = B.idg_create(B.IDG_FP64, 0)
+    configure(ctx, PROBLEMS[name]())
+    assert B.idg_adjoint_workspace_size(ctx) <= ADJOINT[name]
+    B.idg_destroy(ctx)
