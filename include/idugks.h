@@ -309,8 +309,10 @@ idg_status idg_get_wall(idg_ctx *ctx, int side, double *out5, int cap, int *nfac
 
 /* One iteration with a CUDA event recorded between its kernel launches on
  * the caller's stream (synchronises it).  kernel_ms[0..5] receives the
- * device time of: cell prep, interior faces, boundary faces, macroscopic
- * predictor, forward sweep, backward sweep (0 for a kernel not launched). */
+ * device time of: cell prep (moments, coefficients, fb+); reconstruction, face
+ * moments and coefficients; face flux and its moments; macroscopic predictor;
+ * micro residual and forward sweep (explicit: the update); backward sweep (0
+ * for a group not launched). */
 idg_status idg_iterate_profiled(idg_ctx *ctx, void *stream, double *kernel_ms);
 
 /* Launch-shape tuning of the wavefront kernels (after idg_bind_workspace;

@@ -436,7 +436,7 @@ AdjShape adj_shape(const AParams &a)
     // as many velocities side by side as leave every SM a block, at most 8; at
     // most 16 strips a block
     s.G = 8;
-    while (s.G > 1 && (a.Nv / s.G < 152 || (nt + 32 / s.G - 1) / (32 / s.G) > 16)) s.G /= 2;
+    while (s.G > 1 && (a.Nv / s.G < kSMs || (nt + 32 / s.G - 1) / (32 / s.G) > 16)) s.G /= 2;
     const int lw = 32 / s.G;
     s.strips = (nt + lw - 1) / lw;
     s.smem = 64 + (size_t)s.strips * (kAdjRing * s.G * 16 + kAdjAhead * 32 * 40);

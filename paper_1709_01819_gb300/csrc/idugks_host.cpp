@@ -1136,20 +1136,22 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
         k.nsteps_b = c->nsteps_b;
     }
     // k_cell_moments: a warp a cell, two or four from the length on that leaves each
-    // about four chunks of 256 velocities or more; the cells of such a problem are
-    // few thousands and fill few waves of warps (121 x 81 cells x 7921 velocities:
-    // 2.02 waves, 221 us; four warps a cell 173 us.  The face rows, twice as many,
+    // about four chunks of 256 velocities or more.  The line lies in the velocities
+    // alone: a state on the device has few cells where it has many velocities, so
+    // that one warp a cell makes few waves, of which the last costs most (measured
+    // at one size, 121 x 81 cells x 7921 velocities: 2.02 waves,
+    // 221 us; four warps a cell 173 us.  The face rows, twice as many,
     // took 464 + 584 us at one warp and 454 + 565 us at four there, but 201 and
     // 213 us on 128 x 128 x 784 with the code for several in them: they stay at one)
     k.row_warps = c->Nv >= 4096 ? 4 : c->Nv >= 2048 ? 2 : 1;
     // per-(cell, velocity) kernels: four cells a block once that leaves every SM
     // its eight resident blocks, two or one below
     const long long nblocks = (long long)c->N * ((c->Nv + 255) / 256);
-    k.cpb = nblocks >= 4 * 8 * 152 ? 4 : nblocks >= 2 * 8 * 152 ? 2 : 1;
-    // sweep launch shape: cell slots cover the longest hyperplane up to 64
-    // micro sweeps: one thread per cell of the longest hyperplane (of the
-    // longest schedule step on an unstructured mesh) and tv velocities per
-    // CTA (8 by default, more on very narrow blocks)
+    k.cpb = nblocks >= 4 * 8 * idg::kSMs ? 4 : nblocks >= 2 * 8 * idg::kSMs ? 2 : 1;
+    // micro sweeps: a slot per line of a structured block (at most 256) or per
+    // cell of the longest schedule step of an unstructured mesh; the tile here is
+    // the scheduled sweeps' (8 velocities a block, more where the steps are
+    // short), the line sweeps take theirs by size (sweep_shape)
     int maxlen = c->unstr ? c->sched_pc : std::min(c->ni, c->nj);
     if (maxlen > 256) return fail(c, IDG_ERR_ARG, "min(ni, nj) = %d exceeds 256", maxlen);
     k.sweep_pc = maxlen;

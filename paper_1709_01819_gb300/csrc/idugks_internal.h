@@ -11,6 +11,7 @@ constexpr int kMaxVel = 16384;
 constexpr int kMaxHist = 1 << 16;  // residual-history ring (iterations)
 constexpr int kCellP = 16;         // per-cell / per-face coefficient records
 constexpr int kRaw = 11;           // raw velocity moments kept per cell / face
+constexpr int kSMs = 152;  // streaming multiprocessors of a GB300
 constexpr int kNoAllocMaxCells = 16384;  // cell limit of idg_get_moments_noalloc
 
 // Everything one kernel launch needs, passed by value.  Device pointers point
@@ -81,12 +82,12 @@ struct KParams {
     void *mline;    // [6][nslot][4] T: the record as k_macro_lines reads it (null if unstructured), cell slots by line_slot()
     void *mdW;      // [N][4] T increments (Delta W* then Delta W); k_macro_lines: [nslot][4]
     void *mdW2;     // [N][4] T second increment buffer of the point relaxation (else null)
-    double *mpart;  // [ceil(N/256)] block partial sums of ||R/Omega||^2
+    double *mpart;  // [ceil(N/32)] block partial sums of ||R/Omega||^2
     double *res;    // [kMaxHist] absolute residual per iteration
     int *iter;      // [1] device iteration counter
     int *status;    // [1] device status word
     // launch shape of the wavefront kernels: velocities per CTA and cell
-    // slots of the micro sweeps, prefetch depths (hyperplanes; 4 or 8)
+    // slots of the micro sweeps, prefetch depths asked for (steps; 2, 4 or 8)
     int sweep_tv, sweep_pc, sweep_stages, macro_stages;
     int row_warps;   // warps per cell of k_cell_moments (1, 2, 4)
     int cpb;         // cells per block of the per-(cell, velocity) kernels

@@ -110,8 +110,9 @@ class Solver:
         return st == B.IDG_OK, n, r
 
     def iterate_profiled(self) -> np.ndarray:
-        """One iteration; device ms of cell prep, interior faces, boundary faces,
-        macroscopic predictor, forward sweep, backward sweep."""
+        """One iteration; device ms of cell prep, reconstruction with the face moments,
+        face flux, macroscopic predictor, micro residual with the forward sweep,
+        backward sweep."""
         return B.idg_iterate_profiled(self.ctx, self.stream)
 
     def set_tuning(self, **kw):
