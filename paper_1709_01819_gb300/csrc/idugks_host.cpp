@@ -750,20 +750,34 @@ idg_status upload_reference(idg_ctx *c)
             dH[i] = c->K * RT * G - kRTr * gref[q];
         }
     }
+    // per boundary face the outgoing sum of M_ref and the incoming one of the
+    // boundary's Maxwellian, four faces side by side: one sum alone is a chain of
+    // additions
     std::vector<double> bconst((size_t)2 * c->nf, 0.0);
-    for (int f = 0; f < c->nf; ++f) {
-        if (c->fbc[f] < 0) continue;
-        const double *g = &c->fgeo[(size_t)7 * f];
-        double on = c->fL[f] >= 0 ? 1.0 : -1.0;
-        int sd = c->fside[f];
-        double out = 0.0, in = 0.0;
-        for (int q = 0; q < Nv; ++q) {
-            double so = on * (c->ux[q] * g[0] + c->uy[q] * g[1]);
-            if (so > 0) out += c->w[q] * so * gref[q];
-            else if (so < 0) in += c->w[q] * (-so) * bG[(size_t)sd * Nv + q];
+    std::vector<int> bf;
+    for (int f = 0; f < c->nf; ++f)
+        if (c->fbc[f] >= 0) bf.push_back(f);
+    const double *ux = c->ux.data(), *uy = c->uy.data(), *w = c->w.data(), *gr = gref.data();
+    for (size_t i = 0; i < bf.size(); i += 4) {
+        double on[4], gx[4], gy[4], out[4] = {0, 0, 0, 0}, in[4] = {0, 0, 0, 0};
+        const double *bg[4];
+        for (int u = 0; u < 4; ++u) {
+            const int f = bf[std::min(i + u, bf.size() - 1)];
+            on[u] = c->fL[f] >= 0 ? 1.0 : -1.0;
+            gx[u] = c->fgeo[(size_t)7 * f];
+            gy[u] = c->fgeo[(size_t)7 * f + 1];
+            bg[u] = bG.data() + (size_t)c->fside[f] * Nv;
         }
-        bconst[2 * f] = out;
-        bconst[2 * f + 1] = in;
+        for (int q = 0; q < Nv; ++q)
+            for (int u = 0; u < 4; ++u) {
+                const double so = on[u] * (ux[q] * gx[u] + uy[q] * gy[u]);
+                if (so > 0) out[u] += w[q] * so * gr[q];
+                else if (so < 0) in[u] += w[q] * (-so) * bg[u][q];
+            }
+        for (size_t u = 0; u < std::min<size_t>(4, bf.size() - i); ++u) {
+            bconst[2 * (size_t)bf[i + u]] = out[u];
+            bconst[2 * (size_t)bf[i + u] + 1] = in[u];
+        }
     }
     std::vector<float> gf(gref.begin(), gref.end());
     cudaError_t e;
