@@ -3,8 +3,8 @@
 The diagonal D of a cell enters every step of a line, so an error that is the
 same in all its cells adds up along the line: on the mixed solver's 90 x 70
 block G was 0.96e-9 (LU-SGS predictor) and 1.05e-9 (point relaxation) off the
-float64 solver's, rms after 16 iterations, with the outflow's sum rounded by
-itself, and is 0.42e-9 and 0.43e-9 with it added to the cell's base, as it was
+float64 solver's, rms after 16 iterations, with the fluxes' sum rounded by
+itself, and is 0.42e-9 and 0.43e-9 with them added to the cell's base, as it was
 when a hyperplane was swept at a time; 0.6e-9 lies between.
 
 The reciprocal of D is the correctly rounded one for every float whose
