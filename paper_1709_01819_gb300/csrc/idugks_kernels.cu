@@ -2374,8 +2374,8 @@ __global__ void __launch_bounds__(512) k_sweep(Launch L)
 // Bound by the latency of a step (issue a third of the cycles on 64 lines), on
 // large states by the copies.  Measured against one barrier per hyperplane with
 // all neighbours in shared memory, forward + backward, float32: 64 x 64 cells
-// with 1024 velocities 79 + 84 -> 36 + 35 us, 128 x 128 with 784 234 + 326 ->
-// 83 + 89 us, 121 x 81 with 7921 950 + 1436 -> 495 + 671 us; float64 64 x 64
+// with 1024 velocities 79 + 84 -> 36 + 36 us, 128 x 128 with 784 234 + 326 ->
+// 83 + 92 us, 121 x 81 with 7921 950 + 1436 -> 505 + 683 us; float64 64 x 64
 // 462 + 467 -> 359 + 359 us.  Loads into registers instead of cp.async took
 // 53 + 51 us on 64 x 64, a warp running through the steps before its first and
 // after its last cell 57 + 61 us.
