@@ -67,6 +67,7 @@ struct idg_ctx {
     size_t stage_bytes = 0;
     // CUDA graph of kGraphChunk iterations, replayed on a library-owned stream
     // that is event-ordered with the caller's stream
+    int sweep_depth = 8;  // prefetch depth that goes with a tile set by the caller, unless it is set too
     int use_graph = 1;
     cudaStream_t gstream = nullptr;
     cudaGraphExec_t gexec = nullptr;   // kGraphChunk iterations
@@ -1176,7 +1177,9 @@ idg_status idg_bind_workspace(idg_ctx *c, void *dev_ptr, size_t bytes)
     // prefetch depth: 8 hyperplanes where shared memory allows (the plan falls
     // back to 4, then 2); the scheduled sweeps' is 4
     k.macro_stages = 8;
-    k.sweep_stages = c->unstr || !idg::sweep_request_fits(k, c->precision == IDG_FP64) ? 4 : 8;
+    k.sweep_stages = 8;
+    c->sweep_depth = c->unstr || !idg::sweep_request_fits(k, c->precision == IDG_FP64) ? 4 : 8;
+    if (c->unstr) k.sweep_stages = 4;
     // float64: the hyperplane-slot kernel (two threads per cell halve each
     // step's float64 chain); float32 storage: one thread per line of cells
     k.macro_kind = c->precision == IDG_FP64 ? 0 : 1;
@@ -1623,6 +1626,7 @@ idg_status idg_set_tuning(idg_ctx *c, int key, int value)
         if (value != 2 && value != 4 && value != 8) return fail(c, IDG_ERR_ARG, "sweep stages must be 2, 4 or 8");
         if (c->unstr && value != 4) return fail(c, IDG_ERR_ARG, "the scheduled sweeps of an unstructured mesh prefetch 4 steps");
         k.sweep_stages = value;
+        k.sweep_tuned |= 4;
     } else if (key == IDG_TUNE_MACRO_STAGES) {
         if (value != 2 && value != 4 && value != 8) return fail(c, IDG_ERR_ARG, "macro stages must be 2, 4 or 8");
         k.macro_stages = value;
@@ -1634,14 +1638,15 @@ idg_status idg_set_tuning(idg_ctx *c, int key, int value)
     } else {
         return fail(c, IDG_ERR_ARG, "unknown tuning key %d", key);
     }
+    if (key != IDG_TUNE_MACRO_STAGES && key != IDG_TUNE_MACRO_KIND && !(k.sweep_tuned & 4)) k.sweep_stages = c->sweep_depth;
     idg::sweep_shape(k, c->precision == IDG_FP64);
     idg::Plan trial{};
     idg::blocks_per_instance(k, trial.nblocks);
     if (key == IDG_TUNE_MACRO_KIND && !idg::plan_shapes(&k, 1, c->precision == IDG_FP64, trial))
         k.macro_stages = trial.macro_stages;
     const bool sweeps = key == IDG_TUNE_SWEEP_TV || key == IDG_TUNE_SWEEP_VPT || key == IDG_TUNE_SWEEP_STAGES;
-    if ((sweeps && !idg::sweep_request_fits(k, c->precision == IDG_FP64)) ||
-        idg::plan_shapes(&k, 1, c->precision == IDG_FP64, trial) || trial.macro_stages != k.macro_stages)
+    if (idg::plan_shapes(&k, 1, c->precision == IDG_FP64, trial) || trial.macro_stages != k.macro_stages ||
+        (sweeps && trial.sweep_stages != k.sweep_stages && !idg::sweep_request_fits(k, c->precision == IDG_FP64)))
         return fail(c, IDG_ERR_ARG, "launch shape does not fit in shared memory");
     KParams old = c->kp;
     c->kp = k;

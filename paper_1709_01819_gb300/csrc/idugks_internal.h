@@ -91,7 +91,7 @@ struct KParams {
     int sweep_tv, sweep_pc, sweep_stages, macro_stages;
     int row_warps;   // warps per cell of k_cell_moments (1, 2, 4)
     int cpb;         // cells per block of the per-(cell, velocity) kernels
-    int sweep_tuned; // set by the caller: 1 sweep_tv, 2 sweep_vpt
+    int sweep_tuned; // set by the caller: 1 sweep_tv, 2 sweep_vpt, 4 sweep_stages
     // the tile that runs (sweep_shape()): threads per cell of a block and
     // velocities per thread; line sweeps: sweep_g of those threads neighbours in
     // one warp, entries of a border ring

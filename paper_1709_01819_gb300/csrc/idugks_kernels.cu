@@ -2755,7 +2755,7 @@ constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory of a block
 // twelve scalars) and two steps' borders.  The line sweeps may need more, lines
 // padded to whole warps and rings; they then take the next shallower depth
 // (plan_shapes), which idg_get_tuning reads back: at two steps every tile fits
-// that is accepted here.
+// that is accepted here.  (Where they need less, what they can run is taken too.)
 bool sweep_request_fits(const KParams &p, bool fp64)
 {
     const size_t T = fp64 ? 8 : 4, w = (size_t)p.sweep_tv * p.sweep_vpt * 2 * T, st = p.sweep_stages;
@@ -2792,7 +2792,7 @@ void sweep_shape(KParams &p, bool fp64, int vpt)
     // fewer, longer strips with less border between them, as far as 512 threads
     // hold the padded lines
     const int g0 = std::min(p.sweep_ktv, std::max(8, 32 / lines));
-    for (int st = p.sweep_tuned ? p.sweep_stages : 2; st >= 2; st /= 2)
+    for (int st = p.sweep_tuned & 3 ? p.sweep_stages : 2; st >= 2; st /= 2)
         for (p.sweep_g = g0; p.sweep_g >= 1 && 16 * p.sweep_g >= p.sweep_ktv; p.sweep_g /= 2)
             for (p.sweep_ring = 32; p.sweep_ring >= 16; p.sweep_ring /= 2)
                 if (sweep_line_bytes(p, fp64, true, st) <= kMaxSmem) return;

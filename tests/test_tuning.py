@@ -42,7 +42,7 @@ def _request_bytes(lines, tv, vpt, stages, prec):
     return lines * (stages * (2 * tile + 9 * T + 16) + 2 * tile)
 
 
-PROBLEMS = {"square": _block(20, 20), "narrow": I.couette(40, U=0.1, Kn=0.1, nv=8), "three": _block(3, 9), "wide": _block(100, 130),
+PROBLEMS = {"square": _block(20, 20), "lines128": _block(128, 128), "narrow": I.couette(40, U=0.1, Kn=0.1, nv=8), "three": _block(3, 9), "wide": _block(100, 130),
             "many_velocities": _block(65, 66, nv=40), "widest": _block(256, 256, nv=4),
             "triangles": I.tri_cavity(6, nv=8, cfl_imp=10.0)}
 
@@ -73,17 +73,16 @@ def test_a_tile_runs_as_asked_or_is_refused(lines, prec):
                     continue
                 s.set_tuning(sweep_stages=2, sweep_tv=1, sweep_vpt=1)
                 ask = dict(sweep_tv=tv, sweep_vpt=vpt, sweep_stages=st)
-                if _request_bytes(lines, tv, vpt, st, prec) > LIMIT:
-                    with pytest.raises(B.IdgError) as e:
-                        s.set_tuning(**ask)
-                    assert e.value.status == B.IDG_ERR_ARG
+                need = _request_bytes(lines, tv, vpt, st, prec)
+                try:
+                    s.set_tuning(**ask)
+                except B.IdgError as e:
+                    assert e.status == B.IDG_ERR_ARG and need > LIMIT
                     continue
-                s.set_tuning(**ask)
                 got = s.tuning()
                 assert (got["sweep_tv"], got["sweep_vpt"]) == (tv, vpt)
-                assert got["sweep_stages"] <= st
-                if got["sweep_stages"] < st:  # only the padding and the rings stand in the way
-                    assert 1.6 * _request_bytes(lines, tv, vpt, st, prec) > LIMIT
+                if got["sweep_stages"] != st:  # only the padding and the rings stand in the way
+                    assert got["sweep_stages"] < st and need <= LIMIT < 1.6 * need
 
 
 def test_a_refused_call_changes_nothing_and_one_key_leaves_the_others():
@@ -103,6 +102,17 @@ def test_a_refused_call_changes_nothing_and_one_key_leaves_the_others():
     assert auto > 1
     m.set_tuning(sweep_tv=2)
     assert m.tuning()["sweep_vpt"] == auto
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("name", ["lines128", "wide", "widest"])
+def test_one_key_is_taken_by_an_untouched_solver(name, prec):
+    """The depth a solver starts with is one its tile can have: nothing has to be
+    set first."""
+    for key in ("sweep_tv", "sweep_vpt"):
+        s = _solver(PROBLEMS[name], prec)
+        s.set_tuning(**{key: 1})
+        assert s.tuning()[key] == 1
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
